@@ -8,9 +8,6 @@ namespace moesched {
 static thread_local int g_last_cuda_error = 0;
 int& last_cuda_error_slot() { return g_last_cuda_error; }
 
-// Shared memory one CTA may request on sm_100a (227 KB).
-constexpr size_t SMEM_LIMIT = 227 * 1024;
-
 Geometry plan_geometry(int N) {
   Geometry ge;
   ge.cpl = N <= 32 ? 1 : N <= 64 ? 2 : N <= 128 ? 4 : 8;

@@ -1,16 +1,17 @@
 // Birkhoff-von Neumann decomposition (paper Sec. 3.1), one warp per demand matrix.
 //
-// The matrix is balanced by north-west-corner padding, then peeled: the support
-// graph (positive entries) is kept as one row-set bit mask per column in
-// registers; after each subtraction only the rows whose matched entry reached
-// zero are re-matched by an augmenting search that disturbs as few low rows as
-// possible, and canonicalise() restores the lexicographically smallest perfect
-// matching over the window of rows whose column changed (rows before the first
-// changed row provably keep theirs; rows after the last one were settled earlier
-// and removing edges cannot unsettle them).
+// The matrix is balanced by north-west-corner padding, then peeled: after each subtraction the rows whose
+// matched entry reached zero are re-matched and the lexicographically smallest perfect matching is restored
+// (Peeler in peel.cuh).
+//
+// What bounds it: a dependent chain of searches, about 900 instructions per matching at N = 64. A full GPU (4096
+// matrices of 64 ranks) issues 2.5 instructions per cycle and SM, 70 % of the integer pipe; with one warp per scheduler
+// or less the time is the chain's latency (3.7 cycles per instruction). Against one row set per column with an
+// OR-reduction per word of every search level, B200: 4096 x N = 64 37.7 -> 27.9 ms, 1024 x N = 128 244 -> 160 ms,
+// 256 x N = 256 1152 -> 408 ms (that was with a CTA of eight warps per matrix), one N = 64 12.9 -> 8.6 ms.
 #include <atomic>
 
-#include "common.cuh"
+#include "peel.cuh"
 
 namespace moesched {
 
@@ -34,135 +35,136 @@ constexpr unsigned PACE_SLACK = 32;     // entries a warp may be ahead before it
 constexpr unsigned PACE_NS_PER_ENTRY = 2000, PACE_NS_MAX = 200000;
 __device__ unsigned long long g_pace[256][64];   // [SM][warp slot] = launch number << 32 | entries left
 
-template <int CPL, int MODE, bool COUNT, bool PACE = false>
-__global__ void __launch_bounds__(128, CPL <= 2 ? 7 : 0) bvn_kernel(int B, int N, int S, const int32_t* __restrict__ demand, int k_max,
+// The north-west-corner fill needs no walk: with the deficits of the rows and of the columns laid end to end along one line, cell (i, j)
+// gets the overlap of row i's stretch and column j's, so a row's cells are found by its own lanes from two prefix
+// sums while the row is copied (the walk, one cell after the other through memory, was most of the set-up).
+template <int W, int MODE, bool COUNT, bool PACE = false>
+__global__ void __launch_bounds__(128, W <= 2 ? 7 : 0) bvn_kernel(int B, int N, int S, const int32_t* __restrict__ demand, int k_max,
                                                   uint8_t* __restrict__ perm, int32_t* __restrict__ coef,
                                                   int32_t* __restrict__ count, int32_t* __restrict__ aug,
                                                   int32_t* scratch, int32_t* __restrict__ status,
                                                   long long* __restrict__ work_out, unsigned pace_launch = 0u) {
-  constexpr int W = CPL;
   constexpr bool CLUSTER = MODE == 1;
-  constexpr bool USE_MEMO = true;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  WarpCtx cx;
-  if constexpr (MODE == 2) cx = warp_prologue_global<CPL>(B, N, S, demand, scratch, smem_raw);
-  else cx = warp_prologue<CPL, CLUSTER>(B, N, S, demand, smem_raw);
-  if (!cx.worker) { cluster_epilogue<CLUSTER>(); return; }
-  const int lane = cx.lane, b = cx.b;
-  const MatView A = cx.M;
-  short* x = cx.x;
-  unsigned* hist = cx.hist;
-  const bool loaded = cx.loaded;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int b = CLUSTER ? (int)(blockIdx.x >> 1) : (int)(blockIdx.x * (blockDim.x >> 5) + warp);
+  if (b >= B) return;   // (a cluster grid has exactly two CTAs per matrix)
+  PeelMatrix<int, CLUSTER> mem;
+  mem.S = S;
+  mem.split = CLUSTER ? (N + 1) / 2 : N;
+  unsigned char* base = smem_raw;
+  if constexpr (MODE == 2) {
+    base += (size_t)warp * peel_smem_bytes(N, W);
+    mem.near_ = mem.far_ = scratch + (size_t)b * N * S;
+  } else {
+    base += (size_t)warp * (peel_smem_bytes(N, W) + align16((size_t)mem.split * S * 4));
+    mem.near_ = mem.far_ = reinterpret_cast<int*>(base + peel_smem_bytes(N, W));
+  }
+  if constexpr (CLUSTER) {
+    mem.far_ = map_to_cta(mem.near_, 1);
+    cluster_sync_all();
+    if (cluster_ctarank() != 0) { cluster_epilogue<true>(); return; }   // lends its shared memory until the end
+  }
 
   unsigned work[MOESCHED_WORK_FIELDS];
 #pragma unroll
   for (int q = 0; q < MOESCHED_WORK_FIELDS; ++q) work[q] = 0u;
 
-  const bool lane_in = lane * CPL < S;
-  int st_code = loaded ? MOESCHED_ST_OK : MOESCHED_ST_INTERNAL;
-  int k = 0;
-
-  // ---- column sums (registers), row sums (one reduction per row), validation ----
-  long long csum[CPL];
+  // ---- row and column sums, validation: lane c of slot s owns row and column s * 32 + c ----
+  const int32_t* D = demand + (size_t)b * N * N;
+  long long csum[W], rsum[W];
 #pragma unroll
-  for (int s = 0; s < CPL; ++s) csum[s] = 0;
-  long long rsum_mine[CPL];   // row sums of the rows lane*CPL+s
-#pragma unroll
-  for (int s = 0; s < CPL; ++s) rsum_mine[s] = 0;
+  for (int s = 0; s < W; ++s) csum[s] = rsum[s] = 0;
   int neg = 0;
-  for (int r = 0; r < N; ++r) {
-    long long part = 0;
-    if (lane_in) {
-      RowVec<CPL> rv = load_cols<CPL>(A.row(r), lane);
 #pragma unroll
-      for (int s = 0; s < CPL; ++s) {
-        if (lane * CPL + s < N) {
-          neg |= rv.v[s] < 0;
-          csum[s] += rv.v[s];
-          part += rv.v[s];
-        }
+  for (int w = 0; w < W; ++w) {
+#pragma unroll 4
+    for (int q = 0; q < 32; ++q) {
+      const int r = w * 32 + q;
+      if (r >= N) break;
+      unsigned lo = 0u, hi = 0u;   // exact row sum from two 32-bit sums: low and high halves of the entries
+#pragma unroll
+      for (int s = 0; s < W; ++s) {
+        const int v = s * 32 + lane < N ? D[(size_t)r * N + s * 32 + lane] : 0;
+        neg |= v < 0;
+        csum[s] += v;
+        lo += (unsigned)v & 0xffffu;
+        hi += (unsigned)v >> 16;
       }
+      lo = __reduce_add_sync(FULL, lo);
+      hi = __reduce_add_sync(FULL, hi);
+      if (lane == q) rsum[w] = ((long long)hi << 16) + lo;
     }
-    // 64-bit warp sum
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(FULL, part, o);
-    if (lane == r / CPL) put<CPL>(rsum_mine, r % CPL, part);
   }
   neg = __any_sync(FULL, neg);
   long long T = 0;
 #pragma unroll
-  for (int s = 0; s < CPL; ++s) T = max(T, max(csum[s], rsum_mine[s]));
+  for (int s = 0; s < W; ++s) T = max(T, max(csum[s], rsum[s]));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) T = max(T, __shfl_xor_sync(FULL, T, o));
-  if (st_code == MOESCHED_ST_OK && (neg || T > 2147483647LL)) st_code = MOESCHED_ST_BAD_INPUT;
+  int st_code = neg || T > 2147483647LL ? MOESCHED_ST_BAD_INPUT : MOESCHED_ST_OK;
+  int k = 0;
 
   if (st_code == MOESCHED_ST_OK) {
-    // ---- north-west-corner fill of the deficits: lowest row first, then lowest column ----
-    // The staircase visits at most 2N-1 cells; row and column deficits are fetched by shuffle.
+    // ---- deficits as stretches of a line: row r covers [rend - its deficit, rend), and the columns likewise ----
+    long long rend[W], cend[W];
     {
-      int i = 0, j = 0;
-      long long a = 0, bb = 0;
-      bool have_a = false, have_b = false;
-      for (int it = 0; it < 4 * N + 4 && i < N && j < N; ++it) {
-        if (!have_a) { a = T - __shfl_sync(FULL, pick<CPL>(rsum_mine, i % CPL), i / CPL); have_a = true; }
-        if (!have_b) { bb = T - __shfl_sync(FULL, pick<CPL>(csum, j % CPL), j / CPL); have_b = true; }
-        if (a == 0) { ++i; have_a = false; continue; }
-        if (bb == 0) { ++j; have_b = false; continue; }
-        const long long e = min(a, bb);
-        if (lane == 0) A.row(i)[j] += (int)e;
-        a -= e;
-        bb -= e;
-      }
-      __syncwarp();
-    }
-    if (aug != nullptr) {
-      int32_t* ao = aug + (size_t)b * N * N;
-      for (int r = 0; r < N; ++r) {
-        const int* rp = A.row(r);
-        for (int c = lane; c < N; c += 32) ao[(size_t)r * N + c] = rp[c];
+      long long rcarry = 0, ccarry = 0;
+#pragma unroll
+      for (int s = 0; s < W; ++s) {
+        const bool in = s * 32 + lane < N;
+        long long r = in ? T - rsum[s] : 0, c = in ? T - csum[s] : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const long long ur = __shfl_up_sync(FULL, r, o), uc = __shfl_up_sync(FULL, c, o);
+          if (lane >= o) { r += ur; c += uc; }
+        }
+        rend[s] = r + rcarry;
+        cend[s] = c + ccarry;
+        rcarry = __shfl_sync(FULL, rend[s], 31);
+        ccarry = __shfl_sync(FULL, cend[s], 31);
       }
     }
 
-    // ---- support graph: C[s] = rows with a positive entry in the lane's column s ----
-    unsigned C[CPL][CPL];
-#pragma unroll
-    for (int s = 0; s < CPL; ++s)
-#pragma unroll
-      for (int w = 0; w < W; ++w) C[s][w] = 0u;
+    // ---- working copy, support graph: row r starts out, nominally, at position r ----
+    Peeler<W, int, CLUSTER> pl;
+    pl.mem = mem;
+    pl.reset(base, N, lane);
     int nnz = 0;
+    {
+      int32_t* ao = aug != nullptr ? aug + (size_t)b * N * N : nullptr;
+      long long r_from = 0;
 #pragma unroll
-    for (int w = 0; w < W; ++w) {
-      for (int q = 0; q < 32; ++q) {
-        const int r = w * 32 + q;
-        if (r >= N) break;
-        if (lane_in) {
-          RowVec<CPL> rv = load_cols<CPL>(A.row(r), lane);
+      for (int w = 0; w < W; ++w) {
+        for (int q = 0; q < 32; ++q) {
+          const int r = w * 32 + q;
+          if (r >= N) break;
+          const long long r_to = __shfl_sync(FULL, rend[w], q);
+          PosEntry<W> e;
+          e.row8 = (unsigned)r << 8;
 #pragma unroll
-          for (int s = 0; s < CPL; ++s)
-            if (lane * CPL + s < N && rv.v[s] > 0) { C[s][w] |= 1u << q; ++nnz; }
+          for (int s = 0; s < W; ++s) {
+            const int c = s * 32 + lane;
+            int v = 0;
+            if (c < N) {
+              v = D[(size_t)r * N + c];
+              const long long more = min(r_to, cend[s]) - max(r_from, cend[s] - (T - csum[s]));
+              if (more > 0) v += (int)more;
+              *mem.cell(r, c) = v;
+              if (ao != nullptr) ao[(size_t)r * N + c] = v;
+            }
+            e.a[s] = __ballot_sync(FULL, v > 0);
+            nnz += __popc(e.a[s]);
+          }
+          pl.seat(r, e);
+          r_from = r_to;
         }
       }
     }
-    nnz = __reduce_add_sync(FULL, nnz);
-
-    Match<CPL> M;
-    M.reset();
-    CanonMemo<CPL> memo;
-    memo.reset();
-    for (int q = lane; q < N * W; q += 32) hist[(N + 1) * W + q] = 0u;   // per-row memo starts empty
-    for (int r = lane; r < N; r += 32) x[r] = -1;
     __syncwarp();
 
     uint8_t* pout = perm + (size_t)b * k_max * N;
     int32_t* cout_ = coef + (size_t)b * k_max;
-    int lo_changed = 0, hi_changed = N - 1;   // window of rows whose column may not be final
-    unsigned freerows[W];   // uniform: rows without a column
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-      const int lo = w * 32;
-      freerows[w] = N >= lo + 32 ? 0xffffffffu : (N <= lo ? 0u : (0xffffffffu >> (lo + 32 - N)));
-    }
-
     unsigned pace_seen = 0u;   // the largest figure seen at the last look
     while (nnz > 0 && k < k_max) {
       if constexpr (PACE) {
@@ -187,99 +189,37 @@ __global__ void __launch_bounds__(128, CPL <= 2 ? 7 : 0) bvn_kernel(int B, int N
           pace_seen = left;
         }
       }
-      // re-match the free rows: a single row that lost its entry is re-matched canonically at once
-      bool okm = true;
-      if (k > 0) {
-        // rows that lost their entry are re-matched canonically, lowest first, as long as that works
-        for (int it = 0; it < N; ++it) {
-          const int r0 = lowest_bit<W>(freerows);
-          if (r0 < 0) break;
-          int single = 0;
-#pragma unroll
-          for (int w = 0; w < W; ++w) single += __popc(freerows[w]);
-          const int rc = canonical_repair<CPL>(N, lane, r0, C, M, x, hist, hi_changed, memo.changed, work, single == 1,
-                                               lo_changed);
-          if (rc < 0) { okm = false; break; }
-          if (rc == 0) { work[WK_BATCH]++; break; }   // needs rows below r0: the general search below takes over
-          clear_bit<W>(freerows, r0);
-          if (rc == 2) { work[WK_BATCH]++; break; }   // rows below r0 had to move: the window starts at the lowest of them
-          work[WK_TIGHT]++;
-          lo_changed = min(lo_changed, r0 + 1);   // row r0 has its final column; the rows that moved lie above it
-        }
-        if (!okm) { st_code = MOESCHED_ST_INTERNAL; break; }
-      }
-      for (int it = 0; it < N; ++it) {
-        const int f = lowest_bit<W>(freerows);
-        if (f < 0) break;
-        if (!augment_from<CPL>(N, lane, f, C, M, x, lo_changed, hi_changed, memo.changed, work)) { okm = false; break; }
-        clear_bit<W>(freerows, f);
-      }
-      if (!okm || any_bit<W>(freerows)) { st_code = MOESCHED_ST_INTERNAL; break; }
-      work[WK_SKIP] += lo_changed;
-      if (!canonicalise<CPL, USE_MEMO>(N, lane, lo_changed, hi_changed, C, M, x, hist, memo, work)) {
-        st_code = MOESCHED_ST_INTERNAL;
-        break;
-      }
+      unsigned lo8 = (unsigned)N << 8;   // rows below lo8 >> 8 have their final column
+      if (!pl.repair(lo8, work)) { st_code = MOESCHED_ST_INTERNAL; break; }
+      if (k == 0) lo8 = 0u;
+      work[WK_SKIP] += lo8 >> 8;
+      pl.canonicalise(lo8, work);
+      pl.fetch_values();
 
-      // coefficient = smallest matched entry; subtract it along the matching
-      int val[CPL], cmin = INF32;
-      int* cell[CPL];   // the lane's matched entries
+      // coefficient = smallest matched entry; subtract it along the matching; what reaches zero leaves the graph
+      int cmin = INF32;
 #pragma unroll
-      for (int s = 0; s < CPL; ++s) {
-        const int c = lane * CPL + s;
-        val[s] = INF32;
-        cell[s] = nullptr;
-        if (c < N) {
-          // with the working copy in global memory every row is "near": no split to test
-          const int mrow = MS_AT(M.mr[s], N);
-          cell[s] = (MODE == 2 ? A.near_ + (size_t)mrow * A.S : A.row(mrow)) + c;
-          val[s] = *cell[s];
-          cmin = min(cmin, val[s]);
-        }
-      }
+      for (int s = 0; s < W; ++s)
+        if (pl.valid(s)) cmin = min(cmin, pl.val[s]);
       cmin = __reduce_min_sync(FULL, cmin);
-      lo_changed = N;
-      hi_changed = -1;
-      unsigned gone[W];
+      unsigned zero = 0u;
 #pragma unroll
-      for (int w = 0; w < W; ++w) gone[w] = 0u;
-      int zeroed = 0;
-#pragma unroll
-      for (int s = 0; s < CPL; ++s) {
-        const int c = lane * CPL + s;
-        if (c < N) {
-          const int nv = val[s] - cmin;
-          *cell[s] = nv;
-          if (nv == 0) {
-#pragma unroll
-            for (int w = 0; w < W; ++w) C[s][w] &= ~M.word(s, w);
-            M.add_to(gone, s);
-            ++zeroed;
-          }
+      for (int s = 0; s < W; ++s) {
+        pl.val[s] -= cmin;
+        if (pl.valid(s)) {
+          if (pl.val[s] == 0) zero |= 1u << s;
+          pout[MS_AT((int)(pl.key[s] >> 8), N)] = (uint8_t)(s * 32 + lane);
         }
       }
-      for (int r = lane; r < N; r += 32) pout[(size_t)k * N + r] = (uint8_t)x[r];
+      nnz -= pl.drop_edges(zero);
       if (lane == 0) cout_[k] = cmin;
+      pout += N;
       ++k;
       work[WK_MATCH]++;
-      nnz -= __reduce_add_sync(FULL, zeroed);
-#pragma unroll
-      for (int w = 0; w < W; ++w) freerows[w] = __reduce_or_sync(FULL, gone[w]);
-      // unmatch the rows whose entry vanished
-      M.release(freerows);
-      // (x[r] was last read, for the permutation row above, by the lane that clears it here; the barrier after the
-      // loop makes the cleared entries visible to the other lanes, whose later updates of x are made by every lane)
-#pragma unroll
-      for (int q = 0; q < W; ++q) {   // lane l looks after rows l, l + 32, ...
-        const int r = q * 32 + lane;
-        if (r < N && ((freerows[q] >> lane) & 1u)) x[r] = -1;
-      }
-      __syncwarp();
     }
     if (st_code == MOESCHED_ST_OK && nnz > 0) st_code = MOESCHED_ST_TRUNCATED;
   }
 
-  if (st_code == MOESCHED_ST_BAD_INPUT) k = 0;
   if constexpr (PACE) {   // this warp no longer counts (it may have moved on without entering the loop)
     unsigned sm, slot;
     asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
@@ -320,19 +260,14 @@ cudaError_t run_bvn(int B, int N, const int32_t* demand, int k_max, uint8_t* per
     return launch_warp_kernel(bvn_kernel<C, M, false>, ge, B, stream, B, N, ge.S, demand, k_max, perm, coef,  \
                               count, aug, scratch, status, work, 0u);                                         \
   } while (0)
-  // Above 128 ranks a batch that leaves most SMs with a single warp goes to the kernel that puts a
-  // CTA of eight warps on each matrix (measured at N = 256, B = 256: 1.0 s against 1.8 s; at N = 128,
-  // B = 1024 one warp per matrix is the faster of the two, 0.32 s against 0.46 s).
-  if (scratch != nullptr && N > 128 && B < 8 * sm_count())
-    return run_bvn_team(B, N, demand, k_max, perm, coef, count, aug, scratch, status, work, stream);
   if (scratch != nullptr) {
-    // working copy in global memory: four matrices per CTA, shared memory only for hist and x
+    // working copy in global memory: shared memory only for the position table and the search levels
     ge.cluster = false;
     ge.S = bvn_scratch_stride(N);
     // four matrices per CTA once there are enough of them to give every SM several CTAs;
     // a small batch is spread one matrix per CTA so that no SM sits idle
     ge.wpb = B >= 16 * sm_count() ? 4 : 1;
-    ge.smem = warp_smem_bytes_global(N, ge.cpl) * ge.wpb;
+    ge.smem = peel_smem_bytes(N, ge.cpl) * ge.wpb;
     // pacing (see PACE above) when every scheduler gets three warps or more and the whole batch is resident at once
     if (work == nullptr && B >= 12 * sm_count()) {
 #define MOESCHED_PACED(C)                                                                                          \
@@ -361,6 +296,13 @@ cudaError_t run_bvn(int B, int N, const int32_t* demand, int k_max, uint8_t* per
       default: MOESCHED_GO(8, 2);
     }
   }
+  // without scratch the matrix is held in shared memory, split over a 2-CTA cluster where one CTA cannot hold it
+  ge.S = N;
+  ge.smem = peel_smem_bytes(N, ge.cpl) + align16((size_t)N * N * 4);
+  ge.cluster = ge.smem > SMEM_LIMIT;
+  if (ge.cluster) ge.smem = peel_smem_bytes(N, ge.cpl) + align16((size_t)((N + 1) / 2) * N * 4);
+  ge.wpb = !ge.cluster && N <= 32 ? 4 : 1;
+  ge.smem *= ge.wpb;
   if (ge.cluster) MOESCHED_GO(8, 1);
   switch (ge.cpl) {
     case 1: MOESCHED_GO(1, 0);

@@ -490,8 +490,7 @@ __device__ __forceinline__ bool load_rows(int* dst, const int32_t* g, int N, int
 }
 
 // ---- per-warp set-up shared by the kernels ----------------------------------------------------
-// Shared memory of one warp: [matrix rows held here][hist: (N+1)*W words of search levels, then N*W
-// words of per-row memo][x: N shorts][mbarrier][flag].
+// Shared memory of one warp: [matrix rows held here][hist: (N+1)*W words of search levels][x: N shorts][mbarrier][flag].
 // In cluster mode the grid has two CTAs (one warp each) per matrix: CTA 0 of the pair
 // works, CTA 1 loads rows [split, N) into its own shared memory and then only keeps
 // them available to CTA 0 (distributed shared memory) until the final cluster barrier.
@@ -506,7 +505,7 @@ struct WarpCtx {
 };
 
 __host__ __device__ inline size_t align16(size_t v) { return (v + 15) & ~(size_t)15; }
-__host__ __device__ inline size_t hist_bytes_for(int N, int W) { return align16((size_t)(2 * N + 1) * W * 4); }
+__host__ __device__ inline size_t hist_bytes_for(int N, int W) { return align16((size_t)(N + 1) * W * 4); }
 __host__ __device__ inline size_t warp_smem_bytes(int N, int S, int W, bool cluster) {
   const int rows_here = cluster ? (N + 1) / 2 : N;
   return align16((size_t)rows_here * S * 4) + hist_bytes_for(N, W) + align16((size_t)N * 2) + 16;
@@ -552,39 +551,6 @@ __device__ __forceinline__ WarpCtx warp_prologue(int B, int N, int S, const int3
     if (cx.b >= B) { cx.worker = false; return cx; }
     cx.loaded = load_rows(mat, demand + (size_t)cx.b * N * N, N, S, 0, N, cx.lane, mbar);
   }
-  return cx;
-}
-
-// Variant with the working copy of the matrix in caller-provided global memory (row stride
-// S ints, one N x S slab per matrix): shared memory then holds only hist and x, so many more
-// warps fit on an SM. Suits kernels that touch the matrix a few times per matching.
-__host__ __device__ inline size_t warp_smem_bytes_global(int N, int W) {
-  return hist_bytes_for(N, W) + align16((size_t)N * 2);
-}
-
-template <int CPL>
-__device__ __forceinline__ WarpCtx warp_prologue_global(int B, int N, int S, const int32_t* demand,
-                                                        int32_t* scratch, unsigned char* smem_raw) {
-  WarpCtx cx;
-  cx.lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
-  const int wpb = blockDim.x >> 5;
-  unsigned char* base = smem_raw + (size_t)warp * warp_smem_bytes_global(N, CPL);
-  cx.hist = reinterpret_cast<unsigned*>(base);
-  cx.x = reinterpret_cast<short*>(base + hist_bytes_for(N, CPL));
-  cx.b = blockIdx.x * wpb + warp;
-  cx.worker = cx.b < B;
-  cx.loaded = true;
-  cx.M.S = S;
-  cx.M.split = N;
-  cx.M.near_ = cx.M.far_ = nullptr;
-  if (!cx.worker) return cx;
-  int* mat = scratch + (size_t)cx.b * N * S;
-  cx.M.near_ = cx.M.far_ = mat;
-  const int32_t* src = demand + (size_t)cx.b * N * N;
-  for (int r = 0; r < N; ++r)
-    for (int c = cx.lane; c < S; c += 32) mat[(size_t)r * S + c] = c < N ? src[(size_t)r * N + c] : 0;
-  __syncwarp();
   return cx;
 }
 
@@ -747,94 +713,6 @@ __device__ __forceinline__ void candidate_rows(int lane, const unsigned (&C)[CPL
   for (int w = 0; w < W; ++w) cand[w] = __reduce_or_sync(FULL, acc[w]) & __reduce_or_sync(FULL, entered[w]);
 }
 
-// Memo carried from one call to the next when the graph only loses edges between calls
-// (Birkhoff): known = rows whose last search found no lower column and whose searched set
-// (the rows that could reach them) is recorded; desc[r] (shared memory, W words per row,
-// after the level history) = rows that have r in their recorded set. Such a row needs no new
-// search until a row of its recorded set changes column: new alternating steps only lead
-// INTO rows that changed, so a row that reaches it through them would have to pass a changed
-// row that already reached it before. changed = rows whose column changed since the last call.
-template <int W>
-struct CanonMemo {
-  // Up to 128 rows the per-row records live in registers: the lane keeps desc of rows
-  // lane, lane+32, ... (word k of a row set, bit `lane`), so collecting and recording are a
-  // few logic operations and one OR-reduction per word. Above that they live in shared memory.
-  static constexpr bool IN_REGS = W <= 4;
-  unsigned known[W];
-  unsigned changed[W];
-  unsigned dreg[IN_REGS ? W : 1][IN_REGS ? W : 1];
-  __device__ __forceinline__ void reset() {
-#pragma unroll
-    for (int w = 0; w < W; ++w) known[w] = changed[w] = 0u;
-    if constexpr (IN_REGS) {
-#pragma unroll
-      for (int k = 0; k < W; ++k)
-#pragma unroll
-        for (int w = 0; w < W; ++w) dreg[k][w] = 0u;
-    }
-  }
-};
-
-// rows recorded as depending on any row of `rows` are added to out; their entries are consumed
-template <int W>
-__device__ __forceinline__ void collect_dependants(int N, int lane, const unsigned (&rows)[W], unsigned* desc,
-                                                   CanonMemo<W>& memo, unsigned (&out)[W]) {
-  if constexpr (CanonMemo<W>::IN_REGS) {
-    unsigned acc[W];
-#pragma unroll
-    for (int w = 0; w < W; ++w) acc[w] = 0u;
-#pragma unroll
-    for (int k = 0; k < W; ++k) {
-      if ((rows[k] >> lane) & 1u) {
-#pragma unroll
-        for (int w = 0; w < W; ++w) { acc[w] |= memo.dreg[k][w]; memo.dreg[k][w] = 0u; }
-      }
-    }
-#pragma unroll
-    for (int w = 0; w < W; ++w) out[w] |= __reduce_or_sync(FULL, acc[w]);
-  } else {
-    unsigned left[W];
-#pragma unroll
-    for (int w = 0; w < W; ++w) left[w] = rows[w];
-    for (int it = 0; it < N; ++it) {
-      const int r = lowest_bit<W>(left);
-      if (r < 0) break;
-      clear_bit<W>(left, r);
-#pragma unroll
-      for (int w = 0; w < W; ++w) out[w] |= desc[MS_AT(r, N) * W + w];
-    }
-    __syncwarp();
-    // lane l clears the entries of the rows l, l+32, ... that were just read
-#pragma unroll
-    for (int k = 0; k < W; ++k) {
-      if ((rows[k] >> lane) & 1u) {
-#pragma unroll
-        for (int w = 0; w < W; ++w) desc[MS_AT(k * 32 + lane, N) * W + w] = 0u;
-      }
-    }
-    __syncwarp();
-  }
-}
-
-// record that row i (one-hot imask) was searched and depends on the rows of anc
-template <int W>
-__device__ __forceinline__ void record_search(int lane, int i, const unsigned (&imask)[W], const unsigned (&anc)[W],
-                                              unsigned* desc, CanonMemo<W>& memo) {
-#pragma unroll
-  for (int k = 0; k < W; ++k) {
-    if ((anc[k] >> lane) & 1u) {
-      if constexpr (CanonMemo<W>::IN_REGS) {
-#pragma unroll
-        for (int w = 0; w < W; ++w) memo.dreg[k][w] |= imask[w];
-      } else {
-        desc[(k * 32 + lane) * W + (i >> 5)] |= 1u << (i & 31);
-      }
-    }
-    memo.known[k] |= imask[k];
-  }
-  if constexpr (!CanonMemo<W>::IN_REGS) __syncwarp();
-}
-
 // One row set of the search history (W words at hist + level * W). The set is uniform and EVERY lane stores
 // it (same address, same value: one shared-memory transaction), so that a lane which reads the history later
 // reads what it wrote itself, in program order: no warp barrier is needed between the store and the loads. The
@@ -865,29 +743,15 @@ __device__ __forceinline__ void hist_load(const unsigned* hist, int level, unsig
   }
 }
 
-template <int CPL, bool MEMO>
+template <int CPL>
 __device__ __forceinline__ bool canonicalise(int N, int lane, int start, int last,
                                              const unsigned (&C)[CPL][CPL], Match<CPL>& M, short* x,
-                                             unsigned* hist, CanonMemo<CPL>& memo,
-                                             unsigned (&work)[MOESCHED_WORK_FIELDS]) {
+                                             unsigned* hist, unsigned (&work)[MOESCHED_WORK_FIELDS]) {
   constexpr int W = CPL;
-  unsigned* desc = hist + (N + 1) * W;
   bool ok_all = true;
-  unsigned cand[W], stale[W];   // stale: rows whose recorded set contains a changed row
-#pragma unroll
-  for (int w = 0; w < W; ++w) stale[w] = 0u;
-  if constexpr (MEMO) {
-    collect_dependants<W>(N, lane, memo.changed, desc, memo, stale);
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-      stale[w] |= memo.changed[w];
-      memo.known[w] &= ~stale[w];    // rows before `start` keep their column but lose their record
-      memo.changed[w] = 0u;
-    }
-  }
+  unsigned cand[W];
   candidate_rows<CPL>(lane, C, M, cand);
-  // rows still to be looked at: those that could move, from `start` up to the last changed row,
-  // not covered by a record that still holds. Rebuilt only after a rotation; otherwise the row just
+  // rows still to be looked at: those that could move, from `start` up to the last changed row. Rebuilt only after a rotation; otherwise the row just
   // searched is simply struck off.
   unsigned todo[W];
   {
@@ -895,11 +759,7 @@ __device__ __forceinline__ bool canonicalise(int N, int lane, int start, int las
     ge_mask<W>(start, lo);
     ge_mask<W>(last + 1, hi);
 #pragma unroll
-    for (int w = 0; w < W; ++w) {
-      unsigned need = cand[w] & lo[w] & ~hi[w];
-      if constexpr (MEMO) need &= ~memo.known[w];
-      todo[w] = need;
-    }
+    for (int w = 0; w < W; ++w) todo[w] = cand[w] & lo[w] & ~hi[w];
   }
   for (int guard = 0; guard < N; ++guard) {
     const int i = lowest_bit<W>(todo);
@@ -925,23 +785,7 @@ __device__ __forceinline__ bool canonicalise(int N, int lane, int start, int las
     int level = 0;
     work[WK_POP]++;   // row i itself
     hist_store<W>(hist, 0, F, lane);
-    // The lowest column below its own that row i is adjacent to and whose row lies above i: no lower column can
-    // be had, so the search stops as soon as that row is reached (the levels up to there are those of the full
-    // search, hence the same rotation). Used where it was measured to pay: in the Birkhoff steps (most
-    // searches there end in a rotation) with one or two columns per lane (N = 64: 38.6 -> 37.4 ms; at N = 128,
-    // and in the greedy steps, where most searches find nothing, finding the target costs more than it saves).
-    constexpr bool EARLY = MEMO && CPL <= 2;
     int jstar = -1, cur = -1, L = 0, sl = 0;   // the column, the row that gives it up, its lane and slot
-    unsigned target[W];
-#pragma unroll
-    for (int w = 0; w < W; ++w) target[w] = 0u;
-    if constexpr (EARLY) {
-      if (lowest_qualifying_column<CPL>(
-              lane, M, [&](int s) { return lane * CPL + s < xi && M.mr[s] > i && intersects<W>(C[s], imask); },
-              jstar, cur, L, sl))
-        onehot_mask<W>(cur, target);
-    }
-    int early = 0;   // level at which the target row was reached
     for (int it = 0; it < N; ++it) {
       unsigned acc[W];
 #pragma unroll
@@ -967,35 +811,23 @@ __device__ __forceinline__ bool canonicalise(int N, int lane, int start, int las
       ++level;
 #pragma unroll
       for (int w = 0; w < W; ++w) work[WK_POP] += __popc(F[w]);
-      if constexpr (EARLY) {
-        if (intersects<W>(F, target)) { early = level; break; }
-      }
       hist_store<W>(hist, level, F, lane);
     }
-    // otherwise: the lowest column row i may take (its own column always qualifies)
-    if (early == 0 &&
-        !lowest_qualifying_column<CPL>(
+    // the lowest column row i may take (its own column always qualifies)
+    if (!lowest_qualifying_column<CPL>(
             lane, M, [&](int s) { return intersects<W>(C[s], imask) && M.in(anc, s); }, jstar, cur, L, sl)) {
       ok_all = false;
       continue;
     }
-    if (jstar == xi) {
-      // record: row i stays put until one of the rows that can reach it changes column
-      if constexpr (MEMO) record_search<W>(lane, i, imask, anc, desc, memo);
-    } else {
+    if (jstar != xi) {
       // level at which that row was reached
-      int lvl = early > 0 ? early : level_of_row<W>(hist, level, MS_AT(cur, N), lane);
+      int lvl = level_of_row<W>(hist, level, MS_AT(cur, N), lane);
       if (lvl == 0) ok_all = false;
-      unsigned moved[W];
-#pragma unroll
-      for (int w = 0; w < W; ++w) moved[w] = imask[w];
       // walk towards row i: each row takes the column of its successor on the cycle
       while (lvl > 0) {
         unsigned Hm[W], cmask[W];
         onehot_mask<W>(cur, cmask);
         hist_load<W>(hist, lvl - 1, Hm);
-#pragma unroll
-        for (int w = 0; w < W; ++w) moved[w] |= cmask[w];
         int c2, nxt, L2, s2;
         if (!lowest_qualifying_column<CPL>(
                 lane, M, [&](int s) { return M.in(Hm, s) && intersects<W>(C[s], cmask); }, c2, nxt, L2, s2)) {
@@ -1011,25 +843,12 @@ __device__ __forceinline__ bool canonicalise(int N, int lane, int start, int las
       }
       if (lane == L) M.assign(sl, i);
       x[MS_AT(i, N)] = (short)jstar;
-      if constexpr (MEMO) {
-        // the moved rows changed column: every record that contains one of them is void
-        unsigned hit[W];
-#pragma unroll
-        for (int w = 0; w < W; ++w) hit[w] = moved[w];
-        collect_dependants<W>(N, lane, moved, desc, memo, hit);
-#pragma unroll
-        for (int w = 0; w < W; ++w) memo.known[w] &= ~hit[w];
-      }
       candidate_rows<CPL>(lane, C, M, cand);
       unsigned lo[W], hi[W];
       ge_mask<W>(i + 1, lo);
       ge_mask<W>(last + 1, hi);
 #pragma unroll
-      for (int w = 0; w < W; ++w) {
-        unsigned need = cand[w] & lo[w] & ~hi[w];
-        if constexpr (MEMO) need &= ~memo.known[w];
-        todo[w] = need;
-      }
+      for (int w = 0; w < W; ++w) todo[w] = cand[w] & lo[w] & ~hi[w];
     }
   }
   return ok_all;
@@ -1124,210 +943,6 @@ __device__ __forceinline__ bool augment_from(int N, int lane, int f, const unsig
   return false;
 }
 
-// ---- repair of a matching that lost an edge, canonical for the row that lost it -------------------------
-// Birkhoff step: the entry (r0, c0) of a lexicographically smallest perfect matching has just vanished, so
-// row r0 and column c0 are free. Rows below r0 keep their columns (they did so with more edges available).
-// The columns that CAN be handed to r0 without touching rows below it are found by one forward search from
-// the free column(s) over the rows above r0: a row adjacent to a column of the previous level could move
-// there and release its own column. r0 takes the lowest such column it is adjacent to -- which is its column
-// in the lexicographically smallest matching of the new graph -- and the rows on the way each move one step
-// towards a free column. (When several entries vanished at once the free rows are handled lowest first; a
-// free row above r0 releases nothing and is simply passed over. Each row's choice is the lowest among the
-// matchings that leave the other free rows out, hence also among the complete ones if the rest can still be
-// matched above it; if not, the caller's general search lowers the window as far as it has to.) This replaces an arbitrary augmenting path followed by a search (and
-// usually a rotation) for row r0. Returns 1 when done (hi = highest row moved, `changed` gets the moved rows),
-// 0 when r0 cannot be re-matched this way (the caller falls back to augment_from), -1 if an iteration limit
-// was hit.
-// With `may_lower` (the caller passes it when r0 is the only free row) the search does not give up when r0 is
-// adjacent to no column that the rows above it can release: it admits the highest row BELOW r0 that is adjacent
-// to a releasable column, continues from that row's column, and repeats until r0 can be served. The path then
-// disturbs as few low rows as possible (as augment_from's does); r0's column is no longer final, `lo` is lowered
-// to the lowest row that moved, and 2 is returned.
-template <int CPL>
-__device__ __forceinline__ int canonical_repair(int N, int lane, int r0, const unsigned (&C)[CPL][CPL], Match<CPL>& M,
-                                                short* x, unsigned* hist, int& hi, unsigned (&changed)[CPL],
-                                                unsigned (&work)[MOESCHED_WORK_FIELDS], bool may_lower, int& lo) {
-  constexpr int W = CPL;
-  unsigned alive[W], r0mask[W];
-  ge_mask<W>(r0 + 1, alive);        // rows above r0 not reached yet
-  onehot_mask<W>(r0, r0mask);
-  unsigned front = 0u;              // bit s: the lane's column s belongs to the current level
-#pragma unroll
-  for (int s = 0; s < CPL; ++s)
-    if (lane * CPL + s < N && M.mr[s] < 0) front |= 1u << s;
-  if (__ballot_sync(FULL, front != 0u) == 0u) return 0;   // no free column: nothing to hand out
-  unsigned freeable = front;        // bit s: column s is free or can be released
-  int level = 0;
-  bool lowered = false;
-  unsigned below[W];                // rows below r0 not admitted yet
-  {
-    unsigned from_r0[W];
-    ge_mask<W>(r0, from_r0);
-#pragma unroll
-    for (int w = 0; w < W; ++w) below[w] = ~from_r0[w];
-  }
-  int c0 = -1, cur = -1, L = 0, sl = 0;   // r0's column, the row that gives it up, its lane and slot
-  // The lowest column r0 is adjacent to that is free or whose row lies above r0: if that row is reached, r0 can
-  // have nothing lower and the search stops there (with one or two columns per lane, where finding it pays).
-  constexpr bool EARLY = CPL <= 2;
-  unsigned target[W];
-#pragma unroll
-  for (int w = 0; w < W; ++w) target[w] = 0u;
-  int early = 0;
-  int tc = -1, trow = -1, tL = 0, tsl = 0;   // that column, its row, lane and slot
-  if constexpr (EARLY) {
-    if (lowest_qualifying_column<CPL>(
-            lane, M,
-            [&](int s) { return lane * CPL + s < N && (M.mr[s] < 0 || M.mr[s] > r0) && intersects<W>(C[s], r0mask); },
-            tc, trow, tL, tsl)) {
-      if (trow >= 0) onehot_mask<W>(trow, target);
-      else early = -1;   // the free column itself: nothing to search
-    }
-  }
-  for (int round = 0; round <= N && early == 0; ++round) {
-    for (int it = 0; it < N; ++it) {
-      unsigned acc[W];
-#pragma unroll
-      for (int w = 0; w < W; ++w) acc[w] = 0u;
-#pragma unroll
-      for (int s = 0; s < CPL; ++s) {
-        if ((front >> s) & 1u) {
-#pragma unroll
-          for (int w = 0; w < W; ++w) acc[w] |= C[s][w];
-        }
-      }
-      unsigned nw[W];
-      bool grew = false;
-#pragma unroll
-      for (int w = 0; w < W; ++w) {
-        nw[w] = __reduce_or_sync(FULL, acc[w]) & alive[w];
-        alive[w] &= ~nw[w];
-        grew |= nw[w] != 0u;
-      }
-      work[WK_SCAN]++;
-      if (!grew) break;
-      ++level;
-      if constexpr (EARLY) {
-        if (intersects<W>(nw, target)) { early = level; break; }
-      }
-      hist_store<W>(hist, level, nw, lane);
-      front = 0u;
-#pragma unroll
-      for (int s = 0; s < CPL; ++s)
-        if (M.mr[s] >= 0 && M.in(nw, s)) front |= 1u << s;
-      freeable |= front;
-    }
-    if (early != 0) break;
-    // otherwise the lowest column that r0 is adjacent to and that can be released
-    if (lowest_qualifying_column<CPL>(
-            lane, M, [&](int s) { return ((freeable >> s) & 1u) && intersects<W>(C[s], r0mask); }, c0, cur, L, sl))
-      break;
-    c0 = -1;
-    if (!may_lower) return 0;
-    // admit the highest row below r0 that could move to a releasable column
-    unsigned acc[W];
-#pragma unroll
-    for (int w = 0; w < W; ++w) acc[w] = 0u;
-#pragma unroll
-    for (int s = 0; s < CPL; ++s) {
-      if ((freeable >> s) & 1u) {
-#pragma unroll
-        for (int w = 0; w < W; ++w) acc[w] |= C[s][w];
-      }
-    }
-    unsigned waiting[W];
-#pragma unroll
-    for (int w = 0; w < W; ++w) waiting[w] = __reduce_or_sync(FULL, acc[w]) & below[w];
-    const int t = highest_bit<W>(waiting);
-    if (t < 0) return 0;
-    clear_bit<W>(below, t);
-    lowered = true;
-    unsigned tmask[W];
-    onehot_mask<W>(t, tmask);
-    ++level;
-    hist_store<W>(hist, level, tmask, lane);
-    front = 0u;
-#pragma unroll
-    for (int s = 0; s < CPL; ++s)
-      if (M.mr[s] >= 0 && M.in(tmask, s)) front |= 1u << s;
-    freeable |= front;
-    work[WK_SCAN]++;
-  }
-  if (early != 0) { c0 = tc; cur = trow; L = tL; sl = tsl; }
-  if (c0 < 0) return -1;
-  if (lane == L) M.assign(sl, r0);
-  x[MS_AT(r0, N)] = (short)c0;   // every lane (see hist_store)
-  set_bit<W>(changed, r0);
-  hi = max(hi, r0);
-  if (cur < 0) return 1;   // r0 took the free column itself
-  int lvl = early > 0 ? early : level_of_row<W>(hist, level, MS_AT(cur, N), lane);
-  if (lvl == 0) return -1;
-  if (lowered) {
-    // An admitted row joined through a column of ANY earlier level, so a row moves to the lowest column it is
-    // adjacent to whose row was reached at an earlier level (or that is free); the levels still fall strictly.
-    lo = min(lo, r0);
-    for (int it = 0; it <= N; ++it) {
-      unsigned cmask[W], Hm[W];
-      onehot_mask<W>(cur, cmask);
-#pragma unroll
-      for (int w = 0; w < W; ++w) Hm[w] = 0u;
-      for (int d = 1; d < lvl; ++d) {
-        unsigned Hd[W];
-        hist_load<W>(hist, d, Hd);
-#pragma unroll
-        for (int w = 0; w < W; ++w) Hm[w] |= Hd[w];
-      }
-      int c2, nxt, L2, s2;
-      if (!lowest_qualifying_column<CPL>(
-              lane, M,
-              [&](int s) {
-                return lane * CPL + s < N && (M.mr[s] < 0 || M.in(Hm, s)) && intersects<W>(C[s], cmask);
-              },
-              c2, nxt, L2, s2))
-        return -1;
-      if (lane == L2) M.assign(s2, cur);
-      x[MS_AT(cur, N)] = (short)c2;
-      set_bit<W>(changed, cur);
-      hi = max(hi, cur);
-      lo = min(lo, cur);
-      work[WK_AUG]++;
-      if (nxt < 0) return 2;   // took the free column
-      cur = nxt;
-      lvl = level_of_row<W>(hist, level, MS_AT(cur, N), lane);
-      if (lvl == 0) return -1;
-    }
-    return -1;
-  }
-  for (int it = 0; it <= N; ++it) {
-    // cur, reached at level lvl, moves to a column of level lvl - 1 (level 0: the free column)
-    unsigned cmask[W];
-    onehot_mask<W>(cur, cmask);
-    int c2, nxt, L2, s2;
-    bool found;
-    if (lvl == 1) {
-      found = lowest_qualifying_column<CPL>(
-          lane, M, [&](int s) { return lane * CPL + s < N && M.mr[s] < 0 && intersects<W>(C[s], cmask); }, c2, nxt,
-          L2, s2);
-    } else {
-      unsigned Hm[W];
-      hist_load<W>(hist, lvl - 1, Hm);
-      found = lowest_qualifying_column<CPL>(
-          lane, M, [&](int s) { return M.in(Hm, s) && intersects<W>(C[s], cmask); }, c2, nxt, L2, s2);
-    }
-    if (!found) return -1;
-    if (lane == L2) M.assign(s2, cur);
-    x[MS_AT(cur, N)] = (short)c2;
-    set_bit<W>(changed, cur);
-    hi = max(hi, cur);
-    work[WK_AUG]++;
-    if (lvl == 1) return 1;
-    if (nxt < 0) return -1;
-    cur = nxt;
-    --lvl;
-  }
-  return -1;
-}
-
 // Time of one expert batch of g tokens (see moesched_model_t).
 __device__ __forceinline__ long long batch_time_ns(const moesched_model_t& m, long long g) {
   if (g <= 0) return 0;
@@ -1367,16 +982,13 @@ struct Geometry {
   size_t smem;   // dynamic shared memory per CTA
 };
 Geometry plan_geometry(int N);
+constexpr size_t SMEM_LIMIT = 227 * 1024;   // shared memory one CTA may request on sm_100a
 int sm_count();   // SMs of the current device (148 on B200), cached per device
 
 cudaError_t run_mw(int B, int N, const int32_t* demand, int k_max, uint8_t* perm, int32_t* dur, int32_t* count,
                    int32_t* residual, int32_t* status, long long* work, cudaStream_t stream);
 cudaError_t run_bvn(int B, int N, const int32_t* demand, int k_max, uint8_t* perm, int32_t* coef, int32_t* count,
                     int32_t* aug, int32_t* scratch, int32_t* status, long long* work, cudaStream_t stream);
-// the same decomposition with one CTA of several warps per matrix (scratch required, 64 < N <= 256)
-cudaError_t run_bvn_team(int B, int N, const int32_t* demand, int k_max, uint8_t* perm, int32_t* coef,
-                         int32_t* count, int32_t* aug, int32_t* scratch, int32_t* status, long long* work,
-                         cudaStream_t stream);
 // row stride (ints) of the global working copy used by the Birkhoff kernel
 inline int bvn_scratch_stride(int N) { return (N + 7) / 8 * 8; }
 cudaError_t run_eval(int B, int N, const int32_t* demand, int k_stride, const uint8_t* perm, const int32_t* dur,

@@ -281,9 +281,7 @@ __global__ void __launch_bounds__(128) mw_kernel(int B, int N, int S, const int3
       // tight edges: row r is tight to column c iff cost(r,c) - v[c] equals the row minimum
       unsigned C[CPL][CPL];
       tight_graph<CPL, View>(R, N, lane, lane_in, st.v, C);
-      CanonMemo<CPL> memo;   // unused: every greedy step has a new graph
-      memo.reset();
-      if (!canonicalise<CPL, false>(N, lane, 0, N - 1, C, st.M, x, hist, memo, work)) {
+      if (!canonicalise<CPL>(N, lane, 0, N - 1, C, st.M, x, hist, work)) {
         st_code = MOESCHED_ST_INTERNAL;
         break;
       }

@@ -119,7 +119,6 @@ __global__ void __launch_bounds__(32 * NW) mw_team_kernel(int B, int N, const in
   }
   sh.x[t] = -1;
   sh.mr[t] = -1;
-  sh.lvl[t] = -1;
 #pragma unroll
   for (int w = 0; w < W; ++w) ms.search.lvl[w][t] = -1;
   red.open();

@@ -1,6 +1,5 @@
 // Building blocks for the kernels in which a TEAM of NW warps (one CTA) owns one demand matrix.
-// They serve batches with too few matrices to fill the SMs with one warp per matrix (N > 128 in
-// the benchmarked configurations). Thread t of the CTA owns row t and column t of the matrix: its
+// They serve batches with too few matrices to fill the SMs with one warp per matrix. Thread t of the CTA owns row t and column t of the matrix: its
 // adjacency to the columns (Rr) and to the rows (Cc) as bit masks of W = NW words in registers, its
 // matched column and row as scalars. Sets of rows or columns that all threads need are built in
 // shared memory with one atomic per member and read back after a CTA barrier; membership that
@@ -87,20 +86,11 @@ struct TeamShared {
   short x[NT];            // row -> column (-1: none)
   short mr[NT];           // column -> row (-1: none)
   short par[NT];          // augmenting search: row from which a column was reached
-  int lvl[NT];            // stamp of the backward-search level at which a row was reached
   unsigned red[3 * TeamRed::SLOT];
   unsigned tot[NW * NW];  // per-warp column sets of the candidate test
   unsigned ri[NW];        // columns adjacent to the row being searched
   int misc[8];
 };
-
-template <int W>
-__device__ __forceinline__ bool meets(const unsigned (&a)[W], const unsigned (&b)[W]) {
-  unsigned o = 0u;
-#pragma unroll
-  for (int w = 0; w < W; ++w) o |= a[w] & b[w];
-  return o != 0u;
-}
 
 // The matching of one team: who is matched to whom, as the owner thread sees it.
 template <int NW>
@@ -148,180 +138,6 @@ __device__ __forceinline__ bool team_is_candidate(TeamShared<NW>& sh, int t, int
   for (int w = 0; w < W; ++w) o |= m.Rr[w] & above[w] & ~ge_word(m.my_x, w);
   return o != 0u;
 }
-
-// Memo carried from one call of team_canonicalise to the next when the graph only loses edges
-// between calls (Birkhoff), the counterpart of CanonMemo in common.cuh spread over the row owners:
-// known = row t's last search found no lower column and none of the rows that could reach it has
-// changed column since; dep = the searched rows whose recorded set contains row t; changed = row
-// t's column changed since the last call.
-template <int NW>
-struct TeamMemo {
-  bool known, changed;
-  unsigned dep[NW];
-  __device__ __forceinline__ void reset() {
-    known = changed = false;
-#pragma unroll
-    for (int w = 0; w < NW; ++w) dep[w] = 0u;
-  }
-};
-
-// One phase: the rows flagged `moved` void every record that contains them (and their own).
-template <int NW>
-__device__ __forceinline__ void team_void_records(TeamRed& red, int t, bool moved, TeamMemo<NW>& memo) {
-  constexpr int W = NW;
-  red.open();
-  if (moved) {
-    unsigned* s = red.cur() + TeamRed::SET;
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-      const unsigned v = memo.dep[w] | onehot_word(t, w);
-      if (v != 0u) atomicOr(&s[w], v);
-      memo.dep[w] = 0u;
-    }
-  }
-  red.close();
-  if ((red.cur()[TeamRed::SET + (t >> 5)] >> (t & 31)) & 1u) memo.known = false;
-  red.next();
-}
-
-// Lexicographically smallest perfect matching of the graph (Rr / Cc) over the window of rows
-// [start, last], given a perfect matching that already equals the answer below `start` (see
-// canonicalise() in common.cuh for the argument; this is the same procedure with the sets spread
-// over the CTA). For each row i that could move: the rows >= i that reach i by alternating steps
-// are found level by level -- a row joins when it is adjacent to the column of a row of the
-// previous level -- then row i takes the lowest adjacent column whose row was reached and the
-// matching is rotated along the cycle. Returns false if an iteration limit was hit. Uniform.
-template <int NW, bool MEMO>
-__device__ __forceinline__ bool team_canonicalise(TeamShared<NW>& sh, TeamRed& red, int N, int t, int lane, int warp,
-                                                  bool in, TeamMatch<NW>& m, TeamMemo<NW>& memo, int& stamp,
-                                                  int start, int last, unsigned (&work)[MOESCHED_WORK_FIELDS]) {
-  constexpr int W = NW;
-  bool ok_all = true;
-  if constexpr (MEMO) {
-    team_void_records<NW>(red, t, memo.changed, memo);
-    memo.changed = false;
-  }
-  bool cand = team_is_candidate<NW>(sh, t, lane, warp, in, m);
-  int from = start;
-  for (int guard = 0; guard < N; ++guard) {
-    // next row that could move
-    red.open();
-    red.min_key(cand && t >= from && t <= last && !(MEMO && memo.known), t, 0, lane);
-    red.close();
-    const unsigned ikey = red.cur()[TeamRed::MIN];
-    red.next();
-    if (ikey == 0xffffffffu) break;
-    const int i = (int)(ikey >> 16);
-    from = i + 1;
-    if (t == 0) { work[WK_SWEEP]++; work[WK_POP]++; }
-    // Every search takes a fresh range of N + 2 level stamps, so that the marks of earlier searches
-    // never need clearing. Before the stamps could pass 2^31 (after some 8 million searches at
-    // N = 256; a complete worst-case decomposition can get there) all marks are wiped and the
-    // stamps start over. stamp is uniform, so every thread takes this branch or none does.
-    if (stamp > 0x7f000000) {
-      __syncthreads();
-      sh.lvl[t] = -1;
-      stamp = 0;
-      __syncthreads();
-    }
-    stamp += N + 2;
-    // level 0: row i itself. Its adjacency is published for the column choice (read several
-    // barriers later; the previous search's readers are past the barrier above).
-    bool in_anc = t == i;
-    if (t == i) {
-      sh.lvl[i] = stamp;
-#pragma unroll
-      for (int w = 0; w < W; ++w) sh.ri[w] = m.Rr[w];
-    }
-    const int xi = sh.x[i];
-    unsigned xf[W];   // columns of the rows of the current level
-#pragma unroll
-    for (int w = 0; w < W; ++w) xf[w] = onehot_word(xi, w);
-    int level = 0;
-    for (int it = 0; it < N; ++it) {
-      red.open();
-      const bool isnew = in && t > i && !in_anc && meets<W>(m.Rr, xf);
-      if (isnew) {
-        in_anc = true;
-        sh.lvl[t] = stamp + level + 1;
-      }
-      red.add_member<W>(isnew, m.my_x, lane);
-      red.close();
-      red.read_set<W>(xf);
-      red.next();
-      if (t == 0) {
-        work[WK_LEVEL]++;
-#pragma unroll
-        for (int w = 0; w < W; ++w) work[WK_POP] += __popc(xf[w]);
-      }
-      if (!any_bit<W>(xf)) break;
-      ++level;
-    }
-    // lowest column row i may take: adjacent to i, its row reached (its own column always qualifies)
-    red.open();
-    {
-      const bool adj = in && ((sh.ri[t >> 5] >> (t & 31)) & 1u);
-      const bool reached = adj && m.my_mr >= 0 && sh.lvl[MS_AT(m.my_mr, N)] >= stamp;
-      red.min_key(reached, t, m.my_mr, lane);
-    }
-    red.close();
-    const unsigned key = red.cur()[TeamRed::MIN];
-    red.next();
-    if (key == 0xffffffffu) { ok_all = false; continue; }
-    const int jstar = MS_AT((int)(key >> 16), N);
-    if (jstar == xi) {
-      // record: row i stays put until one of the rows that can reach it changes column
-      if constexpr (MEMO) {
-        if (in_anc) {
-#pragma unroll
-          for (int w = 0; w < W; ++w) memo.dep[w] |= onehot_word(i, w);
-        }
-        if (t == i) memo.known = true;
-      }
-      continue;
-    }
-    // rotate along the alternating cycle: the row that gives up column jstar takes the column of
-    // its successor towards row i, and so on down the levels
-    int cur = MS_AT((int)(key & 0xffffu), N);
-    int lvl = sh.lvl[cur] - stamp;
-    if (lvl <= 0 || lvl > level) { ok_all = false; continue; }
-    for (int it = 0; it < N && lvl > 0; ++it) {
-      red.open();
-      const bool q = in && m.my_mr >= 0 && sh.lvl[MS_AT(m.my_mr, N)] == stamp + lvl - 1 && test_bit<W>(m.Cc, cur);
-      red.min_key(q, t, m.my_mr, lane);
-      red.close();
-      const unsigned k2 = red.cur()[TeamRed::MIN];
-      red.next();
-      if (k2 == 0xffffffffu) { ok_all = false; break; }
-      const int c2 = MS_AT((int)(k2 >> 16), N), nxt = MS_AT((int)(k2 & 0xffffu), N);
-      if (t == c2) {
-        m.my_mr = cur;
-        sh.mr[c2] = (short)cur;
-        sh.x[cur] = (short)c2;
-      }
-      last = max(last, cur);
-      cur = nxt;
-      --lvl;
-      if (t == 0) work[WK_ROT]++;
-    }
-    if (t == jstar) {
-      m.my_mr = i;
-      sh.mr[jstar] = (short)i;
-      sh.x[i] = (short)jstar;
-    }
-    __syncthreads();
-    {
-      const int nx = sh.x[t];
-      const bool moved = nx != m.my_x;
-      m.my_x = nx;
-      // the moved rows changed column: every record that contains one of them is void
-      if constexpr (MEMO) team_void_records<NW>(red, t, moved, memo);
-    }
-    cand = team_is_candidate<NW>(sh, t, lane, warp, in, m);
-  }
-  return ok_all;
-}
-
 
 // ---- canonicalisation with one search per WARP, several rows searched at once -----------------------
 //
@@ -477,12 +293,7 @@ __device__ __forceinline__ int warp_rotate(TeamShared<NW>& sh, const TeamSearchS
 
 // Lexicographically smallest perfect matching of the graph (ts.cc / ts.rr, m.Rr) over the rows
 // [start, N), given a perfect matching that already equals the answer below `start`; see
-// canonicalise() in common.cuh for the argument. Same result as team_canonicalise. Uniform.
-// (For the Birkhoff kernel, whose windows hold one to three rows that could move, this scheme, with
-// the search records added, was measured slower than team_canonicalise: 1.85 s against 1.06 s on 256
-// matrices of 256 ranks. With nothing to search side by side, one warp working while seven wait is
-// worse than eight warps sharing every level. It serves the greedy kernel, where every step
-// searches the whole matrix.)
+// canonicalise() in common.cuh for the argument. Uniform.
 template <int NW>
 __device__ __forceinline__ bool team_canonicalise_par(TeamShared<NW>& sh, TeamSearchShared<NW>& ts, TeamRed& red, int N,
                                                       int t, int lane, int warp, bool in, TeamMatch<NW>& m, int& stamp,
