@@ -59,16 +59,6 @@ __device__ __forceinline__ unsigned long long as64(const unsigned (&m)[2]) {
   return ((unsigned long long)m[1] << 32) | m[0];
 }
 template <int W>
-__device__ __forceinline__ bool test_bit(const unsigned (&m)[W], int idx) {
-  if constexpr (W == 2) return ((as64(m) >> idx) & 1ull) != 0ull;
-  const unsigned bit = 1u << (idx & 31);
-  const int wi = idx >> 5;
-  unsigned hit = 0u;
-#pragma unroll
-  for (int k = 0; k < W; ++k) hit |= m[k] & (wi == k ? bit : 0u);
-  return hit != 0u;
-}
-template <int W>
 __device__ __forceinline__ void set_bit(unsigned (&m)[W], int idx) {
   if constexpr (W == 2) {
     const unsigned long long b = 1ull << idx;
@@ -101,185 +91,17 @@ __device__ __forceinline__ bool any_bit(const unsigned (&m)[W]) {
   for (int k = 0; k < W; ++k) o |= m[k];
   return o != 0;
 }
-// lowest set bit of a mask, or -1
-template <int W>
-__device__ __forceinline__ int lowest_bit(const unsigned (&m)[W]) {
-  int r = -1;
-#pragma unroll
-  for (int k = W - 1; k >= 0; --k)
-    if (m[k]) r = k * 32 + __ffs(m[k]) - 1;
-  return r;
-}
-// highest set bit of a mask, or -1
-template <int W>
-__device__ __forceinline__ int highest_bit(const unsigned (&m)[W]) {
-  int r = -1;
-#pragma unroll
-  for (int k = 0; k < W; ++k)
-    if (m[k]) r = k * 32 + 31 - __clz(m[k]);
-  return r;
-}
 // word k of the set {t, t+1, ...}
 __device__ __forceinline__ unsigned ge_word(int t, int k) {
   const int lo = k * 32;
   return t <= lo ? 0xffffffffu : (t >= lo + 32 ? 0u : (0xffffffffu << (t - lo)));
 }
-template <int C, typename T>
-__device__ __forceinline__ T pick(const T (&a)[C], int s) {
-  T v = a[0];
-#pragma unroll
-  for (int k = 1; k < C; ++k)
-    if (s == k) v = a[k];
-  return v;
-}
-template <int C, typename T>
-__device__ __forceinline__ void put(T (&a)[C], int s, T v) {
-#pragma unroll
-  for (int k = 0; k < C; ++k)
-    if (s == k) a[k] = v;
-}
-
-// one-hot word w of the set {idx}; empty for idx < 0
-__device__ __forceinline__ unsigned onehot_word(int idx, int w) {
-  return (idx >> 5) == w ? 1u << (idx & 31) : 0u;
-}
-// The one-hot mask of idx (empty for idx < 0) and the set {t, t+1, ...} as whole masks. With two
-// words (33..64 rows, the headline size) a 64-bit shift does both words at once.
-template <int W>
-__device__ __forceinline__ void onehot_mask(int idx, unsigned (&m)[W]) {
-  if constexpr (W == 2) {
-    const unsigned long long b = idx >= 0 ? 1ull << idx : 0ull;
-    m[0] = (unsigned)b;
-    m[1] = (unsigned)(b >> 32);
-  } else {
-#pragma unroll
-    for (int w = 0; w < W; ++w) m[w] = onehot_word(idx, w);
-  }
-}
-template <int W>
-__device__ __forceinline__ void ge_mask(int t, unsigned (&m)[W]) {
-  if constexpr (W == 2) {
-    const unsigned long long b = t >= 64 ? 0ull : (~0ull << (t > 0 ? t : 0));
-    m[0] = (unsigned)b;
-    m[1] = (unsigned)(b >> 32);
-  } else {
-#pragma unroll
-    for (int w = 0; w < W; ++w) m[w] = ge_word(t, w);
-  }
-}
-
 template <int W>
 __device__ __forceinline__ bool intersects(const unsigned (&a)[W], const unsigned (&b)[W]) {
   unsigned o = 0u;
 #pragma unroll
   for (int k = 0; k < W; ++k) o |= a[k] & b[k];
   return o != 0u;
-}
-
-// The matching as the lane sees it: mr[s] = row matched to the lane's column s (-1 = none).
-// For up to 4 columns per lane the row is also kept as a one-hot mask, so that "is my row in
-// this set" is two logic operations instead of a variable shift and select per word.
-template <int CPL>
-struct Match {
-  static constexpr int W = CPL;
-  static constexpr bool CACHED = CPL <= 4;
-  int mr[CPL];
-  unsigned oh[CACHED ? CPL : 1][CACHED ? CPL : 1];
-
-  __device__ __forceinline__ void reset() {
-#pragma unroll
-    for (int s = 0; s < CPL; ++s) mr[s] = -1;
-    if constexpr (CACHED) {
-#pragma unroll
-      for (int s = 0; s < CPL; ++s)
-#pragma unroll
-        for (int w = 0; w < W; ++w) oh[s][w] = 0u;
-    }
-  }
-  __device__ __forceinline__ unsigned word(int s, int w) const {   // s, w compile-time after unrolling
-    if constexpr (CACHED) return oh[s][w];
-    else return onehot_word(mr[s], w);
-  }
-  // slot chosen at run time
-  __device__ __forceinline__ void assign(int slot, int row) {
-    unsigned rowmask[CPL];
-    if constexpr (CACHED) onehot_mask<CPL>(row, rowmask);
-#pragma unroll
-    for (int s = 0; s < CPL; ++s) {
-      const bool me = s == slot;
-      mr[s] = me ? row : mr[s];
-      if constexpr (CACHED) {
-#pragma unroll
-        for (int w = 0; w < W; ++w) oh[s][w] = me ? rowmask[w] : oh[s][w];
-      }
-    }
-  }
-  __device__ __forceinline__ int row_of(int slot) const { return pick<CPL>(mr, slot); }
-  __device__ __forceinline__ bool in(const unsigned (&set)[CPL], int s) const {
-    unsigned o = 0u;
-#pragma unroll
-    for (int w = 0; w < W; ++w) o |= set[w] & word(s, w);
-    return o != 0u;
-  }
-  __device__ __forceinline__ void add_to(unsigned (&set)[CPL], int s) const {
-#pragma unroll
-    for (int w = 0; w < W; ++w) set[w] |= word(s, w);
-  }
-  // unmatch the columns whose row is in `rows`
-  __device__ __forceinline__ void release(const unsigned (&rows)[CPL]) {
-#pragma unroll
-    for (int s = 0; s < CPL; ++s) {
-      if (in(rows, s)) {
-        mr[s] = -1;
-        if constexpr (CACHED) {
-#pragma unroll
-          for (int w = 0; w < W; ++w) oh[s][w] = 0u;
-        }
-      }
-    }
-  }
-};
-
-// The lowest column, over the whole warp, whose slot qualifies (qualifies(s) is asked for every slot s of the
-// lane), with the row matched to it (-1: the column is free), the lane that owns it and its slot there. Returns
-// false when no column qualifies. With one or two columns per lane, column and row travel packed in one word
-// through a single minimum over the warp (the column, in the upper half, decides); with more columns per lane
-// packing every slot costs more than it saves, and the lowest proposing lane is found by a vote and read by
-// shuffles. (Measured on the Birkhoff kernel, N = 64: 40.5 ms packed against 41.9 ms; N = 128: 278 ms packed
-// against 265 ms.)
-template <int CPL, class Q>
-__device__ __forceinline__ bool lowest_qualifying_column(int lane, const Match<CPL>& M, Q qualifies, int& col,
-                                                         int& row, int& owner_lane, int& slot) {
-  if constexpr (CPL <= 2) {
-    unsigned key = 0xffffffffu;
-#pragma unroll
-    for (int ss = 0; ss < CPL; ++ss) {
-      const int s = CPL - 1 - ss;
-      if (qualifies(s)) key = ((unsigned)(lane * CPL + s) << 16) | ((unsigned)M.mr[s] & 0xffffu);
-    }
-    key = __reduce_min_sync(FULL, key);
-    if (key == 0xffffffffu) return false;
-    col = (int)(key >> 16);
-    const int r = (int)(key & 0xffffu);
-    row = r == 0xffff ? -1 : r;
-    owner_lane = col / CPL;
-    slot = col % CPL;
-    return true;
-  } else {
-    int ms = -1;
-#pragma unroll
-    for (int ss = 0; ss < CPL; ++ss) {
-      const int s = CPL - 1 - ss;
-      if (qualifies(s)) ms = s;
-    }
-    const unsigned ball = __ballot_sync(FULL, ms >= 0);
-    if (ball == 0u) return false;
-    owner_lane = __ffs(ball) - 1;
-    slot = __shfl_sync(FULL, ms, owner_lane);
-    col = owner_lane * CPL + slot;
-    row = __shfl_sync(FULL, M.row_of(slot), owner_lane);
-    return true;
-  }
 }
 
 // Level of the search history (levels 1..level, W words each) that contains row r, 0 if none does. Every row
@@ -643,76 +465,6 @@ __device__ __forceinline__ void cluster_epilogue() {
   if constexpr (CLUSTER) cluster_sync_all();
 }
 
-// ---- lexicographically smallest perfect matching -------------------------------------------
-//
-// State: C[s] = set of rows adjacent to the lane's column s in the graph (tight
-// edges for the greedy step, positive entries for Birkhoff), mr[s] = row matched
-// to that column, x[r] = column matched to row r (shared memory, one entry per
-// row). On entry (mr, x) is some perfect matching of the graph. For each row i
-// in order the routine finds the lowest column that row i can take in a perfect
-// matching that keeps rows < i fixed: an edge (i, j) outside the matching is
-// usable iff row mr[j] reaches row i along alternating steps r -> r' (r adjacent
-// to the column of r') among the rows not yet fixed; the matching is then rotated
-// along that cycle. hist holds one row set per search level to retrace the cycle.
-//
-// Only the window [start, last] of rows is visited. The caller guarantees that the
-// matching already equals the answer on rows < start, and that every row > last
-// was settled by an earlier call, with no row >= it re-matched and no edge added
-// since: its search could only find less now, so its column stands. A rotation at
-// row i moves rows above i and widens the window accordingly.
-// Rows i that have, below their own column, a column they are adjacent to whose row lies
-// above i: only those can move to a lower column. Uniform result. With gt(c) = rows matched
-// to a column > c (a suffix OR over the lanes), row i qualifies through column c iff
-// i is adjacent to c, i < mr[c] and i is in gt(c).
-template <int CPL>
-__device__ __forceinline__ void candidate_rows(int lane, const unsigned (&C)[CPL][CPL], const Match<CPL>& M,
-                                               unsigned (&cand)[CPL]) {
-  constexpr int W = CPL;
-  unsigned own[W];
-#pragma unroll
-  for (int w = 0; w < W; ++w) own[w] = 0u;
-#pragma unroll
-  for (int s = 0; s < CPL; ++s) M.add_to(own, s);
-  unsigned above[W];   // rows matched to the columns of higher lanes
-#pragma unroll
-  for (int w = 0; w < W; ++w) {
-    unsigned v = own[w];
-#pragma unroll
-    // (a lane whose source would lie beyond lane 31 gets its own value back: harmless in an OR)
-    for (int o = 1; o < 32; o <<= 1) v |= __shfl_down_sync(FULL, v, o);
-    // v now covers this lane and all higher ones; every row is matched to one column only, so
-    // taking the lane's own rows out leaves exactly the rows of the higher lanes
-    above[w] = v & ~own[w];
-  }
-  // A row can only move if some row above it is adjacent to its own column (the last step of the
-  // alternating cycle back into it): rows without such a neighbour are dropped here, which spares
-  // them a search that would reach nobody.
-  unsigned acc[W], entered[W];
-#pragma unroll
-  for (int w = 0; w < W; ++w) acc[w] = entered[w] = 0u;
-#pragma unroll
-  for (int ss = 0; ss < CPL; ++ss) {
-    const int s = CPL - 1 - ss;   // from the lane's highest column down, growing gt as we go
-    if (M.mr[s] >= 0) {
-      unsigned higher = 0u, gem[W];
-      ge_mask<W>(M.mr[s], gem);
-#pragma unroll
-      for (int w = 0; w < W; ++w) {
-        const unsigned ge = gem[w];
-        acc[w] |= C[s][w] & above[w] & ~ge;
-        higher |= C[s][w] & ge & ~M.word(s, w);
-      }
-      if (higher != 0u) {
-#pragma unroll
-        for (int w = 0; w < W; ++w) entered[w] |= M.word(s, w);
-      }
-    }
-    M.add_to(above, s);
-  }
-#pragma unroll
-  for (int w = 0; w < W; ++w) cand[w] = __reduce_or_sync(FULL, acc[w]) & __reduce_or_sync(FULL, entered[w]);
-}
-
 // One row set of the search history (W words at hist + level * W). The set is uniform and EVERY lane stores
 // it (same address, same value: one shared-memory transaction), so that a lane which reads the history later
 // reads what it wrote itself, in program order: no warp barrier is needed between the store and the loads. The
@@ -741,206 +493,6 @@ __device__ __forceinline__ void hist_load(const unsigned* hist, int level, unsig
 #pragma unroll
     for (int w = 0; w < W; ++w) H[w] = hist[level * W + w];
   }
-}
-
-template <int CPL>
-__device__ __forceinline__ bool canonicalise(int N, int lane, int start, int last,
-                                             const unsigned (&C)[CPL][CPL], Match<CPL>& M, short* x,
-                                             unsigned* hist, unsigned (&work)[MOESCHED_WORK_FIELDS]) {
-  constexpr int W = CPL;
-  bool ok_all = true;
-  unsigned cand[W];
-  candidate_rows<CPL>(lane, C, M, cand);
-  // rows still to be looked at: those that could move, from `start` up to the last changed row. Rebuilt only after a rotation; otherwise the row just
-  // searched is simply struck off.
-  unsigned todo[W];
-  {
-    unsigned lo[W], hi[W];
-    ge_mask<W>(start, lo);
-    ge_mask<W>(last + 1, hi);
-#pragma unroll
-    for (int w = 0; w < W; ++w) todo[w] = cand[w] & lo[w] & ~hi[w];
-  }
-  for (int guard = 0; guard < N; ++guard) {
-    const int i = lowest_bit<W>(todo);
-    if (i < 0) break;
-    const int xi = x[MS_AT(i, N)];
-    work[WK_SWEEP]++;
-    // backward search from row i among the rows >= i; the one-hot mask of i and the set {i, i+1, ...}
-    // come from isolating the lowest bit of todo
-    unsigned anc[W], F[W], alive[W], imask[W];
-    {
-      bool below = true;   // all lower words of todo are empty
-#pragma unroll
-      for (int w = 0; w < W; ++w) {
-        const unsigned lowbit = todo[w] & (0u - todo[w]);
-        const bool here = below && todo[w] != 0u;
-        imask[w] = here ? lowbit : 0u;
-        alive[w] = here ? (0u - lowbit) & ~lowbit : (below ? 0u : 0xffffffffu);   // rows above i
-        below = below && todo[w] == 0u;
-        todo[w] &= ~imask[w];
-        anc[w] = F[w] = imask[w];
-      }
-    }
-    int level = 0;
-    work[WK_POP]++;   // row i itself
-    hist_store<W>(hist, 0, F, lane);
-    int jstar = -1, cur = -1, L = 0, sl = 0;   // the column, the row that gives it up, its lane and slot
-    for (int it = 0; it < N; ++it) {
-      unsigned acc[W];
-#pragma unroll
-      for (int w = 0; w < W; ++w) acc[w] = 0u;
-#pragma unroll
-      for (int s = 0; s < CPL; ++s) {
-        if (M.in(F, s)) {
-#pragma unroll
-          for (int w = 0; w < W; ++w) acc[w] |= C[s][w];
-        }
-      }
-      bool grew = false;
-#pragma unroll
-      for (int w = 0; w < W; ++w) {
-        const unsigned a = __reduce_or_sync(FULL, acc[w]) & alive[w];   // alive: rows >= i not reached yet
-        alive[w] &= ~a;
-        anc[w] |= a;
-        F[w] = a;
-        grew |= a != 0u;
-      }
-      work[WK_LEVEL]++;
-      if (!grew) break;
-      ++level;
-#pragma unroll
-      for (int w = 0; w < W; ++w) work[WK_POP] += __popc(F[w]);
-      hist_store<W>(hist, level, F, lane);
-    }
-    // the lowest column row i may take (its own column always qualifies)
-    if (!lowest_qualifying_column<CPL>(
-            lane, M, [&](int s) { return intersects<W>(C[s], imask) && M.in(anc, s); }, jstar, cur, L, sl)) {
-      ok_all = false;
-      continue;
-    }
-    if (jstar != xi) {
-      // level at which that row was reached
-      int lvl = level_of_row<W>(hist, level, MS_AT(cur, N), lane);
-      if (lvl == 0) ok_all = false;
-      // walk towards row i: each row takes the column of its successor on the cycle
-      while (lvl > 0) {
-        unsigned Hm[W], cmask[W];
-        onehot_mask<W>(cur, cmask);
-        hist_load<W>(hist, lvl - 1, Hm);
-        int c2, nxt, L2, s2;
-        if (!lowest_qualifying_column<CPL>(
-                lane, M, [&](int s) { return M.in(Hm, s) && intersects<W>(C[s], cmask); }, c2, nxt, L2, s2)) {
-          ok_all = false;
-          break;
-        }
-        if (lane == L2) M.assign(s2, cur);
-        x[MS_AT(cur, N)] = (short)c2;   // every lane (see hist_store)
-        last = max(last, cur);
-        cur = nxt;
-        --lvl;
-        work[WK_ROT]++;
-      }
-      if (lane == L) M.assign(sl, i);
-      x[MS_AT(i, N)] = (short)jstar;
-      candidate_rows<CPL>(lane, C, M, cand);
-      unsigned lo[W], hi[W];
-      ge_mask<W>(i + 1, lo);
-      ge_mask<W>(last + 1, hi);
-#pragma unroll
-      for (int w = 0; w < W; ++w) todo[w] = cand[w] & lo[w] & ~hi[w];
-    }
-  }
-  return ok_all;
-}
-
-// ---- augmenting search on a 0/1 graph --------------------------------------------------------
-// Augmenting search from free row f over alternating paths of the graph C (the support graph of
-// the Birkhoff step, the tight edges of a greedy step).
-// Among all augmenting paths it takes one whose lowest row is as high as possible: the
-// search first uses only rows >= t = f and lowers t to the highest waiting row only when
-// it is stuck, so the rows below the returned path keep their columns. [lo, hi] is widened
-// to cover every row whose column changed. Returns false when no augmenting path exists
-// (cannot happen for a balanced matrix).
-template <int CPL>
-__device__ __forceinline__ bool augment_from(int N, int lane, int f, const unsigned (&C)[CPL][CPL], Match<CPL>& M,
-                                             short* x, int& lo, int& hi, unsigned (&changed)[CPL],
-                                             unsigned (&work)[MOESCHED_WORK_FIELDS]) {
-  constexpr int W = CPL;
-  unsigned F[W], P[W];   // frontier rows; rows met but still below the threshold
-#pragma unroll
-  for (int w = 0; w < W; ++w) F[w] = P[w] = 0u;
-  set_bit<W>(F, f);
-  int t = f;
-  unsigned at_or_above[W];   // rows >= t
-  ge_mask<W>(t, at_or_above);
-  unsigned visited = 0u;
-  int par[CPL];
-#pragma unroll
-  for (int s = 0; s < CPL; ++s) par[s] = -1;
-  int jf = -1;
-  for (int it = 0; it < 2 * N + 2; ++it) {
-    unsigned met[W];
-#pragma unroll
-    for (int w = 0; w < W; ++w) met[w] = 0u;
-    int freeslot = -1;
-#pragma unroll
-    for (int ss = 0; ss < CPL; ++ss) {
-      const int s = CPL - 1 - ss;
-      if (!((visited >> s) & 1u)) {
-        unsigned hit[W];
-#pragma unroll
-        for (int w = 0; w < W; ++w) hit[w] = C[s][w] & F[w];
-        if (any_bit<W>(hit)) {
-          visited |= 1u << s;
-          par[s] = lowest_bit<W>(hit);
-          if (M.mr[s] < 0) freeslot = s;
-          else M.add_to(met, s);
-        }
-      }
-    }
-    work[WK_SCAN]++;
-    const unsigned fb = __ballot_sync(FULL, freeslot >= 0);
-    if (fb) {
-      const int L = __ffs(fb) - 1;
-      jf = L * CPL + __shfl_sync(FULL, freeslot, L);
-      break;
-    }
-    bool grew = false;
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-      const unsigned m = __reduce_or_sync(FULL, met[w]);
-      const unsigned ge = at_or_above[w];
-      F[w] = m & ge;
-      P[w] |= m & ~ge;
-      grew |= F[w] != 0u;
-    }
-    if (!grew) {
-      const int r = highest_bit<W>(P);   // admit the highest waiting row, and only that one
-      if (r < 0) return false;
-      t = r;
-      ge_mask<W>(t, at_or_above);
-      clear_bit<W>(P, r);
-      set_bit<W>(F, r);
-    }
-  }
-  if (jf < 0) return false;
-  int j = jf;
-  for (int it = 0; it <= N; ++it) {
-    const int L = j / CPL, sl = j % CPL;
-    const int i = __shfl_sync(FULL, pick<CPL>(par, sl), L);
-    const int jprev = x[MS_AT(i, N)];
-    if (lane == L) M.assign(sl, i);
-    x[MS_AT(i, N)] = (short)j;   // every lane (see hist_store)
-    lo = min(lo, i);
-    hi = max(hi, i);
-    set_bit<W>(changed, i);
-    work[WK_AUG]++;
-    if (i == f) return true;
-    j = jprev;
-    if (j < 0) return false;
-  }
-  return false;
 }
 
 // Time of one expert batch of g tokens (see moesched_model_t).
@@ -1005,10 +557,6 @@ cudaError_t run_best_budget(int B, int k_stride, const int32_t* count, const lon
                             const long long* prefix_unserved, long long price, int32_t* best_k, long long* best_cost,
                             cudaStream_t stream);
 
-// greedy decomposition with one CTA per matrix, for the matrices whose status holds CLASS_U16 (64 < N <= 256)
-cudaError_t run_mw_team(int B, int N, const int32_t* demand, int k_max, uint8_t* perm, int32_t* dur, int32_t* count,
-                        int32_t* residual, int32_t* status, long long* work, cudaStream_t stream);
-
 // scoring with one CTA per matrix, for the matrices whose status holds CLASS_U16 (64 < N <= 256)
 cudaError_t run_eval_team(int B, int N, const int32_t* demand, int k_stride, const uint8_t* perm, const int32_t* dur,
                           const int32_t* count, const moesched_model_t& model, long long* overlap, long long* serial,
@@ -1018,7 +566,6 @@ cudaError_t run_eval_team(int B, int N, const int32_t* demand, int k_stride, con
 // class codes the pre-pass leaves in status[b] (never equal to a final status)
 constexpr int CLASS_U16 = 64;
 constexpr int CLASS_I32 = 65;
-cudaError_t classify_matrices(int B, int N, const int32_t* demand, int32_t* status, cudaStream_t stream);
 
 bool model_in_range(const moesched_model_t& m);
 cudaError_t run_ideal_a2a(int B, int N, const int32_t* demand, const moesched_model_t& model, long long* comm_ns,

@@ -270,6 +270,25 @@ __global__ void __launch_bounds__(128) eval_kernel(int B, int N, int S, const in
   cluster_epilogue<CLUSTER>();
 }
 
+// Matrices are sorted into two classes by a streaming pre-pass that leaves the class in status[b]:
+// all entries within 16 bits (held as 16-bit values: twice as many matrices per SM) or not.
+__global__ void __launch_bounds__(256) classify_kernel(int B, int N, const int32_t* __restrict__ demand,
+                                                          int32_t* __restrict__ status) {
+  const int lane = threadIdx.x & 31;
+  const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (b >= B) return;
+  const int32_t* D = demand + (size_t)b * N * N;
+  int wide = 0;
+  for (int e = lane; e < N * N; e += 32) wide |= (unsigned)D[e] > 65535u;   // negative entries count as wide
+  wide = __any_sync(FULL, wide);
+  if (lane == 0) status[b] = wide ? CLASS_I32 : CLASS_U16;
+}
+
+static cudaError_t classify_matrices(int B, int N, const int32_t* demand, int32_t* status, cudaStream_t stream) {
+  classify_kernel<<<(B + 7) / 8, 256, 0, stream>>>(B, N, demand, status);
+  return cudaGetLastError();
+}
+
 template <int MODE>
 static cudaError_t launch_eval_mode(const Geometry& ge, int B, int N, const int32_t* demand, int k_stride,
                                     const uint8_t* perm, const int32_t* dur, const int32_t* count,

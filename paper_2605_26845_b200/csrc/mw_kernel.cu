@@ -1,315 +1,472 @@
 // Greedy max-weight decomposition (paper Sec. 3.2), one warp per demand matrix.
 //
-// Each greedy step solves one assignment problem on the residual matrix R by
-// shortest augmenting paths on cost = -R (a Jonker-Volgenant style search that
-// keeps only the column duals v, warm-started from the previous step), derives
-// the row duals, marks the tight edges and hands that graph to canonicalise(),
-// which returns the lexicographically smallest optimal permutation. The matched
-// entries are then served whole; the largest one is the matching's duration.
+// Each greedy step solves one assignment problem on the residual matrix R by shortest augmenting paths on
+// cost = -R (a Jonker-Volgenant style search, column duals v warm-started from the previous step), marks the edges that
+// are tight under the optimal duals and hands that graph to the Peeler (peel.cuh), which returns the lexicographically
+// smallest optimal permutation. The matched entries are then served whole; the largest one is the matching's duration.
+//
+// What bounds it: the column scans of the shortest-path searches, one after the other (160 per matching at N = 64), each
+// a chain of a warp minimum, a load of the settled column's row and a relaxation; a full GPU is bound by
+// their instructions. The search therefore holds every candidate as ONE sortable word, distance above "column is
+// matched" above the row (or column) to go on with, wherever distances fit 23 bits: one minimum over the warp then gives the
+// distance, whether the path ends there, and the row to scan next.
 #include <type_traits>
 
-#include "common.cuh"
+#include "peel.cuh"
 
 namespace moesched {
 
-template <int CPL>
-struct MwState {
-  int v[CPL];     // column duals of the cost problem
-  Match<CPL> M;   // row assigned to each of the lane's columns
+// STORE of the residual matrix: 0 int32 in this CTA's shared memory, 1 int32 split over a 2-CTA cluster, 2 16-bit entries.
+template <int STORE>
+struct Residual {
+  using T = typename std::conditional<STORE == 2, unsigned short, int>::type;
+  T* near_;
+  T* far_;
+  int N, split;
+  __device__ __forceinline__ T* row(int r) const {
+    if constexpr (STORE == 1) return r < split ? near_ + r * N : far_ + (r - split) * N;
+    else return near_ + r * N;
+  }
 };
 
-// Tight edges under the column duals v: T[s] = rows whose smallest reduced cost (cost - v over the
-// row) is attained in the lane's column s.
-template <int CPL, typename View>
-__device__ __forceinline__ void tight_graph(const View& R, int N, int lane, bool lane_in, const int (&v)[CPL],
-                                            unsigned (&T)[CPL][CPL]) {
-  constexpr int W = CPL;
+// Shared memory of one warp next to the matrix and the Peeler's: the assignment by rows and columns, predecessors of the
+// running search, and a scratch word per row or column.
+struct AssignShared {
+  int* urow;         // [row] row dual
+  unsigned* claim;   // [row or column]
+  short* x;          // [row] column
+  short* y;          // [column] row
+  short* pred;       // [column] row from which the running search reached it
+};
+__host__ __device__ inline size_t assign_smem_bytes(int N) {
+  return 2 * align16((size_t)N * 4) + 3 * align16((size_t)N * 2);
+}
+__device__ __forceinline__ AssignShared assign_shared(unsigned char* p, int N) {
+  const size_t words = align16((size_t)N * 4), halves = align16((size_t)N * 2);
+  AssignShared a;
+  a.urow = reinterpret_cast<int*>(p);
+  a.claim = reinterpret_cast<unsigned*>(p + words);
+  a.x = reinterpret_cast<short*>(p + 2 * words);
+  a.y = reinterpret_cast<short*>(p + 2 * words + halves);
+  a.pred = reinterpret_cast<short*>(p + 2 * words + 2 * halves);
+  return a;
+}
+
+// A column's tag is its number while it is free and TAG_MATCHED | its row once it is matched, so that free columns win ties
+// and a minimum that carries a tag along names the row to be scanned next. Rows are tagged likewise where columns choose.
+constexpr unsigned TAG_MATCHED = 0x100u;
+constexpr unsigned TAG_MASK = 0x1ffu;
+constexpr int TAG_BITS = 9;
+// Narrow matrices: distances, which lie within 3 C of zero (C the largest entry), and tag fit one word.
+constexpr int NARROW_BIAS = 1 << 22;
+constexpr int NARROW_MAX_ENTRY = NARROW_BIAS / 4;
+constexpr unsigned NONE = 0xffffffffu;
+
+__device__ __forceinline__ unsigned packed(int dist, unsigned tag) { return ((unsigned)(dist + NARROW_BIAS) << TAG_BITS) | tag; }
+__device__ __forceinline__ int packed_dist(unsigned k) { return (int)(k >> TAG_BITS) - NARROW_BIAS; }
+
+// Smallest distance over the warp with the smallest tag among equals, in two steps (wide matrices). INF32: there is none.
+template <int W>
+__device__ __forceinline__ void nearest(const int (&d)[W], const unsigned (&tag)[W], int& dist, unsigned& who) {
+  int m = INF32;
 #pragma unroll
-  for (int s = 0; s < CPL; ++s)
+  for (int s = 0; s < W; ++s) m = min(m, d[s]);
+  dist = __reduce_min_sync(FULL, m);
+  unsigned t = NONE;
 #pragma unroll
-    for (int w = 0; w < W; ++w) T[s][w] = 0u;
+  for (int s = 0; s < W; ++s)
+    if (d[s] == dist) t = min(t, tag[s]);
+  who = __reduce_min_sync(FULL, t);
+}
+
+// One assignment problem. The column duals v carry over from the previous greedy step (weights only decreased, so they
+// are still feasible); they are shifted so that the largest is zero. Every column of the previous optimum was tight for its
+// row, so v lies within [-C, 0], C the largest entry, and row duals (row minima of cost - v) within [-C, 0] too.
+//   1. Rows: each names the column of its smallest reduced cost; a column goes to the lowest row that names it.
+//   2. Columns left free: each raises its dual to the largest feasible value, min over the rows of cost - row dual (within
+//      [-C, C]), where it becomes tight for a row; if that row is free the two are matched. (N = 64 workload: 15 instead of
+//      21 rows left, 161 instead of 225 column scans per matching.)
+//   3. Rows left over are inserted one by one by a shortest-path search that settles one column per scan, free columns
+//      first among equals, and moves the duals of the settled columns.
+// Distances lie within [-2 C, 3 C]. On return sh.x, sh.y and sh.urow hold the assignment and the row duals. False if a
+// search ran out of columns (an inconsistency).
+template <int W, int STORE, bool WIDE>
+__device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N, int lane, const AssignShared& sh,
+                                                 int (&v)[W], unsigned (&work)[MOESCHED_WORK_FIELDS]) {
+  bool in[W];
+  int vmax = -INF32;
+#pragma unroll
+  for (int s = 0; s < W; ++s) {
+    in[s] = s * 32 + lane < N;
+    if (in[s]) vmax = max(vmax, v[s]);
+  }
+  vmax = __reduce_max_sync(FULL, vmax);
+  unsigned tag[W], base[W];   // of the lane's columns; base: packed(-v, tag), so that base - (entry << TAG_BITS) is a key
+#pragma unroll
+  for (int s = 0; s < W; ++s) {
+    v[s] -= vmax;
+    tag[s] = (unsigned)(s * 32 + lane);
+    base[s] = in[s] ? packed(-v[s], tag[s]) : NONE;
+    if (in[s]) sh.claim[s * 32 + lane] = NONE;
+  }
+  // ---- 1. rows name columns; lane l keeps what rows l, l + 32, ... found ----
+  int u[W];
+  unsigned named[W];
 #pragma unroll
   for (int w = 0; w < W; ++w) {
+    unsigned k_mine = 0u;
+    u[w] = 0;
+    named[w] = 0u;
+#pragma unroll 4
     for (int q = 0; q < 32; ++q) {
       const int r = w * 32 + q;
       if (r >= N) break;
-      RowVec<CPL> rv;
-      if (lane_in) rv = load_cols<CPL>(R.row(r), lane);
-      int red[CPL], lm = INF32;
+      const auto* row = R.row(r);
+      if constexpr (WIDE) {
+        int d[W], dist;
+        unsigned who;
 #pragma unroll
-      for (int s = 0; s < CPL; ++s) {
-        red[s] = (lane * CPL + s < N) ? -rv.v[s] - v[s] : INF32;
-        lm = min(lm, red[s]);
+        for (int s = 0; s < W; ++s) d[s] = in[s] ? -(int)row[s * 32 + lane] - v[s] : INF32;
+        nearest<W>(d, tag, dist, who);
+        if (lane == q) { u[w] = dist; named[w] = who; }
+      } else {
+        unsigned k = NONE;
+#pragma unroll
+        for (int s = 0; s < W; ++s) k = min(k, base[s] - ((unsigned)(in[s] ? row[s * 32 + lane] : 0) << TAG_BITS));
+        k = __reduce_min_sync(FULL, k);
+        if (lane == q) k_mine = k;
       }
-      const int u = __reduce_min_sync(FULL, lm);
-#pragma unroll
-      for (int s = 0; s < CPL; ++s)
-        if (red[s] == u && lane * CPL + s < N) T[s][w] |= 1u << q;
+    }
+    if constexpr (!WIDE) {
+      u[w] = packed_dist(k_mine);
+      named[w] = k_mine & 0xffu;
     }
   }
-}
-
-// One assignment problem. The column duals v carry over from the previous greedy step
-// (weights only decreased, so they are still feasible); they are shifted so that the largest
-// is zero, which keeps every intermediate value within a few multiples of the largest entry.
-// Each row first tries the column that minimises cost - v (lowest column on ties) and keeps
-// it if that column is still free: such a row is matched along a tight edge. When at least half
-// of the rows are left over (sparse, tie-rich residuals), each of them is first offered an
-// augmenting path of tight edges, which matches it without touching the duals (measured on the
-// N = 256 configuration: 2.4 k instead of 13 k column scans per matching; with fewer rows left
-// over the searches cost more than they save). The remaining rows are added one by one by a
-// shortest-augmenting-path search that settles one column per scan and updates only the column
-// duals. Returns false if an iteration limit was hit.
-template <int CPL, typename View>
-__device__ __forceinline__ bool solve_assignment(const View& R, int N, int lane, bool lane_in,
-                                                 MwState<CPL>& st, short* x, unsigned (&work)[MOESCHED_WORK_FIELDS]) {
-  constexpr int W = CPL;
-  bool ok = true;
-  {
-    int vmax = -INF32;
-#pragma unroll
-    for (int s = 0; s < CPL; ++s)
-      if (lane * CPL + s < N) vmax = max(vmax, st.v[s]);
-    vmax = __reduce_max_sync(FULL, vmax);
-#pragma unroll
-    for (int s = 0; s < CPL; ++s) st.v[s] -= vmax;
-    st.M.reset();
-  }
-  for (int r = lane; r < N; r += 32) x[r] = -1;
-  unsigned freerows[W];
-#pragma unroll
-  for (int w = 0; w < W; ++w) freerows[w] = 0u;
+  work[WK_TIGHT] += N;
   __syncwarp();
-  for (int r = 0; r < N; ++r) {
-    RowVec<CPL> rv;
-    if (lane_in) rv = load_cols<CPL>(R.row(r), lane);
-    int lmin = INF32, lslot = 0;
 #pragma unroll
-    for (int ss = 0; ss < CPL; ++ss) {
-      const int s = CPL - 1 - ss;
-      const int d = (lane * CPL + s < N) ? -rv.v[s] - st.v[s] : INF32;
-      if (d <= lmin) { lmin = d; lslot = s; }
+  for (int s = 0; s < W; ++s) {
+    if (in[s]) {
+      sh.urow[s * 32 + lane] = u[s];
+      atomicMin(&sh.claim[MS_AT((int)named[s], N)], (unsigned)(s * 32 + lane));
     }
-    const int u = __reduce_min_sync(FULL, lmin);
-    const unsigned ball = __ballot_sync(FULL, lmin == u);
-    const int L = __ffs(ball) - 1;
-    const int sl = __shfl_sync(FULL, lslot, L);
-    const int owner = __shfl_sync(FULL, st.M.row_of(sl), L);
-    if (owner < 0) {
-      if (lane == L) st.M.assign(sl, r);
-      x[r] = (short)(L * CPL + sl);   // every lane: a lane later reads what it wrote itself (see hist_store)
+  }
+  __syncwarp();
+  bool row_free[W];
+  unsigned owner[W];
+#pragma unroll
+  for (int s = 0; s < W; ++s) {
+    row_free[s] = in[s] && sh.claim[MS_AT((int)named[s], N)] != (unsigned)(s * 32 + lane);
+    if (in[s] && !row_free[s]) sh.x[s * 32 + lane] = (short)named[s];
+    owner[s] = in[s] ? sh.claim[s * 32 + lane] : 0u;
+  }
+  __syncwarp();
+  // the rows as the free columns see them: packed(-u, tag of the row), or just the tag
+#pragma unroll
+  for (int s = 0; s < W; ++s) {
+    if (in[s]) {
+      if (owner[s] != NONE) {
+        tag[s] = TAG_MATCHED | owner[s];
+        sh.y[s * 32 + lane] = (short)owner[s];
+      }
+      const unsigned rt = (row_free[s] ? 0u : TAG_MATCHED) | (unsigned)(s * 32 + lane);
+      sh.claim[s * 32 + lane] = WIDE ? rt : packed(-u[s], rt);
+    }
+  }
+  __syncwarp();
+  // ---- 2. free columns raise their duals ----
+  {
+    int best[W];
+    unsigned by[W];
+    if constexpr (WIDE) {
+#pragma unroll
+      for (int s = 0; s < W; ++s) { best[s] = INF32; by[s] = NONE; }
+      for (int i = 0; i < N; ++i) {
+        const auto* row = R.row(i);
+        const int ui = sh.urow[i];
+        const unsigned ti = sh.claim[i];
+#pragma unroll
+        for (int s = 0; s < W; ++s) {
+          const int t = -(int)(in[s] ? row[s * 32 + lane] : 0) - ui;
+          if (t < best[s] || (t == best[s] && ti < by[s])) { best[s] = t; by[s] = ti; }
+        }
+      }
     } else {
-      set_bit<W>(freerows, r);
+      unsigned k[W];
+#pragma unroll
+      for (int s = 0; s < W; ++s) k[s] = NONE;
+#pragma unroll 4
+      for (int i = 0; i < N; ++i) {
+        const auto* row = R.row(i);
+        const unsigned from = sh.claim[i];
+#pragma unroll
+        for (int s = 0; s < W; ++s) k[s] = min(k[s], from - ((unsigned)(in[s] ? row[s * 32 + lane] : 0) << TAG_BITS));
+      }
+#pragma unroll
+      for (int s = 0; s < W; ++s) {
+        best[s] = packed_dist(k[s]);
+        by[s] = k[s] & TAG_MASK;
+      }
     }
-    work[WK_TIGHT]++;
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < W; ++s)
+      if (in[s]) sh.claim[s * 32 + lane] = NONE;
+    __syncwarp();
+    bool asks[W];
+#pragma unroll
+    for (int s = 0; s < W; ++s) {
+      const bool is_free = in[s] && tag[s] < TAG_MATCHED;
+      if (is_free) v[s] = best[s];
+      asks[s] = is_free && by[s] < TAG_MATCHED;
+      if (asks[s]) atomicMin(&sh.claim[MS_AT((int)by[s], N)], (unsigned)(s * 32 + lane));
+    }
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < W; ++s) {
+      if (asks[s] && sh.claim[by[s]] == (unsigned)(s * 32 + lane)) {
+        tag[s] = TAG_MATCHED | by[s];
+        sh.y[s * 32 + lane] = (short)by[s];
+        sh.x[by[s]] = (short)(s * 32 + lane);
+      }
+      if (in[s] && sh.claim[s * 32 + lane] != NONE) row_free[s] = false;
+    }
+  }
+  unsigned left[W];
+#pragma unroll
+  for (int s = 0; s < W; ++s) left[s] = __ballot_sync(FULL, row_free[s]);
+  work[WK_SKIP] += N;   // (rows left over are taken off again below)
+  __syncwarp();
+  // ---- 3. shortest augmenting paths ----
+  while (any_bit<W>(left)) {
+    const int f = first_of<W>(left);
+    clear_bit<W>(left, f);
+    work[WK_SKIP]--;
+    work[WK_AUG]++;
+    int pred[W], settled_at[W], mu;
+    unsigned done = 0u, who;   // done: bit s: the lane's column s is settled; who: tag of the column reached
+#pragma unroll
+    for (int s = 0; s < W; ++s) {
+      pred[s] = f;
+      settled_at[s] = 0;
+    }
+    if constexpr (WIDE) {
+      int d[W];
+      const auto* first = R.row(MS_AT(f, N));
+#pragma unroll
+      for (int s = 0; s < W; ++s) d[s] = in[s] ? -(int)first[s * 32 + lane] - v[s] : INF32;
+      while (true) {   // every scan settles one more column
+        nearest<W>(d, tag, mu, who);
+        work[WK_SCAN]++;
+        if (mu == INF32) return false;
+        if (who < TAG_MATCHED) break;
+        const int i = MS_AT((int)(who & 0xffu), N);
+        const auto* row = R.row(i);
+        const int h = sh.urow[i] - mu;
+#pragma unroll
+        for (int s = 0; s < W; ++s) {
+          if (tag[s] == who) { done |= 1u << s; settled_at[s] = mu; d[s] = INF32; }
+          if (in[s] && !((done >> s) & 1u)) {
+            const int nd = -(int)row[s * 32 + lane] - v[s] - h;
+            if (nd < d[s]) { d[s] = nd; pred[s] = i; }
+          }
+        }
+      }
+    } else {
+      // a settled column's key is all ones from then on: `closed` keeps new keys from undercutting it
+      unsigned key[W], closed[W], k;
+      const auto* first = R.row(MS_AT(f, N));
+#pragma unroll
+      for (int s = 0; s < W; ++s) {
+        closed[s] = in[s] ? 0u : NONE;
+        base[s] = in[s] ? packed(-v[s], tag[s]) : NONE;
+        key[s] = base[s] - ((unsigned)(in[s] ? first[s * 32 + lane] : 0) << TAG_BITS);
+      }
+      while (true) {   // every scan settles one more column
+        k = key[0];
+#pragma unroll
+        for (int s = 1; s < W; ++s) k = min(k, key[s]);
+        k = __reduce_min_sync(FULL, k);
+        work[WK_SCAN]++;
+        if ((k & TAG_MATCHED) == 0u) break;
+        if (k == NONE) return false;
+        const int i = MS_AT((int)(k & 0xffu), N);
+        const auto* row = R.row(i);
+        const unsigned h = (unsigned)(sh.urow[i] - packed_dist(k));
+#pragma unroll
+        for (int s = 0; s < W; ++s) {
+          if (key[s] == k) {   // (rows differ, so only the settled column has this key)
+            settled_at[s] = packed_dist(k);
+            key[s] = closed[s] = NONE;
+          }
+          const unsigned nk = (base[s] - (((unsigned)(in[s] ? row[s * 32 + lane] : 0) + h) << TAG_BITS)) | closed[s];
+          if (nk < key[s]) { key[s] = nk; pred[s] = i; }
+        }
+      }
+      mu = packed_dist(k);
+      who = k & TAG_MASK;
+#pragma unroll
+      for (int s = 0; s < W; ++s) done |= closed[s] & (1u << s);
+    }
+    // settled columns move their dual so that the shortest-path tree stays tight, and their rows' duals with them
+#pragma unroll
+    for (int s = 0; s < W; ++s) {
+      if (in[s]) {
+        if ((done >> s) & 1u) {
+          v[s] += settled_at[s] - mu;
+          sh.urow[tag[s] & 0xffu] += mu - settled_at[s];
+        }
+        sh.pred[s * 32 + lane] = (short)pred[s];
+      }
+    }
+    sh.urow[f] = mu;   // every lane
+    __syncwarp();
+    // flip the path back to row f (every lane makes every update)
+    int j = MS_AT((int)who, N);
+    for (int it = 0; it <= N; ++it) {
+      const int i = MS_AT((int)sh.pred[j], N);
+      const int from = i == f ? j : MS_AT((int)sh.x[i], N);
+      __syncwarp();
+      sh.y[j] = (short)i;
+      sh.x[i] = (short)j;
+      if (i == f) break;
+      j = from;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < W; ++s)
+      if (in[s] && (tag[s] >= TAG_MATCHED || tag[s] == who)) tag[s] = TAG_MATCHED | (unsigned)sh.y[s * 32 + lane];
+  }
+  return true;
+}
+
+// Tight edges under the optimal duals, row by row into the position table: entry (r, c) is tight iff its reduced cost
+// equals the row's dual. One vote per 32 columns gives a row's edges as a set.
+template <int W, int STORE>
+__device__ __forceinline__ void tight_graph(const Residual<STORE>& R, int N, int lane, const AssignShared& sh,
+                                            const int (&v)[W], const PosTable<W>& tab) {
+#pragma unroll 4
+  for (int r = 0; r < N; ++r) {
+    const auto* row = R.row(r);
+    const int ur = sh.urow[r];
+    PosEntry<W> e;
+    e.row8 = (unsigned)r << 8;
+#pragma unroll
+    for (int s = 0; s < W; ++s) {
+      const int c = s * 32 + lane;
+      const int sum = c < N ? (int)row[c] + v[s] + ur : 1;
+      e.a[s] = __ballot_sync(FULL, sum == 0);
+    }
+    tab.store(MS_AT((int)sh.x[r], N), e);
   }
   __syncwarp();
-  {
-    int nfree = 0;
-#pragma unroll
-    for (int w = 0; w < W; ++w) nfree += __popc(freerows[w]);
-    if (2 * nfree >= N) {
-      unsigned T[CPL][CPL];
-      tight_graph<CPL, View>(R, N, lane, lane_in, st.v, T);
-      unsigned left[W];
-#pragma unroll
-      for (int w = 0; w < W; ++w) { left[w] = freerows[w]; freerows[w] = 0u; }
-      unsigned search_work[MOESCHED_WORK_FIELDS], moved[W];   // not reported: the search's own counters
-      int lo = 0, hi = 0;
-      for (int it = 0; it < N; ++it) {
-        const int f = lowest_bit<W>(left);
-        if (f < 0) break;
-        clear_bit<W>(left, f);
-        if (augment_from<CPL>(N, lane, f, T, st.M, x, lo, hi, moved, search_work)) work[WK_SKIP]++;
-        else set_bit<W>(freerows, f);
-      }
-      __syncwarp();
-    }
-  }
-  for (int outer = 0; outer < N; ++outer) {
-    const int f = lowest_bit<W>(freerows);
-    if (f < 0) break;
-    clear_bit<W>(freerows, f);
-    int dist[CPL], pred[CPL];
-    unsigned scanned = 0u;     // bit s: the lane's column s is settled
-    {
-      RowVec<CPL> rv;
-      if (lane_in) rv = load_cols<CPL>(R.row(MS_AT(f, N)), lane);
-#pragma unroll
-      for (int s = 0; s < CPL; ++s) {
-        bool valid = lane * CPL + s < N;
-        dist[s] = valid ? -rv.v[s] - st.v[s] : INF32;
-        pred[s] = f;
-        if (!valid) scanned |= 1u << s;
-      }
-    }
-    int jfin = -1, mu = 0;
-    for (int it = 0; it < N; ++it) {
-      int lmin = INF32, lslot = 0;
-#pragma unroll
-      for (int ss = 0; ss < CPL; ++ss) {
-        const int s = CPL - 1 - ss;
-        int d = ((scanned >> s) & 1u) ? INF32 : dist[s];
-        if (d <= lmin) { lmin = d; lslot = s; }
-      }
-      mu = __reduce_min_sync(FULL, lmin);
-      const unsigned ball = __ballot_sync(FULL, lmin == mu);
-      const int L = __ffs(ball) - 1;
-      const int sl = __shfl_sync(FULL, lslot, L);
-      if (lane == L) scanned |= 1u << sl;
-      const int i = __shfl_sync(FULL, st.M.row_of(sl), L);
-      work[WK_SCAN]++;
-      if (i < 0) { jfin = L * CPL + sl; break; }
-      RowVec<CPL> rv;
-      if (lane_in) rv = load_cols<CPL>(R.row(MS_AT(i, N)), lane);
-      // the owner of the settled column forms h from its own entry and dual: one broadcast instead of two
-      const int h = __shfl_sync(FULL, -pick<CPL>(rv.v, sl) - pick<CPL>(st.v, sl) - mu, L);
-#pragma unroll
-      for (int s = 0; s < CPL; ++s) {
-        int nd = -rv.v[s] - st.v[s] - h;
-        if (!((scanned >> s) & 1u) && nd < dist[s]) { dist[s] = nd; pred[s] = i; }
-      }
-    }
-    if (jfin < 0) { ok = false; break; }
-    // settled columns move their dual so that the new shortest-path tree stays tight
-#pragma unroll
-    for (int s = 0; s < CPL; ++s)
-      if (((scanned >> s) & 1u) && lane * CPL + s < N) st.v[s] += dist[s] - mu;
-    // flip the path back to row f
-    int j = jfin;
-    for (int it = 0; it <= N; ++it) {
-      const int L = j / CPL, sl = j % CPL;
-      const int i = __shfl_sync(FULL, pick<CPL>(pred, sl), L);
-      const int jprev = x[MS_AT(i, N)];
-      if (lane == L) st.M.assign(sl, i);
-      x[MS_AT(i, N)] = (short)j;   // every lane
-      if (i == f) break;
-      j = jprev;
-      if (j < 0) { ok = false; break; }
-    }
-    work[WK_AUG]++;
-  }
-  if (any_bit<W>(freerows)) ok = false;
-  return ok;
 }
 
-// Matrices are sorted into two classes by a streaming pre-pass that leaves the class in status[b]:
-// all entries within 16 bits (held as 16-bit values: twice as many matrices per SM) or not.
-__global__ void __launch_bounds__(256) mw_classify_kernel(int B, int N, const int32_t* __restrict__ demand,
-                                                          int32_t* __restrict__ status) {
-  const int lane = threadIdx.x & 31;
-  const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (b >= B) return;
-  const int32_t* D = demand + (size_t)b * N * N;
-  int wide = 0;
-  for (int e = lane; e < N * N; e += 32) wide |= (unsigned)D[e] > 65535u;   // negative entries count as wide
-  wide = __any_sync(FULL, wide);
-  if (lane == 0) status[b] = wide ? CLASS_I32 : CLASS_U16;
-}
-
-// MODE 0: matrix in this CTA's shared memory as int32; 1: split over a 2-CTA cluster; 2: 16-bit entries.
-// only_class != 0: handle only the matrices whose status[b] holds that class.
+// STORE 2 leaves a matrix with entries beyond 16 bits alone, its status marked CLASS_I32, for a launch with another STORE
+// and only_class set, which handles nothing else.
 // COUNT: the per-matrix work counters are wanted (register increments the compiler drops otherwise).
-template <int CPL, int MODE, bool COUNT>
-__global__ void __launch_bounds__(128) mw_kernel(int B, int N, int S, const int32_t* __restrict__ demand, int k_max,
+template <int W, int STORE, bool COUNT>
+__global__ void __launch_bounds__(128) mw_kernel(int B, int N, const int32_t* __restrict__ demand, int k_max,
                                                  uint8_t* __restrict__ perm, int32_t* __restrict__ dur,
                                                  int32_t* __restrict__ count, int32_t* __restrict__ residual,
                                                  int32_t* status, long long* __restrict__ work_out, int only_class) {
-  constexpr bool CLUSTER = MODE == 1;
+  constexpr bool CLUSTER = STORE == 1;
+  using T = typename Residual<STORE>::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (only_class != 0) {
-    const int bb = CLUSTER ? (int)(blockIdx.x >> 1) : (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
-    if (bb < B && status[bb] != only_class) return;   // both CTAs of a cluster see the same class
-  }
-  using View = typename std::conditional<MODE == 2, MatView16, MatView>::type;
-  View R;
-  int lane, b;
-  short* x;
-  unsigned* hist;
-  bool loaded = true;
-  if constexpr (MODE == 2) {
-    WarpCtx16 cx = warp_prologue16<CPL, false>(B, N, S, demand, smem_raw);
-    if (!cx.worker) return;
-    lane = cx.lane; b = cx.b; R = cx.M; x = cx.x; hist = cx.hist; loaded = cx.loaded;
-  } else {
-    WarpCtx cx = warp_prologue<CPL, CLUSTER>(B, N, S, demand, smem_raw);
-    if (!cx.worker) { cluster_epilogue<CLUSTER>(); return; }
-    lane = cx.lane; b = cx.b; R = cx.M; x = cx.x; hist = cx.hist; loaded = cx.loaded;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int b = CLUSTER ? (int)(blockIdx.x >> 1) : (int)(blockIdx.x * (blockDim.x >> 5) + warp);
+  if (b >= B) return;   // (a cluster grid has exactly two CTAs per matrix)
+  if (only_class != 0 && status[b] != only_class) return;   // both CTAs of a cluster see the same class
+  Residual<STORE> R;
+  R.N = N;
+  R.split = CLUSTER ? (N + 1) / 2 : N;
+  const size_t mat_bytes = align16((size_t)R.split * N * sizeof(T));
+  unsigned char* base = smem_raw + (size_t)warp * (mat_bytes + peel_smem_bytes(N, W) + assign_smem_bytes(N));
+  R.near_ = R.far_ = reinterpret_cast<T*>(base);
+  Peeler<W, int, false> pl;
+  pl.reset(base + mat_bytes, N, lane);
+  const AssignShared sh = assign_shared(base + mat_bytes + peel_smem_bytes(N, W), N);
+  if constexpr (CLUSTER) {
+    R.far_ = reinterpret_cast<T*>(map_to_cta(reinterpret_cast<int*>(R.near_), 1));
+    cluster_sync_all();
+    if (cluster_ctarank() != 0) { cluster_epilogue<true>(); return; }   // lends its shared memory until the end
   }
 
   unsigned work[MOESCHED_WORK_FIELDS];
 #pragma unroll
   for (int q = 0; q < MOESCHED_WORK_FIELDS; ++q) work[q] = 0u;
 
-  const bool lane_in = lane * CPL < S;
-  int st_code = MOESCHED_ST_OK;
-  int k = 0;
-
-  // validate, find the largest entry, count the non-zero entries
-  int nnz = 0;
+  // ---- matrix into shared memory; validate, find the largest entry, count the non-zero entries ----
+  int nnz = 0, mx = 0;
   {
-    int mx = 0, neg = 0, cnt = 0;
-    for (int r = 0; r < N; ++r) {
-      if (lane_in) {
-        RowVec<CPL> rv = load_cols<CPL>(R.row(r), lane);
+    const int32_t* D = demand + (size_t)b * N * N;
+    int neg = 0;
 #pragma unroll
-        for (int s = 0; s < CPL; ++s) {
-          if (lane * CPL + s < N) {
-            neg |= rv.v[s] < 0;
-            mx = max(mx, rv.v[s]);
-            cnt += rv.v[s] != 0;
-          }
+    for (int s = 0; s < W; ++s) {
+      const int c = s * 32 + lane;
+      if (c < N) {
+#pragma unroll 8
+        for (int r = 0; r < N; ++r) {
+          const int val = D[(size_t)r * N + c];
+          neg |= val < 0;
+          mx = max(mx, val);
+          nnz += val != 0;
+          R.row(r)[c] = (T)val;
         }
       }
     }
     neg = __any_sync(FULL, neg);
-    mx = __reduce_max_sync(FULL, mx);
-    nnz = __reduce_add_sync(FULL, cnt);
-    if (neg || mx > MOESCHED_MW_MAX_ENTRY) st_code = MOESCHED_ST_BAD_INPUT;
-    if (!loaded) st_code = MOESCHED_ST_INTERNAL;
+    mx = neg ? INF32 : __reduce_max_sync(FULL, mx);
+    nnz = __reduce_add_sync(FULL, nnz);
+    __syncwarp();
+    if (STORE == 2 && mx > 65535) {
+      if (lane == 0) status[b] = CLASS_I32;
+      return;
+    }
   }
+  int st_code = mx > MOESCHED_MW_MAX_ENTRY ? MOESCHED_ST_BAD_INPUT : MOESCHED_ST_OK;
+  int k = 0;
 
   if (st_code == MOESCHED_ST_OK) {
-    MwState<CPL> st;
+    const bool wide = STORE != 2 && mx > NARROW_MAX_ENTRY;
+    int v[W];
 #pragma unroll
-    for (int s = 0; s < CPL; ++s) st.v[s] = 0;
-    st.M.reset();
+    for (int s = 0; s < W; ++s) v[s] = 0;
     uint8_t* pout = perm + (size_t)b * k_max * N;
     int32_t* dout = dur + (size_t)b * k_max;
     while (k < k_max && nnz > 0) {
-      if (!solve_assignment<CPL, View>(R, N, lane, lane_in, st, x, work)) { st_code = MOESCHED_ST_INTERNAL; break; }
-      // tight edges: row r is tight to column c iff cost(r,c) - v[c] equals the row minimum
-      unsigned C[CPL][CPL];
-      tight_graph<CPL, View>(R, N, lane, lane_in, st.v, C);
-      if (!canonicalise<CPL>(N, lane, 0, N - 1, C, st.M, x, hist, work)) {
-        st_code = MOESCHED_ST_INTERNAL;
-        break;
-      }
+      bool ok;
+      if (wide) ok = solve_assignment<W, STORE, STORE != 2>(R, N, lane, sh, v, work);
+      else ok = solve_assignment<W, STORE, false>(R, N, lane, sh, v, work);
+      if (!ok) { st_code = MOESCHED_ST_INTERNAL; break; }
+      tight_graph<W, STORE>(R, N, lane, sh, v, pl.tab);
+      pl.adopt();
+      pl.canonicalise(0u, work);
       // serve: the heaviest matched pair sets the duration; matched entries are sent whole
       int dmax = 0, served = 0;
 #pragma unroll
-      for (int s = 0; s < CPL; ++s) {
-        const int c = lane * CPL + s;
-        if (c < N && st.M.mr[s] >= 0) {
-          auto* p = R.row(MS_AT(st.M.mr[s], N)) + c;
+      for (int s = 0; s < W; ++s) {
+        if (pl.valid(s)) {
+          const int r = MS_AT((int)(pl.key[s] >> 8), N);
+          T* p = R.row(r) + s * 32 + lane;
           const int val = *p;
           dmax = max(dmax, val);
           served += val != 0;
-          *p = 0;
+          *p = (T)0;
+          pout[r] = (uint8_t)(s * 32 + lane);
         }
       }
       dmax = __reduce_max_sync(FULL, dmax);
       nnz -= __reduce_add_sync(FULL, served);
-      __syncwarp();
-      for (int r = lane; r < N; r += 32) pout[(size_t)k * N + r] = (uint8_t)x[r];
       if (lane == 0) dout[k] = dmax;
+      __syncwarp();
+      pout += N;
       ++k;
       work[WK_MATCH]++;
     }
     if (st_code == MOESCHED_ST_OK && nnz > 0) st_code = MOESCHED_ST_TRUNCATED;
   }
 
-  if (st_code == MOESCHED_ST_BAD_INPUT) k = 0;
   if (lane == 0) {
     count[b] = k;
     status[b] = st_code;
@@ -317,7 +474,7 @@ __global__ void __launch_bounds__(128) mw_kernel(int B, int N, int S, const int3
   if (residual != nullptr && st_code != MOESCHED_ST_BAD_INPUT) {
     int32_t* ro = residual + (size_t)b * N * N;
     for (int r = 0; r < N; ++r) {
-      const auto* rp = R.row(r);
+      const T* rp = R.row(r);
       for (int c = lane; c < N; c += 32) ro[(size_t)r * N + c] = rp[c];
     }
   }
@@ -330,65 +487,55 @@ __global__ void __launch_bounds__(128) mw_kernel(int B, int N, int S, const int3
   cluster_epilogue<CLUSTER>();
 }
 
-cudaError_t classify_matrices(int B, int N, const int32_t* demand, int32_t* status, cudaStream_t stream) {
-  mw_classify_kernel<<<(B + 7) / 8, 256, 0, stream>>>(B, N, demand, status);
-  return cudaGetLastError();
-}
-
 // ---- host side ---------------------------------------------------------------------------
 
-template <int MODE>
-static cudaError_t launch_mw_mode(Geometry ge, int B, int N, const int32_t* demand, int k_max, uint8_t* perm,
-                                  int32_t* dur, int32_t* count, int32_t* residual, int32_t* status, long long* work,
-                                  int only_class, cudaStream_t stream) {
-#define MOESCHED_GO(C)                                                                                         \
-  do {                                                                                                         \
-    if (work != nullptr)                                                                                       \
-      return launch_warp_kernel(mw_kernel<C, MODE, true>, ge, B, stream, B, N, ge.S, demand, k_max, perm, dur, \
-                                count, residual, status, work, only_class);                                    \
-    return launch_warp_kernel(mw_kernel<C, MODE, false>, ge, B, stream, B, N, ge.S, demand, k_max, perm, dur,  \
-                              count, residual, status, work, only_class);                                      \
+static size_t mw_smem_per_warp(int N, int W, int store) {
+  const int rows = store == 1 ? (N + 1) / 2 : N;
+  return align16((size_t)rows * N * (store == 2 ? 2 : 4)) + peel_smem_bytes(N, W) + assign_smem_bytes(N);
+}
+
+template <int STORE>
+static cudaError_t launch_mw(int B, int N, const int32_t* demand, int k_max, uint8_t* perm, int32_t* dur,
+                             int32_t* count, int32_t* residual, int32_t* status, long long* work, int only_class,
+                             cudaStream_t stream) {
+  Geometry ge = plan_geometry(N);
+  ge.cluster = STORE == 1;
+  ge.wpb = STORE == 0 && N <= 32 ? 4 : 1;   // several small matrices share a CTA so that an SM can hold 64 warps
+  ge.smem = mw_smem_per_warp(N, ge.cpl, STORE) * ge.wpb;
+#define MOESCHED_GO(C)                                                                                             \
+  do {                                                                                                             \
+    if (work != nullptr)                                                                                           \
+      return launch_warp_kernel(mw_kernel<C, STORE, true>, ge, B, stream, B, N, demand, k_max, perm, dur, count,   \
+                                residual, status, work, only_class);                                               \
+    return launch_warp_kernel(mw_kernel<C, STORE, false>, ge, B, stream, B, N, demand, k_max, perm, dur, count,    \
+                              residual, status, work, only_class);                                                 \
   } while (0)
-  switch (ge.cpl) {
-    case 1: MOESCHED_GO(1);
-    case 2: MOESCHED_GO(2);
-    case 4: MOESCHED_GO(4);
-    default: MOESCHED_GO(8);
+  if constexpr (STORE == 1) {
+    MOESCHED_GO(8);
+  } else {
+    switch (ge.cpl) {
+      case 1: MOESCHED_GO(1);
+      case 2: MOESCHED_GO(2);
+      case 4: MOESCHED_GO(4);
+      default: MOESCHED_GO(8);
+    }
   }
 #undef MOESCHED_GO
 }
 
-// Batches with fewer matrices per SM than this go to the CTA-per-matrix kernel (N > 64). Measured on a
-// B200: N = 256, B = 256 (1.7 per SM): 294 ms against 613 ms for one warp per matrix; N = 128, B = 1024
-// (6.9 per SM): 91 ms against 63 ms -- with that many matrices per SM the warps of different matrices
-// already fill the issue slots and the CTA's barriers only cost.
-constexpr int MW_TEAM_MAX_PER_SM = 4;
-
 cudaError_t run_mw(int B, int N, const int32_t* demand, int k_max, uint8_t* perm, int32_t* dur, int32_t* count,
                    int32_t* residual, int32_t* status, long long* work, cudaStream_t stream) {
-  const Geometry ge = plan_geometry(N);
-  int only_class = 0;
-  if (N >= 48) {
-    // Shared memory limits how many matrices an SM holds: first the matrices that fit 16-bit entries
-    // (one CTA each at any N), then the rest as int32 (a 2-CTA cluster above N = 232).
-    cudaError_t e = classify_matrices(B, N, demand, status, stream);
-    if (e != cudaSuccess) return e;
-    if (N > 64 && B < MW_TEAM_MAX_PER_SM * sm_count()) {
-      // few large matrices: one CTA per matrix instead of one warp
-      e = run_mw_team(B, N, demand, k_max, perm, dur, count, residual, status, work, stream);
-    } else {
-      Geometry g16 = ge;
-      g16.cluster = false;
-      g16.wpb = 1;
-      g16.smem = warp_smem_bytes16(N, g16.S, g16.cpl);
-      e = launch_mw_mode<2>(g16, B, N, demand, k_max, perm, dur, count, residual, status, work, CLASS_U16, stream);
-    }
-    if (e != cudaSuccess) return e;
-    only_class = CLASS_I32;
-  }
-  if (ge.cluster) return launch_mw_mode<1>(ge, B, N, demand, k_max, perm, dur, count, residual, status, work,
-                                           only_class, stream);
-  return launch_mw_mode<0>(ge, B, N, demand, k_max, perm, dur, count, residual, status, work, only_class, stream);
+  const size_t as_int32 = mw_smem_per_warp(N, plan_geometry(N).cpl, 0);
+  // Shared memory limits how many matrices an SM holds. Where all of them are resident at once as int32 anyway, one launch
+  // takes every matrix; otherwise they are held as 16-bit entries, and a second launch takes those that do not fit (as int32,
+  // over a 2-CTA cluster where one CTA cannot hold the matrix).
+  if (N < 48 || (as_int32 <= SMEM_LIMIT && B <= (long long)sm_count() * (long long)(SMEM_LIMIT / (as_int32 + 1024))))
+    return launch_mw<0>(B, N, demand, k_max, perm, dur, count, residual, status, work, 0, stream);
+  cudaError_t e = launch_mw<2>(B, N, demand, k_max, perm, dur, count, residual, status, work, 0, stream);
+  if (e != cudaSuccess) return e;
+  if (as_int32 > SMEM_LIMIT)
+    return launch_mw<1>(B, N, demand, k_max, perm, dur, count, residual, status, work, CLASS_I32, stream);
+  return launch_mw<0>(B, N, demand, k_max, perm, dur, count, residual, status, work, CLASS_I32, stream);
 }
 
 }  // namespace moesched

@@ -197,6 +197,31 @@ struct Peeler {
     }
   }
 
+  // Takes over a complete matching from the table, as the graph of a new problem: nothing is known about it yet.
+  __device__ __forceinline__ void adopt() {
+    broken_count = 0;
+    const unsigned low = (1u << lane) - 1u;
+#pragma unroll
+    for (int s = 0; s < W; ++s) {
+      key[s] = 0u;
+      chance[s] = IN_VAIN;
+#pragma unroll
+      for (int w = 0; w < W; ++w) A[s][w] = rec[s][w] = 0u;
+      if (valid(s)) {
+        const PosEntry<W> e = tab.load(s * 32 + lane);
+        key[s] = e.row8 | (unsigned)(s * 32 + lane);
+        unsigned lower = e.a[s] & low;
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+          A[s][w] = e.a[w];
+          if (w < s) lower |= e.a[w];
+        }
+        chance[s] = lower != 0u ? UNKNOWN : 0;
+      }
+    }
+    __syncwarp();
+  }
+
   // Row e takes column q (single: the set {q}) from row old8 >> 8: the table, the owner's registers, and the chances of
   // the rows between the two that are adjacent to q and sit above it.
   __device__ __forceinline__ void shift(int q, const unsigned (&single)[W], const PosEntry<W>& e, unsigned old8) {
