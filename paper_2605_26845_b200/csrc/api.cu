@@ -11,17 +11,10 @@ int& last_cuda_error_slot() { return g_last_cuda_error; }
 Geometry plan_geometry(int N) {
   Geometry ge;
   ge.cpl = N <= 32 ? 1 : N <= 64 ? 2 : N <= 128 ? 4 : 8;
-  ge.S = (N + ge.cpl - 1) / ge.cpl * ge.cpl;
+  ge.S = N;
   ge.cluster = false;
-  size_t per_warp = warp_smem_bytes(N, ge.S, ge.cpl, false);
-  if (per_warp > SMEM_LIMIT) {
-    ge.cluster = true;
-    per_warp = warp_smem_bytes(N, ge.S, ge.cpl, true);
-  }
-  // several small matrices share a CTA so that an SM can hold up to 64 warps
   ge.wpb = 1;
-  if (!ge.cluster && N <= 32) ge.wpb = 4;
-  ge.smem = per_warp * ge.wpb;
+  ge.smem = 0;
   return ge;
 }
 
