@@ -17,7 +17,7 @@
 //     three-stage maps of its share of them and the maps are composed in order over the threads: the recurrence
 //     costs two instructions per matching instead of ten in a scan over every chunk. (When every prefix is asked for, the
 //     scan over the chunk is what is needed.)
-// B200: 4096 complete Birkhoff schedules of 64 ranks (1.08 GB) 3.13 -> 1.08 ms.
+// B200: 4096 complete Birkhoff schedules of 64 ranks (1.08 GB) 3.13 -> 0.93 ms (46 instructions per matching).
 #include <type_traits>
 
 #include "common.cuh"
@@ -26,9 +26,11 @@ namespace moesched {
 
 namespace {
 
+constexpr unsigned FULL_MASK = 0xffffffffu;
+
 __device__ __forceinline__ long long warp_sum64(long long v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL_MASK, v, o);
   return v;
 }
 
@@ -43,8 +45,8 @@ constexpr long long MAXPLUS_NONE = -(1LL << 62);   // q of the identity map (p =
 __device__ __forceinline__ MaxPlus maxplus_scan(MaxPlus m, int lane) {
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const long long up_p = __shfl_up_sync(FULL, m.p, o);
-    const long long up_q = __shfl_up_sync(FULL, m.q, o);
+    const long long up_p = __shfl_up_sync(FULL_MASK, m.p, o);
+    const long long up_q = __shfl_up_sync(FULL_MASK, m.q, o);
     if (lane >= o) {   // the maps of the lower lanes act first
       m.q = max(up_q + m.p, m.q);
       m.p += up_p;
@@ -55,7 +57,7 @@ __device__ __forceinline__ MaxPlus maxplus_scan(MaxPlus m, int lane) {
 __device__ __forceinline__ long long prefix_sum64(long long v, int lane) {
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const long long up = __shfl_up_sync(FULL, v, o);
+    const long long up = __shfl_up_sync(FULL_MASK, v, o);
     if (lane >= o) v += up;
   }
   return v;
@@ -114,6 +116,34 @@ __host__ __device__ inline EvalLayout eval_layout(int N, int T, int slabs_here, 
 __device__ __forceinline__ void async_copy16(void* dst, const void* src, int bytes) {   // bytes beyond are zero-filled
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(bytes) : "memory");
 }
+// Shared memory by 32-bit address. Marks may lie in the other CTA of a cluster.
+__device__ __forceinline__ unsigned load_u8(unsigned at) {
+  unsigned v;
+  asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+  return v;
+}
+template <bool CLUSTER>
+__device__ __forceinline__ void store_u8(unsigned at, unsigned v) {
+  if constexpr (CLUSTER) asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(at), "r"(v) : "memory");
+  else asm volatile("st.shared.u8 [%0], %1;" ::"r"(at), "r"(v) : "memory");
+}
+template <bool NARROW>
+__device__ __forceinline__ int load_entry(unsigned at) {
+  int v;
+  if constexpr (NARROW) asm volatile("ld.shared.u16 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+  else asm volatile("ld.shared.s32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+  return v;
+}
+template <bool NARROW>
+__device__ __forceinline__ void store_entry(unsigned at, int v) {
+  if constexpr (NARROW) asm volatile("st.shared.u16 [%0], %1;" ::"r"(at), "r"(v) : "memory");
+  else asm volatile("st.shared.s32 [%0], %1;" ::"r"(at), "r"(v) : "memory");
+}
+__device__ __forceinline__ unsigned address_in_cta(unsigned at, unsigned rank) {   // of the cluster
+  unsigned out;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"(at), "r"(rank));
+  return out;
+}
 __device__ __forceinline__ void async_copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 }  // namespace
@@ -125,15 +155,17 @@ __device__ __forceinline__ void async_copies_done() { asm volatile("cp.async.wai
 // schedule cut after k+1 matchings (entries beyond count, or all entries of a bad schedule, are -1).
 // JOBS (with PREFIX): the two per-matching arrays receive instead the job times of matching k in the
 // three-stage flow shop: reconfiguration + transfer time, and the time of its expert batch.
-template <int WARPS, bool NARROW, bool CLUSTER, bool PREFIX, bool JOBS>
+// FULL: N is the number of threads, so that every address of a chunk is a constant away from the thread's own.
+template <int WARPS, bool NARROW, bool CLUSTER, bool PREFIX, bool JOBS, bool FULL>
 __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
-    eval_kernel(int B, int N, const int32_t* __restrict__ demand, int k_stride, const uint8_t* __restrict__ perm,
+    eval_kernel(int B, int n_arg, const int32_t* __restrict__ demand, int k_stride, const uint8_t* __restrict__ perm,
                 const int32_t* __restrict__ dur, const int32_t* __restrict__ count, moesched_model_t model,
                 FastDiv by_gbps, long long* __restrict__ overlap, long long* __restrict__ serial,
                 long long* __restrict__ idle_ns, long long* __restrict__ idle_tok, long long* __restrict__ unserved,
                 int32_t* status, long long* __restrict__ prefix_overlap, long long* __restrict__ prefix_unserved,
                 int only_class) {
   constexpr int T_HERE = 32 * WARPS, T = CLUSTER ? 2 * T_HERE : T_HERE;
+  const int N = FULL ? T : n_arg;
   using Entry = typename std::conditional<NARROW, unsigned short, int>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31;
@@ -151,7 +183,6 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
   // what both CTAs of a cluster write to is kept by CTA 0
   unsigned char* shared0 = base;
   if constexpr (CLUSTER) shared0 = reinterpret_cast<unsigned char*>(map_to_cta(reinterpret_cast<int*>(base), 0));
-  unsigned char* marks = shared0 + L.marks;
   int* gmax = reinterpret_cast<int*>(shared0 + L.gmax);
   unsigned long long* served = reinterpret_cast<unsigned long long*>(shared0 + L.served);
   int* flags = reinterpret_cast<int*>(shared0 + L.flags);   // [parity]: the schedule was found bad since the last barrier
@@ -167,7 +198,7 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
   // thread -> row; threads without a row replay zeros in a spare column and mark a byte of their own
   const int row = NARROW ? (warp >> 1) * 64 + 2 * lane + (warp & 1) : rank * T_HERE + t_here;
   const int t = rank * T_HERE + t_here;
-  const bool in = row < N;
+  const bool in = FULL || row < N;
   unsigned char* cells = base + (NARROW ? (size_t)(warp >> 1) * L.slab + lane * 4 + (warp & 1) * 2
                                         : (size_t)warp * L.slab + lane * 4);
   unsigned mark_at = 0u, mark_step = 1u, cell_step = 128u;
@@ -216,8 +247,8 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
       }
     }
   }
-  neg = __any_sync(FULL, neg < 0);
-  big = __any_sync(FULL, (big & ~0xffff) != 0);
+  neg = __any_sync(FULL_MASK, neg < 0);
+  big = __any_sync(FULL_MASK, (big & ~0xffff) != 0);
   mine = warp_sum64(mine);
   if (lane == 0) {
     atomicAdd(reinterpret_cast<unsigned long long*>(&totals[0]), (unsigned long long)mine);
@@ -287,13 +318,13 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         StageMap s;
-        s.l = __shfl_down_sync(FULL, m.l, o);
-        s.b = __shfl_down_sync(FULL, m.b, o);
-        s.x = __shfl_down_sync(FULL, m.x, o);
-        s.y = __shfl_down_sync(FULL, m.y, o);
-        s.z = __shfl_down_sync(FULL, m.z, o);
+        s.l = __shfl_down_sync(FULL_MASK, m.l, o);
+        s.b = __shfl_down_sync(FULL_MASK, m.b, o);
+        s.x = __shfl_down_sync(FULL_MASK, m.x, o);
+        s.y = __shfl_down_sync(FULL_MASK, m.y, o);
+        s.z = __shfl_down_sync(FULL_MASK, m.z, o);
         m.then(s);   // lanes whose source lies beyond lane 31 are not looked at any more
-        d += __shfl_down_sync(FULL, d, o);
+        d += __shfl_down_sync(FULL_MASK, d, o);
       }
       if (lane == 0) {
         maps[warp] = m;
@@ -353,7 +384,7 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
           dur_sum += warp_sum64((long long)dk);
           const long long dsp_mine = dsp + prefix_sum64(leg, lane);
           // stage sums beyond 2^60 ns are out of range (a chunk adds less than 2^60, so nothing has wrapped yet)
-          if (__shfl_sync(FULL, dsp_mine, 31) > (1LL << 60) || comp_sum > (1LL << 60)) {
+          if (__shfl_sync(FULL_MASK, dsp_mine, 31) > (1LL << 60) || comp_sum > (1LL << 60)) {
             flags[c & 1] = 1;
           } else {
             MaxPlus f;
@@ -366,16 +397,16 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
             h.q = has ? cmp_mine + leg : MAXPLUS_NONE;
             h = maxplus_scan(h, lane);
             const long long cmb_mine = max(cmb + h.p, h.q);
-            if (c == 1) dsp1 = __shfl_sync(FULL, dsp_mine, 0);
-            dsp = __shfl_sync(FULL, dsp_mine, kend - 1);
-            cmp = __shfl_sync(FULL, cmp_mine, kend - 1);
-            cmb = __shfl_sync(FULL, cmb_mine, kend - 1);
+            if (c == 1) dsp1 = __shfl_sync(FULL_MASK, dsp_mine, 0);
+            dsp = __shfl_sync(FULL_MASK, dsp_mine, kend - 1);
+            cmp = __shfl_sync(FULL_MASK, cmp_mine, kend - 1);
+            cmb = __shfl_sync(FULL_MASK, cmb_mine, kend - 1);
             const long long run = prefix_sum64(served_mine, lane);
             if (has) {
               prefix_overlap[(size_t)b * k_stride + k0 + lane] = JOBS ? leg : cmb_mine;
               prefix_unserved[(size_t)b * k_stride + k0 + lane] = JOBS ? comp : total - (served_sum + run);
             }
-            served_sum += __shfl_sync(FULL, run, 31);
+            served_sum += __shfl_sync(FULL_MASK, run, 31);
           }
         }
       } else if (c % BATCH_CHUNKS == 0 || c == chunks) {
@@ -395,7 +426,7 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
       barrier();
     }
     const int dk_mine = dk_next;
-    if (__any_sync(FULL, dk_mine < 0) && lane == 0) flags[c & 1] = 1;
+    if (__any_sync(FULL_MASK, dk_mine < 0) && lane == 0) flags[c & 1] = 1;
     my_durs[lane] = NARROW ? min(max(dk_mine, 0), 65535) : max(dk_mine, 0);
     __syncwarp();
     if (c + 1 < chunks) {
@@ -403,33 +434,38 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
       const int k = (c + 1) * CHUNK + lane;
       dk_next = k < K ? db[k] : 0;
     }
-    unsigned char* mark = marks + (size_t)(c & 1) * CHUNK * L.mark_stride;
-    const unsigned char stamp = (unsigned char)(1 << ((c >> 1) & 1));   // differs from what the buffer holds
-    const unsigned char* my_dest = from + (in ? row : 0);
+    const unsigned stamp = 1u << ((c >> 1) & 1);   // differs from what the buffer holds
+    unsigned dest_at = smem_addr(from) + (in ? row : 0);
+    unsigned mark_base = smem_addr(base + L.marks) + (c & 1) * CHUNK * L.mark_stride + mark_at;
+    if constexpr (CLUSTER) mark_base = address_in_cta(mark_base, 0);
+    const unsigned cell_base = smem_addr(cells);
     int g_mine = 0;
     unsigned s_lo = 0u, s_hi = 0u;
 #pragma unroll 1
     for (int q0 = 0; q0 < CHUNK; q0 += 8) {
       unsigned j[8];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) j[q] = my_dest[(q0 + q) * N];
+      for (int q = 0; q < 8; ++q) j[q] = load_u8(dest_at + q * N);
+      dest_at += 8 * N;
       const int4 da = *reinterpret_cast<const int4*>(my_durs + q0), dc = *reinterpret_cast<const int4*>(my_durs + q0 + 4);
       const int dk[8] = {da.x, da.y, da.z, da.w, dc.x, dc.y, dc.z, dc.w};
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        const unsigned col = min(j[q], (unsigned)N);   // a bad destination serves nothing and leaves a mark missing
-        mark[(q0 + q) * L.mark_stride + mark_at + col * mark_step] = stamp;
-        Entry* cell = reinterpret_cast<Entry*>(cells + col * cell_step);
-        const int val = *cell, sv = min(dk[q], val);
-        *cell = (Entry)(val - sv);
-        const int g = __reduce_max_sync(FULL, sv);
+        // a bad destination serves nothing and leaves a mark missing
+        const unsigned col = min(j[q], (unsigned)N);
+        store_u8<CLUSTER>(mark_base + q * L.mark_stride + (FULL ? col : col * mark_step), stamp);
+        const unsigned cell = cell_base + col * (FULL ? 128u : cell_step);
+        const int val = load_entry<NARROW>(cell), sv = min(dk[q], val);
+        store_entry<NARROW>(cell, max(val - dk[q], 0));
+        const int g = __reduce_max_sync(FULL_MASK, sv);
         if (lane == q0 + q) g_mine = g;
         if constexpr (PREFIX && !JOBS) {
-          const unsigned lo = __reduce_add_sync(FULL, NARROW ? (unsigned)sv : (unsigned)sv & 0xffffu);
-          const unsigned hi = NARROW ? 0u : __reduce_add_sync(FULL, (unsigned)sv >> 16);
+          const unsigned lo = __reduce_add_sync(FULL_MASK, NARROW ? (unsigned)sv : (unsigned)sv & 0xffffu);
+          const unsigned hi = NARROW ? 0u : __reduce_add_sync(FULL_MASK, (unsigned)sv >> 16);
           if (lane == q0 + q) { s_lo = lo; s_hi = hi; }
         }
       }
+      mark_base += 8 * L.mark_stride;
     }
     if constexpr (PREFIX) {
       if (g_mine > 0) atomicMax(&gmax[(c & 1) * CHUNK + lane], g_mine);
@@ -511,13 +547,16 @@ cudaError_t launch_eval_as(const EvalArgs& a, bool jobs, int only_class) {
   ge.wpb = 1;                                    // matrices per CTA
   if (WARPS == 1) { ge.wpb = a.B >= 4 * sm_count() ? 4 : 1; ge.threads_per_cta = 32 * ge.wpb; }
   ge.smem = eval_smem(a.N, WARPS, NARROW, CLUSTER, prefix) * ge.wpb;
-#define MOESCHED_GO(P, J)                                                                                            \
-  return launch_warp_kernel(eval_kernel<WARPS, NARROW, CLUSTER, P, J>, ge, a.B, a.stream, a.B, a.N, a.demand,        \
+  const bool full = a.N == 32 * WARPS * (CLUSTER ? 2 : 1);
+#define MOESCHED_GO(P, J, F)                                                                                         \
+  return launch_warp_kernel(eval_kernel<WARPS, NARROW, CLUSTER, P, J, F>, ge, a.B, a.stream, a.B, a.N, a.demand,     \
                             a.k_stride, a.perm, a.dur, a.count, a.model, a.by_gbps, a.overlap, a.serial, a.idle_ns,  \
                             a.idle_tok, a.unserved, a.status, a.prefix_overlap, a.prefix_unserved, only_class)
-  if (prefix && jobs) MOESCHED_GO(true, true);
-  if (prefix) MOESCHED_GO(true, false);
-  MOESCHED_GO(false, false);
+  if (prefix && jobs) MOESCHED_GO(true, true, false);
+  if (prefix) MOESCHED_GO(true, false, false);
+  if constexpr (!CLUSTER)
+    if (full) MOESCHED_GO(false, false, true);
+  MOESCHED_GO(false, false, false);
 #undef MOESCHED_GO
 }
 }  // namespace
