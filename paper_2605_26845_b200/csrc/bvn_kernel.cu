@@ -7,10 +7,10 @@
 // What bounds it: a dependent chain of searches, about 900 instructions per matching at N = 64. A full GPU (4096
 // matrices of 64 ranks) issues 2.5 instructions per cycle and SM, 70 % of the integer pipe; with one warp per scheduler
 // or less the time is the chain's latency (3.7 cycles per instruction). Against one row set per column with an
-// OR-reduction per word of every search level, B200: 4096 x N = 64 37.7 -> 27.9 ms, 1024 x N = 128 244 -> 160 ms,
-// 256 x N = 256 1152 -> 408 ms (that was with a CTA of eight warps per matrix), one N = 64 12.9 -> 8.6 ms.
-#include <atomic>
-
+// OR-reduction per word of every search level, B200: 4096 x N = 64 37.7 -> 27.3 ms, 1024 x N = 128 244 -> 150 ms,
+// 256 x N = 256 1152 -> 690 ms (that was with a CTA of eight warps per matrix), one N = 64 12.9 -> 8.3 ms.
+// (Warps that slept while they were ahead of the others on their scheduler gained 4 % when a matching took 1700
+// instructions; now a full GPU takes 27.3 ms without and 27.4 ms with it.)
 #include "peel.cuh"
 
 namespace moesched {
@@ -20,30 +20,16 @@ namespace moesched {
 // COUNT: the per-matrix work counters are wanted (they are plain register increments that the
 // compiler drops, registers included, when nothing reads them).
 //
-// PACE. The warp schedulers of an SM serve their resident warps in a fixed order of preference. With several
-// equally long decompositions per scheduler the preferred warps run at full speed and finish early, and the
-// others are left to finish alone, each stalled on its own dependent chain with most issue slots empty
-// (measured, N = 64, B = 4096, all warps resident from the start: the warps in the first four slots of an SM
-// finish after 22.7 ms, those in the last four after 39.3 ms). When the whole batch is resident at once the
-// launcher therefore switches pacing on: every warp publishes, every PACE_EVERY matchings, how many entries its
-// matrix has left, reads the figures of the warps that share its scheduler (warp slot modulo 4), and sleeps for a
-// moment when it is well ahead of the slowest of them. The slots go to the warps behind and all finish together
-// (40.5 -> 38.9 ms). A sleep is a plain delay, never a wait for another warp: results and termination do not
-// depend on it. Entries carry the launch's number, so figures left by another launch are ignored.
-constexpr int PACE_EVERY = 16;          // matchings between two looks (a power of two)
-constexpr unsigned PACE_SLACK = 32;     // entries a warp may be ahead before it sleeps
-constexpr unsigned PACE_NS_PER_ENTRY = 2000, PACE_NS_MAX = 200000;
-__device__ unsigned long long g_pace[256][64];   // [SM][warp slot] = launch number << 32 | entries left
-
-// The north-west-corner fill needs no walk: with the deficits of the rows and of the columns laid end to end along one line, cell (i, j)
-// gets the overlap of row i's stretch and column j's, so a row's cells are found by its own lanes from two prefix
-// sums while the row is copied (the walk, one cell after the other through memory, was most of the set-up).
-template <int W, int MODE, bool COUNT, bool PACE = false>
+// The north-west-corner fill needs no walk: with the deficits of the rows and of the columns laid end to end along one
+// line, cell (i, j) gets the overlap of row i's stretch and column j's, so a row's cells are found by its own lanes
+// from two prefix sums while the row is copied (the walk, one cell after the other through memory, was most of the
+// set-up).
+template <int W, int MODE, bool COUNT>
 __global__ void __launch_bounds__(128, W <= 2 ? 7 : 0) bvn_kernel(int B, int N, int S, const int32_t* __restrict__ demand, int k_max,
                                                   uint8_t* __restrict__ perm, int32_t* __restrict__ coef,
                                                   int32_t* __restrict__ count, int32_t* __restrict__ aug,
                                                   int32_t* scratch, int32_t* __restrict__ status,
-                                                  long long* __restrict__ work_out, unsigned pace_launch = 0u) {
+                                                  long long* __restrict__ work_out) {
   constexpr bool CLUSTER = MODE == 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -165,30 +151,7 @@ __global__ void __launch_bounds__(128, W <= 2 ? 7 : 0) bvn_kernel(int B, int N, 
 
     uint8_t* pout = perm + (size_t)b * k_max * N;
     int32_t* cout_ = coef + (size_t)b * k_max;
-    unsigned pace_seen = 0u;   // the largest figure seen at the last look
     while (nnz > 0 && k < k_max) {
-      if constexpr (PACE) {
-        if ((k & (PACE_EVERY - 1)) == 0) {
-          unsigned pace_sm, pace_slot;   // read afresh every time rather than kept in registers across the loop
-          asm volatile("mov.u32 %0, %%smid;" : "=r"(pace_sm));
-          asm volatile("mov.u32 %0, %%warpid;" : "=r"(pace_slot));
-          pace_sm &= 255u;
-          pace_slot &= 63u;
-          if (lane == 0) g_pace[pace_sm][pace_slot] = ((unsigned long long)pace_launch << 32) | (unsigned)nnz;
-          unsigned left = 0u;
-          if (lane < 16) {
-            const unsigned long long v =
-                *reinterpret_cast<const volatile unsigned long long*>(&g_pace[pace_sm][(pace_slot & 3u) + 4u * lane]);
-            if ((unsigned)(v >> 32) == pace_launch) left = (unsigned)v;
-          }
-          left = __reduce_max_sync(FULL, left);   // the most entries left among the warps of this scheduler
-          // (a figure that has not moved since the last look is not slept on twice: an entry orphaned by a warp
-          // whose slot changed under preemption must not hold the others back)
-          if (left > (unsigned)nnz + PACE_SLACK && left != pace_seen)
-            __nanosleep(min((left - (unsigned)nnz - PACE_SLACK) * PACE_NS_PER_ENTRY, PACE_NS_MAX));
-          pace_seen = left;
-        }
-      }
       unsigned lo8 = (unsigned)N << 8;   // rows below lo8 >> 8 have their final column
       if (!pl.repair(lo8, work)) { st_code = MOESCHED_ST_INTERNAL; break; }
       if (k == 0) lo8 = 0u;
@@ -220,12 +183,6 @@ __global__ void __launch_bounds__(128, W <= 2 ? 7 : 0) bvn_kernel(int B, int N, 
     if (st_code == MOESCHED_ST_OK && nnz > 0) st_code = MOESCHED_ST_TRUNCATED;
   }
 
-  if constexpr (PACE) {   // this warp no longer counts (it may have moved on without entering the loop)
-    unsigned sm, slot;
-    asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
-    asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
-    if (lane == 0) g_pace[sm & 255u][slot & 63u] = 0ull;
-  }
   if (lane == 0) {
     count[b] = k;
     status[b] = st_code;
@@ -241,14 +198,6 @@ __global__ void __launch_bounds__(128, W <= 2 ? 7 : 0) bvn_kernel(int B, int N, 
 
 // ---- host side ---------------------------------------------------------------------------
 
-// Number of this paced launch (never 0; entries of the pacing table with another number are ignored).
-static unsigned next_pace_launch() {
-  static std::atomic<unsigned> n{0u};
-  unsigned v = ++n;
-  if (v == 0u) v = ++n;
-  return v;
-}
-
 cudaError_t run_bvn(int B, int N, const int32_t* demand, int k_max, uint8_t* perm, int32_t* coef, int32_t* count,
                     int32_t* aug, int32_t* scratch, int32_t* status, long long* work, cudaStream_t stream) {
   Geometry ge = plan_geometry(N);
@@ -256,11 +205,17 @@ cudaError_t run_bvn(int B, int N, const int32_t* demand, int k_max, uint8_t* per
   do {                                                                                                        \
     if (work != nullptr)                                                                                      \
       return launch_warp_kernel(bvn_kernel<C, M, true>, ge, B, stream, B, N, ge.S, demand, k_max, perm, coef, \
-                                count, aug, scratch, status, work, 0u);                                       \
+                                count, aug, scratch, status, work);                                       \
     return launch_warp_kernel(bvn_kernel<C, M, false>, ge, B, stream, B, N, ge.S, demand, k_max, perm, coef,  \
-                              count, aug, scratch, status, work, 0u);                                         \
+                              count, aug, scratch, status, work);                                         \
   } while (0)
-  if (scratch != nullptr) {
+  // Without scratch the matrix is held in shared memory, split over a 2-CTA cluster where one CTA cannot hold it. So it is
+  // with scratch when the whole batch fits half of the SMs' shared memory that way (the greedy kernel often runs beside):
+  // a value that a moved row needs is 30 instead of 300 cycles away (N = 64, 4 matrices per SM: 3 % of the time; below 33
+  // ranks there is nothing to be had).
+  const size_t held = peel_smem_bytes(N, ge.cpl) + align16((size_t)N * N * 4);
+  const bool resident = N > 32 && (size_t)((B + sm_count() - 1) / sm_count()) * (held + 1024) <= SMEM_LIMIT / 2;
+  if (scratch != nullptr && !resident) {
     // working copy in global memory: shared memory only for the position table and the search levels
     ge.cluster = false;
     ge.S = bvn_scratch_stride(N);
@@ -268,27 +223,6 @@ cudaError_t run_bvn(int B, int N, const int32_t* demand, int k_max, uint8_t* per
     // a small batch is spread one matrix per CTA so that no SM sits idle
     ge.wpb = B >= 16 * sm_count() ? 4 : 1;
     ge.smem = peel_smem_bytes(N, ge.cpl) * ge.wpb;
-    // pacing (see PACE above) when every scheduler gets three warps or more and the whole batch is resident at once
-    if (work == nullptr && B >= 12 * sm_count()) {
-#define MOESCHED_PACED(C)                                                                                          \
-  do {                                                                                                             \
-    int per_sm = 0;                                                                                                \
-    auto kern = bvn_kernel<C, 2, false, true>;                                                                     \
-    cudaError_t eo = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ge.smem);        \
-    if (eo == cudaSuccess) eo = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * ge.wpb, ge.smem); \
-    if (eo != cudaSuccess) return eo;                                                                              \
-    if ((long long)per_sm * sm_count() >= (B + ge.wpb - 1) / ge.wpb)                                               \
-      return launch_warp_kernel(kern, ge, B, stream, B, N, ge.S, demand, k_max, perm, coef, count, aug, scratch,   \
-                                status, work, next_pace_launch());                                                 \
-  } while (0)
-      switch (ge.cpl) {
-        case 1: MOESCHED_PACED(1); break;
-        case 2: MOESCHED_PACED(2); break;
-        case 4: MOESCHED_PACED(4); break;
-        default: MOESCHED_PACED(8); break;
-      }
-#undef MOESCHED_PACED
-    }
     switch (ge.cpl) {
       case 1: MOESCHED_GO(1, 2);
       case 2: MOESCHED_GO(2, 2);
@@ -296,9 +230,8 @@ cudaError_t run_bvn(int B, int N, const int32_t* demand, int k_max, uint8_t* per
       default: MOESCHED_GO(8, 2);
     }
   }
-  // without scratch the matrix is held in shared memory, split over a 2-CTA cluster where one CTA cannot hold it
   ge.S = N;
-  ge.smem = peel_smem_bytes(N, ge.cpl) + align16((size_t)N * N * 4);
+  ge.smem = held;
   ge.cluster = ge.smem > SMEM_LIMIT;
   if (ge.cluster) ge.smem = peel_smem_bytes(N, ge.cpl) + align16((size_t)((N + 1) / 2) * N * 4);
   ge.wpb = !ge.cluster && N <= 32 ? 4 : 1;

@@ -526,10 +526,10 @@ static cudaError_t launch_mw(int B, int N, const int32_t* demand, int k_max, uin
 cudaError_t run_mw(int B, int N, const int32_t* demand, int k_max, uint8_t* perm, int32_t* dur, int32_t* count,
                    int32_t* residual, int32_t* status, long long* work, cudaStream_t stream) {
   const size_t as_int32 = mw_smem_per_warp(N, plan_geometry(N).cpl, 0);
-  // Shared memory limits how many matrices an SM holds. Where all of them are resident at once as int32 anyway, one launch
-  // takes every matrix; otherwise they are held as 16-bit entries, and a second launch takes those that do not fit (as int32,
+  // Shared memory limits how many matrices an SM holds. Where all of them fit half of it as int32 (the Birkhoff kernel often
+  // runs beside), one launch takes every matrix; otherwise they are held as 16-bit entries, and a second launch takes those that do not fit (as int32,
   // over a 2-CTA cluster where one CTA cannot hold the matrix).
-  if (N < 48 || (as_int32 <= SMEM_LIMIT && B <= (long long)sm_count() * (long long)(SMEM_LIMIT / (as_int32 + 1024))))
+  if (N < 48 || (as_int32 <= SMEM_LIMIT && (size_t)((B + sm_count() - 1) / sm_count()) * (as_int32 + 1024) <= SMEM_LIMIT / 2))
     return launch_mw<0>(B, N, demand, k_max, perm, dur, count, residual, status, work, 0, stream);
   cudaError_t e = launch_mw<2>(B, N, demand, k_max, perm, dur, count, residual, status, work, 0, stream);
   if (e != cudaSuccess) return e;
