@@ -406,6 +406,31 @@ int moesched_bvn_decompose_static(int B, int N, const int32_t* d_demand, int k_m
                                   int32_t* d_status, int64_t* d_work, void* stream);
 
 /*
+ * The whole path for one batch in one call: greedy and Birkhoff-von Neumann decomposition, both scored
+ * (moesched_mw_decompose, moesched_bvn_decompose and moesched_schedule_eval with the buffers named here). The two
+ * decompositions do not depend on each other. With `overlap` the greedy one and its scoring are enqueued on
+ * side_stream, which first waits for what `stream` holds at the time of the call (fork_event) and which `stream` waits
+ * for at the end (join_event); without it, or with side_stream NULL, everything goes to `stream`. The streams and
+ * events belong to the caller (cudaStream_t, cudaEvent_t); a call that finds the same side_stream busy queues up behind it.
+ *
+ *   B, N         in   size of this batch; all buffers hold at least B matrices of N x N, budgets k_mw and k_bvn
+ *   scores       out  five int64 arrays each: overlap, serial, compute idle, link idle tokens, unserved tokens,
+ *                     score_stride elements apart
+ *   d_work       out  as in the decompositions, may be NULL
+ */
+typedef struct moesched_path {
+  int64_t k_mw, k_bvn, score_stride;
+  uint8_t *d_mw_perm, *d_bvn_perm;
+  int32_t *d_mw_dur, *d_mw_count, *d_mw_status, *d_mw_eval_status;
+  int32_t *d_bvn_coef, *d_bvn_count, *d_bvn_status, *d_bvn_eval_status;
+  int64_t *d_mw_work, *d_bvn_work, *d_mw_scores, *d_bvn_scores;
+  int32_t* d_bvn_scratch;
+  void *side_stream, *fork_event, *join_event;
+} moesched_path_t;
+int moesched_path_run(const moesched_path_t* h_path, int B, int N, const int32_t* d_demand,
+                      const moesched_model_t* h_model, int overlap, void* stream);
+
+/*
  * Measurement aid (no counterpart in the paper): enqueue a kernel of `blocks` CTAs of 256
  * threads, each thread running 8 independent chains of add / min / xor for `iters`
  * iterations, and return the number of integer lane-operations it executes

@@ -34,7 +34,29 @@ class _Model(ctypes.Structure):
                 ("expert_ps_per_token", ctypes.c_int64), ("expert_knee_tokens", ctypes.c_int64)]
 
 
+class _PathArgs(ctypes.Structure):
+    """moesched_path_t of include/moesched.h."""
+    _fields_ = ([(n, ctypes.c_int64) for n in ("k_mw", "k_bvn", "score_stride")] +
+                [(n, ctypes.c_void_p) for n in (
+                    "mw_perm", "bvn_perm", "mw_dur", "mw_count", "mw_status", "mw_eval_status", "bvn_coef", "bvn_count",
+                    "bvn_status", "bvn_eval_status", "mw_work", "bvn_work", "mw_scores", "bvn_scores", "bvn_scratch",
+                    "side_stream", "fork_event", "join_event")])
+
+
 _lib = None
+
+# Argument types of the entry points: i = int, p = pointer (an address, or None), q = int64, d = double. With them declared,
+# addresses go in as plain integers.
+_ARGTYPES = {"i": ctypes.c_int, "p": ctypes.c_void_p, "q": ctypes.c_int64, "d": ctypes.c_double}
+_SIGNATURES = {
+    "moesched_mw_decompose": "iipippppppp", "moesched_bvn_decompose": "iipipppppppp",
+    "moesched_bvn_decompose_static": "iipippppppp", "moesched_schedule_eval": "iipippp" + "p" * 8,
+    "moesched_schedule_prefix_eval": "iipippp" + "p" * 10, "moesched_ideal_a2a": "iipppppp",
+    "moesched_sinkhorn_scale": "iipidipppppp", "moesched_sinkhorn_durations": "iipppipp",
+    "moesched_schedule_order": "iipippp" + "p" * 8, "moesched_schedule_permute": "iiipppppp",
+    "moesched_best_budget": "iipppqppp", "moesched_bvn_real_decompose": "iipdipppppppp",
+    "moesched_path_run": "piippip", "moesched_last_cuda_error": "",
+}
 
 
 def _open(path):
@@ -45,12 +67,9 @@ def _open(path):
     lib.moesched_strerror.restype = ctypes.c_char_p
     lib.moesched_status_str.restype = ctypes.c_char_p
     lib.moesched_workspace_bytes.restype = ctypes.c_size_t
-    for name in ("moesched_mw_decompose", "moesched_bvn_decompose", "moesched_bvn_decompose_static",
-                 "moesched_schedule_eval", "moesched_schedule_prefix_eval", "moesched_ideal_a2a",
-                 "moesched_sinkhorn_scale", "moesched_sinkhorn_durations", "moesched_last_cuda_error",
-                 "moesched_schedule_order", "moesched_schedule_permute", "moesched_best_budget",
-                 "moesched_bvn_real_decompose"):
-        getattr(lib, name).restype = ctypes.c_int
+    for name, signature in _SIGNATURES.items():
+        fn = getattr(lib, name)
+        fn.restype, fn.argtypes = ctypes.c_int, [_ARGTYPES[c] for c in signature]
     lib.moesched_bvn_scratch_bytes.restype = ctypes.c_size_t
     lib.moesched_order_scratch_bytes.restype = ctypes.c_size_t
     lib.moesched_probe_int_ops.restype = ctypes.c_longlong
@@ -96,11 +115,21 @@ def _dev(t, dtype, what):
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
-def _stream(device):
-    return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+def _call(name, device, *args):
+    """Entry point `name` with `args` and the current stream of `device`, with that device current."""
+    index = device.index
+    stream = torch._C._cuda_getCurrentRawStream(index)
+    fn = getattr(load_library(), name)
+    if torch.cuda.current_device() == index:
+        rc = fn(*args, stream)
+    else:
+        with torch.cuda.device(device):
+            rc = fn(*args, stream)
+    if rc != 0:
+        _check(rc, name)
 
 
 @dataclass
@@ -136,17 +165,12 @@ def _check_demand(demand):
 
 def mw_decompose(demand, k_max, want_residual=False, want_work=False, out=None) -> Schedule:
     """Greedy max-weight decomposition of every matrix of `demand` [B, N, N] int32 (CUDA)."""
-    lib = load_library()
     demand = _check_demand(demand)
     B, N, _ = demand.shape
-    dev = demand.device
     if out is None:
         out = _new_schedule(demand, int(k_max), want_residual, want_work)
-    with torch.cuda.device(dev):
-        rc = lib.moesched_mw_decompose(B, N, _ptr(demand), int(k_max), _ptr(out.perm), _ptr(out.dur),
-                                       _ptr(out.count), _ptr(out.extra), _ptr(out.status), _ptr(out.work),
-                                       _stream(dev))
-    _check(rc, "moesched_mw_decompose")
+    _call("moesched_mw_decompose", demand.device, B, N, _ptr(demand), int(k_max), _ptr(out.perm), _ptr(out.dur),
+          _ptr(out.count), _ptr(out.extra), _ptr(out.status), _ptr(out.work))
     return out
 
 
@@ -169,7 +193,6 @@ def bvn_decompose(demand, k_max=None, want_aug=False, want_work=False, out=None,
 
     scratch: True allocates the working buffer of the fast path, a uint8 CUDA tensor of at least
     bvn_scratch_bytes(B, N) bytes is used as given, False / None selects the shared-memory path."""
-    lib = load_library()
     demand = _check_demand(demand)
     B, N, _ = demand.shape
     dev = demand.device
@@ -185,11 +208,8 @@ def bvn_decompose(demand, k_max=None, want_aug=False, want_work=False, out=None,
         _dev(scratch, torch.uint8, "scratch")
         if scratch.numel() < bvn_scratch_bytes(B, N):
             raise MoeschedError("scratch is smaller than bvn_scratch_bytes(B, N)")
-    with torch.cuda.device(dev):
-        rc = lib.moesched_bvn_decompose(B, N, _ptr(demand), int(k_max), _ptr(out.perm), _ptr(out.dur),
-                                        _ptr(out.count), _ptr(out.extra), _ptr(scratch), _ptr(out.status),
-                                        _ptr(out.work), _stream(dev))
-    _check(rc, "moesched_bvn_decompose")
+    _call("moesched_bvn_decompose", dev, B, N, _ptr(demand), int(k_max), _ptr(out.perm), _ptr(out.dur), _ptr(out.count),
+          _ptr(out.extra), _ptr(scratch), _ptr(out.status), _ptr(out.work))
     return out
 
 
@@ -202,15 +222,10 @@ def bvn_decompose_static(demand, out: Schedule) -> Schedule:
     latency-critical loop). `out` must be a complete, caller-made Schedule; the working copy sits
     in the library's built-in 16 MiB array, so B * N * roundup(N, 8) * 4 must fit in it. Calls
     that may overlap on one GPU share that array and must be serialised."""
-    lib = load_library()
     demand = _check_demand(demand)
     B, N, _ = demand.shape
-    dev = demand.device
-    with torch.cuda.device(dev):
-        rc = lib.moesched_bvn_decompose_static(B, N, _ptr(demand), int(out.perm.shape[1]), _ptr(out.perm),
-                                               _ptr(out.dur), _ptr(out.count), _ptr(out.extra),
-                                               _ptr(out.status), _ptr(out.work), _stream(dev))
-    _check(rc, "moesched_bvn_decompose_static")
+    _call("moesched_bvn_decompose_static", demand.device, B, N, _ptr(demand), int(out.perm.shape[1]), _ptr(out.perm),
+          _ptr(out.dur), _ptr(out.count), _ptr(out.extra), _ptr(out.status), _ptr(out.work))
     return out
 
 
@@ -224,7 +239,8 @@ def probe_int_rate(device=None, blocks=148 * 8, iters=20000, reps=3) -> float:
         for _ in range(reps + 1):
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             e0.record()
-            ops = lib.moesched_probe_int_ops(blocks, iters, _ptr(out), _stream(dev))
+            ops = lib.moesched_probe_int_ops(blocks, iters, ctypes.c_void_p(_ptr(out)),
+                                             ctypes.c_void_p(torch.cuda.current_stream(dev).cuda_stream))
             e1.record()
             if ops < 0:
                 _check(int(ops), "moesched_probe_int_ops")
@@ -251,11 +267,8 @@ def sinkhorn_scale(demand, iters=20, smooth=0.5, scale_bits=20, out=None) -> dic
         _dev(out["fixed"], torch.int32, "out['fixed']")
         if out["scaled"].shape != demand.shape or out["fixed"].shape != demand.shape:
             raise MoeschedError("out has the wrong shape")
-    rc = load_library().moesched_sinkhorn_scale(B, N, _ptr(demand), int(iters), ctypes.c_double(float(smooth)),
-                                                int(scale_bits), _ptr(out["scaled"]), _ptr(out["fixed"]),
-                                                _ptr(out["stretch"]), _ptr(out["row_err"]), _ptr(out["status"]),
-                                                _stream(dev))
-    _check(rc, "moesched_sinkhorn_scale")
+    _call("moesched_sinkhorn_scale", dev, B, N, _ptr(demand), int(iters), float(smooth), int(scale_bits),
+          _ptr(out["scaled"]), _ptr(out["fixed"]), _ptr(out["stretch"]), _ptr(out["row_err"]), _ptr(out["status"]))
     return out
 
 
@@ -268,9 +281,8 @@ def sinkhorn_durations(coef, count, stretch, scale_bits=20, out=None) -> torch.T
     B, K = coef.shape
     if out is None:
         out = torch.zeros_like(coef)
-    rc = load_library().moesched_sinkhorn_durations(B, K, _ptr(coef), _ptr(count), _ptr(stretch), int(scale_bits),
-                                                    _ptr(_dev(out, torch.int32, "out")), _stream(coef.device))
-    _check(rc, "moesched_sinkhorn_durations")
+    _call("moesched_sinkhorn_durations", coef.device, B, K, _ptr(coef), _ptr(count), _ptr(stretch), int(scale_bits),
+          _ptr(_dev(out, torch.int32, "out")))
     return out
 
 
@@ -278,7 +290,6 @@ def bvn_real_decompose(matrix, k_max=None, tol=1e-12) -> dict:
     """Real-valued Birkhoff-von Neumann decomposition A = sum_k lambda_k P_k (paper Sec. 3.1) of [B, N, N]
     float64 matrices, e.g. sinkhorn_scale(...)["scaled"]. Returns perm [B, k_max, N] uint8, lam [B, k_max]
     float64, count, sum_lambda, max_left (largest entry remaining) and status [B]."""
-    lib = load_library()
     matrix = _dev(matrix, torch.float64, "matrix")
     if matrix.dim() != 3 or matrix.shape[1] != matrix.shape[2]:
         raise MoeschedError("matrix must have shape [B, N, N]")
@@ -292,33 +303,37 @@ def bvn_real_decompose(matrix, k_max=None, tol=1e-12) -> dict:
                max_left=torch.empty(B, dtype=torch.float64, device=dev),
                status=torch.empty(B, dtype=torch.int32, device=dev))
     scratch = torch.empty(max(1, B * N * ((N + 7) // 8 * 8)), dtype=torch.float64, device=dev)
-    with torch.cuda.device(dev):
-        rc = lib.moesched_bvn_real_decompose(B, N, _ptr(matrix), ctypes.c_double(float(tol)), k_max, _ptr(out["perm"]),
-                                             _ptr(out["lam"]), _ptr(out["count"]), _ptr(out["sum_lambda"]),
-                                             _ptr(out["max_left"]), _ptr(scratch), _ptr(out["status"]), _stream(dev))
-    _check(rc, "moesched_bvn_real_decompose")
+    _call("moesched_bvn_real_decompose", dev, B, N, _ptr(matrix), float(tol), k_max, _ptr(out["perm"]), _ptr(out["lam"]),
+          _ptr(out["count"]), _ptr(out["sum_lambda"]), _ptr(out["max_left"]), _ptr(scratch), _ptr(out["status"]))
     return out
 
 
+_models = {}    # the few models a program uses, as the C structure; never changed once made
+
+
 def _model(model):
-    return _Model(**{k: int(v) for k, v in (model or DEFAULT_MODEL).items()})
+    """Address of the C form of a model dict."""
+    key = tuple((model or DEFAULT_MODEL).items())
+    made = _models.get(key)
+    if made is None:
+        if len(_models) >= 256:
+            _models.clear()
+        made = _Model(**{k: int(v) for k, v in key})
+        made = _models[key] = (made, ctypes.addressof(made))
+    return made
 
 
 def ideal_a2a(demand, model=None) -> dict:
     """Idealised congestion-free all-to-all of every matrix: 'comm_ns' (one exchange at line rate of
     the busiest port), 'makespan_ns' (dispatch + compute + combine, run to completion), 'status'."""
-    lib = load_library()
     demand = _check_demand(demand)
     B, N, _ = demand.shape
     dev = demand.device
     m = _model(model)
-    out = torch.empty((2, B), dtype=torch.int64, device=dev)
+    comm, makespan = torch.empty((2, B), dtype=torch.int64, device=dev).unbind(0)
     status = torch.empty(B, dtype=torch.int32, device=dev)
-    with torch.cuda.device(dev):
-        rc = lib.moesched_ideal_a2a(B, N, _ptr(demand), ctypes.byref(m), _ptr(out[0]), _ptr(out[1]), _ptr(status),
-                                    _stream(dev))
-    _check(rc, "moesched_ideal_a2a")
-    return {"comm_ns": out[0], "makespan_ns": out[1], "status": status}
+    _call("moesched_ideal_a2a", dev, B, N, _ptr(demand), m[1], _ptr(comm), _ptr(makespan), _ptr(status))
+    return {"comm_ns": comm, "makespan_ns": makespan, "status": status}
 
 
 SCORE_FIELDS = ("makespan_overlap_ns", "makespan_serial_ns", "compute_idle_ns", "link_idle_tokens",
@@ -331,7 +346,6 @@ def schedule_eval(demand, perm, dur, count, model=None, out=None, status=None, p
     `status` a [B] int32 tensor. With prefix=True the dict also holds 'prefix_overlap_ns' and
     'prefix_unserved_tokens', [B, k_stride] int64: the scores of the schedule cut after each
     matching (-1 beyond count)."""
-    lib = load_library()
     demand = _dev(demand, torch.int32, "demand")
     perm = _dev(perm, torch.uint8, "perm")
     dur = _dev(dur, torch.int32, "dur")
@@ -346,17 +360,15 @@ def schedule_eval(demand, perm, dur, count, model=None, out=None, status=None, p
         status = torch.empty(B, dtype=torch.int32, device=dev)
     K = int(perm.shape[1])
     pre = torch.empty((2, B, K), dtype=torch.int64, device=dev) if prefix else None
-    with torch.cuda.device(dev):
-        args = (B, N, _ptr(demand), K, _ptr(perm), _ptr(dur), _ptr(count), ctypes.byref(m), _ptr(scores[0]),
-                _ptr(scores[1]), _ptr(scores[2]), _ptr(scores[3]), _ptr(scores[4]), _ptr(status))
-        if prefix:
-            rc = lib.moesched_schedule_prefix_eval(*args, _ptr(pre[0]), _ptr(pre[1]), _stream(dev))
-        else:
-            rc = lib.moesched_schedule_eval(*args, _stream(dev))
-    _check(rc, "moesched_schedule_eval")
-    res = {name: scores[i] for i, name in enumerate(SCORE_FIELDS)}
+    rows = scores.unbind(0)
+    args = (B, N, _ptr(demand), K, _ptr(perm), _ptr(dur), _ptr(count), m[1], *(r.data_ptr() for r in rows), _ptr(status))
+    res = dict(zip(SCORE_FIELDS, rows))
     if prefix:
-        res["prefix_overlap_ns"], res["prefix_unserved_tokens"] = pre[0], pre[1]
+        overlap, unserved = pre.unbind(0)
+        _call("moesched_schedule_prefix_eval", dev, *args, _ptr(overlap), _ptr(unserved))
+        res["prefix_overlap_ns"], res["prefix_unserved_tokens"] = overlap, unserved
+    else:
+        _call("moesched_schedule_eval", dev, *args)
     res["status"] = status
     return res
 
@@ -380,45 +392,36 @@ def schedule_order(demand, perm, dur, count, model=None) -> dict:
     dev = demand.device
     m = _model(model)
     order = torch.empty((B, K), dtype=torch.int32, device=dev)
-    times = torch.empty((2, B), dtype=torch.int64, device=dev)
-    small = torch.empty((2, B), dtype=torch.int32, device=dev)
+    makespan, emission = torch.empty((2, B), dtype=torch.int64, device=dev).unbind(0)
+    rule, status = torch.empty((2, B), dtype=torch.int32, device=dev).unbind(0)
     scratch = torch.empty(max(8, int(lib.moesched_order_scratch_bytes(B, K))), dtype=torch.uint8, device=dev)
-    with torch.cuda.device(dev):
-        rc = lib.moesched_schedule_order(B, N, _ptr(demand), K, _ptr(perm), _ptr(dur), _ptr(count), ctypes.byref(m),
-                                         _ptr(order), _ptr(times[0]), _ptr(times[1]), _ptr(small[0]), _ptr(small[1]),
-                                         _ptr(scratch), _stream(dev))
-    _check(rc, "moesched_schedule_order")
-    return {"order": order, "makespan_ns": times[0], "emission_ns": times[1], "rule": small[0], "status": small[1]}
+    _call("moesched_schedule_order", dev, B, N, _ptr(demand), K, _ptr(perm), _ptr(dur), _ptr(count), m[1], _ptr(order),
+          _ptr(makespan), _ptr(emission), _ptr(rule), _ptr(status), _ptr(scratch))
+    return {"order": order, "makespan_ns": makespan, "emission_ns": emission, "rule": rule, "status": status}
 
 
 def schedule_permute(perm, dur, order):
     """(perm, dur) with the matchings in the given order; positions whose order entry is -1 hold zeros."""
-    lib = load_library()
     perm = _dev(perm, torch.uint8, "perm")
     dur = _dev(dur, torch.int32, "dur")
     order = _dev(order, torch.int32, "order")
     B, K, N = perm.shape
     perm_out, dur_out = torch.zeros_like(perm), torch.zeros_like(dur)
-    with torch.cuda.device(perm.device):
-        rc = lib.moesched_schedule_permute(B, N, K, _ptr(perm), _ptr(dur), _ptr(order), _ptr(perm_out), _ptr(dur_out),
-                                           _stream(perm.device))
-    _check(rc, "moesched_schedule_permute")
+    _call("moesched_schedule_permute", perm.device, B, N, K, _ptr(perm), _ptr(dur), _ptr(order), _ptr(perm_out),
+          _ptr(dur_out))
     return perm_out, dur_out
 
 
 def best_budget(count, prefix_overlap_ns, prefix_unserved_tokens, ns_per_unserved_token) -> dict:
     """Number of matchings (1..count) minimising prefix makespan + price * unserved tokens."""
-    lib = load_library()
     count = _dev(count, torch.int32, "count")
     po = _dev(prefix_overlap_ns, torch.int64, "prefix_overlap_ns")
     pu = _dev(prefix_unserved_tokens, torch.int64, "prefix_unserved_tokens")
     B, K = po.shape
     best_k = torch.empty(B, dtype=torch.int32, device=po.device)
     best_cost = torch.empty(B, dtype=torch.int64, device=po.device)
-    with torch.cuda.device(po.device):
-        rc = lib.moesched_best_budget(B, K, _ptr(count), _ptr(po), _ptr(pu), ctypes.c_int64(int(ns_per_unserved_token)),
-                                      _ptr(best_k), _ptr(best_cost), _stream(po.device))
-    _check(rc, "moesched_best_budget")
+    _call("moesched_best_budget", po.device, B, K, _ptr(count), _ptr(po), _ptr(pu), int(ns_per_unserved_token),
+          _ptr(best_k), _ptr(best_cost))
     return {"best_k": best_k, "best_cost": best_cost}
 
 
@@ -426,10 +429,10 @@ class Path:
     """The whole path for batches of one shape: greedy max-weight and BvN decomposition, both scored.
 
     All buffers (schedules, scores, BvN scratch) are allocated once here. The two decompositions do not
-    depend on each other: run() forks them onto two streams -- BvN and its scoring first, greedy and its
-    scoring second -- and joins them back into the caller's current stream, so that the greedy warps fill
-    the SMs as the BvN matrices finish at different times (measured on a B200, headline workload: 70 ms
-    per step against 77 ms on one stream). run(overlap=False) keeps everything on the current stream."""
+    depend on each other: run() enqueues BvN and its scoring on the caller's current stream and greedy and its
+    scoring on a side stream forked from it and joined back, so that the greedy warps fill the SMs beside the BvN
+    warps. run(overlap=False) keeps everything on the current stream. The launches, the fork and the join are
+    one call into the library (moesched_path_run), since a small batch is done in microseconds."""
 
     def __init__(self, B, N, k_mw, k_bvn=None, device=None, want_work=False):
         dev = torch.device("cuda", torch.cuda.current_device()) if device is None else torch.device(device)
@@ -449,23 +452,22 @@ class Path:
         self.eval_status_mw = torch.empty(B, dtype=torch.int32, device=dev)
         self.eval_status_bvn = torch.empty(B, dtype=torch.int32, device=dev)
         self.scratch = torch.empty(max(1, bvn_scratch_bytes(B, N)), dtype=torch.uint8, device=dev)
-        self._side = (torch.cuda.Stream(dev), torch.cuda.Stream(dev))
-        self._fork = torch.cuda.Event()
-        self._join = (torch.cuda.Event(), torch.cuda.Event())
+        with torch.cuda.device(dev):
+            self._side = torch.cuda.Stream(dev)
+            self._events = (torch.cuda.Event(), torch.cuda.Event())      # fork, join
+            for event in self._events:
+                event.record()                                           # an event gets its handle when first recorded
+        self._args = _PathArgs(
+            self.k_mw, self.k_bvn, B, _ptr(self.mw.perm), _ptr(self.bvn.perm), _ptr(self.mw.dur), _ptr(self.mw.count),
+            _ptr(self.mw.status), _ptr(self.eval_status_mw), _ptr(self.bvn.dur), _ptr(self.bvn.count),
+            _ptr(self.bvn.status), _ptr(self.eval_status_bvn), _ptr(self.mw.work), _ptr(self.bvn.work),
+            _ptr(self.score_mw), _ptr(self.score_bvn), _ptr(self.scratch), self._side.cuda_stream,
+            self._events[0].cuda_event, self._events[1].cuda_event)
+        self._args_at = ctypes.addressof(self._args)
 
     def outputs(self):
         return [self.mw.perm, self.mw.dur, self.mw.count, self.mw.status, self.bvn.perm, self.bvn.dur,
                 self.bvn.count, self.bvn.status, self.score_mw, self.score_bvn]
-
-    def _greedy(self, demand, model):
-        mw_decompose(demand, self.k_mw, out=self.mw)
-        schedule_eval(demand, self.mw.perm, self.mw.dur, self.mw.count, model, out=self.score_mw,
-                      status=self.eval_status_mw)
-
-    def _bvn(self, demand, model):
-        bvn_decompose(demand, self.k_bvn, out=self.bvn, scratch=self.scratch)
-        schedule_eval(demand, self.bvn.perm, self.bvn.dur, self.bvn.count, model, out=self.score_bvn,
-                      status=self.eval_status_bvn)
 
     def run_graph(self, demand, model=None):
         """The same launches replayed from a CUDA graph: for small matrices the step is a handful of
@@ -484,19 +486,11 @@ class Path:
 
     def run(self, demand, model=None, overlap=True):
         """Enqueue the four kernels; results are ready when the caller's current stream reaches this point."""
-        if not overlap:
-            self._greedy(demand, model)
-            self._bvn(demand, model)
-            return self
-        cur = torch.cuda.current_stream(self.device)
-        self._fork.record(cur)
-        for side, work, done in ((self._side[0], self._bvn, self._join[0]), (self._side[1], self._greedy, self._join[1])):
-            side.wait_event(self._fork)
-            with torch.cuda.stream(side):
-                work(demand, model)
-                done.record(side)
-        for done in self._join:
-            cur.wait_event(done)
+        demand = _check_demand(demand)
+        B, N, _ = demand.shape
+        if B > self.B or N > self.N:
+            raise MoeschedError("demand is larger than the Path was made for")
+        _call("moesched_path_run", demand.device, self._args_at, B, N, _ptr(demand), _model(model)[1], int(overlap))
         return self
 
 
@@ -504,7 +498,7 @@ class HostPipeline:
     """The whole path for batches that live in host memory, double-buffered.
 
     submit() enqueues, for one batch: the copy of the demand from (pinned) host memory to the device
-    on an upload stream, the four kernels on a compute stream, and the copy of all schedules and scores
+    on an upload stream, the four kernels on the slot's compute stream, and the copy of all schedules and scores
     back to pinned host memory on a download stream. With two slots the download of one batch and the
     upload of the next overlap the kernels of the batch in between, so a stream of batches runs at the
     speed of the slowest of the three stages instead of their sum."""
@@ -515,7 +509,13 @@ class HostPipeline:
         self.paths = [Path(B, N, k_mw, k_bvn, device=dev) for _ in range(slots)]
         self.d_in = [torch.empty((B, N, N), dtype=torch.int32, device=dev) for _ in range(slots)]
         self.h_out = [[torch.empty(t.shape, dtype=t.dtype, pin_memory=True) for t in p.outputs()] for p in self.paths]
-        self.up, self.compute, self.down = (torch.cuda.Stream(dev) for _ in range(3))
+        self.up, self.down = torch.cuda.Stream(dev), torch.cuda.Stream(dev)
+        # A batch that leaves the schedulers with little to choose from is bound by the latency of its chains, so two of
+        # them run side by side, a compute stream per slot; larger ones would only
+        # get in each other's way.
+        sms = torch.cuda.get_device_properties(dev).multi_processor_count
+        shared = None if B < 12 * sms else torch.cuda.Stream(dev)
+        self.compute = [shared or torch.cuda.Stream(dev) for _ in range(slots)]
         self.ev_in = [torch.cuda.Event() for _ in range(slots)]
         self.ev_done = [torch.cuda.Event() for _ in range(slots)]
         self.ev_out = [torch.cuda.Event() for _ in range(slots)]
@@ -532,10 +532,11 @@ class HostPipeline:
         with torch.cuda.stream(self.up):
             self.d_in[s].copy_(demand_host, non_blocking=True)
             self.ev_in[s].record(self.up)
-        self.compute.wait_event(self.ev_in[s])
-        with torch.cuda.stream(self.compute):
+        compute = self.compute[s]
+        compute.wait_event(self.ev_in[s])
+        with torch.cuda.stream(compute):
             self.paths[s].run(self.d_in[s], model)
-            self.ev_done[s].record(self.compute)
+            self.ev_done[s].record(compute)
         self.down.wait_event(self.ev_done[s])
         with torch.cuda.stream(self.down):
             for h, t in zip(self.h_out[s], self.paths[s].outputs()):

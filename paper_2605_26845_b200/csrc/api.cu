@@ -150,6 +150,44 @@ int moesched_schedule_prefix_eval(int B, int N, const int32_t* d_demand, int k_s
                             d_status, d_prefix_overlap_ns, d_prefix_unserved_tokens, stream);
 }
 
+int moesched_path_run(const moesched_path_t* p, int B, int N, const int32_t* d_demand, const moesched_model_t* h_model,
+                      int overlap, void* stream) {
+  if (p == nullptr || B < 0 || p->k_mw < 1 || p->k_mw > 0x7fffffff || p->k_bvn < 1 || p->k_bvn > 0x7fffffff || p->score_stride < B)
+    return MOESCHED_EINVAL;
+  if (B == 0) return MOESCHED_OK;
+  if (!p->d_mw_scores || !p->d_bvn_scores) return MOESCHED_EINVAL;
+  const bool fork = overlap != 0 && p->side_stream != nullptr;
+  if (fork && (!p->fork_event || !p->join_event)) return MOESCHED_EINVAL;
+  const cudaStream_t main = static_cast<cudaStream_t>(stream);
+  const cudaStream_t side = fork ? static_cast<cudaStream_t>(p->side_stream) : main;
+  if (fork) {
+    cudaError_t e = cudaEventRecord(static_cast<cudaEvent_t>(p->fork_event), main);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(side, static_cast<cudaEvent_t>(p->fork_event), 0);
+    if (e != cudaSuccess) return fail_cuda(e);
+  }
+  // the Birkhoff decomposition is the longer one: it goes first, and on the caller's stream, so that no event stands
+  // between it and what comes before and after
+  const size_t st = (size_t)p->score_stride;
+  int64_t *sb = p->d_bvn_scores, *sm = p->d_mw_scores;
+  int rc = moesched_bvn_decompose(B, N, d_demand, (int)p->k_bvn, p->d_bvn_perm, p->d_bvn_coef, p->d_bvn_count, nullptr,
+                                  p->d_bvn_scratch, p->d_bvn_status, p->d_bvn_work, main);
+  if (rc == MOESCHED_OK)
+    rc = moesched_mw_decompose(B, N, d_demand, (int)p->k_mw, p->d_mw_perm, p->d_mw_dur, p->d_mw_count, nullptr,
+                               p->d_mw_status, p->d_mw_work, side);
+  if (rc == MOESCHED_OK)
+    rc = moesched_schedule_eval(B, N, d_demand, (int)p->k_mw, p->d_mw_perm, p->d_mw_dur, p->d_mw_count, h_model, sm, sm + st,
+                                sm + 2 * st, sm + 3 * st, sm + 4 * st, p->d_mw_eval_status, side);
+  if (rc == MOESCHED_OK)
+    rc = moesched_schedule_eval(B, N, d_demand, (int)p->k_bvn, p->d_bvn_perm, p->d_bvn_coef, p->d_bvn_count, h_model, sb,
+                                sb + st, sb + 2 * st, sb + 3 * st, sb + 4 * st, p->d_bvn_eval_status, main);
+  if (fork) {   // also after an error: what was enqueued on the side stream is joined
+    cudaError_t e = cudaEventRecord(static_cast<cudaEvent_t>(p->join_event), side);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(main, static_cast<cudaEvent_t>(p->join_event), 0);
+    if (e != cudaSuccess && rc == MOESCHED_OK) return fail_cuda(e);
+  }
+  return rc;
+}
+
 size_t moesched_order_scratch_bytes(int B, int k_stride) {
   if (B < 0 || k_stride < 1 || k_stride > MOESCHED_ORDER_MAX_K) return 0;
   return (size_t)B * (2 * (size_t)k_stride + 5) * sizeof(int64_t) + (((size_t)B * sizeof(int32_t) + 7) & ~(size_t)7);

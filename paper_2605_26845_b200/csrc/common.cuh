@@ -250,8 +250,10 @@ cudaError_t run_bvn_real(int B, int N, const double* matrix, double tol, int k_m
 // Launch helper shared by the three kernels.
 template <typename Kernel, typename... Args>
 cudaError_t launch_warp_kernel(Kernel kern, const Geometry& ge, int B, cudaStream_t stream, Args... args) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ge.smem);
-  if (e != cudaSuccess) return e;
+  if (ge.smem > 48 * 1024) {   // up to that much needs no permission
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ge.smem);
+    if (e != cudaSuccess) return e;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(ge.threads_per_cta != 0 ? ge.threads_per_cta : 32 * ge.wpb);
   cfg.dynamicSmemBytes = ge.smem;
