@@ -36,19 +36,19 @@ struct AssignShared {
   unsigned* claim;   // [row or column]
   short* x;          // [row] column
   short* y;          // [column] row
-  short* pred;       // [column] row from which the running search reached it
+  unsigned* pred;    // [column] row from which the running search reached it, and that row's column << 16
 };
 __host__ __device__ inline size_t assign_smem_bytes(int N) {
-  return 2 * align16((size_t)N * 4) + 3 * align16((size_t)N * 2);
+  return 3 * align16((size_t)N * 4) + 2 * align16((size_t)N * 2);
 }
 __device__ __forceinline__ AssignShared assign_shared(unsigned char* p, int N) {
   const size_t words = align16((size_t)N * 4), halves = align16((size_t)N * 2);
   AssignShared a;
   a.urow = reinterpret_cast<int*>(p);
   a.claim = reinterpret_cast<unsigned*>(p + words);
-  a.x = reinterpret_cast<short*>(p + 2 * words);
-  a.y = reinterpret_cast<short*>(p + 2 * words + halves);
-  a.pred = reinterpret_cast<short*>(p + 2 * words + 2 * halves);
+  a.pred = reinterpret_cast<unsigned*>(p + 2 * words);
+  a.x = reinterpret_cast<short*>(p + 3 * words);
+  a.y = reinterpret_cast<short*>(p + 3 * words + halves);
   return a;
 }
 
@@ -57,10 +57,13 @@ __device__ __forceinline__ AssignShared assign_shared(unsigned char* p, int N) {
 constexpr unsigned TAG_MATCHED = 0x100u;
 constexpr unsigned TAG_MASK = 0x1ffu;
 constexpr int TAG_BITS = 9;
-// Narrow matrices: distances, which lie within 3 C of zero (C the largest entry), and tag fit one word.
+// Narrow matrices: distances, which lie within 3 C of zero (C the largest entry), and tag fit one word. Wide ones: so does,
+// nearly always, the distance from the row's dual, which no column of the search undercuts; it saturates at FAR, and a search
+// that gets there is done over with distances of their own.
 constexpr int NARROW_BIAS = 1 << 22;
 constexpr int NARROW_MAX_ENTRY = NARROW_BIAS / 4;
 constexpr unsigned NONE = 0xffffffffu;
+constexpr unsigned FAR = (1u << (32 - TAG_BITS)) - 1u;
 
 __device__ __forceinline__ unsigned packed(int dist, unsigned tag) { return ((unsigned)(dist + NARROW_BIAS) << TAG_BITS) | tag; }
 __device__ __forceinline__ int packed_dist(unsigned k) { return (int)(k >> TAG_BITS) - NARROW_BIAS; }
@@ -109,7 +112,8 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
     base[s] = in[s] ? packed(-v[s], tag[s]) : NONE;
     if (in[s]) sh.claim[s * 32 + lane] = NONE;
   }
-  // ---- 1. rows name columns; lane l keeps what rows l, l + 32, ... found ----
+  // ---- 1. rows name columns, several at a time; lane l keeps what rows l, l + 32, ... found ----
+  constexpr int ROWS = W <= 2 ? 8 : W == 4 ? 4 : 2;
   int u[W];
   unsigned named[W];
 #pragma unroll
@@ -117,24 +121,32 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
     unsigned k_mine = 0u;
     u[w] = 0;
     named[w] = 0u;
-#pragma unroll 4
-    for (int q = 0; q < 32; ++q) {
-      const int r = w * 32 + q;
-      if (r >= N) break;
-      const auto* row = R.row(r);
+    for (int q0 = 0; q0 < 32 && w * 32 + q0 < N; q0 += ROWS) {   // (the last row again beyond the end)
       if constexpr (WIDE) {
-        int d[W], dist;
-        unsigned who;
 #pragma unroll
-        for (int s = 0; s < W; ++s) d[s] = in[s] ? -(int)row[s * 32 + lane] - v[s] : INF32;
-        nearest<W>(d, tag, dist, who);
-        if (lane == q) { u[w] = dist; named[w] = who; }
+        for (int q = 0; q < ROWS; ++q) {
+          const auto* row = R.row(min(w * 32 + q0 + q, N - 1));
+          int d[W], dist;
+          unsigned who;
+#pragma unroll
+          for (int s = 0; s < W; ++s) d[s] = in[s] ? -(int)row[s * 32 + lane] - v[s] : INF32;
+          nearest<W>(d, tag, dist, who);
+          if (lane == q0 + q) { u[w] = dist; named[w] = who; }
+        }
       } else {
-        unsigned k = NONE;
+        unsigned k[ROWS];
 #pragma unroll
-        for (int s = 0; s < W; ++s) k = min(k, base[s] - ((unsigned)(in[s] ? row[s * 32 + lane] : 0) << TAG_BITS));
-        k = __reduce_min_sync(FULL, k);
-        if (lane == q) k_mine = k;
+        for (int q = 0; q < ROWS; ++q) {
+          const auto* row = R.row(min(w * 32 + q0 + q, N - 1));
+          k[q] = NONE;
+#pragma unroll
+          for (int s = 0; s < W; ++s) k[q] = min(k[q], base[s] - ((unsigned)(in[s] ? row[s * 32 + lane] : 0) << TAG_BITS));
+        }
+#pragma unroll
+        for (int q = 0; q < ROWS; ++q) {
+          k[q] = __reduce_min_sync(FULL, k[q]);
+          if (lane == q0 + q) k_mine = k[q];
+        }
       }
     }
     if constexpr (!WIDE) {
@@ -244,79 +256,106 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
     work[WK_SKIP]--;
     work[WK_AUG]++;
     int pred[W], settled_at[W], mu;
-    unsigned done = 0u, who;   // done: bit s: the lane's column s is settled; who: tag of the column reached
+    unsigned closed[W], who;   // closed: all ones for a settled column; who: tag of the column reached
 #pragma unroll
     for (int s = 0; s < W; ++s) {
       pred[s] = f;
       settled_at[s] = 0;
+      closed[s] = in[s] ? 0u : NONE;
     }
+    // Candidates are keys, distance above tag. A settled column's key is all ones from then on; `closed` keeps new keys from
+    // undercutting it. There is a free column as long as there is a free row, so a search always ends at one.
+    unsigned key[W], k;
+    const auto* first = R.row(MS_AT(f, N));
+    const int off = sh.urow[MS_AT(f, N)];
     if constexpr (WIDE) {
-      int d[W];
-      const auto* first = R.row(MS_AT(f, N));
 #pragma unroll
-      for (int s = 0; s < W; ++s) d[s] = in[s] ? -(int)first[s * 32 + lane] - v[s] : INF32;
-      while (true) {   // every scan settles one more column
-        nearest<W>(d, tag, mu, who);
-        work[WK_SCAN]++;
-        if (mu == INF32) return false;
-        if (who < TAG_MATCHED) break;
-        const int i = MS_AT((int)(who & 0xffu), N);
-        const auto* row = R.row(i);
-        const int h = sh.urow[i] - mu;
-#pragma unroll
-        for (int s = 0; s < W; ++s) {
-          if (tag[s] == who) { done |= 1u << s; settled_at[s] = mu; d[s] = INF32; }
-          if (in[s] && !((done >> s) & 1u)) {
-            const int nd = -(int)row[s * 32 + lane] - v[s] - h;
-            if (nd < d[s]) { d[s] = nd; pred[s] = i; }
-          }
-        }
-      }
+      for (int s = 0; s < W; ++s)
+        key[s] = (min((unsigned)(-(int)(in[s] ? first[s * 32 + lane] : 0) - v[s] - off), FAR) << TAG_BITS) | tag[s] | closed[s];
     } else {
-      // a settled column's key is all ones from then on: `closed` keeps new keys from undercutting it
-      unsigned key[W], closed[W], k;
-      const auto* first = R.row(MS_AT(f, N));
 #pragma unroll
       for (int s = 0; s < W; ++s) {
-        closed[s] = in[s] ? 0u : NONE;
-        base[s] = in[s] ? packed(-v[s], tag[s]) : NONE;
-        key[s] = base[s] - ((unsigned)(in[s] ? first[s * 32 + lane] : 0) << TAG_BITS);
+        base[s] = ((unsigned)-v[s] << TAG_BITS) + tag[s];
+        key[s] = (base[s] + ((unsigned)(NARROW_BIAS - (in[s] ? (int)first[s * 32 + lane] : 0)) << TAG_BITS)) | closed[s];
       }
-      while (true) {   // every scan settles one more column
-        k = key[0];
+    }
+    while (true) {   // every scan settles one more column
+      k = key[0];
 #pragma unroll
-        for (int s = 1; s < W; ++s) k = min(k, key[s]);
-        k = __reduce_min_sync(FULL, k);
-        work[WK_SCAN]++;
-        if ((k & TAG_MATCHED) == 0u) break;
-        if (k == NONE) return false;
-        const int i = MS_AT((int)(k & 0xffu), N);
-        const auto* row = R.row(i);
-        const unsigned h = (unsigned)(sh.urow[i] - packed_dist(k));
+      for (int s = 1; s < W; ++s) k = min(k, key[s]);
+      k = __reduce_min_sync(FULL, k);
+      work[WK_SCAN]++;
+      if ((k & TAG_MATCHED) == 0u || k >= (WIDE ? FAR << TAG_BITS : NONE)) break;
+      const int i = MS_AT((int)(k & 0xffu), N);
+      const auto* row = R.row(i);
+      const int ui = sh.urow[i];
+#pragma unroll
+      for (int s = 0; s < W; ++s) {
+        if (key[s] == k) {   // (rows differ, so only the settled column has this key)
+          settled_at[s] = (int)(k >> TAG_BITS);
+          key[s] = closed[s] = NONE;
+        }
+        const int entry = in[s] ? (int)row[s * 32 + lane] : 0;
+        unsigned nk;
+        if constexpr (WIDE)
+          nk = (min((unsigned)((int)(k >> TAG_BITS) - v[s] - ui - entry), FAR) << TAG_BITS) | tag[s] | closed[s];
+        else
+          nk = ((k & ~TAG_MASK) + base[s] - ((unsigned)ui << TAG_BITS) - ((unsigned)entry << TAG_BITS)) | closed[s];
+        if (nk < key[s]) pred[s] = i;
+        key[s] = min(key[s], nk);
+      }
+    }
+    who = k & TAG_MASK;
+    mu = (int)(k >> TAG_BITS);
+    if constexpr (!WIDE) {
+      if (k == NONE) return false;
+      mu -= NARROW_BIAS;
+#pragma unroll
+      for (int s = 0; s < W; ++s) settled_at[s] -= NARROW_BIAS;
+    } else {
+      mu += off;
+#pragma unroll
+      for (int s = 0; s < W; ++s) settled_at[s] += off;
+      if (k >= FAR << TAG_BITS) {   // too far for a key
+        int d[W];
 #pragma unroll
         for (int s = 0; s < W; ++s) {
-          if (key[s] == k) {   // (rows differ, so only the settled column has this key)
-            settled_at[s] = packed_dist(k);
-            key[s] = closed[s] = NONE;
+          pred[s] = f;
+          closed[s] = in[s] ? 0u : NONE;
+          d[s] = in[s] ? -(int)first[s * 32 + lane] - v[s] : INF32;
+        }
+        while (true) {   // every scan settles one more column
+          nearest<W>(d, tag, mu, who);
+          work[WK_SCAN]++;
+          if (mu == INF32) return false;
+          if (who < TAG_MATCHED) break;
+          const int i = MS_AT((int)(who & 0xffu), N);
+          const auto* row = R.row(i);
+          const int h = sh.urow[i] - mu;
+#pragma unroll
+          for (int s = 0; s < W; ++s) {
+            if (tag[s] == who) {
+              closed[s] = NONE;
+              settled_at[s] = mu;
+              d[s] = INF32;
+            }
+            if (closed[s] == 0u) {
+              const int nd = -(int)row[s * 32 + lane] - v[s] - h;
+              if (nd < d[s]) { d[s] = nd; pred[s] = i; }
+            }
           }
-          const unsigned nk = (base[s] - (((unsigned)(in[s] ? row[s * 32 + lane] : 0) + h) << TAG_BITS)) | closed[s];
-          if (nk < key[s]) { key[s] = nk; pred[s] = i; }
         }
       }
-      mu = packed_dist(k);
-      who = k & TAG_MASK;
-#pragma unroll
-      for (int s = 0; s < W; ++s) done |= closed[s] & (1u << s);
     }
     // settled columns move their dual so that the shortest-path tree stays tight, and their rows' duals with them
 #pragma unroll
     for (int s = 0; s < W; ++s) {
       if (in[s]) {
-        if ((done >> s) & 1u) {
+        if (closed[s] != 0u) {
           v[s] += settled_at[s] - mu;
           sh.urow[tag[s] & 0xffu] += mu - settled_at[s];
         }
-        sh.pred[s * 32 + lane] = (short)pred[s];
+        sh.pred[s * 32 + lane] = (unsigned)pred[s] | (unsigned)(pred[s] == f ? 0 : sh.x[MS_AT(pred[s], N)]) << 16;
       }
     }
     sh.urow[f] = mu;   // every lane
@@ -324,13 +363,12 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
     // flip the path back to row f (every lane makes every update)
     int j = MS_AT((int)who, N);
     for (int it = 0; it <= N; ++it) {
-      const int i = MS_AT((int)sh.pred[j], N);
-      const int from = i == f ? j : MS_AT((int)sh.x[i], N);
-      __syncwarp();
+      const unsigned back = sh.pred[j];
+      const int i = MS_AT((int)(back & 0xffffu), N);
       sh.y[j] = (short)i;
       sh.x[i] = (short)j;
       if (i == f) break;
-      j = from;
+      j = MS_AT((int)(back >> 16), N);
     }
     __syncwarp();
 #pragma unroll
@@ -345,19 +383,26 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
 template <int W, int STORE>
 __device__ __forceinline__ void tight_graph(const Residual<STORE>& R, int N, int lane, const AssignShared& sh,
                                             const int (&v)[W], const PosTable<W>& tab) {
-#pragma unroll 4
-  for (int r = 0; r < N; ++r) {
-    const auto* row = R.row(r);
-    const int ur = sh.urow[r];
-    PosEntry<W> e;
-    e.row8 = (unsigned)r << 8;
+  constexpr int ROWS = W <= 4 ? 8 : 4;   // at a time (the last one again beyond the end)
+  for (int r0 = 0; r0 < N; r0 += ROWS) {
+    PosEntry<W> e[ROWS];
+    int at[ROWS];
 #pragma unroll
-    for (int s = 0; s < W; ++s) {
-      const int c = s * 32 + lane;
-      const int sum = c < N ? (int)row[c] + v[s] + ur : 1;
-      e.a[s] = __ballot_sync(FULL, sum == 0);
+    for (int q = 0; q < ROWS; ++q) {
+      const int r = min(r0 + q, N - 1);
+      const auto* row = R.row(r);
+      const int ur = sh.urow[r];
+      e[q].row8 = (unsigned)r << 8;
+      at[q] = MS_AT((int)sh.x[r], N);
+#pragma unroll
+      for (int s = 0; s < W; ++s) {
+        const int c = s * 32 + lane;
+        const int sum = c < N ? (int)row[c] + v[s] + ur : 1;
+        e[q].a[s] = __ballot_sync(FULL, sum == 0);
+      }
     }
-    tab.store(MS_AT((int)sh.x[r], N), e);
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) tab.store(at[q], e[q]);
   }
   __syncwarp();
 }
@@ -529,7 +574,7 @@ cudaError_t run_mw(int B, int N, const int32_t* demand, int k_max, uint8_t* perm
   // Shared memory limits how many matrices an SM holds. Where all of them fit half of it as int32 (the Birkhoff kernel often
   // runs beside), one launch takes every matrix; otherwise they are held as 16-bit entries, and a second launch takes those that do not fit (as int32,
   // over a 2-CTA cluster where one CTA cannot hold the matrix).
-  if (N < 48 || (as_int32 <= SMEM_LIMIT && (size_t)((B + sm_count() - 1) / sm_count()) * (as_int32 + 1024) <= SMEM_LIMIT / 2))
+  if (N <= 32 || (as_int32 <= SMEM_LIMIT && (size_t)((B + sm_count() - 1) / sm_count()) * (as_int32 + 1024) <= SMEM_LIMIT / 2))
     return launch_mw<0>(B, N, demand, k_max, perm, dur, count, residual, status, work, 0, stream);
   cudaError_t e = launch_mw<2>(B, N, demand, k_max, perm, dur, count, residual, status, work, 0, stream);
   if (e != cudaSuccess) return e;
