@@ -379,10 +379,13 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
 }
 
 // Tight edges under the optimal duals, row by row into the position table: entry (r, c) is tight iff its reduced cost
-// equals the row's dual. One vote per 32 columns gives a row's edges as a set.
+// equals the row's dual. One vote per 32 columns gives a row's edges as a set. highest: the highest row adjacent to each of
+// the lane's columns.
 template <int W, int STORE>
 __device__ __forceinline__ void tight_graph(const Residual<STORE>& R, int N, int lane, const AssignShared& sh,
-                                            const int (&v)[W], const PosTable<W>& tab) {
+                                            const int (&v)[W], const PosTable<W>& tab, int (&highest)[W]) {
+#pragma unroll
+  for (int s = 0; s < W; ++s) highest[s] = -1;
   constexpr int ROWS = W <= 4 ? 8 : 4;   // at a time (the last one again beyond the end)
   for (int r0 = 0; r0 < N; r0 += ROWS) {
     PosEntry<W> e[ROWS];
@@ -399,6 +402,7 @@ __device__ __forceinline__ void tight_graph(const Residual<STORE>& R, int N, int
         const int c = s * 32 + lane;
         const int sum = c < N ? (int)row[c] + v[s] + ur : 1;
         e[q].a[s] = __ballot_sync(FULL, sum == 0);
+        if (sum == 0) highest[s] = r;
       }
     }
 #pragma unroll
@@ -484,8 +488,9 @@ __global__ void __launch_bounds__(128) mw_kernel(int B, int N, const int32_t* __
       if (wide) ok = solve_assignment<W, STORE, STORE != 2>(R, N, lane, sh, v, work);
       else ok = solve_assignment<W, STORE, false>(R, N, lane, sh, v, work);
       if (!ok) { st_code = MOESCHED_ST_INTERNAL; break; }
-      tight_graph<W, STORE>(R, N, lane, sh, v, pl.tab);
-      pl.adopt();
+      int highest[W];
+      tight_graph<W, STORE>(R, N, lane, sh, v, pl.tab, highest);
+      pl.adopt(highest);
       pl.canonicalise(0u, work);
       // serve: the heaviest matched pair sets the duration; matched entries are sent whole
       int dmax = 0, served = 0;

@@ -197,8 +197,9 @@ struct Peeler {
     }
   }
 
-  // Takes over a complete matching from the table, as the graph of a new problem: nothing is known about it yet.
-  __device__ __forceinline__ void adopt() {
+  // Takes over a complete matching from the table, as the graph of a new problem. A row cannot move unless a row above it
+  // (highest: the highest one adjacent to the lane's column) could take its column; nothing more is known yet.
+  __device__ __forceinline__ void adopt(const int (&highest)[W]) {
     broken_count = 0;
     const unsigned low = (1u << lane) - 1u;
 #pragma unroll
@@ -216,7 +217,7 @@ struct Peeler {
           A[s][w] = e.a[w];
           if (w < s) lower |= e.a[w];
         }
-        chance[s] = lower != 0u ? UNKNOWN : 0;
+        chance[s] = highest[s] <= (int)(e.row8 >> 8) ? IN_VAIN : lower != 0u ? UNKNOWN : 0;
       }
     }
     __syncwarp();
