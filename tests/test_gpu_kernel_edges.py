@@ -1,0 +1,120 @@
+"""Sizes and values at which the kernels change their way of working, against the CPU oracle, bit for bit: whole warps and
+slabs of rows, chunks and batches of matchings, 16-bit and 32-bit entries, one-word and two-step distances, the quick and
+the ordinary division. (All results are whole numbers or defined operation by operation, so equality is the tolerance.)"""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2605_26845_b200 as ms
+from paper_2605_26845_b200.workload import DEFAULT_MODEL, PROFILED_MODEL, bvn_capacity, random_matrices
+
+pytestmark = pytest.mark.gpu
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def random_schedule(B, K, N, seed, high):
+    rng = np.random.default_rng(seed)
+    perm = np.argsort(rng.random((B, K, N)), axis=2).astype(np.uint8)
+    dur = rng.integers(0, high, size=(B, K)).astype(np.int32)
+    return perm, dur
+
+
+@pytest.mark.parametrize("K", [1, 31, 32, 33, 255, 256, 257, 520])
+@pytest.mark.parametrize("N,B,high", [(1, 3, 50), (32, 3, 900), (33, 700, 900), (64, 3, 900), (64, 1600, 900), (65, 3, 90000),
+                                      (128, 3, 900), (128, 320, 900), (192, 3, 90000), (193, 3, 900), (193, 3, 90000),
+                                      (256, 3, 900), (256, 3, 90000)])
+def test_scoring_at_the_edges_of_chunks_and_layouts(N, B, high, K):
+    """Batches that are resident with 32-bit entries, that are not, and matrices that need them split over two CTAs."""
+    few = 3
+    D = random_matrices(few, N, seed=100 * N + K, high=high)
+    perm, dur = random_schedule(few, K, N, N + K, 40)
+    count = np.array([K, max(0, K - 1), K // 2], np.int32)
+    which = np.arange(B) % few
+    d, p, q, c = dev(D[which]), dev(perm[which]), dev(dur[which]), dev(count[which])
+    for prefix in (False, True):
+        s = ms.schedule_eval(d, p, q, c, PROFILED_MODEL, prefix=prefix)
+        r = oracle.schedule_eval(D, perm, dur, count, PROFILED_MODEL, threads=8)
+        for name in ms.SCORE_FIELDS + ("status",):
+            assert (s[name].cpu().numpy() == r[name][which]).all(), name
+        if prefix:
+            rp = oracle.schedule_prefix_eval(D, perm, dur, count, PROFILED_MODEL, threads=8)
+            for name in ("prefix_overlap_ns", "prefix_unserved_tokens"):
+                assert (s[name].cpu().numpy() == rp[name][which]).all(), name
+
+
+@pytest.mark.parametrize("N", [5, 33, 64, 100])
+@pytest.mark.parametrize("offset", [1, 4, 15])
+def test_scoring_of_a_schedule_at_any_address(N, offset):
+    """The schedule is fetched in aligned groups of 16 bytes; its first byte may lie anywhere in one."""
+    B, K = 4, 70
+    D = random_matrices(B, N, seed=N, high=500)
+    perm, dur = random_schedule(B, K, N, N, 30)
+    count = np.array([70, 64, 33, 1], np.int32)
+    room = torch.zeros(perm.size + offset, dtype=torch.uint8, device="cuda")
+    p = room[offset:].view(B, K, N)
+    p.copy_(dev(perm))
+    perm[2, 5, 0] = perm[2, 5, 1] if N > 1 else 7            # one faulty schedule
+    p[2, 5, 0] = p[2, 5, 1]
+    s = ms.schedule_eval(dev(D), p, dev(dur), dev(count), DEFAULT_MODEL)
+    r = oracle.schedule_eval(D, perm, dur, count, DEFAULT_MODEL, threads=4)
+    assert list(r["status"]) == [0, 0, -1, 0]
+    for name in ms.SCORE_FIELDS + ("status",):
+        assert (s[name].cpu().numpy() == r[name]).all(), name
+
+
+@pytest.mark.parametrize("N", [4, 32, 33, 64, 72, 129, 200, 256])
+@pytest.mark.parametrize("high", [65535, 65536, 1 << 20, (1 << 20) + 1, 1 << 28])
+def test_greedy_at_the_edges_of_its_distances(N, high):
+    """Largest entries on either side of 16 bits and of the one-word distances, and so large that a search leaves the
+    range of a saturating one-word distance."""
+    D = random_matrices(2, N, seed=N, high=high)
+    D[0, 0, 0] = high
+    D[1] = np.where(D[1] % 3 == 0, 0, D[1])
+    K = 6 if N > 64 else 12
+    g = ms.mw_decompose(dev(D), K, want_residual=True)
+    r = oracle.mw_decompose(D, K, threads=8)
+    assert (g.status.cpu().numpy() == r["status"]).all() and (g.count.cpu().numpy() == r["count"]).all()
+    kk = np.arange(K)[None, :] < r["count"][:, None]
+    assert (g.perm.cpu().numpy()[kk] == r["perm"][kk]).all() and (g.dur.cpu().numpy()[kk] == r["dur"][kk]).all()
+    assert (g.extra.cpu().numpy() == r["residual"]).all()
+
+
+@pytest.mark.parametrize("N,smooth,iters", [(3, 0.0, 1200), (8, 0.0, 400), (16, 1e300, 3), (64, 1e-300, 3), (7, 0.5, 40),
+                                            (96, 0.5, 4), (97, 0.5, 4), (128, 0.5, 4), (160, 0.5, 3), (161, 0.5, 3)])
+def test_scaling_at_the_ends_of_the_exponent_range_and_of_the_layouts(N, smooth, iters):
+    """Without a perfect matching in the support some entries halve in every sweep, down to the subnormal numbers and zero."""
+    D = random_matrices(3, N, seed=N, high=300, zero_frac=0.0 if smooth == 0.0 else 0.3)
+    if smooth == 0.0:
+        D[:] = D + 1
+        D[:, :2, 1:] = 0                                     # two rows that reach the first column only
+        D[2] = np.triu(D[2] + 1)
+    g = ms.sinkhorn_scale(dev(D), iters, smooth, 20)
+    r = oracle.sinkhorn_scale(D, iters, smooth, 20, threads=8)
+    assert (g["status"].cpu().numpy() == r["status"]).all()
+    for name in ("scaled", "fixed", "stretch", "row_err"):
+        assert (g[name].cpu().numpy() == r[name]).all(), name
+
+
+def test_path_takes_smaller_batches_and_refuses_larger_ones():
+    path = ms.Path(40, 24, 10)
+    for B, N in ((40, 24), (7, 24), (9, 11)):
+        D = random_matrices(B, N, seed=B, high=400)
+        d = dev(D)
+        cap = path.k_bvn
+        for overlap in (True, False):
+            path.run(d, DEFAULT_MODEL, overlap=overlap)
+            r = oracle.bvn_decompose(D, cap, threads=8)
+            assert (path.bvn.count.cpu().numpy()[:B] == r["count"]).all()
+            perm = path.bvn.perm.view(-1)[:B * cap * N].view(B, cap, N).cpu().numpy()
+            kk = np.arange(cap)[None, :] < r["count"][:, None]
+            assert (perm[kk] == r["perm"][kk]).all()
+            rs = oracle.schedule_eval(D, r["perm"], r["coef"], r["count"], DEFAULT_MODEL, threads=8)
+            for i, name in enumerate(ms.SCORE_FIELDS):
+                assert (path.score_bvn[i, :B].cpu().numpy() == rs[name]).all(), name
+    with pytest.raises(ms.MoeschedError):
+        path.run(dev(random_matrices(41, 24, seed=1)))
+    assert bvn_capacity(24) == path.k_bvn
