@@ -223,33 +223,48 @@ struct Peeler {
     __syncwarp();
   }
 
-  // Row e takes column q (single: the set {q}) from row old8 >> 8: the table, the owner's registers, and the chances of
-  // the rows between the two that are adjacent to q and sit above it.
-  __device__ __forceinline__ void shift(int q, const unsigned (&single)[W], const PosEntry<W>& e, unsigned old8) {
-    tab.store(q, e);
-    const unsigned now = e.row8 | 0xffu, before = old8 | 0xffu, low = (1u << lane) - 1u;
-    const int change = e.row8 > old8 ? 1 : -1;
-    unsigned under[W];
-    below_mask<W>(single, under);
-    int own = 0;
+  // reaches[s]: the row at position s is adjacent to column q (single: the set {q}), which lies below its own.
+  __device__ __forceinline__ void adjacent_from_above(const unsigned (&single)[W], bool (&reaches)[W]) const {
+    const unsigned low = (1u << lane) - 1u;
 #pragma unroll
     for (int s = 0; s < W; ++s) {
       unsigned t = A[s][s] & single[s] & low;
 #pragma unroll
       for (int w = 0; w < s; ++w) t |= A[s][w] & single[w];
-      const bool above = key[s] > now;
-      if (t != 0u && above != (key[s] > before)) chance[s] += change;
-      own += __popc(__ballot_sync(FULL, above) & e.a[s] & under[s]);
+      reaches[s] = t != 0u;
     }
+  }
+  // The owner of position q (single: the set {q}) takes over row e.
+  __device__ __forceinline__ void settle(const unsigned (&single)[W], const PosEntry<W>& e, int its_chance) {
 #pragma unroll
     for (int s = 0; s < W; ++s) {
       if (mine(single, s)) {
         key[s] = e.row8 | (unsigned)(s * 32 + lane);
-        chance[s] = own;
+        chance[s] = its_chance;
 #pragma unroll
         for (int w = 0; w < W; ++w) A[s][w] = e.a[w];
       }
     }
+  }
+
+  // Row e takes column q (single: the set {q}) from row old8 >> 8: the table, the owner's registers, and the chances of
+  // the rows between the two that are adjacent to q and sit above it.
+  __device__ __forceinline__ void shift(int q, const unsigned (&single)[W], const PosEntry<W>& e, unsigned old8) {
+    tab.store(q, e);
+    const unsigned now = e.row8 | 0xffu, before = old8 | 0xffu;
+    const int change = e.row8 > old8 ? 1 : -1;
+    unsigned under[W];
+    below_mask<W>(single, under);
+    bool reaches[W];
+    adjacent_from_above(single, reaches);
+    int own = 0;
+#pragma unroll
+    for (int s = 0; s < W; ++s) {
+      const bool above = key[s] > now;
+      if (reaches[s] && above != (key[s] > before)) chance[s] += change;
+      own += __popc(__ballot_sync(FULL, above) & e.a[s] & under[s]);
+    }
+    settle(single, e, own);
   }
 
   // One search level: the positions of `alive` whose row is adjacent to a column of F become the new F. Returns the new
@@ -280,40 +295,24 @@ struct Peeler {
                                            const unsigned (&target)[W], const PosEntry<W>& f, bool settled) {
     tab.store(q, e);
     tab.store(p, f);
-    const unsigned ki = e.row8 | 0xffu, ku = f.row8 | 0xffu, low = (1u << lane) - 1u;
+    const unsigned ki = e.row8 | 0xffu, ku = f.row8 | 0xffu;
     unsigned under[W];
     below_mask<W>(root, under);
+    bool reaches_p[W], reaches_q[W];
+    adjacent_from_above(root, reaches_p);
+    adjacent_from_above(target, reaches_q);
     int own = 0;
 #pragma unroll
     for (int s = 0; s < W; ++s) {
-      unsigned tp = A[s][s] & root[s] & low, tq = A[s][s] & target[s] & low;
-#pragma unroll
-      for (int w = 0; w < s; ++w) {
-        tp |= A[s][w] & root[w];
-        tq |= A[s][w] & target[w];
-      }
       const bool above = key[s] > ku;
       own += __popc(__ballot_sync(FULL, above) & f.a[s] & under[s]);
       if (!above && key[s] > ki) {   // between the two: column q now holds a lower row, column p a higher one
-        if (tq != 0u) --chance[s];
-        if (tp != 0u) ++chance[s];
+        if (reaches_q[s]) --chance[s];
+        if (reaches_p[s]) ++chance[s];
       }
     }
-#pragma unroll
-    for (int s = 0; s < W; ++s) {
-      if (mine(target, s)) {
-        key[s] = e.row8 | (unsigned)(s * 32 + lane);
-        chance[s] = settled ? 0 : UNKNOWN;
-#pragma unroll
-        for (int w = 0; w < W; ++w) A[s][w] = e.a[w];
-      }
-      if (mine(root, s)) {
-        key[s] = f.row8 | (unsigned)(s * 32 + lane);
-        chance[s] = own;
-#pragma unroll
-        for (int w = 0; w < W; ++w) A[s][w] = f.a[w];
-      }
-    }
+    settle(target, e, settled ? 0 : UNKNOWN);
+    settle(root, f, own);
   }
 
   // Row e (of position p, single: root) takes column q (single: target), which its search has reached at `level`; the row
