@@ -398,10 +398,12 @@ struct Peeler {
   // repair_any(). Rows below lo8 >> 8 have their final column. False: some row cannot be matched any more (the matching of
   // the others is unchanged).
   __device__ __forceinline__ bool repair(unsigned& lo8, unsigned (&work)[MOESCHED_WORK_FIELDS]) {
+    unsigned alive[W];
+    int searched = -1;   // levels of a search that found nothing for the only free row
     if (broken_count == 1) {
       const int p = MS_AT(first_of<W>(broken), N);
       const PosEntry<W> e = tab.load(p);
-      unsigned alive[W], F[W], want[W], target[W], any = 0u;
+      unsigned F[W], want[W], target[W], any = 0u;
 #pragma unroll
       for (int s = 0; s < W; ++s) {
         alive[s] = __ballot_sync(FULL, key[s] > (e.row8 | 0xffu));   // the rows above r0
@@ -409,7 +411,7 @@ struct Peeler {
         want[s] = e.a[s] & alive[s];
         any |= want[s];
       }
-      if (any != 0u && !intersects<W>(broken, e.a)) {
+      if (any != 0u) {
         int q = first_of<W>(want, target), level = 0;
         unsigned pops = 0u;
         const bool hit = search(F, alive, target, level, work[WK_SCAN], pops);
@@ -430,15 +432,20 @@ struct Peeler {
           broken_count = 0;
           return true;
         }
+        // (with more words, what this keeps alive costs more than the search: N = 8 1.28 -> 1.15 us a matching, N = 100
+        // 4.39 -> 4.46, N = 256 17.9 -> 23.2)
+        if constexpr (W == 1) searched = level;
       }
     }
-    return repair_any(lo8, work);
+    return repair_any(lo8, searched, alive, work);
   }
 
   // The general case: free rows lowest first, each from all free columns. A row that is adjacent to none of the columns that
   // can be released above it: the highest row below r0 that could move to one of them is admitted, the search continues from
   // its column, and so on: the path disturbs as few low rows as possible, and lo8 drops to the lowest row it moves.
-  __device__ __forceinline__ bool repair_any(unsigned& lo8, unsigned (&work)[MOESCHED_WORK_FIELDS]) {
+  // searched >= 0: the only free row has been searched for so many levels; `left` are the rows above it that were not reached.
+  __device__ __forceinline__ bool repair_any(unsigned& lo8, int searched, const unsigned (&left)[W],
+                                             unsigned (&work)[MOESCHED_WORK_FIELDS]) {
     for (; broken_count > 0; --broken_count) {
       unsigned k = 0xffffffffu;
 #pragma unroll
@@ -453,18 +460,19 @@ struct Peeler {
       for (int s = 0; s < W; ++s) {
         above[s] = __ballot_sync(FULL, key[s] > (r8 | 0xffu));
         F[s] = broken[s];
-        alive[s] = above[s] & ~F[s];
+        alive[s] = searched >= 0 ? left[s] : above[s] & ~F[s];
         can[s] = e.a[s] & (above[s] | F[s]);
         any |= can[s];
         target[s] = admitted[s] = 0u;
       }
-      int q = any != 0u ? first_of<W>(can, target) : 0, level = 0;
+      int q = any != 0u ? first_of<W>(can, target) : 0, level = max(searched, 0);
       hist_store<W>(hist, 0, F, lane);
       bool lowered = false, settled = intersects<W>(F, target);
       unsigned pops = 0u;
       while (!settled) {
-        settled = search(F, alive, target, level, work[WK_SCAN], pops);
+        if (searched < 0) settled = search(F, alive, target, level, work[WK_SCAN], pops);
         if (settled) break;
+        searched = -1;
         unsigned released[W];
         any = 0u;
 #pragma unroll
