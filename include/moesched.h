@@ -112,10 +112,9 @@ typedef struct moesched_model {
  *                   0 shortest-path column scans, 1 augmentations, 2 rows
  *                   tried against their best column, 3 canonicalisation
  *                   sweeps that searched, 4 search levels, 5 rotation steps,
- *                   6 matchings, 7 rows matched along tight edges before the
- *                   shortest-path phase, 8 rows expanded by the canonicalisation
- *                   searches (frontier pops), 9 groups of columns settled together
- *                   (CTA-per-matrix kernel only; there 0 counts the rows relaxed)
+ *                   6 matchings, 7 rows matched before the shortest-path
+ *                   phase, 8 rows expanded by the canonicalisation searches
+ *                   (frontier pops), 9 not used (0)
  */
 int moesched_mw_decompose(int B, int N, const int32_t* d_demand, int k_max, uint8_t* d_perm,
                           int32_t* d_dur, int32_t* d_count, int32_t* d_residual,

@@ -4,13 +4,16 @@
 // matched entry reached zero are re-matched and the lexicographically smallest perfect matching is restored
 // (Peeler in peel.cuh).
 //
-// What bounds it: a dependent chain of searches, about 900 instructions per matching at N = 64. A full GPU (4096
+// What bounds it: a dependent chain of searches, about 1200 instructions per matching at N = 64. A full GPU (4096
 // matrices of 64 ranks) issues 2.5 instructions per cycle and SM, 70 % of the integer pipe; with one warp per scheduler
-// or less the time is the chain's latency (3.7 cycles per instruction). Against one row set per column with an
-// OR-reduction per word of every search level, B200: 4096 x N = 64 37.7 -> 27.3 ms, 1024 x N = 128 244 -> 150 ms,
-// 256 x N = 256 1152 -> 690 ms (that was with a CTA of eight warps per matrix), one N = 64 12.9 -> 8.3 ms.
+// or less the time is the chain's latency (3.3 cycles per instruction). Against one row set per column with an
+// OR-reduction per word of every search level, B200: 4096 x N = 64 37.7 -> 27.0 ms, 1024 x N = 128 244 -> 123 ms,
+// 256 x N = 256 1152 -> 523 ms (that was with a CTA of eight warps per matrix), one N = 64 12.9 -> 7.8 ms.
 // (Warps that slept while they were ahead of the others on their scheduler gained 4 % when a matching took 1700
-// instructions; now a full GPU takes 27.3 ms without and 27.4 ms with it.)
+// instructions; now a full GPU takes the same time with and without it. A team of two, four or eight warps per matrix that
+// exchanges its votes through shared memory is slower at every size, however few the matrices: 148 of 256 ranks, 1200
+// matchings, 20.7 -> 28.1, 25.2, 29.3 ms; three of 100 ranks 39.9 -> 57 ms with two. Every warp has to repeat the arithmetic
+// on whole sets, and a barrier per vote costs more than the divided tests save.)
 #include "peel.cuh"
 
 namespace moesched {
