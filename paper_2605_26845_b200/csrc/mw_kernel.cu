@@ -279,28 +279,45 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
         key[s] = (base[s] + ((unsigned)(NARROW_BIAS - (in[s] ? (int)first[s * 32 + lane] : 0)) << TAG_BITS)) | closed[s];
       }
     }
+    // AHEAD: the row is asked for before it is known whether the search goes on (a free column's number is a row's number
+    // too), so that the load and the test overlap: 148 x 256 ranks 42.9 -> 36.5 ms, 20 x 200 ranks 61.1 -> 54.4 ms, 1024 x 16 ranks
+    // 99 -> 95 us; with two words (4.8 -> 5.3 ms, 4096 x 64 ranks) and four (20.6 -> 22.1 ms, 1024 x 128) it does not pay.
+    // With two words the whole row is asked for after the test, then used: 4.83 -> 4.56 ms, one plan of 16 matchings 415 -> 389 us;
+    // with four that costs registers (20.1 -> 20.9 ms).
+    constexpr bool AHEAD = W == 1 || W == 8;
     while (true) {   // every scan settles one more column
       k = key[0];
 #pragma unroll
       for (int s = 1; s < W; ++s) k = min(k, key[s]);
       k = __reduce_min_sync(FULL, k);
       work[WK_SCAN]++;
-      if ((k & TAG_MATCHED) == 0u || k >= (WIDE ? FAR << TAG_BITS : NONE)) break;
-      const int i = MS_AT((int)(k & 0xffu), N);
+      const int i = MS_AT((int)(AHEAD ? min(k & 0xffu, (unsigned)(N - 1)) : k & 0xffu), N);   // (no row if k is NONE)
       const auto* row = R.row(i);
-      const int ui = sh.urow[i];
+      int ui, entry[W];
+      auto fetch = [&] {   // (the empty statements keep the loads where they are)
+        ui = sh.urow[i];
+        asm volatile("" : "+r"(ui));
+#pragma unroll
+        for (int s = 0; s < W; ++s) entry[s] = in[s] ? (int)row[s * 32 + lane] : 0;
+#pragma unroll
+        for (int s = 0; s < W; ++s) asm volatile("" : "+r"(entry[s]));
+      };
+      if constexpr (AHEAD) fetch();
+      if ((k & TAG_MATCHED) == 0u || k >= (WIDE ? FAR << TAG_BITS : NONE)) break;
+      if constexpr (W == 2) fetch();
+      if constexpr (W == 4) ui = sh.urow[i];
 #pragma unroll
       for (int s = 0; s < W; ++s) {
         if (key[s] == k) {   // (rows differ, so only the settled column has this key)
           settled_at[s] = (int)(k >> TAG_BITS);
           key[s] = closed[s] = NONE;
         }
-        const int entry = in[s] ? (int)row[s * 32 + lane] : 0;
+        if constexpr (W == 4) entry[s] = in[s] ? (int)row[s * 32 + lane] : 0;
         unsigned nk;
         if constexpr (WIDE)
-          nk = (min((unsigned)((int)(k >> TAG_BITS) - v[s] - ui - entry), FAR) << TAG_BITS) | tag[s] | closed[s];
+          nk = (min((unsigned)((int)(k >> TAG_BITS) - v[s] - ui - entry[s]), FAR) << TAG_BITS) | tag[s] | closed[s];
         else
-          nk = ((k & ~TAG_MASK) + base[s] - ((unsigned)ui << TAG_BITS) - ((unsigned)entry << TAG_BITS)) | closed[s];
+          nk = ((k & ~TAG_MASK) + base[s] - ((unsigned)ui << TAG_BITS) - ((unsigned)entry[s] << TAG_BITS)) | closed[s];
         if (nk < key[s]) pred[s] = i;
         key[s] = min(key[s], nk);
       }
