@@ -229,7 +229,11 @@ cudaError_t run_bvn(int B, int N, const int32_t* demand, int k_max, uint8_t* per
     switch (ge.cpl) {
       case 1: MOESCHED_GO(1, 2);
       case 2: MOESCHED_GO(2, 2);
+      case 3: MOESCHED_GO(3, 2);
       case 4: MOESCHED_GO(4, 2);
+      case 5: MOESCHED_GO(5, 2);
+      case 6: MOESCHED_GO(6, 2);
+      case 7: MOESCHED_GO(7, 2);
       default: MOESCHED_GO(8, 2);
     }
   }
@@ -243,7 +247,11 @@ cudaError_t run_bvn(int B, int N, const int32_t* demand, int k_max, uint8_t* per
   switch (ge.cpl) {
     case 1: MOESCHED_GO(1, 0);
     case 2: MOESCHED_GO(2, 0);
+    case 3: MOESCHED_GO(3, 0);
     case 4: MOESCHED_GO(4, 0);
+    case 5: MOESCHED_GO(5, 0);
+    case 6: MOESCHED_GO(6, 0);
+    case 7: MOESCHED_GO(7, 0);
     default: MOESCHED_GO(8, 0);
   }
 #undef MOESCHED_GO

@@ -147,7 +147,11 @@ cudaError_t run_bvn_real(int B, int N, const double* matrix, double tol, int k_m
   switch (ge.cpl) {
     case 1: MOESCHED_GO(1);
     case 2: MOESCHED_GO(2);
+    case 3: MOESCHED_GO(3);
     case 4: MOESCHED_GO(4);
+    case 5: MOESCHED_GO(5);
+    case 6: MOESCHED_GO(6);
+    case 7: MOESCHED_GO(7);
     default: MOESCHED_GO(8);
   }
 #undef MOESCHED_GO

@@ -140,16 +140,17 @@ __device__ __forceinline__ void cluster_epilogue() {
 // One row set of the search history (W words at hist + level * W). The set is uniform and EVERY lane stores
 // it (same address, same value: one shared-memory transaction), so that a lane which reads the history later
 // reads what it wrote itself, in program order: no warp barrier is needed between the store and the loads. The
-// matching x[] is kept the same way (every lane makes every update). Two words go in one 8-byte store, four
-// or eight in 16-byte stores (hist is 16-byte aligned and W * 4 divides 16 or is a multiple of it).
+// matching x[] is kept the same way (every lane makes every update). Four
+// or eight words go in 16-byte stores, two or six in 8-byte stores (hist is 16-byte aligned).
 template <int W>
 __device__ __forceinline__ void hist_store(unsigned* hist, int level, const unsigned (&F)[W], int /*lane*/) {
-  if constexpr (W == 2) {
-    *reinterpret_cast<uint2*>(hist + level * 2) = make_uint2(F[0], F[1]);
-  } else if constexpr (W % 4 == 0) {
+  if constexpr (W % 4 == 0) {
 #pragma unroll
     for (int q = 0; q < W; q += 4)
       *reinterpret_cast<uint4*>(hist + level * W + q) = make_uint4(F[q], F[q + 1], F[q + 2], F[q + 3]);
+  } else if constexpr (W % 2 == 0) {
+#pragma unroll
+    for (int q = 0; q < W; q += 2) *reinterpret_cast<uint2*>(hist + level * W + q) = make_uint2(F[q], F[q + 1]);
   } else {
 #pragma unroll
     for (int w = 0; w < W; ++w) hist[level * W + w] = F[w];
@@ -199,7 +200,7 @@ __device__ __forceinline__ long long fast_div(long long x, const FastDiv& f) {
 
 // ---- host-side launch geometry ---------------------------------------------------------------
 struct Geometry {
-  int cpl;       // columns per lane: 1, 2, 4 or 8
+  int cpl;       // columns per lane, 1 .. 8
   int S;         // shared-memory row stride in ints
   bool cluster;  // matrix split over a 2-CTA cluster
   int wpb;       // matrices per CTA

@@ -113,7 +113,7 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
     if (in[s]) sh.claim[s * 32 + lane] = NONE;
   }
   // ---- 1. rows name columns, several at a time; lane l keeps what rows l, l + 32, ... found ----
-  constexpr int ROWS = W <= 2 ? 8 : W == 4 ? 4 : 2;
+  constexpr int ROWS = W <= 2 ? 8 : W <= 4 ? 4 : 2;
   int u[W];
   unsigned named[W];
 #pragma unroll
@@ -284,7 +284,7 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
     // 99 -> 95 us; with two words (4.8 -> 5.3 ms, 4096 x 64 ranks) and four (20.6 -> 22.1 ms, 1024 x 128) it does not pay.
     // With two words the whole row is asked for after the test, then used: 4.83 -> 4.56 ms, one plan of 16 matchings 415 -> 389 us;
     // with four that costs registers (20.1 -> 20.9 ms).
-    constexpr bool AHEAD = W == 1 || W == 8;
+    constexpr bool AHEAD = W == 1 || W > 4;
     while (true) {   // every scan settles one more column
       k = key[0];
 #pragma unroll
@@ -305,14 +305,14 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
       if constexpr (AHEAD) fetch();
       if ((k & TAG_MATCHED) == 0u || k >= (WIDE ? FAR << TAG_BITS : NONE)) break;
       if constexpr (W == 2) fetch();
-      if constexpr (W == 4) ui = sh.urow[i];
+      if constexpr (W == 3 || W == 4) ui = sh.urow[i];
 #pragma unroll
       for (int s = 0; s < W; ++s) {
         if (key[s] == k) {   // (rows differ, so only the settled column has this key)
           settled_at[s] = (int)(k >> TAG_BITS);
           key[s] = closed[s] = NONE;
         }
-        if constexpr (W == 4) entry[s] = in[s] ? (int)row[s * 32 + lane] : 0;
+        if constexpr (W == 3 || W == 4) entry[s] = in[s] ? (int)row[s * 32 + lane] : 0;
         unsigned nk;
         if constexpr (WIDE)
           nk = (min((unsigned)((int)(k >> TAG_BITS) - v[s] - ui - entry[s]), FAR) << TAG_BITS) | tag[s] | closed[s];
@@ -583,7 +583,11 @@ static cudaError_t launch_mw(int B, int N, const int32_t* demand, int k_max, uin
     switch (ge.cpl) {
       case 1: MOESCHED_GO(1);
       case 2: MOESCHED_GO(2);
+      case 3: MOESCHED_GO(3);
       case 4: MOESCHED_GO(4);
+      case 5: MOESCHED_GO(5);
+      case 6: MOESCHED_GO(6);
+      case 7: MOESCHED_GO(7);
       default: MOESCHED_GO(8);
     }
   }

@@ -85,7 +85,8 @@ struct PosEntry {
 };
 template <int W>
 struct PosTable {
-  static constexpr int WORDS = W == 1 ? 2 : W == 2 ? 4 : W == 4 ? 8 : 12;   // per entry
+  static constexpr int WORDS = W == 1 ? 2 : (W + 4) / 4 * 4;   // per entry
+  static constexpr int WHOLE = W / 4 * 4;   // words of the mask that fill groups of 16 bytes
   unsigned* base;
   __device__ __forceinline__ PosEntry<W> load(int q) const {
     const unsigned* p = base + q * WORDS;
@@ -93,16 +94,23 @@ struct PosTable {
     if constexpr (W == 1) {
       const uint2 v = *reinterpret_cast<const uint2*>(p);
       e.a[0] = v.x; e.row8 = v.y;
-    } else if constexpr (W == 2) {
-      const uint4 v = *reinterpret_cast<const uint4*>(p);
-      e.a[0] = v.x; e.a[1] = v.y; e.row8 = v.z;
     } else {
 #pragma unroll
-      for (int k = 0; k < W; k += 4) {
+      for (int k = 0; k < WHOLE; k += 4) {
         const uint4 v = *reinterpret_cast<const uint4*>(p + k);
         e.a[k] = v.x; e.a[k + 1] = v.y; e.a[k + 2] = v.z; e.a[k + 3] = v.w;
       }
-      e.row8 = p[W];
+      if constexpr (W % 4 == 0) {
+        e.row8 = p[W];
+      } else if constexpr (W % 4 == 1) {
+        const uint2 v = *reinterpret_cast<const uint2*>(p + WHOLE);
+        e.a[WHOLE] = v.x; e.row8 = v.y;
+      } else {
+        const uint4 v = *reinterpret_cast<const uint4*>(p + WHOLE);
+        e.a[WHOLE] = v.x; e.a[WHOLE + 1] = v.y;
+        if constexpr (W % 4 == 3) { e.a[WHOLE + 2] = v.z; e.row8 = v.w; }
+        else e.row8 = v.z;
+      }
     }
     return e;
   }
@@ -111,20 +119,21 @@ struct PosTable {
     unsigned* p = base + q * WORDS;
     if constexpr (W == 1) {
       *reinterpret_cast<uint2*>(p) = make_uint2(e.a[0], e.row8);
-    } else if constexpr (W == 2) {
-      *reinterpret_cast<uint4*>(p) = make_uint4(e.a[0], e.a[1], e.row8, 0u);
     } else {
 #pragma unroll
-      for (int k = 0; k < W; k += 4)
+      for (int k = 0; k < WHOLE; k += 4)
         *reinterpret_cast<uint4*>(p + k) = make_uint4(e.a[k], e.a[k + 1], e.a[k + 2], e.a[k + 3]);
-      p[W] = e.row8;
+      if constexpr (W % 4 == 0) p[W] = e.row8;
+      else if constexpr (W % 4 == 1) *reinterpret_cast<uint2*>(p + WHOLE) = make_uint2(e.a[WHOLE], e.row8);
+      else if constexpr (W % 4 == 2) *reinterpret_cast<uint4*>(p + WHOLE) = make_uint4(e.a[WHOLE], e.a[WHOLE + 1], e.row8, 0u);
+      else *reinterpret_cast<uint4*>(p + WHOLE) = make_uint4(e.a[WHOLE], e.a[WHOLE + 1], e.a[WHOLE + 2], e.row8);
     }
   }
 };
 
 // Shared memory of one warp: position table, then the search levels (0 .. N).
 __host__ __device__ inline size_t peel_smem_bytes(int N, int W) {
-  const int words = W == 1 ? 2 : W == 2 ? 4 : W == 4 ? 8 : 12;
+  const int words = W == 1 ? 2 : (W + 4) / 4 * 4;
   return align16((size_t)N * words * 4) + align16((size_t)(N + 1) * W * 4);
 }
 

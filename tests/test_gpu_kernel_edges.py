@@ -118,3 +118,15 @@ def test_path_takes_smaller_batches_and_refuses_larger_ones():
     with pytest.raises(ms.MoeschedError):
         path.run(dev(random_matrices(41, 24, seed=1)))
     assert bvn_capacity(24) == path.k_bvn
+
+
+@pytest.mark.parametrize("N", [65, 95, 96, 97, 128, 129, 159, 160, 161, 191, 192, 193, 223, 224, 225])
+@pytest.mark.parametrize("high", [3, 2000, 90000])
+def test_decomposers_at_the_edges_of_their_words(N, high):
+    """One kernel per number of 32-column words a row set takes; tie-rich, 16-bit and 32-bit entries."""
+    D = random_matrices(2, N, seed=N + high, high=high)
+    for K, gpu, cpu, value in ((20, ms.mw_decompose, oracle.mw_decompose, "dur"), (60, ms.bvn_decompose, oracle.bvn_decompose, "coef")):
+        g, r = gpu(dev(D), K), cpu(D, K, threads=2)
+        assert (g.status.cpu().numpy() == r["status"]).all() and (g.count.cpu().numpy() == r["count"]).all()
+        kk = np.arange(K)[None, :] < r["count"][:, None]
+        assert (g.perm.cpu().numpy()[kk] == r["perm"][kk]).all() and (g.dur.cpu().numpy()[kk] == r[value][kk]).all()
