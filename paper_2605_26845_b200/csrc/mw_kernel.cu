@@ -282,9 +282,10 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
     // AHEAD: the row is asked for before it is known whether the search goes on (a free column's number is a row's number
     // too), so that the load and the test overlap: 148 x 256 ranks 42.9 -> 36.5 ms, 20 x 200 ranks 61.1 -> 54.4 ms, 1024 x 16 ranks
     // 99 -> 95 us; with two words (4.8 -> 5.3 ms, 4096 x 64 ranks) and four (20.6 -> 22.1 ms, 1024 x 128) it does not pay.
-    // With two words the whole row is asked for after the test, then used: 4.83 -> 4.56 ms, one plan of 16 matchings 415 -> 389 us;
-    // with four that costs registers (20.1 -> 20.9 ms).
-    constexpr bool AHEAD = W == 1 || W > 4;
+    // With two or three words the whole row is asked for after the test, then used: 4.83 -> 4.56 ms, one plan of 16 matchings
+    // 415 -> 389 us; with four to six that costs registers (20.1 -> 20.9 ms), and asking ahead is no better there (100 x 160 ranks
+    // 8.3 -> 9.1 ms).
+    constexpr bool AHEAD = W == 1 || W > 6;
     while (true) {   // every scan settles one more column
       k = key[0];
 #pragma unroll
@@ -304,15 +305,15 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
       };
       if constexpr (AHEAD) fetch();
       if ((k & TAG_MATCHED) == 0u || k >= (WIDE ? FAR << TAG_BITS : NONE)) break;
-      if constexpr (W == 2) fetch();
-      if constexpr (W == 3 || W == 4) ui = sh.urow[i];
+      if constexpr (W == 2 || W == 3) fetch();
+      if constexpr (W >= 4 && W <= 6) ui = sh.urow[i];
 #pragma unroll
       for (int s = 0; s < W; ++s) {
         if (key[s] == k) {   // (rows differ, so only the settled column has this key)
           settled_at[s] = (int)(k >> TAG_BITS);
           key[s] = closed[s] = NONE;
         }
-        if constexpr (W == 3 || W == 4) entry[s] = in[s] ? (int)row[s * 32 + lane] : 0;
+        if constexpr (W >= 4 && W <= 6) entry[s] = in[s] ? (int)row[s * 32 + lane] : 0;
         unsigned nk;
         if constexpr (WIDE)
           nk = (min((unsigned)((int)(k >> TAG_BITS) - v[s] - ui - entry[s]), FAR) << TAG_BITS) | tag[s] | closed[s];
@@ -403,10 +404,11 @@ __device__ __forceinline__ void tight_graph(const Residual<STORE>& R, int N, int
                                             const int (&v)[W], const PosTable<W>& tab, int (&highest)[W]) {
 #pragma unroll
   for (int s = 0; s < W; ++s) highest[s] = -1;
-  constexpr int ROWS = W <= 4 ? 8 : 4;   // at a time (the last one again beyond the end)
+  // Several at a time (the last one again beyond the end), all sums before the first vote: 1024 x 16 ranks 95 -> 90 us.
+  constexpr int ROWS = W <= 4 ? 8 : 4;
   for (int r0 = 0; r0 < N; r0 += ROWS) {
     PosEntry<W> e[ROWS];
-    int at[ROWS];
+    int at[ROWS], sum[ROWS][W];
 #pragma unroll
     for (int q = 0; q < ROWS; ++q) {
       const int r = min(r0 + q, N - 1);
@@ -417,10 +419,14 @@ __device__ __forceinline__ void tight_graph(const Residual<STORE>& R, int N, int
 #pragma unroll
       for (int s = 0; s < W; ++s) {
         const int c = s * 32 + lane;
-        const int sum = c < N ? (int)row[c] + v[s] + ur : 1;
-        e[q].a[s] = __ballot_sync(FULL, sum == 0);
-        if (sum == 0) highest[s] = r;
+        sum[q][s] = c < N ? (int)row[c] + v[s] + ur : 1;
+        if (sum[q][s] == 0) highest[s] = r;
       }
+    }
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) {
+#pragma unroll
+      for (int s = 0; s < W; ++s) e[q].a[s] = __ballot_sync(FULL, sum[q][s] == 0);
     }
 #pragma unroll
     for (int q = 0; q < ROWS; ++q) tab.store(at[q], e[q]);

@@ -172,10 +172,10 @@ struct Peeler {
   // whether the lane's position s is in the set
   __device__ __forceinline__ bool mine(const unsigned (&set)[W], int s) const { return (set[s] & (1u << lane)) != 0u; }
 
-  // Up to four words, the tests of all words are evaluated before the first vote, so that the votes follow one another and
+  // Up to six words, the tests of all words are evaluated before the first vote, so that the votes follow one another and
   // their latencies overlap, in place of a test and a vote in turn: one matrix of N = 64 8.13 -> 7.84 ms, three of N = 100
-  // 41.0 -> 39.7, 1024 of N = 128 18.7 -> 18.4. (With eight words, what this keeps alive costs more: 33.5 -> 34.7.)
-  static constexpr bool VOTES_LAST = W <= 4;
+  // 41.0 -> 39.7, 1024 of N = 128 18.7 -> 18.4, 100 of N = 160 13.4 -> 12.0. (With eight words, what this keeps alive costs more: 33.5 -> 34.7.)
+  static constexpr bool VOTES_LAST = W <= 6;
 
   // positions whose row is higher than that of key k
   __device__ __forceinline__ void rows_above(unsigned k, unsigned (&out)[W]) const {
@@ -381,10 +381,10 @@ struct Peeler {
         hist_load<W>(hist, level, h);
 #pragma unroll
         for (int w = 0; w < W; ++w) h[w] = level == 0 ? root[w] : h[w] & e.a[w];
-        if constexpr (W <= 4) {
+        if constexpr (W <= 6) {
           // rather a column that the row can have without displacing a lower one: that row would be searched again (N = 128:
           // 4.5 instead of 5.2 searches per matching, 23.5 -> 19.4 ms over 1024 x 3000 matchings; N = 64 27.9 -> 27.5 ms;
-          // at 256 columns the votes cost what the searches save)
+          // 100 x N = 192 17.0 -> 16.1 ms; with seven and eight words the votes cost what the searches save)
           unsigned G[W], some = 0u;
           rows_above(e.row8, G);
 #pragma unroll
