@@ -472,8 +472,9 @@ class Path:
     def run_graph(self, demand, model=None):
         """The same launches replayed from a CUDA graph: for small matrices the step is a handful of
         microsecond kernels and the cost of launching them one by one dominates. The graph is captured
-        on first use and again whenever the demand tensor's address or the model changes."""
-        key = (demand.data_ptr(), tuple(sorted((model or DEFAULT_MODEL).items())))
+        on first use and again whenever the demand tensor's address, its shape or the model changes."""
+        demand = _check_demand(demand)                   # also where the graph is replayed
+        key = (demand.data_ptr(), demand.device, demand.shape, tuple(sorted((model or DEFAULT_MODEL).items())))
         if getattr(self, "_graph_key", None) != key:
             self.run(demand, model)                      # first-use set-up outside the capture
             torch.cuda.current_stream(self.device).synchronize()
@@ -485,7 +486,11 @@ class Path:
         return self
 
     def run(self, demand, model=None, overlap=True):
-        """Enqueue the four kernels; results are ready when the caller's current stream reaches this point."""
+        """Enqueue the four kernels; results are ready when the caller's current stream reaches this point.
+
+        A smaller batch is taken too. Its results lie densely packed at the start of the buffers ([B, k, N] with its own
+        B and N), so with fewer matrices of the Path's own N they are rows 0 .. B-1 of outputs(); what lies behind them is
+        left as it was."""
         demand = _check_demand(demand)
         B, N, _ = demand.shape
         if B > self.B or N > self.N:

@@ -454,3 +454,33 @@ def test_graph_replay_gives_the_same_schedules():
         kk = torch.arange(a.perm.shape[1], device="cuda")[None, :] < b.count[:, None]
         assert (a.count == b.count).all() and (a.perm[kk] == b.perm[kk]).all() and (a.dur[kk] == b.dur[kk]).all()
     assert (path.score_bvn == other.score_bvn).all() and (path.score_mw == other.score_mw).all()
+
+
+def test_graph_replay_follows_the_shape_of_the_batch():
+    """Batches of several shapes can start at one address: a graph serves the shape that it was captured for only, and a
+    replay checks its input as a first call does."""
+    N, budget = 8, 8
+    D = make_demand(1, 64)
+    buf = dev(D)
+    path = ms.Path(64, N, budget)
+
+    def check(d):
+        B, n, _ = d.shape
+        for t in path.outputs():
+            t.fill_(77)
+        path.run_graph(d, DEFAULT_MODEL)
+        torch.cuda.synchronize()
+        for s, ref, key in ((path.mw, oracle.mw_decompose(d.cpu().numpy(), budget), "dur"),
+                            (path.bvn, oracle.bvn_decompose(d.cpu().numpy(), path.k_bvn), "coef")):
+            k = s.perm.shape[1]
+            part = ms.Schedule(s.perm.view(-1)[:B * k * n].view(B, k, n), s.dur[:B], s.count[:B], s.status[:B])
+            assert_schedule_equal(part, ref, key)
+            assert (s.count[B:] == 77).all()
+
+    other = buf.view(-1)[:5 * 6 * 6].view(5, 6, 6)
+    for d in (buf[:8], buf, buf[:40], buf, other, buf):
+        check(d)
+    for wrong in (buf.view(torch.float32), buf.transpose(1, 2), buf[0]):
+        assert wrong.data_ptr() == buf.data_ptr()
+        with pytest.raises(ms.MoeschedError):
+            path.run_graph(wrong, DEFAULT_MODEL)
