@@ -360,7 +360,8 @@ def schedule_eval(demand, perm, dur, count, model=None, out=None, status=None, p
         status = torch.empty(B, dtype=torch.int32, device=dev)
     K = int(perm.shape[1])
     pre = torch.empty((2, B, K), dtype=torch.int64, device=dev) if prefix else None
-    rows = scores.unbind(0)
+    # (a caller's own may be a sequence, and hold more)
+    rows = scores.unbind(0) if out is None else [out[i] for i in range(len(SCORE_FIELDS))]
     args = (B, N, _ptr(demand), K, _ptr(perm), _ptr(dur), _ptr(count), m[1], *(r.data_ptr() for r in rows), _ptr(status))
     res = dict(zip(SCORE_FIELDS, rows))
     if prefix:

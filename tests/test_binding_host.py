@@ -1,0 +1,36 @@
+"""What the Python binding hands to the library, seen from the host side (no GPU: the native call is recorded)."""
+import pytest
+import torch
+
+import paper_2605_26845_b200 as ms
+
+
+@pytest.fixture
+def calls(monkeypatch):
+    """Native calls made by the binding, as (name, arguments without the stream); CPU tensors are let through."""
+    made = []
+    monkeypatch.setattr(ms, "_dev", lambda t, dtype, what: t)
+    monkeypatch.setattr(ms, "_call", lambda name, device, *args: made.append((name, args)))
+    return made
+
+
+def schedule(B, N, K):
+    return (torch.zeros((B, N, N), dtype=torch.int32), torch.zeros((B, K, N), dtype=torch.uint8),
+            torch.zeros((B, K), dtype=torch.int32), torch.zeros(B, dtype=torch.int32))
+
+
+@pytest.mark.parametrize("prefix", [False, True])
+@pytest.mark.parametrize("form", ["five", "seven", "list", "slice"])
+def test_scores_go_where_the_caller_wants_them(calls, form, prefix):
+    """`out` may have rows to spare, be a sequence of tensors, or a part of a wider array."""
+    B = 3
+    out = {"five": torch.zeros((5, B), dtype=torch.int64), "seven": torch.zeros((7, B), dtype=torch.int64),
+           "list": [torch.zeros(B, dtype=torch.int64) for _ in range(5)],
+           "slice": torch.zeros((5, 2 * B), dtype=torch.int64)[:, B:]}[form]
+    status = torch.zeros(B, dtype=torch.int32)
+    res = ms.schedule_eval(*schedule(B, 4, 2), out=out, status=status, prefix=prefix)
+    (name, args), = calls
+    assert len(args) + 1 == len(ms._SIGNATURES[name])            # (the stream comes last)
+    assert list(args[8:13]) == [out[i].data_ptr() for i in range(5)] and args[13] == status.data_ptr()
+    for i, field in enumerate(ms.SCORE_FIELDS):
+        assert res[field].data_ptr() == out[i].data_ptr() and res[field].shape == (B,)
