@@ -308,19 +308,10 @@ def bvn_real_decompose(matrix, k_max=None, tol=1e-12) -> dict:
     return out
 
 
-_models = {}    # the few models a program uses, as the C structure; never changed once made
-
-
 def _model(model):
-    """Address of the C form of a model dict."""
-    key = tuple((model or DEFAULT_MODEL).items())
-    made = _models.get(key)
-    if made is None:
-        if len(_models) >= 256:
-            _models.clear()
-        made = _Model(**{k: int(v) for k, v in key})
-        made = _models[key] = (made, ctypes.addressof(made))
-    return made
+    """Reference to the C form of a model dict; it keeps the structure alive for as long as it is held itself, which a call's
+    arguments do until the call is over."""
+    return ctypes.byref(_Model(**{k: int(v) for k, v in (model or DEFAULT_MODEL).items()}))
 
 
 def ideal_a2a(demand, model=None) -> dict:
@@ -332,7 +323,7 @@ def ideal_a2a(demand, model=None) -> dict:
     m = _model(model)
     comm, makespan = torch.empty((2, B), dtype=torch.int64, device=dev).unbind(0)
     status = torch.empty(B, dtype=torch.int32, device=dev)
-    _call("moesched_ideal_a2a", dev, B, N, _ptr(demand), m[1], _ptr(comm), _ptr(makespan), _ptr(status))
+    _call("moesched_ideal_a2a", dev, B, N, _ptr(demand), m, _ptr(comm), _ptr(makespan), _ptr(status))
     return {"comm_ns": comm, "makespan_ns": makespan, "status": status}
 
 
@@ -362,7 +353,7 @@ def schedule_eval(demand, perm, dur, count, model=None, out=None, status=None, p
     pre = torch.empty((2, B, K), dtype=torch.int64, device=dev) if prefix else None
     # (a caller's own may be a sequence, and hold more)
     rows = scores.unbind(0) if out is None else [out[i] for i in range(len(SCORE_FIELDS))]
-    args = (B, N, _ptr(demand), K, _ptr(perm), _ptr(dur), _ptr(count), m[1], *(r.data_ptr() for r in rows), _ptr(status))
+    args = (B, N, _ptr(demand), K, _ptr(perm), _ptr(dur), _ptr(count), m, *(r.data_ptr() for r in rows), _ptr(status))
     res = dict(zip(SCORE_FIELDS, rows))
     if prefix:
         overlap, unserved = pre.unbind(0)
@@ -396,7 +387,7 @@ def schedule_order(demand, perm, dur, count, model=None) -> dict:
     makespan, emission = torch.empty((2, B), dtype=torch.int64, device=dev).unbind(0)
     rule, status = torch.empty((2, B), dtype=torch.int32, device=dev).unbind(0)
     scratch = torch.empty(max(8, int(lib.moesched_order_scratch_bytes(B, K))), dtype=torch.uint8, device=dev)
-    _call("moesched_schedule_order", dev, B, N, _ptr(demand), K, _ptr(perm), _ptr(dur), _ptr(count), m[1], _ptr(order),
+    _call("moesched_schedule_order", dev, B, N, _ptr(demand), K, _ptr(perm), _ptr(dur), _ptr(count), m, _ptr(order),
           _ptr(makespan), _ptr(emission), _ptr(rule), _ptr(status), _ptr(scratch))
     return {"order": order, "makespan_ns": makespan, "emission_ns": emission, "rule": rule, "status": status}
 
@@ -496,7 +487,7 @@ class Path:
         B, N, _ = demand.shape
         if B > self.B or N > self.N:
             raise MoeschedError("demand is larger than the Path was made for")
-        _call("moesched_path_run", demand.device, self._args_at, B, N, _ptr(demand), _model(model)[1], int(overlap))
+        _call("moesched_path_run", demand.device, self._args_at, B, N, _ptr(demand), _model(model), int(overlap))
         return self
 
 

@@ -34,3 +34,24 @@ def test_scores_go_where_the_caller_wants_them(calls, form, prefix):
     assert list(args[8:13]) == [out[i].data_ptr() for i in range(5)] and args[13] == status.data_ptr()
     for i, field in enumerate(ms.SCORE_FIELDS):
         assert res[field].data_ptr() == out[i].data_ptr() and res[field].shape == (B,)
+
+
+def test_a_call_owns_its_model(calls):
+    """The structure that the library reads belongs to the call that made it, whatever other models are used meanwhile, and
+    holds the values that the dict has at the time of the call."""
+    d, perm, dur, count = schedule(2, 4, 2)
+    link = torch.tensor(400)
+    model = dict(ms.DEFAULT_MODEL, link_gbps=link)
+    made = {}
+    for gbps in (400, 800):
+        link.fill_(gbps)
+        ms.schedule_eval(d, perm, dur, count, model)
+        ms.schedule_order(d, perm, dur, count, model)
+        ms.ideal_a2a(d, model)
+        made[gbps] = [args[at] for (_, args), at in zip(calls[-3:], (7, 7, 3))]
+    for other in range(300):
+        ms.ideal_a2a(d, dict(ms.DEFAULT_MODEL, reconfig_ns=other))
+    for gbps, structures in made.items():
+        for m in structures:
+            assert isinstance(m._obj, ms._Model) and m._obj.link_gbps == gbps
+            assert m._obj.bytes_per_token == ms.DEFAULT_MODEL["bytes_per_token"]
