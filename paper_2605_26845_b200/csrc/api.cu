@@ -57,6 +57,22 @@ void register_fault_reader(FaultReader reader) { fault_readers().push_back(reade
 static bool aligned4(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 3) == 0; }
 static bool aligned8(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 7) == 0; }
 
+// The argument checks of the entry points that moesched_path_run is made of.
+static bool size_ok(int B, int N, int k) { return B >= 0 && N >= 1 && N <= MOESCHED_MAX_N && k >= 1; }
+static bool mw_pointers_ok(const void* demand, const void* perm, const void* dur, const void* count, const void* residual,
+                           const void* status, const void* work) {
+  return demand && perm && dur && count && status && aligned4(demand) && aligned4(dur) && aligned4(count) &&
+         aligned4(status) && aligned4(residual) && aligned8(work);
+}
+static bool bvn_pointers_ok(const void* demand, const void* perm, const void* coef, const void* count, const void* aug,
+                            const void* scratch, const void* status, const void* work) {
+  return demand && perm && coef && count && status && aligned4(demand) && aligned4(coef) && aligned4(count) &&
+         aligned4(status) && aligned4(aug) && aligned8(work) && (reinterpret_cast<uintptr_t>(scratch) & 31) == 0;
+}
+static bool eval_pointers_ok(const void* demand, const void* perm, const void* dur, const void* count, const void* status) {
+  return demand && perm && dur && count && status && aligned4(demand) && aligned4(dur) && aligned4(count) && aligned4(status);
+}
+
 }  // namespace moesched
 
 using namespace moesched;
@@ -66,12 +82,9 @@ extern "C" {
 int moesched_mw_decompose(int B, int N, const int32_t* d_demand, int k_max, uint8_t* d_perm, int32_t* d_dur,
                           int32_t* d_count, int32_t* d_residual, int32_t* d_status, int64_t* d_work,
                           void* stream) {
-  if (B < 0 || N < 1 || N > MOESCHED_MAX_N || k_max < 1) return MOESCHED_EINVAL;
+  if (!size_ok(B, N, k_max)) return MOESCHED_EINVAL;
   if (B == 0) return MOESCHED_OK;
-  if (!d_demand || !d_perm || !d_dur || !d_count || !d_status) return MOESCHED_EINVAL;
-  if (!aligned4(d_demand) || !aligned4(d_dur) || !aligned4(d_count) || !aligned4(d_status) ||
-      !aligned4(d_residual) || !aligned8(d_work))
-    return MOESCHED_EINVAL;
+  if (!mw_pointers_ok(d_demand, d_perm, d_dur, d_count, d_residual, d_status, d_work)) return MOESCHED_EINVAL;
   cudaError_t e = run_mw(B, N, d_demand, k_max, d_perm, d_dur, d_count, d_residual, d_status,
                          reinterpret_cast<long long*>(d_work), static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? MOESCHED_OK : fail_cuda(e);
@@ -90,12 +103,9 @@ size_t moesched_workspace_bytes(int B, int N, int k_max) {
 int moesched_bvn_decompose(int B, int N, const int32_t* d_demand, int k_max, uint8_t* d_perm, int32_t* d_coef,
                            int32_t* d_count, int32_t* d_aug, int32_t* d_scratch, int32_t* d_status,
                            int64_t* d_work, void* stream) {
-  if (B < 0 || N < 1 || N > MOESCHED_MAX_N || k_max < 1) return MOESCHED_EINVAL;
+  if (!size_ok(B, N, k_max)) return MOESCHED_EINVAL;
   if (B == 0) return MOESCHED_OK;
-  if (!d_demand || !d_perm || !d_coef || !d_count || !d_status) return MOESCHED_EINVAL;
-  if (!aligned4(d_demand) || !aligned4(d_coef) || !aligned4(d_count) || !aligned4(d_status) || !aligned4(d_aug) ||
-      !aligned8(d_work) || (reinterpret_cast<uintptr_t>(d_scratch) & 31) != 0)
-    return MOESCHED_EINVAL;
+  if (!bvn_pointers_ok(d_demand, d_perm, d_coef, d_count, d_aug, d_scratch, d_status, d_work)) return MOESCHED_EINVAL;
   cudaError_t e = run_bvn(B, N, d_demand, k_max, d_perm, d_coef, d_count, d_aug, d_scratch, d_status,
                           reinterpret_cast<long long*>(d_work), static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? MOESCHED_OK : fail_cuda(e);
@@ -107,13 +117,12 @@ static int schedule_eval_impl(int B, int N, const int32_t* d_demand, int k_strid
                               int64_t* d_compute_idle_ns, int64_t* d_link_idle_tokens, int64_t* d_unserved_tokens,
                               int32_t* d_status, int64_t* d_prefix_overlap_ns, int64_t* d_prefix_unserved_tokens,
                               void* stream) {
-  if (B < 0 || N < 1 || N > MOESCHED_MAX_N || k_stride < 1) return MOESCHED_EINVAL;
+  if (!size_ok(B, N, k_stride)) return MOESCHED_EINVAL;
   if (B == 0) return MOESCHED_OK;
-  if (!d_demand || !d_perm || !d_dur || !d_count || !h_model || !d_makespan_overlap_ns ||
-      !d_makespan_serial_ns || !d_compute_idle_ns || !d_link_idle_tokens || !d_unserved_tokens || !d_status)
+  if (!eval_pointers_ok(d_demand, d_perm, d_dur, d_count, d_status) || !h_model || !d_makespan_overlap_ns ||
+      !d_makespan_serial_ns || !d_compute_idle_ns || !d_link_idle_tokens || !d_unserved_tokens)
     return MOESCHED_EINVAL;
-  if (!aligned4(d_demand) || !aligned4(d_dur) || !aligned4(d_count) || !aligned4(d_status) ||
-      !aligned8(d_makespan_overlap_ns) || !aligned8(d_makespan_serial_ns) || !aligned8(d_compute_idle_ns) ||
+  if (!aligned8(d_makespan_overlap_ns) || !aligned8(d_makespan_serial_ns) || !aligned8(d_compute_idle_ns) ||
       !aligned8(d_link_idle_tokens) || !aligned8(d_unserved_tokens) || !aligned8(d_prefix_overlap_ns) ||
       !aligned8(d_prefix_unserved_tokens))
     return MOESCHED_EINVAL;
@@ -155,12 +164,21 @@ int moesched_schedule_prefix_eval(int B, int N, const int32_t* d_demand, int k_s
 
 int moesched_path_run(const moesched_path_t* p, int B, int N, const int32_t* d_demand, const moesched_model_t* h_model,
                       int overlap, void* stream) {
-  if (p == nullptr || B < 0 || p->k_mw < 1 || p->k_mw > 0x7fffffff || p->k_bvn < 1 || p->k_bvn > 0x7fffffff || p->score_stride < B)
+  // everything is checked before anything is enqueued
+  if (p == nullptr || p->k_mw > 0x7fffffff || p->k_bvn > 0x7fffffff || p->k_mw < 1 || p->k_bvn < 1 || !size_ok(B, N, 1) ||
+      p->score_stride < B)
     return MOESCHED_EINVAL;
   if (B == 0) return MOESCHED_OK;
-  if (!p->d_mw_scores || !p->d_bvn_scores) return MOESCHED_EINVAL;
   const bool fork = overlap != 0 && p->side_stream != nullptr;
   if (fork && (!p->fork_event || !p->join_event)) return MOESCHED_EINVAL;
+  if (!bvn_pointers_ok(d_demand, p->d_bvn_perm, p->d_bvn_coef, p->d_bvn_count, nullptr, p->d_bvn_scratch, p->d_bvn_status,
+                       p->d_bvn_work) ||
+      !mw_pointers_ok(d_demand, p->d_mw_perm, p->d_mw_dur, p->d_mw_count, nullptr, p->d_mw_status, p->d_mw_work) ||
+      !eval_pointers_ok(d_demand, p->d_bvn_perm, p->d_bvn_coef, p->d_bvn_count, p->d_bvn_eval_status) ||
+      !eval_pointers_ok(d_demand, p->d_mw_perm, p->d_mw_dur, p->d_mw_count, p->d_mw_eval_status) ||
+      !p->d_mw_scores || !p->d_bvn_scores || !aligned8(p->d_mw_scores) || !aligned8(p->d_bvn_scores))
+    return MOESCHED_EINVAL;
+  if (h_model == nullptr || !model_in_range(*h_model)) return MOESCHED_EINVAL;
   const cudaStream_t main = static_cast<cudaStream_t>(stream);
   const cudaStream_t side = fork ? static_cast<cudaStream_t>(p->side_stream) : main;
   if (fork) {
