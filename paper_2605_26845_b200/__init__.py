@@ -449,13 +449,21 @@ class Path:
             self._events = (torch.cuda.Event(), torch.cuda.Event())      # fork, join
             for event in self._events:
                 event.record()                                           # an event gets its handle when first recorded
-        self._args = _PathArgs(
-            self.k_mw, self.k_bvn, B, _ptr(self.mw.perm), _ptr(self.bvn.perm), _ptr(self.mw.dur), _ptr(self.mw.count),
-            _ptr(self.mw.status), _ptr(self.eval_status_mw), _ptr(self.bvn.dur), _ptr(self.bvn.count),
-            _ptr(self.bvn.status), _ptr(self.eval_status_bvn), _ptr(self.mw.work), _ptr(self.bvn.work),
-            _ptr(self.score_mw), _ptr(self.score_bvn), _ptr(self.scratch), self._side.cuda_stream,
-            self._events[0].cuda_event, self._events[1].cuda_event)
-        self._args_at = ctypes.addressof(self._args)
+        self._made = (None, None)                                        # addresses, and the C form made of them
+
+    def _arguments(self):
+        """The C form of the buffers as they are at this call: a caller may have put others of the same shapes and types in
+        their place."""
+        mw, bvn = self.mw, self.bvn
+        at = (mw.perm.data_ptr(), bvn.perm.data_ptr(), mw.dur.data_ptr(), mw.count.data_ptr(), mw.status.data_ptr(),
+              self.eval_status_mw.data_ptr(), bvn.dur.data_ptr(), bvn.count.data_ptr(), bvn.status.data_ptr(),
+              self.eval_status_bvn.data_ptr(), _ptr(mw.work), _ptr(bvn.work), self.score_mw.data_ptr(),
+              self.score_bvn.data_ptr(), self.scratch.data_ptr())
+        made_of, args = self._made
+        if made_of != at:
+            args = _PathArgs(self.k_mw, self.k_bvn, self.B, *at, self._side.cuda_stream, *(e.cuda_event for e in self._events))
+            self._made = (at, args)
+        return args
 
     def outputs(self):
         return [self.mw.perm, self.mw.dur, self.mw.count, self.mw.status, self.bvn.perm, self.bvn.dur,
@@ -464,9 +472,9 @@ class Path:
     def run_graph(self, demand, model=None):
         """The same launches replayed from a CUDA graph: for small matrices the step is a handful of
         microsecond kernels and the cost of launching them one by one dominates. The graph is captured
-        on first use and again whenever the demand tensor's address, its shape or the model changes."""
+        on first use and again whenever the demand tensor's address, its shape, the model or one of the buffers changes."""
         demand = _check_demand(demand)                   # also where the graph is replayed
-        key = (demand.data_ptr(), demand.device, demand.shape, tuple(sorted((model or DEFAULT_MODEL).items())))
+        key = (demand.data_ptr(), demand.device, demand.shape, bytes(_model(model)._obj), bytes(self._arguments()))
         if getattr(self, "_graph_key", None) != key:
             self.run(demand, model)                      # first-use set-up outside the capture
             torch.cuda.current_stream(self.device).synchronize()
@@ -487,7 +495,7 @@ class Path:
         B, N, _ = demand.shape
         if B > self.B or N > self.N:
             raise MoeschedError("demand is larger than the Path was made for")
-        _call("moesched_path_run", demand.device, self._args_at, B, N, _ptr(demand), _model(model), int(overlap))
+        _call("moesched_path_run", demand.device, ctypes.byref(self._arguments()), B, N, _ptr(demand), _model(model), int(overlap))
         return self
 
 

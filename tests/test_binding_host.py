@@ -1,4 +1,6 @@
 """What the Python binding hands to the library, seen from the host side (no GPU: the native call is recorded)."""
+import contextlib
+
 import pytest
 import torch
 
@@ -55,3 +57,57 @@ def test_a_call_owns_its_model(calls):
         for m in structures:
             assert isinstance(m._obj, ms._Model) and m._obj.link_gbps == gbps
             assert m._obj.bytes_per_token == ms.DEFAULT_MODEL["bytes_per_token"]
+
+
+class FakeStream:
+    cuda_stream = 8
+
+
+class FakeEvent:
+    cuda_event = 16
+
+    def record(self, stream=None):
+        pass
+
+
+@pytest.fixture
+def path(calls, monkeypatch):
+    monkeypatch.setattr(torch.cuda, "device", lambda dev: contextlib.nullcontext())
+    monkeypatch.setattr(torch.cuda, "Stream", lambda *a, **k: FakeStream())
+    monkeypatch.setattr(torch.cuda, "Event", lambda *a, **k: FakeEvent())
+    return ms.Path(3, 4, 2, device="cpu", want_work=True)
+
+
+def test_a_path_uses_the_buffers_that_it_has_at_the_time_of_the_call(calls, path):
+    """Buffers are public: one that was replaced between two runs must neither be missed nor written to once it is gone."""
+    demand = torch.zeros((3, 4, 4), dtype=torch.int32)
+
+    def passed():
+        path.run(demand)
+        given = calls[-1][1][0]
+        args = ms._PathArgs.from_address(given) if isinstance(given, int) else given._obj
+        return {name: getattr(args, name) for name, _ in ms._PathArgs._fields_}
+
+    def expected():
+        return {"mw_perm": path.mw.perm, "bvn_perm": path.bvn.perm, "mw_dur": path.mw.dur, "mw_count": path.mw.count,
+                "mw_status": path.mw.status, "mw_eval_status": path.eval_status_mw, "bvn_coef": path.bvn.dur,
+                "bvn_count": path.bvn.count, "bvn_status": path.bvn.status, "bvn_eval_status": path.eval_status_bvn,
+                "mw_work": path.mw.work, "bvn_work": path.bvn.work, "mw_scores": path.score_mw,
+                "bvn_scores": path.score_bvn, "bvn_scratch": path.scratch}
+
+    def check():
+        got = passed()
+        for name, tensor in expected().items():
+            assert got[name] == (None if tensor is None else tensor.data_ptr()), name
+        assert (got["k_mw"], got["k_bvn"], got["score_stride"]) == (path.k_mw, path.k_bvn, 3)
+
+    check()
+    old = []
+    for holder, names in ((path.mw, ("perm", "dur", "count", "status", "work")), (path.bvn, ("perm", "dur", "count", "status", "work")),
+                          (path, ("score_mw", "score_bvn", "eval_status_mw", "eval_status_bvn", "scratch"))):
+        for name in names:
+            old.append(getattr(holder, name))
+            setattr(holder, name, torch.empty_like(old[-1]))
+            check()
+    path.mw.work = path.bvn.work = None
+    check()
