@@ -410,7 +410,9 @@ int moesched_bvn_decompose_static(int B, int N, const int32_t* d_demand, int k_m
  * decompositions do not depend on each other. With `overlap` the greedy one and its scoring are enqueued on
  * side_stream, which first waits for what `stream` holds at the time of the call (fork_event) and which `stream` waits
  * for at the end (join_event); without it, or with side_stream NULL, everything goes to `stream`. The streams and
- * events belong to the caller (cudaStream_t, cudaEvent_t); a call that finds the same side_stream busy queues up behind it.
+ * events belong to the caller (cudaStream_t, cudaEvent_t). Calls with the same buffers may come on different streams: with
+ * done_event, `stream` first waits for the last of them that was not captured, and done_event marks the end of this one (a
+ * captured call neither waits nor marks). With done_event NULL the caller keeps such calls apart.
  *
  *   B, N         in   size of this batch; all buffers hold at least B matrices of N x N, budgets k_mw and k_bvn
  *   scores       out  five int64 arrays each: overlap, serial, compute idle, link idle tokens, unserved tokens,
@@ -424,7 +426,7 @@ typedef struct moesched_path {
   int32_t *d_bvn_coef, *d_bvn_count, *d_bvn_status, *d_bvn_eval_status;
   int64_t *d_mw_work, *d_bvn_work, *d_mw_scores, *d_bvn_scores;
   int32_t* d_bvn_scratch;
-  void *side_stream, *fork_event, *join_event;
+  void *side_stream, *fork_event, *join_event, *done_event;
 } moesched_path_t;
 int moesched_path_run(const moesched_path_t* h_path, int B, int N, const int32_t* d_demand,
                       const moesched_model_t* h_model, int overlap, void* stream);

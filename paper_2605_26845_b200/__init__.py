@@ -40,7 +40,7 @@ class _PathArgs(ctypes.Structure):
                 [(n, ctypes.c_void_p) for n in (
                     "mw_perm", "bvn_perm", "mw_dur", "mw_count", "mw_status", "mw_eval_status", "bvn_coef", "bvn_count",
                     "bvn_status", "bvn_eval_status", "mw_work", "bvn_work", "mw_scores", "bvn_scores", "bvn_scratch",
-                    "side_stream", "fork_event", "join_event")])
+                    "side_stream", "fork_event", "join_event", "done_event")])
 
 
 _lib = None
@@ -446,7 +446,7 @@ class Path:
         self.scratch = torch.empty(max(1, bvn_scratch_bytes(B, N)), dtype=torch.uint8, device=dev)
         with torch.cuda.device(dev):
             self._side = torch.cuda.Stream(dev)
-            self._events = (torch.cuda.Event(), torch.cuda.Event())      # fork, join
+            self._events = tuple(torch.cuda.Event() for _ in range(3))   # fork, join, done
             for event in self._events:
                 event.record()                                           # an event gets its handle when first recorded
         self._made = (None, None)                                        # addresses, and the C form made of them
@@ -486,7 +486,8 @@ class Path:
         return self
 
     def run(self, demand, model=None, overlap=True):
-        """Enqueue the four kernels; results are ready when the caller's current stream reaches this point.
+        """Enqueue the four kernels; results are ready when the caller's current stream reaches this point. Runs of one Path
+        follow one another whatever streams they are called on (captured ones are ordered by their graph alone).
 
         A smaller batch is taken too. Its results lie densely packed at the start of the buffers ([B, k, N] with its own
         B and N), so with fewer matrices of the Path's own N they are rows 0 .. B-1 of outputs(); what lies behind them is

@@ -181,6 +181,16 @@ int moesched_path_run(const moesched_path_t* p, int B, int N, const int32_t* d_d
   if (h_model == nullptr || !model_in_range(*h_model)) return MOESCHED_EINVAL;
   const cudaStream_t main = static_cast<cudaStream_t>(stream);
   const cudaStream_t side = fork ? static_cast<cudaStream_t>(p->side_stream) : main;
+  // The Birkhoff part runs on the caller's stream, which need not be the one of the last call with these buffers.
+  // (An event from outside a capture must not be waited for inside, nor one from inside outside.)
+  cudaEvent_t done = static_cast<cudaEvent_t>(p->done_event);
+  if (done != nullptr) {
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(main, &capturing);
+    if (e == cudaSuccess && capturing != cudaStreamCaptureStatusNone) done = nullptr;
+    else if (e == cudaSuccess) e = cudaStreamWaitEvent(main, done, 0);
+    if (e != cudaSuccess) return fail_cuda(e);
+  }
   if (fork) {
     cudaError_t e = cudaEventRecord(static_cast<cudaEvent_t>(p->fork_event), main);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(side, static_cast<cudaEvent_t>(p->fork_event), 0);
@@ -204,7 +214,11 @@ int moesched_path_run(const moesched_path_t* p, int B, int N, const int32_t* d_d
   if (fork) {   // also after an error: what was enqueued on the side stream is joined
     cudaError_t e = cudaEventRecord(static_cast<cudaEvent_t>(p->join_event), side);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(main, static_cast<cudaEvent_t>(p->join_event), 0);
-    if (e != cudaSuccess && rc == MOESCHED_OK) return fail_cuda(e);
+    if (e != cudaSuccess && rc == MOESCHED_OK) rc = fail_cuda(e);
+  }
+  if (done != nullptr) {
+    cudaError_t e = cudaEventRecord(done, main);
+    if (e != cudaSuccess && rc == MOESCHED_OK) rc = fail_cuda(e);
   }
   return rc;
 }

@@ -64,7 +64,7 @@ def test_the_path_call_checks_everything_before_it_enqueues_anything(lib):
         p = ms._PathArgs(**dict(valid, **dict(args)))
         return lib.moesched_path_run(ctypes.byref(p), B, N, demand, ctypes.byref(m), overlap, None)
 
-    optional = {"mw_work", "bvn_work", "bvn_scratch", "side_stream"}
+    optional = {"mw_work", "bvn_work", "bvn_scratch", "side_stream", "done_event"}
     for overlap in (0, 1):
         for name in set(pointers) - optional - (set() if overlap else {"fork_event", "join_event"}):
             assert call(overlap=overlap, args={name: None}) == -1, name

@@ -484,3 +484,28 @@ def test_graph_replay_follows_the_shape_of_the_batch():
         assert wrong.data_ptr() == buf.data_ptr()
         with pytest.raises(ms.MoeschedError):
             path.run_graph(wrong, DEFAULT_MODEL)
+
+
+@pytest.mark.parametrize("overlap", [True, False])
+def test_runs_of_one_path_on_different_streams_follow_one_another(overlap):
+    """The caller does not order the streams that it runs a Path on: the buffers hold the results of the last run, with a
+    long run on another stream before it, and around a capture."""
+    N, B = 64, 40
+    long, short = dev(make_demand(3, B)), dev(random_matrices(3, 20, seed=3, high=50))
+    path = ms.Path(B, N, 16)
+    want = oracle.bvn_decompose(short.cpu().numpy(), path.k_bvn, threads=8)
+    greedy = oracle.mw_decompose(short.cpu().numpy(), 16, threads=8)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    torch.cuda.synchronize()
+    for capture in (False, True, False):
+        if capture:
+            path.run_graph(long)
+            torch.cuda.synchronize()
+        for stream, d in zip(streams, (long, short)):
+            with torch.cuda.stream(stream):
+                path.run(d, overlap=overlap)
+        streams[1].synchronize()
+        for s, ref, key in ((path.bvn, want, "coef"), (path.mw, greedy, "dur")):
+            k = s.perm.shape[1]
+            part = ms.Schedule(s.perm.view(-1)[:3 * k * 20].view(3, k, 20), s.dur[:3], s.count[:3], s.status[:3])
+            assert_schedule_equal(part, ref, key)
