@@ -21,6 +21,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "schedule_read.h"
 
 namespace moesched {
 
@@ -270,16 +271,18 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
   const int skew = (int)(reinterpret_cast<uintptr_t>(pb) & 15);   // a chunk is a multiple of 16 bytes: the same for all
   unsigned char* stage = base + L.stage;
   const size_t stage_bytes = align16((size_t)CHUNK * N + 16);
-  auto fetch = [&](int c) {   // chunk c into its buffer, as aligned groups of 16 bytes; nothing outside the schedule is read
+  const int lead = (int)min((size_t)15, (size_t)(pb - perm));   // bytes of the array that precede the matrix's
+  auto fetch = [&](int c) {   // chunk c into its buffer, as aligned groups of 16 bytes; nothing outside the schedules is read
     const int bytes = min(CHUNK, K - c * CHUNK) * N;
     const uint8_t* first = pb + (size_t)c * CHUNK * N;
     unsigned char* dst = stage + (c & 1) * stage_bytes;
     for (int g = t_here; g * 16 < bytes + skew; g += T_HERE) {
-      const int from = g * 16 - skew;   // offset of the group from the first byte
-      if (from < 0 && c == 0 && b == 0) {
-        for (int q = skew; q < 16 && q - skew < bytes; ++q) dst[q] = first[q - skew];
+      const int at = g * 16 - skew;   // offset of the group from the first byte
+      const ByteSpan s = group_span(c == 0 ? lead : 15, bytes, at);
+      if (s.from > 0) {
+        for (int q = s.from; q < s.to; ++q) dst[q] = first[at + q];   // (the first group: dst itself)
       } else {
-        async_copy16(dst + g * 16, first + from, min(16, bytes - from));
+        async_copy16(dst + g * 16, first + at, s.to);
       }
     }
   };

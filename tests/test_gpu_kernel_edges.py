@@ -66,6 +66,24 @@ def test_scoring_of_a_schedule_at_any_address(N, offset):
         assert (s[name].cpu().numpy() == r[name]).all(), name
 
 
+@pytest.mark.parametrize("N", [1, 2, 3, 4, 7])
+@pytest.mark.parametrize("K", [1, 2, 3])
+def test_scoring_of_schedules_shorter_than_a_group_of_bytes(N, K):
+    """Several matrices lie in the first 16 bytes; the array may begin anywhere in them."""
+    B = 9
+    D = random_matrices(B, N, seed=N, high=500)
+    perm, dur = random_schedule(B, K, N, 10 * N + K, 30)
+    count = (np.arange(B) % (K + 1)).astype(np.int32)
+    r = oracle.schedule_eval(D, perm, dur, count, DEFAULT_MODEL, threads=4)
+    for offset in range(16):
+        room = torch.full((perm.size + offset,), 255, dtype=torch.uint8, device="cuda")
+        p = room[offset:].view(B, K, N)
+        p.copy_(dev(perm))
+        s = ms.schedule_eval(dev(D), p, dev(dur), dev(count), DEFAULT_MODEL)
+        for name in ms.SCORE_FIELDS + ("status",):
+            assert (s[name].cpu().numpy() == r[name]).all(), (name, offset)
+
+
 @pytest.mark.parametrize("N", [4, 32, 33, 64, 72, 129, 200, 256])
 @pytest.mark.parametrize("high", [65535, 65536, 1 << 20, (1 << 20) + 1, 1 << 28])
 def test_greedy_at_the_edges_of_its_distances(N, high):
