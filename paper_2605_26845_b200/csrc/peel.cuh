@@ -12,8 +12,11 @@
 //   * a search record (the set of rows that could reach the searched one) stays with the position and is void as soon
 //     as one of its positions changes hands.
 // When a row moves to another column its mask and number move to another lane: a table in shared memory (one entry
-// per position, rewritten by every lane with the same values, so that a lane reads back its own stores and no
-// barrier is needed) makes them available to all lanes with one vector load.
+// per position, rewritten by every lane with the same values, so that a lane reads back its own stores) makes them
+// available to all lanes with one vector load. An entry is overwritten only once every lane has read what it held: a
+// vote keeps the lanes together but orders no memory, so shift(), exchange() and drop_edges() begin with a warp barrier
+// (three matrices of N = 100 41.3 -> 41.8 ms; barrier and stores at their end 42.0).
+// (What a search leaves in the history is likewise read before the rows are moved, and so before the next search.)
 // The matched values live in registers; the matrix in memory is touched only where a row moves (the value of the pair
 // that is given up goes back, the value of the new pair is fetched, and is not needed before the end of the step).
 // Against a layout that keeps, per column, the set of adjacent rows (rows stay where they are, a level needs an
@@ -28,9 +31,13 @@ namespace moesched {
 
 // 1 << n, and 0 for n outside 0 .. 31 (the shift of the machine clamps; the language leaves it open)
 __device__ __forceinline__ unsigned one_shl(int n) {
+#ifdef __CUDACC__
   unsigned r;
   asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(n));
   return r;
+#else   // (the CPU tests)
+  return n < 0 || n > 31 ? 0u : 1u << n;
+#endif
 }
 template <int W>
 __device__ __forceinline__ void single_mask(int q, unsigned (&m)[W]) {
@@ -278,6 +285,7 @@ struct Peeler {
   // Row e takes column q (single: the set {q}) from row old8 >> 8: the table, the owner's registers, and the chances of
   // the rows between the two that are adjacent to q and sit above it.
   __device__ __forceinline__ void shift(int q, const unsigned (&single)[W], const PosEntry<W>& e, unsigned old8) {
+    __syncwarp();   // the entry of q, and the levels that led there, have been read
     tab.store(q, e);
     const unsigned now = e.row8 | 0xffu, before = old8 | 0xffu;
     const int change = e.row8 > old8 ? 1 : -1;
@@ -329,6 +337,7 @@ struct Peeler {
   // holds a row above it.
   __device__ __forceinline__ void exchange(int p, const unsigned (&root)[W], const PosEntry<W>& e, int q,
                                            const unsigned (&target)[W], const PosEntry<W>& f, bool settled) {
+    __syncwarp();   // both entries, and the levels that led there, have been read
     tab.store(q, e);
     tab.store(p, f);
     const unsigned ki = e.row8 | 0xffu, ku = f.row8 | 0xffu;
@@ -359,7 +368,6 @@ struct Peeler {
   __device__ __forceinline__ void walk(int p, const unsigned (&root)[W], PosEntry<W> e, int q, unsigned (&target)[W], int level,
                                        bool settled) {
     unsigned P[W];
-    __syncwarp();
     q = MS_AT(q, N);
     if (level == 1) {
       const PosEntry<W> f = tab.load(q);
@@ -552,7 +560,6 @@ struct Peeler {
       unsigned P[W], lowest8 = r8;
 #pragma unroll
       for (int w = 0; w < W; ++w) P[w] = 0u;
-      __syncwarp();
       while (true) {
         const PosEntry<W> old = tab.load(MS_AT(q, N));
         shift(q, target, e, old.row8);
@@ -677,6 +684,7 @@ struct Peeler {
   // edges out and returns how many there were (uniform).
   __device__ __forceinline__ int drop_edges(unsigned zero) {
     broken_count = 0;
+    __syncwarp();   // every lane is done with the entries as they were
 #pragma unroll
     for (int s = 0; s < W; ++s) {
       const bool z = (zero >> s) & 1u;
