@@ -365,19 +365,19 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
         }
       }
     }
+#pragma unroll
+    for (int s = 0; s < W; ++s)
+      if (in[s]) sh.pred[s * 32 + lane] = (unsigned)pred[s] | (unsigned)(pred[s] == f ? 0 : sh.x[MS_AT(pred[s], N)]) << 16;
+    __syncwarp();   // (also: the scans have read the row duals)
     // settled columns move their dual so that the shortest-path tree stays tight, and their rows' duals with them
 #pragma unroll
     for (int s = 0; s < W; ++s) {
-      if (in[s]) {
-        if (closed[s] != 0u) {
-          v[s] += settled_at[s] - mu;
-          sh.urow[tag[s] & 0xffu] += mu - settled_at[s];
-        }
-        sh.pred[s * 32 + lane] = (unsigned)pred[s] | (unsigned)(pred[s] == f ? 0 : sh.x[MS_AT(pred[s], N)]) << 16;
+      if (in[s] && closed[s] != 0u) {
+        v[s] += settled_at[s] - mu;
+        sh.urow[tag[s] & 0xffu] += mu - settled_at[s];
       }
     }
     sh.urow[f] = mu;   // every lane
-    __syncwarp();
     // flip the path back to row f (every lane makes every update)
     int j = MS_AT((int)who, N);
     for (int it = 0; it <= N; ++it) {
