@@ -450,6 +450,7 @@ class Path:
             for event in self._events:
                 event.record()                                           # an event gets its handle when first recorded
         self._made = (None, None)                                        # addresses, and the C form made of them
+        self._arguments()
 
     def _arguments(self):
         """The C form of the buffers as they are at this call: a caller may have put others of the same shapes and types in
