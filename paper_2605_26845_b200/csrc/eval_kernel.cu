@@ -271,25 +271,24 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
   const int skew = (int)(reinterpret_cast<uintptr_t>(pb) & 15);   // a chunk is a multiple of 16 bytes: the same for all
   unsigned char* stage = base + L.stage;
   const size_t stage_bytes = align16((size_t)CHUNK * N + 16);
-  const int lead = (int)min((size_t)15, (size_t)(pb - perm));   // bytes of the array that precede the matrix's
-  auto fetch = [&](int c) {   // chunk c into its buffer, as aligned groups of 16 bytes; nothing outside the schedules is read
+  // chunk c into its buffer, as aligned groups of 16 bytes; nothing outside the schedules is read
+  auto fetch = [&](int c, auto is_first) {
     const int bytes = min(CHUNK, K - c * CHUNK) * N;
     const uint8_t* first = pb + (size_t)c * CHUNK * N;
     unsigned char* dst = stage + (c & 1) * stage_bytes;
     for (int g = t_here; g * 16 < bytes + skew; g += T_HERE) {
-      const int at = g * 16 - skew;   // offset of the group from the first byte
-      const ByteSpan s = group_span(c == 0 ? lead : 15, bytes, at);
-      if (s.from > 0) {
-        for (int q = s.from; q < s.to; ++q) dst[q] = first[at + q];   // (the first group: dst itself)
+      const int from = g * 16 - skew;   // offset of the group from the first byte
+      if (is_first && from < 0 && begins_before_the_array(pb - perm, skew)) {
+        for (int q = skew; q < 16 && q - skew < bytes; ++q) dst[q] = first[q - skew];
       } else {
-        async_copy16(dst + g * 16, first + at, s.to);
+        async_copy16(dst + g * 16, first + from, min(16, bytes - from));
       }
     }
   };
   const int chunks = bad ? 0 : (K + CHUNK - 1) / CHUNK;
   int dk_next = 0;
   if (chunks > 0) {
-    fetch(0);
+    fetch(0, std::true_type{});
     dk_next = lane < K ? db[lane] : 0;
   }
 
@@ -433,7 +432,7 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
     my_durs[lane] = NARROW ? min(max(dk_mine, 0), 65535) : max(dk_mine, 0);
     __syncwarp();
     if (c + 1 < chunks) {
-      fetch(c + 1);
+      fetch(c + 1, std::false_type{});
       const int k = (c + 1) * CHUNK + lane;
       dk_next = k < K ? db[k] : 0;
     }

@@ -3,22 +3,14 @@
 
 namespace moesched {
 
-struct ByteSpan {
-  int from, to;   // bytes [from, to) of a group of 16
-};
-
-// A chunk of `bytes` bytes that begins `ahead` bytes into the array (15 stands for all above) is read in groups of 16 aligned bytes; the group that
-// begins `at` bytes after the chunk's first byte (at > -16) is read in this span. A group may reach back into what precedes
-// the chunk as long as that belongs to the array; where it would begin before the array it is read from the chunk's
-// first byte on. Nothing behind the chunk is read.
+// A matrix's schedule is read in groups of 16 aligned bytes, the first of which begins `skew` bytes before it. That may be
+// part of the matrix before; where fewer than `skew` bytes of the array precede the schedule, the group would begin before
+// the array, and only the part from the schedule's first byte on is read.
 #ifdef __CUDACC__
 __host__ __device__
 #endif
-inline ByteSpan group_span(int ahead, int bytes, int at) {
-  ByteSpan s;
-  s.from = at + ahead < 0 ? -at : 0;
-  s.to = bytes - at < 16 ? bytes - at : 16;
-  return s;
+inline bool begins_before_the_array(long long ahead, int skew) {
+  return ahead < skew;
 }
 
 }  // namespace moesched

@@ -17,20 +17,19 @@ static int faults(int B, int N, int K, int used, int offset) {
       const long long ahead = (long long)b * K * N + (long long)c * 32 * N;
       const int bytes = (used - c * 32 < 32 ? used - c * 32 : 32) * N, skew = (int)((offset + ahead) & 15);
       for (int g = 0; g * 16 < bytes + skew; ++g) {
-        const int at = g * 16 - skew;
-        const moesched::ByteSpan s = moesched::group_span(ahead < 15 ? (int)ahead : 15, bytes, at);
-        if (s.from < 0 || s.from >= s.to || s.to > 16) return 1;
-        if (s.from > 0 && (g != 0 || s.from != skew)) return 2;   // only the first group is read in part, from the chunk on
-        for (int q = s.from; q < s.to; ++q) {
+        const int at = g * 16 - skew;   // offset of the group from the chunk's first byte
+        const bool cut = at < 0 && c == 0 && moesched::begins_before_the_array(ahead, skew);
+        const int from = cut ? skew : 0, to = bytes - at < 16 ? bytes - at : 16;
+        for (int q = from; q < to; ++q) {
           const long long byte = ahead + at + q;
-          if (byte < 0 || byte >= ahead + bytes) return 3;
+          if (byte < 0 || byte >= ahead + bytes) return 1;
           ++read[byte];
         }
       }
     }
   for (int b = 0; b < B; ++b)
     for (int i = 0; i < used * N; ++i)
-      if (read[(size_t)b * K * N + i] == 0) return 4;
+      if (read[(size_t)b * K * N + i] == 0) return 2;
   return 0;
 }
 int main() {
