@@ -308,10 +308,24 @@ def bvn_real_decompose(matrix, k_max=None, tol=1e-12) -> dict:
     return out
 
 
+_models = {}    # models of plain ints that have been used lately, in their C form (never changed once made)
+
+
 def _model(model):
     """Reference to the C form of a model dict; it keeps the structure alive for as long as it is held itself, which a call's
     arguments do until the call is over."""
-    return ctypes.byref(_Model(**{k: int(v) for k, v in (model or DEFAULT_MODEL).items()}))
+    items = tuple((model or DEFAULT_MODEL).items())
+    try:
+        made = _models.get(items)
+    except TypeError:           # a value that has no hash
+        made = None
+    if made is None:
+        made = _Model(**{k: int(v) for k, v in items})
+        if all(type(v) is int for _, v in items):   # (what else is equal to them has the same values)
+            if len(_models) >= 256:
+                _models.clear()
+            _models[items] = made
+    return ctypes.byref(made)
 
 
 def ideal_a2a(demand, model=None) -> dict:

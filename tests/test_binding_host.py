@@ -1,6 +1,7 @@
 """What the Python binding hands to the library, seen from the host side (no GPU: the native call is recorded)."""
 import contextlib
 
+import numpy as np
 import pytest
 import torch
 
@@ -57,6 +58,12 @@ def test_a_call_owns_its_model(calls):
         for m in structures:
             assert isinstance(m._obj, ms._Model) and m._obj.link_gbps == gbps
             assert m._obj.bytes_per_token == ms.DEFAULT_MODEL["bytes_per_token"]
+    for value in (torch.tensor(500), np.array(500), np.int64(500), 500.0):     # with a hash or without
+        ms.ideal_a2a(d, dict(ms.DEFAULT_MODEL, link_gbps=value))
+        assert calls[-1][1][3]._obj.link_gbps == 500
+    ms.ideal_a2a(d, dict(ms.DEFAULT_MODEL, link_gbps=400.9))
+    ms.ideal_a2a(d, dict(ms.DEFAULT_MODEL, link_gbps=401))
+    assert [args[3]._obj.link_gbps for _, args in calls[-2:]] == [400, 401]
 
 
 class FakeStream:
