@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
     unsigned char* dst = stage + (c & 1) * stage_bytes;
     for (int g = t_here; g * 16 < bytes + skew; g += T_HERE) {
       const int from = g * 16 - skew;   // offset of the group from the first byte
-      if (is_first && from < 0 && begins_before_the_array(pb - perm, skew)) {
+      if (decltype(is_first)::value && from < 0 && begins_before_the_array(pb - perm, skew)) {
         for (int q = skew; q < 16 && q - skew < bytes; ++q) dst[q] = first[q - skew];
       } else {
         async_copy16(dst + g * 16, first + from, min(16, bytes - from));
