@@ -206,6 +206,7 @@ cudaError_t run_bvn(int B, int N, const int32_t* demand, int k_max, uint8_t* per
   Geometry ge = plan_geometry(N);
 #define MOESCHED_GO(C, M)                                                                                     \
   do {                                                                                                        \
+    if (ge.max_shared) prefer_shared_memory(work != nullptr ? bvn_kernel<C, M, true> : bvn_kernel<C, M, false>); \
     if (work != nullptr)                                                                                      \
       return launch_warp_kernel(bvn_kernel<C, M, true>, ge, B, stream, B, N, ge.S, demand, k_max, perm, coef, \
                                 count, aug, scratch, status, work);                                       \
@@ -226,6 +227,10 @@ cudaError_t run_bvn(int B, int N, const int32_t* demand, int k_max, uint8_t* per
     // a small batch is spread one matrix per CTA so that no SM sits idle
     ge.wpb = B >= 16 * sm_count() ? 4 : 1;
     ge.smem = peel_smem_bytes(N, ge.cpl) * ge.wpb;
+    // Left to itself the driver divides an SM's memory for this kernel alone, and a greedy CTA of the same batch (149 KB at 256
+    // ranks) does not fit what is left beside a single one of these (18 KB of 164): the greedy part then waits until SMs
+    // are empty (whole path, 256 matrices of 256 ranks, 565 -> 646 ms).
+    ge.max_shared = ge.cpl == 8;
     switch (ge.cpl) {
       case 1: MOESCHED_GO(1, 2);
       case 2: MOESCHED_GO(2, 2);

@@ -206,6 +206,7 @@ struct Geometry {
   int wpb;       // matrices per CTA
   size_t smem;   // dynamic shared memory per CTA
   int threads_per_cta = 0;   // 0: one warp per matrix
+  bool max_shared = false;   // shared memory rather than L1, for kernels that run beside this one
 };
 Geometry plan_geometry(int N);
 constexpr size_t SMEM_LIMIT = 227 * 1024;   // shared memory one CTA may request on sm_100a
@@ -247,6 +248,13 @@ cudaError_t run_sinkhorn_durations(int B, int k_stride, const int32_t* coef, con
 cudaError_t run_bvn_real(int B, int N, const double* matrix, double tol, int k_max, uint8_t* perm, double* lambda,
                          int32_t* count, double* sum_lambda, double* max_left, double* scratch, int32_t* status,
                          cudaStream_t stream);
+
+// All of an SM's memory that can be shared memory is, while the kernel runs there. (A preference: failing is harmless.)
+template <typename Kernel>
+void prefer_shared_memory(Kernel kern) {
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess)
+    (void)cudaGetLastError();
+}
 
 // Launch helper shared by the three kernels.
 template <typename Kernel, typename... Args>

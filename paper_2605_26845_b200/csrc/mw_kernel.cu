@@ -41,6 +41,11 @@ struct AssignShared {
 __host__ __device__ inline size_t assign_smem_bytes(int N) {
   return 3 * align16((size_t)N * 4) + 2 * align16((size_t)N * 2);
 }
+// With eight words it lies in the Peeler's search levels: the assignment is done with once the tight edges are in the table,
+// before the first search, and the levels take 32 bytes a rank, so that a matrix of 232 ranks still fits as int32.
+__host__ __device__ inline size_t state_smem_bytes(int N, int W) {
+  return peel_smem_bytes(N, W) + (W == 8 ? 0 : assign_smem_bytes(N));
+}
 __device__ __forceinline__ AssignShared assign_shared(unsigned char* p, int N) {
   const size_t words = align16((size_t)N * 4), halves = align16((size_t)N * 2);
   AssignShared a;
@@ -453,11 +458,11 @@ __global__ void __launch_bounds__(128) mw_kernel(int B, int N, const int32_t* __
   R.N = N;
   R.split = CLUSTER ? (N + 1) / 2 : N;
   const size_t mat_bytes = align16((size_t)R.split * N * sizeof(T));
-  unsigned char* base = smem_raw + (size_t)warp * (mat_bytes + peel_smem_bytes(N, W) + assign_smem_bytes(N));
+  unsigned char* base = smem_raw + (size_t)warp * (mat_bytes + state_smem_bytes(N, W));
   R.near_ = R.far_ = reinterpret_cast<T*>(base);
   Peeler<W, int, false> pl;
   pl.reset(base + mat_bytes, N, lane);
-  const AssignShared sh = assign_shared(base + mat_bytes + peel_smem_bytes(N, W), N);
+  const AssignShared sh = assign_shared(base + mat_bytes + (W == 8 ? table_bytes(N, W) : peel_smem_bytes(N, W)), N);
   if constexpr (CLUSTER) {
     R.far_ = reinterpret_cast<T*>(map_to_cta(reinterpret_cast<int*>(R.near_), 1));
     cluster_sync_all();
@@ -564,7 +569,7 @@ __global__ void __launch_bounds__(128) mw_kernel(int B, int N, const int32_t* __
 
 static size_t mw_smem_per_warp(int N, int W, int store) {
   const int rows = store == 1 ? (N + 1) / 2 : N;
-  return align16((size_t)rows * N * (store == 2 ? 2 : 4)) + peel_smem_bytes(N, W) + assign_smem_bytes(N);
+  return align16((size_t)rows * N * (store == 2 ? 2 : 4)) + state_smem_bytes(N, W);
 }
 
 template <int STORE>

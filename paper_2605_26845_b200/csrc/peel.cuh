@@ -90,11 +90,18 @@ struct PosEntry {
   unsigned a[W];   // columns adjacent to the row
   unsigned row8;   // row << 8
 };
+// With eight words the row numbers lie apart, behind the masks: a padded entry would take 48 bytes, and a matrix of 230 to 232
+// ranks held as int32 next to the table would no longer fit one CTA (148 greedy ones of 232 ranks 55.8 -> 76.6 ms over two).
+__host__ __device__ constexpr int table_words(int W) { return W == 1 ? 2 : W == 8 ? 8 : (W + 4) / 4 * 4; }   // per entry
+__host__ __device__ inline size_t table_bytes(int N, int W) {
+  return align16((size_t)N * table_words(W) * 4) + (W == 8 ? align16((size_t)N * 4) : 0);
+}
 template <int W>
 struct PosTable {
-  static constexpr int WORDS = W == 1 ? 2 : (W + 4) / 4 * 4;   // per entry
+  static constexpr int WORDS = table_words(W);
   static constexpr int WHOLE = W / 4 * 4;   // words of the mask that fill groups of 16 bytes
   unsigned* base;
+  unsigned* rows;   // eight words only
   __device__ __forceinline__ PosEntry<W> load(int q) const {
     const unsigned* p = base + q * WORDS;
     PosEntry<W> e;
@@ -107,7 +114,9 @@ struct PosTable {
         const uint4 v = *reinterpret_cast<const uint4*>(p + k);
         e.a[k] = v.x; e.a[k + 1] = v.y; e.a[k + 2] = v.z; e.a[k + 3] = v.w;
       }
-      if constexpr (W % 4 == 0) {
+      if constexpr (W == 8) {
+        e.row8 = rows[q];
+      } else if constexpr (W % 4 == 0) {
         e.row8 = p[W];
       } else if constexpr (W % 4 == 1) {
         const uint2 v = *reinterpret_cast<const uint2*>(p + WHOLE);
@@ -130,7 +139,8 @@ struct PosTable {
 #pragma unroll
       for (int k = 0; k < WHOLE; k += 4)
         *reinterpret_cast<uint4*>(p + k) = make_uint4(e.a[k], e.a[k + 1], e.a[k + 2], e.a[k + 3]);
-      if constexpr (W % 4 == 0) p[W] = e.row8;
+      if constexpr (W == 8) rows[q] = e.row8;
+      else if constexpr (W % 4 == 0) p[W] = e.row8;
       else if constexpr (W % 4 == 1) *reinterpret_cast<uint2*>(p + WHOLE) = make_uint2(e.a[WHOLE], e.row8);
       else if constexpr (W % 4 == 2) *reinterpret_cast<uint4*>(p + WHOLE) = make_uint4(e.a[WHOLE], e.a[WHOLE + 1], e.row8, 0u);
       else *reinterpret_cast<uint4*>(p + WHOLE) = make_uint4(e.a[WHOLE], e.a[WHOLE + 1], e.a[WHOLE + 2], e.row8);
@@ -140,8 +150,7 @@ struct PosTable {
 
 // Shared memory of one warp: position table, then the search levels (0 .. N).
 __host__ __device__ inline size_t peel_smem_bytes(int N, int W) {
-  const int words = W == 1 ? 2 : (W + 4) / 4 * 4;
-  return align16((size_t)N * words * 4) + align16((size_t)(N + 1) * W * 4);
+  return table_bytes(N, W) + align16((size_t)(N + 1) * W * 4);
 }
 
 // The matrix in memory: rows [0, split) at near_, the rest in the partner CTA of a cluster (CLUSTER only).
@@ -202,7 +211,8 @@ struct Peeler {
     N = N_;
     lane = lane_;
     tab.base = reinterpret_cast<unsigned*>(smem);
-    hist = reinterpret_cast<unsigned*>(smem + align16((size_t)N * PosTable<W>::WORDS * 4));
+    tab.rows = tab.base + (size_t)N * PosTable<W>::WORDS;
+    hist = reinterpret_cast<unsigned*>(smem + table_bytes(N, W));
     broken_count = N;
 #pragma unroll
     for (int s = 0; s < W; ++s) {

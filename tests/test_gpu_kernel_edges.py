@@ -148,3 +148,16 @@ def test_decomposers_at_the_edges_of_their_words(N, high):
         assert (g.status.cpu().numpy() == r["status"]).all() and (g.count.cpu().numpy() == r["count"]).all()
         kk = np.arange(K)[None, :] < r["count"][:, None]
         assert (g.perm.cpu().numpy()[kk] == r["perm"][kk]).all() and (g.dur.cpu().numpy()[kk] == r[value][kk]).all()
+
+
+@pytest.mark.parametrize("N", [229, 230, 231, 232, 233])
+def test_where_one_cta_no_longer_holds_a_matrix(N):
+    """Up to 232 ranks an int32 matrix and the state of its warp fit the shared memory of one CTA, above they take two: greedy
+    with entries beyond 16 bits, Birkhoff without scratch."""
+    D = random_matrices(3, N, seed=N, high=300000, zero_frac=0.4)
+    for K, gpu, cpu, value in ((12, ms.mw_decompose, oracle.mw_decompose, "dur"),
+                               (40, lambda d, k: ms.bvn_decompose(d, k, scratch=False), oracle.bvn_decompose, "coef")):
+        g, r = gpu(dev(D), K), cpu(D, K, threads=3)
+        assert (g.status.cpu().numpy() == r["status"]).all() and (g.count.cpu().numpy() == r["count"]).all()
+        kk = np.arange(K)[None, :] < r["count"][:, None]
+        assert (g.perm.cpu().numpy()[kk] == r["perm"][kk]).all() and (g.dur.cpu().numpy()[kk] == r[value][kk]).all()

@@ -20,7 +20,7 @@ def program(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("N,pieces,k_max", [(3, 4, 9), (8, 14, 60), (17, 40, 30), (33, 60, 10), (64, 90, 8), (70, 40, 6)])
+@pytest.mark.parametrize("N,pieces,k_max", [(3, 4, 9), (8, 14, 60), (17, 40, 30), (33, 60, 10), (64, 90, 8), (70, 40, 6), (230, 12, 3)])
 def test_lanes_that_run_apart_find_the_same_schedule(program, N, pieces, k_max):
     rng = np.random.default_rng(N)
     A = np.zeros((N, N), np.int32)

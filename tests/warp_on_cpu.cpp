@@ -116,7 +116,7 @@ int main() {
   memory.resize(peel_smem_bytes(N, W) + 64);
   std::vector<std::thread> warp;
   for (int lane = 0; lane < 32; ++lane)
-    warp.emplace_back(W == 1 ? lane_main<1> : W == 2 ? lane_main<2> : lane_main<3>, lane);
+    warp.emplace_back(W == 1 ? lane_main<1> : W == 2 ? lane_main<2> : W == 3 ? lane_main<3> : lane_main<8>, lane);
   for (auto& t : warp) t.join();
   std::fwrite(&found, 4, 1, stdout);
   std::fwrite(coef.data(), 4, found, stdout);
