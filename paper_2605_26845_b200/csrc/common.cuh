@@ -1,7 +1,7 @@
 // Device-side building blocks shared by the kernels, and what the launchers share.
 //
 // In the decomposition kernels one warp owns one demand matrix; sets of rows or columns are bit masks of W 32-bit
-// words (W = 1, 2, 4 or 8), one bit per row or column; masks that every lane holds identically are "uniform".
+// words (W = 1 .. 8), one bit per row or column; masks that every lane holds identically are "uniform".
 #pragma once
 
 #include <cuda_runtime.h>
@@ -52,19 +52,6 @@ enum WorkField { WK_SCAN = 0, WK_AUG = 1, WK_TIGHT = 2, WK_SWEEP = 3, WK_LEVEL =
 // (Two-word masks take a 64-bit path: one wide shift instead of per-word selects.)
 __device__ __forceinline__ unsigned long long as64(const unsigned (&m)[2]) {
   return ((unsigned long long)m[1] << 32) | m[0];
-}
-template <int W>
-__device__ __forceinline__ void set_bit(unsigned (&m)[W], int idx) {
-  if constexpr (W == 2) {
-    const unsigned long long b = 1ull << idx;
-    m[0] |= (unsigned)b;
-    m[1] |= (unsigned)(b >> 32);
-    return;
-  }
-  const unsigned bit = 1u << (idx & 31);
-  const int wi = idx >> 5;
-#pragma unroll
-  for (int k = 0; k < W; ++k) m[k] |= (wi == k ? bit : 0u);
 }
 template <int W>
 __device__ __forceinline__ void clear_bit(unsigned (&m)[W], int idx) {
@@ -139,11 +126,11 @@ __device__ __forceinline__ void cluster_epilogue() {
 
 // One row set of the search history (W words at hist + level * W). The set is uniform and EVERY lane stores
 // it (same address, same value: one shared-memory transaction), so that a lane which reads the history later
-// reads what it wrote itself, in program order: no warp barrier is needed between the store and the loads. The
-// matching x[] is kept the same way (every lane makes every update). Four
+// reads what it wrote itself, in program order: no warp barrier is needed between the store and the loads (one is before
+// the next store there, see peel.cuh). The matching x[] is kept the same way (every lane makes every update). Four
 // or eight words go in 16-byte stores, two or six in 8-byte stores (hist is 16-byte aligned).
 template <int W>
-__device__ __forceinline__ void hist_store(unsigned* hist, int level, const unsigned (&F)[W], int /*lane*/) {
+__device__ __forceinline__ void hist_store(unsigned* hist, int level, const unsigned (&F)[W]) {
   if constexpr (W % 4 == 0) {
 #pragma unroll
     for (int q = 0; q < W; q += 4)

@@ -94,13 +94,12 @@ constexpr int BATCH = CHUNK * BATCH_CHUNKS;
 
 // Layout of the shared memory of one matrix. T: threads of the group (all CTAs of a cluster together), t_here: of this CTA.
 struct EvalLayout {
-  int column_bytes;   // entry (r, j) of a 32-bit slab (32 rows) or 16-bit slab (64 rows) at j * 128 in the slab
-  size_t slab, stage, marks, gmax, served, durs, maps, flags, total;
+  size_t slab,   // entry (r, j) of a 32-bit slab (32 rows) or 16-bit slab (64 rows) lies at j * 128 in it
+       stage, marks, gmax, served, durs, maps, flags, total;
   int mark_stride;
 };
 __host__ __device__ inline EvalLayout eval_layout(int N, int T, int slabs_here, int warps_here, bool prefix) {
   EvalLayout L;
-  L.column_bytes = 128;
   L.slab = (size_t)(N + 1) * 128;   // one column more than there are: where rows beyond N and bad destinations end up
   L.stage = (size_t)slabs_here * L.slab;
   L.mark_stride = T + 16;           // (a bad destination's mark may go behind the T bytes that are looked at)
@@ -156,8 +155,8 @@ __device__ __forceinline__ void async_copies_done() { asm volatile("cp.async.wai
 // schedule cut after k+1 matchings (entries beyond count, or all entries of a bad schedule, are -1).
 // JOBS (with PREFIX): the two per-matching arrays receive instead the job times of matching k in the
 // three-stage flow shop: reconfiguration + transfer time, and the time of its expert batch.
-// FULL: N is the number of threads, so that every address of a chunk is a constant away from the thread's own.
-template <int WARPS, bool NARROW, bool CLUSTER, bool PREFIX, bool JOBS, bool FULL>
+// EXACT: N is the number of threads, so that every address of a chunk is a constant away from the thread's own.
+template <int WARPS, bool NARROW, bool CLUSTER, bool PREFIX, bool JOBS, bool EXACT>
 __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
     eval_kernel(int B, int n_arg, const int32_t* __restrict__ demand, int k_stride, const uint8_t* __restrict__ perm,
                 const int32_t* __restrict__ dur, const int32_t* __restrict__ count, moesched_model_t model,
@@ -166,7 +165,7 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
                 int32_t* status, long long* __restrict__ prefix_overlap, long long* __restrict__ prefix_unserved,
                 int only_class) {
   constexpr int T_HERE = 32 * WARPS, T = CLUSTER ? 2 * T_HERE : T_HERE;
-  const int N = FULL ? T : n_arg;
+  const int N = EXACT ? T : n_arg;
   using Entry = typename std::conditional<NARROW, unsigned short, int>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31;
@@ -199,7 +198,7 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
   // thread -> row; threads without a row replay zeros in a spare column and mark a byte of their own
   const int row = NARROW ? (warp >> 1) * 64 + 2 * lane + (warp & 1) : rank * T_HERE + t_here;
   const int t = rank * T_HERE + t_here;
-  const bool in = FULL || row < N;
+  const bool in = EXACT || row < N;
   unsigned char* cells = base + (NARROW ? (size_t)(warp >> 1) * L.slab + lane * 4 + (warp & 1) * 2
                                         : (size_t)warp * L.slab + lane * 4);
   unsigned mark_at = 0u, mark_step = 1u, cell_step = 128u;
@@ -455,8 +454,8 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
       for (int q = 0; q < 8; ++q) {
         // a bad destination serves nothing and leaves a mark missing
         const unsigned col = min(j[q], (unsigned)N);
-        store_u8<CLUSTER>(mark_base + q * L.mark_stride + (FULL ? col : col * mark_step), stamp);
-        const unsigned cell = cell_base + col * (FULL ? 128u : cell_step);
+        store_u8<CLUSTER>(mark_base + q * L.mark_stride + (EXACT ? col : col * mark_step), stamp);
+        const unsigned cell = cell_base + col * (EXACT ? 128u : cell_step);
         const int val = load_entry<NARROW>(cell), sv = min(dk[q], val);
         store_entry<NARROW>(cell, max(val - dk[q], 0));
         const int g = __reduce_max_sync(FULL_MASK, sv);

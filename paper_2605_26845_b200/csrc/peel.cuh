@@ -442,7 +442,7 @@ struct Peeler {
       const bool hit = intersects<W>(F, target);
       level += any != 0u ? 1 : 0;
       if (hit || any == 0u) return hit;
-      hist_store<W>(hist, level, F, lane);
+      hist_store<W>(hist, level, F);
     }
   }
 
@@ -525,7 +525,7 @@ struct Peeler {
         target[s] = admitted[s] = 0u;
       }
       int q = any != 0u ? first_of<W>(can, target) : 0, level = max(searched, 0);
-      hist_store<W>(hist, 0, F, lane);
+      hist_store<W>(hist, 0, F);
       bool lowered = false, settled = intersects<W>(F, target);
       unsigned pops = 0u;
       while (!settled) {
@@ -558,7 +558,7 @@ struct Peeler {
         lowered = true;
         single_mask<W>((int)(k & 0xffu), F);
         ++level;
-        hist_store<W>(hist, level, F, lane);
+        hist_store<W>(hist, level, F);
         settled = intersects<W>(F, e.a);   // r0 is adjacent to the admitted row's own column
         q = settled ? (int)(k & 0xffu) : q;
 #pragma unroll
