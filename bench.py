@@ -117,16 +117,17 @@ def measured_peaks():
 
 
 def captured_traffic(name):
-    """DRAM bytes per launch from the committed ncu capture, or None once the kernel's source has
-    changed since the counters were taken."""
+    """DRAM bytes per launch from the committed ncu capture, or None once one of the files that make up the
+    kernel has changed since the counters were taken."""
     import hashlib
-    src = {"bvn_decompose": "bvn_kernel.cu", "mw_decompose": "mw_kernel.cu", "schedule_eval(bvn)": "eval_kernel.cu"}
+    src = {"bvn_decompose": ("peel.cuh", "bvn_kernel.cu"), "mw_decompose": ("peel.cuh", "mw_kernel.cu"),
+           "schedule_eval(bvn)": ("schedule_read.h", "eval_kernel.cu")}
     path = os.path.join(ROOT, "profiles", "dram_traffic_config3.txt")
     if name not in src or not os.path.exists(path):
         return None
     csrc = os.path.join(ROOT, "paper_2605_26845_b200", "csrc")
     h = hashlib.sha256()
-    for f in ("common.cuh", src[name]):
+    for f in ("common.cuh", *src[name]):
         with open(os.path.join(csrc, f), "rb") as fh:
             h.update(fh.read())
     for line in open(path):
@@ -161,7 +162,7 @@ def scalar_model_ops(work_mw, work_bvn, N):
 
 
 WORK_NAMES_MW = ("column_scans", "augmentations", "rows_bid", "searches", "search_levels", "rotation_steps",
-                 "matchings", "rows_matched_on_tight_edges", "frontier_pops", "settled_groups")
+                 "matchings", "rows_matched_before_the_searches", "frontier_pops", "unused")
 WORK_NAMES_BVN = ("repair_levels", "repair_path_steps", "canonical_repairs", "searches", "search_levels",
                   "rotation_steps", "matchings", "rows_skipped_as_prefix", "frontier_pops", "repair_fallbacks")
 

@@ -16,8 +16,8 @@
  *     (a cudaStream_t passed as void*, NULL = default stream) and the call
  *     returns at once. Buffers must stay alive until the stream has drained.
  *   - Matrices are int32, row major, [B][N][N], densely packed. 1 <= N <= 256.
- *     d_demand should be 16-byte aligned (it then takes the bulk-copy path for
- *     even N; any 4-byte aligned pointer is still accepted).
+ *     d_demand should be 16-byte aligned (scoring then loads 16 bytes at a time
+ *     where N is a multiple of 4; any 4-byte aligned pointer is accepted).
  *   - A matching is a permutation pi stored as N bytes: pi[i] = destination
  *     rank of source rank i. Schedules are [B][k_max][N] uint8 plus
  *     [B][k_max] int32 durations (in tokens); only the first count[b]
@@ -142,11 +142,12 @@ int moesched_mw_decompose(int B, int N, const int32_t* d_demand, int k_max, uint
  *   d_count    out  [B] int32
  *   d_aug      out  [B][N][N] int32 the balanced matrix A; may be NULL
  *   d_scratch  tmp  moesched_bvn_scratch_bytes(B, N) bytes of device memory, 32-byte
- *                   aligned, or NULL. With scratch the working copy of every matrix
- *                   lives there (it stays in L2) and shared memory is left for
+ *                   aligned, or NULL. With scratch the working copies of a large batch
+ *                   live there (they stay in L2) and shared memory is left for
  *                   bookkeeping, so several times more matrices are in flight per SM:
- *                   the fast path. Without it the matrix is held in shared memory
- *                   (a 2-CTA cluster for N > 232). Results are identical. Contents
+ *                   the fast path. Without it, and where the whole batch fits half of
+ *                   the SMs' shared memory (above 32 ranks), the matrix is held in shared
+ *                   memory (a 2-CTA cluster for N > 232). Results are identical. Contents
  *                   are undefined afterwards; calls that overlap in time need
  *                   separate scratch.
  *   d_status   out  [B] int32
