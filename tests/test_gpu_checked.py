@@ -80,8 +80,7 @@ def test_every_kernel_stays_in_bounds_and_agrees_with_the_oracle(checked, N):
 
 @pytest.mark.parametrize("cfg,B", [(3, 160), (5, 3)])
 def test_complete_decompositions_stay_in_bounds(checked, cfg, B):
-    """The late, sparse phase of a complete Birkhoff run, and a complete greedy run at 256 ranks (one
-    CTA per matrix), under the checks."""
+    """The late, sparse phase of a complete Birkhoff run, and a complete greedy run at 256 ranks, under the checks."""
     D = make_demand(cfg, B)
     d = dev(D)
     N = D.shape[1]
@@ -97,4 +96,35 @@ def test_complete_decompositions_stay_in_bounds(checked, cfg, B):
         kk = torch.arange(a.perm.shape[1], device="cuda")[None, :] < a.count[:, None]
         assert (a.count == b.count).all() and (a.status == b.status).all() and (a.status == 0).all()
         assert (a.perm[kk] == b.perm[kk]).all() and (a.dur[kk] == b.dur[kk]).all()
+    assert checked.debug_index_faults() == 0
+
+
+def many(D):
+    """The matrices over and over, until a batch held as int32 would take more than half of the SMs' shared memory."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    B = sms * (227 * 512 // (4 * D.shape[1] ** 2 + 1024)) + 1
+    return np.arange(B) % len(D)
+
+
+@pytest.mark.parametrize("N", [33, 64, 65, 100, 128, 160])
+def test_batches_that_are_not_resident_stay_in_bounds(checked, N):
+    """The launches of large batches: Birkhoff with its working copy in global memory, greedy with 16-bit entries."""
+    D = random_matrices(5, N, seed=12500 + N, kind="uniform", high=900, zero_frac=0.3)
+    which = many(D)
+    for K, gpu, cpu, value in ((12, checked.mw_decompose, oracle.mw_decompose, "dur"),
+                               (120, checked.bvn_decompose, oracle.bvn_decompose, "coef")):
+        same(gpu(dev(D[which]), K), {k: v[which] for k, v in cpu(D, K, threads=5).items() if k in ("status", "count", "perm", value)},
+             value)
+    assert checked.debug_index_faults() == 0
+
+
+def test_complete_decompositions_of_a_large_batch_stay_in_bounds(checked):
+    """64 ranks as the headline batch has them, every matching."""
+    D = make_demand(3, 24)
+    which = many(D)
+    v = checked.bvn_decompose(dev(D[which]), bvn_capacity(64))
+    g = checked.mw_decompose(dev(D[which]), 64)
+    for s, value, ref in ((v, "coef", oracle.bvn_decompose(D, bvn_capacity(64), threads=8)),
+                          (g, "dur", oracle.mw_decompose(D, 64, threads=8))):
+        same(s, {k: ref[k][which] for k in ("status", "count", "perm", value)}, value)
     assert checked.debug_index_faults() == 0

@@ -6,7 +6,7 @@ coefficient of up to 24 thousand matchings per matrix; written by tests/golden/m
 which calls the oracle only). Here the GPU result of the launch shape bench.py times is hashed the
 same way: the late, sparse phase of a Birkhoff run, where the records of earlier searches live
 longest, is compared with the oracle bit for bit and not only through invariants. The other
-placements of the working copy (shared memory / 2-CTA cluster, one warp or one CTA per matrix) must
+placements of the working copy (shared memory, 2-CTA cluster, a larger batch) must
 give the same bits as the benchmarked one on EVERY matrix at full depth.
 """
 import hashlib
@@ -78,9 +78,7 @@ def test_bvn_complete_schedules_match_the_oracle_digests(cfg, min_rows):
     same_schedules(other, s)
     del other
     if cfg == 5:
-        # 256 matrices go to the CTA-per-matrix kernel; a batch of at least eight matrices per SM takes
-        # the one-warp kernel with the working copy in global memory and its search records in shared
-        # memory: five copies of the batch make such a launch
+        # five copies of the batch make a launch with more matrices than the GPU holds at once
         reps = -(-8 * torch.cuda.get_device_properties(0).multi_processor_count // D.shape[0])
         big = d.repeat(reps, 1, 1)
         wide = ms.bvn_decompose(big, bvn_capacity(N))

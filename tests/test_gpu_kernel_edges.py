@@ -161,3 +161,19 @@ def test_where_one_cta_no_longer_holds_a_matrix(N):
         assert (g.status.cpu().numpy() == r["status"]).all() and (g.count.cpu().numpy() == r["count"]).all()
         kk = np.arange(K)[None, :] < r["count"][:, None]
         assert (g.perm.cpu().numpy()[kk] == r["perm"][kk]).all() and (g.dur.cpu().numpy()[kk] == r[value][kk]).all()
+
+
+@pytest.mark.parametrize("N", [33, 64, 65, 96, 97, 128, 129, 160, 161])
+def test_decomposers_in_batches_that_are_not_resident(N):
+    """A batch that does not fit half of the SMs' shared memory as int32 has its Birkhoff working copy in global memory and its
+    greedy residual as 16-bit entries, here with some matrices that do not fit those."""
+    D = random_matrices(5, N, seed=17 * N, high=3000)
+    D[3] *= 50
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    which = np.arange(sms * (227 * 512 // (4 * N * N + 1024)) + 1) % 5
+    for K, gpu, cpu, value in ((16, ms.mw_decompose, oracle.mw_decompose, "dur"), (70, ms.bvn_decompose, oracle.bvn_decompose, "coef")):
+        g, r = gpu(dev(D[which]), K), cpu(D, K, threads=5)
+        assert (g.status.cpu().numpy() == r["status"][which]).all() and (g.count.cpu().numpy() == r["count"][which]).all()
+        kk = (np.arange(K)[None, :] < r["count"][:, None])[which]
+        assert (g.perm.cpu().numpy()[kk] == r["perm"][which][kk]).all()
+        assert (g.dur.cpu().numpy()[kk] == r[value][which][kk]).all()

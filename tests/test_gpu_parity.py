@@ -39,7 +39,10 @@ def check_all(D, k_mw, k_bvn, model=DEFAULT_MODEL, threads=8):
     assert (g.extra.cpu().numpy()[ok] == rg["residual"][ok]).all()
     rv = oracle.bvn_decompose(D, k_bvn, threads=threads)
     ok = rv["status"] >= 0
-    for scratch in (True, False):       # global working copy / shared-memory (cluster) path
+    # Without scratch the matrix is held in shared memory (above 232 ranks by two CTAs). With it a small batch of 33 to about
+    # 160 ranks is too; larger ones and other sizes have their working copy in global memory (test_gpu_kernel_edges.py
+    # has batches that are not resident at each number of words).
+    for scratch in (True, False):
         v = ms.bvn_decompose(d, k_bvn, want_aug=True, scratch=scratch)
         assert_schedule_equal(v, rv, "coef")
         assert (v.extra.cpu().numpy()[ok] == rv["aug"][ok]).all()
@@ -72,9 +75,8 @@ def test_large_matrices_prefix(N, kw):
 
 @pytest.mark.parametrize("N,kw", [(129, KINDS[0]), (200, KINDS[2]), (256, KINDS[0]), (256, KINDS[1])])
 def test_team_kernel_deep_prefix(N, kw):
-    """Above 128 ranks a small batch runs the Birkhoff kernel that puts a CTA of eight warps on each
-    matrix: several hundred matchings deep against the oracle, and against the one-warp kernel
-    (shared-memory placement) on the same inputs."""
+    """Above 128 ranks, several hundred matchings deep against the oracle, with the working copy in global memory (from
+    about 160 ranks) and in shared memory."""
     D = random_matrices(2, N, seed=7000 + N, **kw)
     d = dev(D)
     K = 400
@@ -88,10 +90,8 @@ def test_team_kernel_deep_prefix(N, kw):
 
 @pytest.mark.parametrize("N,kw", [(129, KINDS[2]), (256, KINDS[0])])
 def test_one_warp_kernel_above_128_ranks_in_a_large_batch(N, kw):
-    """Above 128 ranks a batch of at least eight matrices per SM keeps one warp per matrix, with the
-    working copy in global memory and the search records in shared memory; a small batch of the same
-    matrices takes the CTA-per-matrix kernel. Both against the oracle on a sample, and against each
-    other on every matrix."""
+    """Above 128 ranks, a batch of at least eight matrices per SM, and a small batch of the same matrices (which at 129 ranks
+    is held in shared memory): every matrix against the oracle."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     base = random_matrices(37, N, seed=8100 + N, **kw)
     reps = -(-8 * sms // base.shape[0])
@@ -110,9 +110,8 @@ def test_one_warp_kernel_above_128_ranks_in_a_large_batch(N, kw):
 
 @pytest.mark.parametrize("N,per_sm", [(16, 14), (64, 13), (64, 27)])
 def test_paced_launch_of_a_resident_batch_gives_the_same_schedules(N, per_sm):
-    """From twelve matrices per SM up, when the whole batch is resident at once, the warps that share a
-    scheduler pace one another (a warp that is ahead sleeps). Timing only: the complete schedules must equal
-    those of the same matrices decomposed in a small, unpaced batch, and the oracle's."""
+    """Twelve and more matrices per SM, all resident at once: the complete schedules must equal those of the same matrices
+    decomposed in a small batch, and the oracle's, run after run."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     base = random_matrices(29, N, seed=8300 + N, **(KINDS[2] if N == 16 else KINDS[0]))
     reps = -(-per_sm * sms // base.shape[0])
@@ -122,7 +121,7 @@ def test_paced_launch_of_a_resident_batch_gives_the_same_schedules(N, per_sm):
     rv = oracle.bvn_decompose(base, K, threads=8)
     small = ms.bvn_decompose(dev(base), K)
     assert_schedule_equal(small, rv, "coef")
-    for _ in range(2):   # twice: entries of the pacing table left by the first launch must not matter
+    for _ in range(2):
         wide = ms.bvn_decompose(dev(D), K)
         torch.cuda.synchronize()
         for q in range(reps):
@@ -219,10 +218,10 @@ def test_link_time_for_any_link_speed_and_token_size(gbps):
 
 @pytest.mark.parametrize("N", [100, 129, 200, 256])
 def test_large_matrix_scoring_rejects_bad_schedules_and_scores_long_ones(N):
-    """Few large matrices are scored by the kernel that puts one CTA on each matrix: faulty schedules,
+    """Few large matrices: faulty schedules,
     a mix of narrow and wide matrices, and a schedule several chunks long, all against the oracle."""
     D = random_matrices(6, N, seed=9000 + N, kind="uniform", high=3000)
-    D[5, 1, 2] = 70000                        # one wide matrix: scored by the one-warp kernel
+    D[5, 1, 2] = 70000                        # one wide matrix
     d = dev(D)
     K = 75
     g = ms.mw_decompose(d, K)
@@ -245,7 +244,7 @@ def test_large_matrix_scoring_rejects_bad_schedules_and_scores_long_ones(N):
 @pytest.mark.parametrize("N", [4, 64, 200])
 def test_stage_sums_out_of_range_are_rejected_like_the_oracle_does(N):
     """Slowest link, largest token: transfer times that add up beyond 2^60 ns give BAD_INPUT, not a wrapped
-    makespan; just below the limit the 64-bit sums are still exact (one-warp and CTA-per-matrix kernels)."""
+    makespan; just below the limit the 64-bit sums are still exact."""
     K = 600
     D = random_matrices(3, N, seed=31 + N, kind="uniform", high=100)
     perm = np.tile(np.arange(N, dtype=np.uint8), (3, K, 1))

@@ -50,8 +50,7 @@ def test_static_entry_point_matches_regular_one_twice_in_a_row():
 def test_static_entry_point_against_the_oracle_without_touching_device_memory():
     """Checked against the CPU oracle here, not against the sibling entry point; and the call must leave the
     amount of free device memory exactly as it found it, which is the whole point for a caller
-    that cannot allocate. Two shapes: small matrices (one warp per matrix, four matrices per
-    CTA) and 200 ranks in a batch of two (one CTA of eight warps per matrix)."""
+    that cannot allocate. Two shapes: small matrices and 200 ranks in a batch of two."""
     cases = [(random_matrices(40, 24, seed=11, kind="uniform", high=50, zero_frac=0.4), bvn_capacity(24)),
              (random_matrices(2, 200, seed=12, kind="uniform", high=9, zero_frac=0.6), 300)]
     for D, k_max in cases:
