@@ -145,10 +145,22 @@ __device__ __forceinline__ void hist_store(unsigned* hist, int level, const unsi
 }
 template <int W>
 __device__ __forceinline__ void hist_load(const unsigned* hist, int level, unsigned (&H)[W]) {
-  if constexpr (W == 2) {
-    const uint2 v = *reinterpret_cast<const uint2*>(hist + level * 2);
-    H[0] = v.x;
-    H[1] = v.y;
+  if constexpr (W % 4 == 0) {
+#pragma unroll
+    for (int q = 0; q < W; q += 4) {
+      const uint4 v = *reinterpret_cast<const uint4*>(hist + level * W + q);
+      H[q] = v.x;
+      H[q + 1] = v.y;
+      H[q + 2] = v.z;
+      H[q + 3] = v.w;
+    }
+  } else if constexpr (W % 2 == 0) {
+#pragma unroll
+    for (int q = 0; q < W; q += 2) {
+      const uint2 v = *reinterpret_cast<const uint2*>(hist + level * W + q);
+      H[q] = v.x;
+      H[q + 1] = v.y;
+    }
   } else {
 #pragma unroll
     for (int w = 0; w < W; ++w) H[w] = hist[level * W + w];

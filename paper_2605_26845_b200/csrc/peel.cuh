@@ -192,6 +192,25 @@ struct Peeler {
   // their latencies overlap, in place of a test and a vote in turn: one matrix of N = 64 8.13 -> 7.84 ms, three of N = 100
   // 41.0 -> 39.7, 1024 of N = 128 18.7 -> 18.4, 100 of N = 160 13.4 -> 12.0. (With eight words, what this keeps alive costs more: 33.5 -> 34.7.)
   static constexpr bool VOTES_LAST = W <= 6;
+  // A row that has moved is read back from the table by the lane that it has moved to. Up to six words, where the row is needed again
+  // sooner than the load returns, that lane selects it from the copy that all lanes have. (Selecting, with seven and eight words:
+  // 100 of N = 224 334 ms, reading back 307; 256 of N = 256 531 and 530; with two words 10.6 and 11.9 for 1024 of N = 64.)
+  static constexpr bool RELOAD = W >= 7;
+  // The chances of a row that has moved are counted, or it is just looked at when its turn comes: a look in vain costs the same few
+  // operations per word for any W, counting grows with it (100 of N = 160 158.6 -> 154.7 ms, 100 of N = 192 171.4 -> 168.9, 256 of
+  // N = 256 530 -> 520, but one of N = 64 7.48 -> 7.75; with four words there is nothing in it).
+  static constexpr bool COUNTED = W <= 4;
+  // A branch that all lanes take together costs about 20 cycles of the chain, so the ways out of a search lead straight to what comes
+  // next instead of through a common test (one of N = 64 7.84 -> 7.47 ms, 4096 27.1 -> 25.9, 256 of N = 256 530 -> 514). Likewise:
+  // the first level, where most searches end, is taken apart and followed by the exchange (1024 of N = 16 271 -> 267 us, one of
+  // N = 64 7.47 -> 7.24 ms, 148 of N = 96 27.1 -> 26.4, 100 of N = 192 168.9 -> 165.3; 1024 of N = 128 123.7 -> 124.9; with eight words the
+  // code that this adds costs more: 514 -> 581);
+  static constexpr bool FIRST_APART = W <= 6;
+  // a first level without members has a way of its own (267 -> 261 us, 4096 of N = 64 26.0 -> 25.7 ms; 100 of N = 160 153.9 -> 158.3);
+  static constexpr bool NONE_APART = W <= 2;
+  // the lowest column wanted is found before it is known whether there is one (one of N = 64 7.20 -> 7.18 ms, 1024 10.48 -> 10.41, 148
+  // of N = 96 26.5 -> 26.4, 1024 of N = 128 124.9 -> 123.5; 1024 of N = 16 261 -> 265 us, 100 of N = 160 153.8 -> 157.8 ms).
+  static constexpr bool WANT_EARLY = W >= 2 && W <= 4;
 
   // positions whose row is higher than that of key k
   __device__ __forceinline__ void rows_above(unsigned k, unsigned (&out)[W]) const {
@@ -279,6 +298,18 @@ struct Peeler {
       reaches[s] = t != 0u;
     }
   }
+  // The owners of the positions of a set take over what the table says.
+  __device__ __forceinline__ void reload(const unsigned (&set)[W]) {
+#pragma unroll
+    for (int s = 0; s < W; ++s) {
+      if (mine(set, s)) {
+        const PosEntry<W> e = tab.load(s * 32 + lane);
+        key[s] = e.row8 | (unsigned)(s * 32 + lane);
+#pragma unroll
+        for (int w = 0; w < W; ++w) A[s][w] = e.a[w];
+      }
+    }
+  }
   // The owner of position q (single: the set {q}) takes over row e.
   __device__ __forceinline__ void settle(const unsigned (&single)[W], const PosEntry<W>& e, int its_chance) {
 #pragma unroll
@@ -303,16 +334,23 @@ struct Peeler {
     below_mask<W>(single, under);
     bool reaches[W];
     adjacent_from_above(single, reaches);
-    int own = 0;
+    int own = COUNTED ? 0 : UNKNOWN;
     unsigned higher[W];
-    if (VOTES_LAST) rows_above(now, higher);
+    if (VOTES_LAST && COUNTED) rows_above(now, higher);
 #pragma unroll
     for (int s = 0; s < W; ++s) {
       const bool above = key[s] > now;
       if (reaches[s] && above != (key[s] > before)) chance[s] += change;
-      own += __popc((VOTES_LAST ? higher[s] : __ballot_sync(FULL, above)) & e.a[s] & under[s]);
+      if constexpr (COUNTED) own += __popc((VOTES_LAST ? higher[s] : __ballot_sync(FULL, above)) & e.a[s] & under[s]);
     }
-    settle(single, e, own);
+    if constexpr (RELOAD) {
+      reload(single);
+#pragma unroll
+      for (int s = 0; s < W; ++s)
+        if (mine(single, s)) chance[s] = own;
+    } else {
+      settle(single, e, own);
+    }
   }
 
   // One search level: the positions of `alive` whose row is adjacent to a column of F become the new F. Returns the new
@@ -346,7 +384,7 @@ struct Peeler {
   // places: what a walk of one step comes to, and most walks are. `settled`: no column below q that row i is adjacent to
   // holds a row above it.
   __device__ __forceinline__ void exchange(int p, const unsigned (&root)[W], const PosEntry<W>& e, int q,
-                                           const unsigned (&target)[W], const PosEntry<W>& f, bool settled) {
+                                           const unsigned (&target)[W], const PosEntry<W>& f, bool settled = true) {
     __syncwarp();   // both entries, and the levels that led there, have been read
     tab.store(q, e);
     tab.store(p, f);
@@ -356,20 +394,36 @@ struct Peeler {
     bool reaches_p[W], reaches_q[W];
     adjacent_from_above(root, reaches_p);
     adjacent_from_above(target, reaches_q);
-    int own = 0;
+    int own = COUNTED ? 0 : UNKNOWN;
     unsigned higher[W];
-    if (VOTES_LAST) rows_above(ku, higher);
+    if (VOTES_LAST && COUNTED) rows_above(ku, higher);
 #pragma unroll
     for (int s = 0; s < W; ++s) {
       const bool above = key[s] > ku;
-      own += __popc((VOTES_LAST ? higher[s] : __ballot_sync(FULL, above)) & f.a[s] & under[s]);
+      if constexpr (COUNTED) own += __popc((VOTES_LAST ? higher[s] : __ballot_sync(FULL, above)) & f.a[s] & under[s]);
       if (!above && key[s] > ki) {   // between the two: column q now holds a lower row, column p a higher one
         if (reaches_q[s]) --chance[s];
         if (reaches_p[s]) ++chance[s];
       }
     }
-    settle(target, e, settled ? 0 : UNKNOWN);
-    settle(root, f, own);
+    if constexpr (RELOAD) {
+      unsigned both[W];
+#pragma unroll
+      for (int w = 0; w < W; ++w) both[w] = root[w] | target[w];
+      reload(both);
+#pragma unroll
+      for (int s = 0; s < W; ++s) {
+        if (mine(target, s)) chance[s] = settled ? 0 : UNKNOWN;
+        if (mine(root, s)) chance[s] = own;
+      }
+    } else {
+      settle(target, e, settled ? 0 : UNKNOWN);
+      settle(root, f, own);
+    }
+    unsigned P[W];
+#pragma unroll
+    for (int w = 0; w < W; ++w) P[w] = root[w] | target[w];
+    void_records(P);
   }
 
   // Row e (of position p, single: root) takes column q (single: target), which its search has reached at `level`; the row
@@ -378,43 +432,42 @@ struct Peeler {
   __device__ __forceinline__ void walk(int p, const unsigned (&root)[W], PosEntry<W> e, int q, unsigned (&target)[W], int level,
                                        bool settled) {
     unsigned P[W];
-    q = MS_AT(q, N);
-    if (level == 1) {
-      const PosEntry<W> f = tab.load(q);
-      exchange(p, root, e, q, target, f, settled);
-#pragma unroll
-      for (int w = 0; w < W; ++w) P[w] = root[w] | target[w];
-    } else {
-#pragma unroll
-      for (int w = 0; w < W; ++w) P[w] = 0u;
-      while (true) {
-        const PosEntry<W> old = tab.load(q);
-        shift(q, target, e, old.row8);
-#pragma unroll
-        for (int w = 0; w < W; ++w) P[w] |= target[w];
-        e = old;
-        if (level == 0) break;
-        --level;
-        unsigned h[W];
-        hist_load<W>(hist, level, h);
-#pragma unroll
-        for (int w = 0; w < W; ++w) h[w] = level == 0 ? root[w] : h[w] & e.a[w];
-        if constexpr (W <= 6) {
-          // rather a column that the row can have without displacing a lower one: that row would be searched again (N = 128:
-          // 4.5 instead of 5.2 searches per matching, 23.5 -> 19.4 ms over 1024 x 3000 matchings; N = 64 27.9 -> 27.5 ms;
-          // 100 x N = 192 17.0 -> 16.1 ms; with seven and eight words the votes cost what the searches save)
-          unsigned G[W], some = 0u;
-          rows_above(e.row8, G);
-#pragma unroll
-          for (int w = 0; w < W; ++w) {
-            G[w] &= h[w];
-            some |= G[w];
-          }
-#pragma unroll
-          for (int w = 0; w < W; ++w) h[w] = some != 0u && level != 0 ? G[w] : h[w];
-        }
-        q = (int)min((unsigned)first_of<W>(h, target), (unsigned)(N - 1));
+    PosEntry<W> f = tab.load(q);
+    if constexpr (!FIRST_APART) {
+      if (level == 1) {
+        exchange(p, root, e, q, target, f, settled);
+        return;
       }
+    }
+#pragma unroll
+    for (int w = 0; w < W; ++w) P[w] = 0u;
+    while (true) {
+      shift(q, target, e, f.row8);
+#pragma unroll
+      for (int w = 0; w < W; ++w) P[w] |= target[w];
+      e = f;
+      if (level == 0) break;
+      --level;
+      unsigned h[W];
+      hist_load<W>(hist, level, h);
+#pragma unroll
+      for (int w = 0; w < W; ++w) h[w] = level == 0 ? root[w] : h[w] & e.a[w];
+      if constexpr (W <= 6) {
+        // rather a column that the row can have without displacing a lower one: that row would be searched again (N = 128:
+        // 4.5 instead of 5.2 searches per matching, 23.5 -> 19.4 ms over 1024 x 3000 matchings; N = 64 27.9 -> 27.5 ms;
+        // 100 x N = 192 17.0 -> 16.1 ms; with seven and eight words the votes cost what the searches save)
+        unsigned G[W], some = 0u;
+        rows_above(e.row8, G);
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+          G[w] &= h[w];
+          some |= G[w];
+        }
+#pragma unroll
+        for (int w = 0; w < W; ++w) h[w] = some != 0u && level != 0 ? G[w] : h[w];
+      }
+      q = (int)min((unsigned)first_of<W>(h, target), (unsigned)(N - 1));
+      f = tab.load(q);
     }
     void_records(P);
   }
@@ -435,15 +488,25 @@ struct Peeler {
   __device__ __forceinline__ bool search(unsigned (&F)[W], unsigned (&alive)[W], const unsigned (&target)[W], int& level,
                                          unsigned& levels, unsigned& pops) const {
     while (true) {   // every level takes its members out of `alive`
-      const unsigned any = grow(F, alive);
-      ++levels;
-#pragma unroll
-      for (int w = 0; w < W; ++w) pops += __popc(F[w]);
-      const bool hit = intersects<W>(F, target);
-      level += any != 0u ? 1 : 0;
-      if (hit || any == 0u) return hit;
+      unsigned hit;
+      if (!step(F, alive, target, hit, levels, pops)) return false;
+      ++level;
+      if (hit != 0u) return true;
       hist_store<W>(hist, level, F);
     }
+  }
+  // One level of it; whether it has members. hit: not zero if one of them is the one searched for.
+  __device__ __forceinline__ bool step(unsigned (&F)[W], unsigned (&alive)[W], const unsigned (&target)[W], unsigned& hit,
+                                       unsigned& levels, unsigned& pops) const {
+    const unsigned any = grow(F, alive);
+    ++levels;
+    hit = 0u;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      pops += __popc(F[w]);
+      hit |= F[w] & target[w];
+    }
+    return any != 0u;
   }
 
   // ---- repair: every row that lost its entry gets a column again ----------------------------------
@@ -470,16 +533,35 @@ struct Peeler {
         any |= want[s];
       }
       if (any != 0u) {
-        int q = first_of<W>(want, target), level = 0;
-        unsigned pops = 0u;
-        const bool hit = search(F, alive, target, level, work[WK_SCAN], pops);
+        int q = MS_AT(first_of<W>(want, target), N), level = 0;
+        unsigned pops = 0u, hit1;
+        bool hit;
+        if constexpr (FIRST_APART) {
+          const bool some = step(F, alive, target, hit1, work[WK_SCAN], pops);
+          if (some && hit1 != 0u) {
+            work[WK_AUG]++;
+            work[WK_TIGHT]++;
+            exchange(p, broken, e, q, target, tab.load(q));
+            lo8 = min(lo8, e.row8 + 0x100u);
+            broken_count = 0;
+            return true;
+          }
+          hit = false;
+          if (some) {
+            level = 1;
+            hist_store<W>(hist, 1, F);
+            hit = search(F, alive, target, level, work[WK_SCAN], pops);
+          }
+        } else {
+          hit = search(F, alive, target, level, work[WK_SCAN], pops);
+        }
         if (!hit) {
           any = 0u;
 #pragma unroll
           for (int w = 0; w < W; ++w) { want[w] &= ~alive[w]; any |= want[w]; }
           if (any != 0u) {   // the next best column
-            q = first_of<W>(want, target);
-            level = level_of_row<W>(hist, level, MS_AT(q, N), lane);
+            q = MS_AT(first_of<W>(want, target), N);
+            level = level_of_row<W>(hist, level, q, lane);
           }
         }
         if (hit || any != 0u) {
@@ -524,7 +606,7 @@ struct Peeler {
         any |= can[s];
         target[s] = admitted[s] = 0u;
       }
-      int q = any != 0u ? first_of<W>(can, target) : 0, level = max(searched, 0);
+      int q = any != 0u ? MS_AT(first_of<W>(can, target), N) : 0, level = max(searched, 0);
       hist_store<W>(hist, 0, F);
       bool lowered = false, settled = intersects<W>(F, target);
       unsigned pops = 0u;
@@ -640,6 +722,8 @@ struct Peeler {
         any |= want[s];
         F[s] = root[s];
       }
+      int q = 0, level = FIRST_APART ? 1 : 0;
+      if constexpr (WANT_EARLY) q = first_of<W>(want, target);   // (meaningless if there is none)
       if (any == 0u) {   // (after a record has become void) none: counted from here on
 #pragma unroll
         for (int s = 0; s < W; ++s)
@@ -648,8 +732,35 @@ struct Peeler {
       }
       work[WK_SWEEP]++;
       work[WK_POP]++;
-      int q = first_of<W>(want, target), level = 0;
-      const bool hit = search(F, alive, target, level, work[WK_LEVEL], work[WK_POP]);
+      if constexpr (!WANT_EARLY) q = first_of<W>(want, target);
+      q = MS_AT(q, N);
+      bool hit = false;
+      if constexpr (FIRST_APART) {
+        unsigned hit1;
+        const bool some = step(F, alive, target, hit1, work[WK_LEVEL], work[WK_POP]);
+        if (NONE_APART && !some) {   // nobody can take its column
+#pragma unroll
+          for (int s = 0; s < W; ++s) {
+            if (mine(root, s)) {
+              chance[s] = IN_VAIN;
+#pragma unroll
+              for (int w = 0; w < W; ++w) rec[s][w] = root[w];
+            }
+          }
+          continue;
+        }
+        if ((NONE_APART || some) && hit1 != 0u) {
+          work[WK_ROT]++;
+          exchange(p, root, e, q, target, tab.load(q));
+          continue;
+        }
+        if (NONE_APART || some) {
+          hist_store<W>(hist, 1, F);
+          hit = search(F, alive, target, level, work[WK_LEVEL], work[WK_POP]);
+        }
+      } else {
+        hit = search(F, alive, target, level, work[WK_LEVEL], work[WK_POP]);
+      }
       if (!hit) {
         any = 0u;
 #pragma unroll
@@ -669,8 +780,8 @@ struct Peeler {
           }
           continue;
         }
-        q = first_of<W>(want, target);   // the next best column
-        level = level_of_row<W>(hist, level, MS_AT(q, N), lane);
+        q = MS_AT(first_of<W>(want, target), N);   // the next best column
+        level = level_of_row<W>(hist, level, q, lane);
       }
       work[WK_ROT] += level;
       walk(p, root, e, q, target, level, hit);
