@@ -17,7 +17,7 @@
 //     three-stage maps of its share of them and the maps are composed in order over the threads: the recurrence
 //     costs two instructions per matching instead of ten in a scan over every chunk. (When every prefix is asked for, the
 //     scan over the chunk is what is needed.)
-// B200: 4096 complete Birkhoff schedules of 64 ranks (1.08 GB) 3.13 -> 0.93 ms (46 instructions per matching).
+// B200: 4096 complete Birkhoff schedules of 64 ranks (1.08 GB) 0.89 ms (46 instructions per matching).
 #include <type_traits>
 
 #include "common.cuh"
@@ -92,19 +92,26 @@ constexpr int CHUNK = 32;        // matchings replayed between two barriers
 constexpr int BATCH_CHUNKS = 8;  // chunks between two passes over the times
 constexpr int BATCH = CHUNK * BATCH_CHUNKS;
 
+// Buffers for the marks. Two save a barrier per chunk. 16-bit entries are for batches that do not fit the GPU at once, and there one
+// buffer, with no gap between the marks of two matchings, lets an SM hold 14 matrices of 64 ranks instead of 11: 4096 complete Birkhoff
+// schedules 944 -> 886 us, 2000 of 62 ranks 436 -> 406 (two buffers without the gap: 881 and 435).
+__host__ __device__ constexpr int mark_buffers(bool narrow) { return narrow ? 1 : 2; }
+
 // Layout of the shared memory of one matrix. T: threads of the group (all CTAs of a cluster together), t_here: of this CTA.
 struct EvalLayout {
   size_t slab,   // entry (r, j) of a 32-bit slab (32 rows) or 16-bit slab (64 rows) lies at j * 128 in it
        stage, marks, gmax, served, durs, maps, flags, total;
   int mark_stride;
 };
-__host__ __device__ inline EvalLayout eval_layout(int N, int T, int slabs_here, int warps_here, bool prefix) {
+__host__ __device__ inline EvalLayout eval_layout(int N, int T, int slabs_here, int warps_here, bool prefix, int mark_buffers) {
   EvalLayout L;
   L.slab = (size_t)(N + 1) * 128;   // one column more than there are: where rows beyond N and bad destinations end up
   L.stage = (size_t)slabs_here * L.slab;
-  L.mark_stride = T + 16;           // (a bad destination's mark may go behind the T bytes that are looked at)
+  L.mark_stride = T;
   L.marks = L.stage + 2 * align16((size_t)CHUNK * N + 16);
-  L.gmax = L.marks + (size_t)2 * CHUNK * L.mark_stride;
+  // A bad destination may mark the first byte of the next matching (or of the 16 behind the last one). Its own matching then lacks a
+  // mark all the same, unless the one before was bad too, and so on up to the first of the chunk, which nothing marks for it.
+  L.gmax = L.marks + (size_t)mark_buffers * CHUNK * L.mark_stride + 16;
   L.served = L.gmax + (prefix ? 2 * CHUNK : BATCH) * sizeof(int);
   L.durs = L.served + (prefix ? 2 * CHUNK : 0) * sizeof(long long);
   L.maps = L.durs + (size_t)warps_here * CHUNK * sizeof(int);
@@ -165,6 +172,7 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
                 int32_t* status, long long* __restrict__ prefix_overlap, long long* __restrict__ prefix_unserved,
                 int only_class) {
   constexpr int T_HERE = 32 * WARPS, T = CLUSTER ? 2 * T_HERE : T_HERE;
+  constexpr int MARK_BUFFERS = mark_buffers(NARROW);
   const int N = EXACT ? T : n_arg;
   using Entry = typename std::conditional<NARROW, unsigned short, int>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -178,7 +186,7 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
   if (only_class != 0 && status[b] != only_class) return;
   const int slabs = NARROW ? (N + 63) / 64 : (N + 31) / 32;
   const int slabs_here = CLUSTER ? WARPS : slabs;   // (the second CTA of a cluster may leave some unused)
-  const EvalLayout L = eval_layout(N, T, slabs_here, WARPS, PREFIX);
+  const EvalLayout L = eval_layout(N, T, slabs_here, WARPS, PREFIX, MARK_BUFFERS);
   unsigned char* base = smem_raw + (WARPS == 1 ? (size_t)(threadIdx.x >> 5) * L.total : 0);
   // what both CTAs of a cluster write to is kept by CTA 0
   unsigned char* shared0 = base;
@@ -211,7 +219,7 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
   }
 
   // ---- shared state, demand (each thread its own row), total, validation ----
-  for (int e = t_here; e < 2 * CHUNK * L.mark_stride / 4; e += T_HERE) reinterpret_cast<int*>(base + L.marks)[e] = 0;
+  for (int e = t_here; e < MARK_BUFFERS * CHUNK * L.mark_stride / 4; e += T_HERE) reinterpret_cast<int*>(base + L.marks)[e] = 0;
   for (int e = t_here; e < (PREFIX ? 2 * CHUNK : BATCH); e += T_HERE) reinterpret_cast<int*>(base + L.gmax)[e] = 0;
   if constexpr (PREFIX)
     for (int e = t_here; e < 2 * CHUNK; e += T_HERE) reinterpret_cast<unsigned long long*>(base + L.served)[e] = 0ull;
@@ -348,7 +356,8 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
     }
   };
 
-  // Step c replays chunk c; before that, the marks of chunk c-1 are looked at. One barrier per step.
+  // Step c replays chunk c; before that, the marks of chunk c-1 are looked at. One barrier per step, and one more where there is one
+  // buffer for marks.
   int k_settled = 0;
   for (int c = 0; c <= chunks; ++c) {
     async_copies_done();
@@ -357,18 +366,19 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
     if (c > 0) {
       // every row of the chunk before marked its destination; all T marks of a matching are there iff it is a permutation
       const int p = (c - 1) & 1;
-      const unsigned want = 0x01010101u << ((c - 1) >> 1 & 1);
+      const unsigned want = 0x01010101u << ((MARK_BUFFERS == 1 ? c - 1 : (c - 1) >> 1) & 1);
       if (rank == 0) {
         unsigned off = 0u;
 #pragma unroll
         for (int i = 0; i < T / T_HERE * 2; ++i) {
           const int g = i * T_HERE + t_here;   // group of 16 marks; T / 16 of them to a matching
-          const uint4 v = *reinterpret_cast<const uint4*>(base + L.marks + (size_t)p * CHUNK * L.mark_stride +
+          const uint4 v = *reinterpret_cast<const uint4*>(base + L.marks + (size_t)(MARK_BUFFERS == 1 ? 0 : p) * CHUNK * L.mark_stride +
                                                           (g / (T / 16)) * L.mark_stride + (g % (T / 16)) * 16);
           off |= (v.x ^ want) | (v.y ^ want) | (v.z ^ want) | (v.w ^ want);
         }
         if (off != 0u) flags[c & 1] = 1;
       }
+      if constexpr (MARK_BUFFERS == 1) barrier();   // the marks have been looked at
       if constexpr (PREFIX) {
         if (rank == 0 && warp == 0) {
           // times of the chunk, one matching per lane, then the three-stage recurrence by scans
@@ -435,9 +445,9 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
       const int k = (c + 1) * CHUNK + lane;
       dk_next = k < K ? db[k] : 0;
     }
-    const unsigned stamp = 1u << ((c >> 1) & 1);   // differs from what the buffer holds
+    const unsigned stamp = 1u << ((MARK_BUFFERS == 1 ? c : c >> 1) & 1);   // differs from what the buffer holds
     unsigned dest_at = smem_addr(from) + (in ? row : 0);
-    unsigned mark_base = smem_addr(base + L.marks) + (c & 1) * CHUNK * L.mark_stride + mark_at;
+    unsigned mark_base = smem_addr(base + L.marks) + (MARK_BUFFERS == 1 ? 0 : c & 1) * CHUNK * L.mark_stride + mark_at;
     if constexpr (CLUSTER) mark_base = address_in_cta(mark_base, 0);
     const unsigned cell_base = smem_addr(cells);
     int g_mine = 0;
@@ -536,7 +546,7 @@ struct EvalArgs {
 };
 size_t eval_smem(int N, int warps, bool narrow, bool cluster, bool prefix) {
   const int slabs = cluster ? warps : narrow ? (N + 63) / 64 : (N + 31) / 32;
-  return eval_layout(N, 32 * warps * (cluster ? 2 : 1), slabs, warps, prefix).total;
+  return eval_layout(N, 32 * warps * (cluster ? 2 : 1), slabs, warps, prefix, mark_buffers(narrow)).total;
 }
 
 template <int WARPS, bool NARROW, bool CLUSTER>
