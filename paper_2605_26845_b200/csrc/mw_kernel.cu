@@ -518,8 +518,9 @@ __global__ void __launch_bounds__(128) mw_kernel(int B, int N, const int32_t* __
       if (!ok) { st_code = MOESCHED_ST_INTERNAL; break; }
       int highest[W];
       tight_graph<W, STORE>(R, N, lane, sh, v, pl.tab, highest);
-      pl.adopt(highest);
-      pl.canonicalise(0u, work);
+      unsigned left[W];
+      pl.adopt(highest, left);
+      pl.canonicalise(0u, left, work);
       // serve: the heaviest matched pair sets the duration; matched entries are sent whole
       int dmax = 0, served = 0;
 #pragma unroll
