@@ -35,11 +35,10 @@ struct AssignShared {
   int* urow;         // [row] row dual
   unsigned* claim;   // [row or column]
   short* x;          // [row] column
-  short* y;          // [column] row
   unsigned* pred;    // [column] row from which the running search reached it, and that row's column << 16
 };
 __host__ __device__ inline size_t assign_smem_bytes(int N) {
-  return 3 * align16((size_t)N * 4) + 2 * align16((size_t)N * 2);
+  return 3 * align16((size_t)N * 4) + align16((size_t)N * 2);
 }
 // With eight words it lies in the Peeler's search levels: the assignment is done with once the tight edges are in the table,
 // before the first search, and the levels take 32 bytes a rank, so that a matrix of 232 ranks still fits as int32.
@@ -47,13 +46,12 @@ __host__ __device__ inline size_t state_smem_bytes(int N, int W) {
   return peel_smem_bytes(N, W) + (W == 8 ? 0 : assign_smem_bytes(N));
 }
 __device__ __forceinline__ AssignShared assign_shared(unsigned char* p, int N) {
-  const size_t words = align16((size_t)N * 4), halves = align16((size_t)N * 2);
+  const size_t words = align16((size_t)N * 4);
   AssignShared a;
   a.urow = reinterpret_cast<int*>(p);
   a.claim = reinterpret_cast<unsigned*>(p + words);
   a.pred = reinterpret_cast<unsigned*>(p + 2 * words);
   a.x = reinterpret_cast<short*>(p + 3 * words);
-  a.y = reinterpret_cast<short*>(p + 3 * words + halves);
   return a;
 }
 
@@ -96,7 +94,7 @@ __device__ __forceinline__ void nearest(const int (&d)[W], const unsigned (&tag)
 //      21 rows left, 161 instead of 225 column scans per matching.)
 //   3. Rows left over are inserted one by one by a shortest-path search that settles one column per scan, free columns
 //      first among equals, and moves the duals of the settled columns.
-// Distances lie within [-2 C, 3 C]. On return sh.x, sh.y and sh.urow hold the assignment and the row duals. False if a
+// Distances lie within [-2 C, 3 C]. On return sh.x and sh.urow hold the assignment and the row duals. False if a
 // search ran out of columns (an inconsistency).
 template <int W, int STORE, bool WIDE>
 __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N, int lane, const AssignShared& sh,
@@ -182,10 +180,7 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
 #pragma unroll
   for (int s = 0; s < W; ++s) {
     if (in[s]) {
-      if (owner[s] != NONE) {
-        tag[s] = TAG_MATCHED | owner[s];
-        sh.y[s * 32 + lane] = (short)owner[s];
-      }
+      if (owner[s] != NONE) tag[s] = TAG_MATCHED | owner[s];
       const unsigned rt = (row_free[s] ? 0u : TAG_MATCHED) | (unsigned)(s * 32 + lane);
       sh.claim[s * 32 + lane] = WIDE ? rt : packed(-u[s], rt);
     }
@@ -243,7 +238,6 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
     for (int s = 0; s < W; ++s) {
       if (asks[s] && sh.claim[by[s]] == (unsigned)(s * 32 + lane)) {
         tag[s] = TAG_MATCHED | by[s];
-        sh.y[s * 32 + lane] = (short)by[s];
         sh.x[by[s]] = (short)(s * 32 + lane);
       }
       if (in[s] && sh.claim[s * 32 + lane] != NONE) row_free[s] = false;
@@ -370,33 +364,42 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
         }
       }
     }
+    int j = MS_AT((int)who, N);
+    // (Loads first, stores when they have come back, and the next step of the path is on its way before it is known whether there is
+    // one: an augmentation costs 400 instead of 700 cycles at N = 64. One plan of 16 matchings 357 -> 323 us, 1024 x 128 ranks 17.9 ->
+    // 16.2 ms, 256 x 256 ranks 65.4 -> 63.5 ms. The flip names the rows of its columns itself: 323 -> 319 us, 16.2 -> 16.0, 63.5 -> 62.6;
+    // only entries beyond 23 bits lose, 60 x 72 ranks 2.16 -> 2.25 ms.)
+    int at[W], ud[W];
+#pragma unroll
+    for (int s = 0; s < W; ++s) {
+      at[s] = in[s] ? (int)sh.x[MS_AT(pred[s], N)] : 0;
+      ud[s] = in[s] ? sh.urow[tag[s] & 0xffu] : 0;   // (of no interest for a free column)
+    }
 #pragma unroll
     for (int s = 0; s < W; ++s)
-      if (in[s]) sh.pred[s * 32 + lane] = (unsigned)pred[s] | (unsigned)(pred[s] == f ? 0 : sh.x[MS_AT(pred[s], N)]) << 16;
+      if (in[s]) sh.pred[s * 32 + lane] = (unsigned)pred[s] | (unsigned)(pred[s] == f ? 0 : at[s]) << 16;
     __syncwarp();   // (also: the scans have read the row duals)
+    unsigned back = sh.pred[j];
     // settled columns move their dual so that the shortest-path tree stays tight, and their rows' duals with them
 #pragma unroll
     for (int s = 0; s < W; ++s) {
       if (in[s] && closed[s] != 0u) {
         v[s] += settled_at[s] - mu;
-        sh.urow[tag[s] & 0xffu] += mu - settled_at[s];
+        sh.urow[tag[s] & 0xffu] = ud[s] + mu - settled_at[s];
       }
     }
     sh.urow[f] = mu;   // every lane
     // flip the path back to row f (every lane makes every update)
-    int j = MS_AT((int)who, N);
     for (int it = 0; it <= N; ++it) {
-      const unsigned back = sh.pred[j];
-      const int i = MS_AT((int)(back & 0xffffu), N);
-      sh.y[j] = (short)i;
+      const int i = MS_AT((int)(back & 0xffffu), N), before = MS_AT((int)(back >> 16), N);
+      back = sh.pred[before];
       sh.x[i] = (short)j;
+#pragma unroll
+      for (int s = 0; s < W; ++s) tag[s] = j == s * 32 + lane ? TAG_MATCHED | (unsigned)i : tag[s];
       if (i == f) break;
-      j = MS_AT((int)(back >> 16), N);
+      j = before;
     }
     __syncwarp();
-#pragma unroll
-    for (int s = 0; s < W; ++s)
-      if (in[s] && (tag[s] >= TAG_MATCHED || tag[s] == who)) tag[s] = TAG_MATCHED | (unsigned)sh.y[s * 32 + lane];
   }
   return true;
 }
