@@ -7,8 +7,8 @@ import sys
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
-SOURCES = ["api.cu", "mw_kernel.cu", "bvn_kernel.cu", "bvn_real_kernel.cu", "eval_kernel.cu", "order_kernel.cu", "bvn_static.cu", "probe.cu", "a2a_kernel.cu", "sinkhorn_kernel.cu"]
-HEADERS = [os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "peel.cuh"), os.path.join(CSRC, "schedule_read.h"), os.path.join(HERE, "..", "include", "moesched.h")]
+SOURCES = ["api.cu", "mw_kernel.cu", "bvn_kernel.cu", "bvn_small.cu", "bvn_real_kernel.cu", "eval_kernel.cu", "order_kernel.cu", "bvn_static.cu", "probe.cu", "a2a_kernel.cu", "sinkhorn_kernel.cu"]
+HEADERS = [os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "peel.cuh"), os.path.join(CSRC, "small.cuh"), os.path.join(CSRC, "schedule_read.h"), os.path.join(HERE, "..", "include", "moesched.h")]
 LIB = os.path.join(HERE, "libmoesched.so")
 LIB_CHECKED = os.path.join(HERE, "libmoesched_checked.so")   # the same sources with -DMOESCHED_CHECKED
 

@@ -15,6 +15,7 @@
 // matchings, 20.7 -> 28.1, 25.2, 29.3 ms; three of 100 ranks 39.9 -> 57 ms with two. Every warp has to repeat the arithmetic
 // on whole sets, and a barrier per vote costs more than the divided tests save.)
 #include "peel.cuh"
+#include "small.cuh"
 
 namespace moesched {
 
@@ -203,6 +204,8 @@ __global__ void __launch_bounds__(128, W <= 2 ? 7 : 0) bvn_kernel(int B, int N, 
 
 cudaError_t run_bvn(int B, int N, const int32_t* demand, int k_max, uint8_t* perm, int32_t* coef, int32_t* count,
                     int32_t* aug, int32_t* scratch, int32_t* status, long long* work, cudaStream_t stream) {
+  // (Work counters count searches, of which the kernel for few ranks has none: with them it is this kernel for any N.)
+  if (N <= SMALL_MAX_N && work == nullptr) return run_bvn_small(B, N, demand, k_max, perm, coef, count, aug, status, stream);
   Geometry ge = plan_geometry(N);
 #define MOESCHED_GO(C, M)                                                                                     \
   do {                                                                                                        \

@@ -177,3 +177,25 @@ def test_decomposers_in_batches_that_are_not_resident(N):
         kk = (np.arange(K)[None, :] < r["count"][:, None])[which]
         assert (g.perm.cpu().numpy()[kk] == r["perm"][which][kk]).all()
         assert (g.dur.cpu().numpy()[kk] == r[value][which][kk]).all()
+
+
+@pytest.mark.parametrize("N", range(1, 13))
+@pytest.mark.parametrize("kind", [dict(high=9000), dict(kind="ties"), dict(high=5, zero_frac=0.6)])
+def test_birkhoff_decomposition_of_few_ranks(N, kind):
+    """Up to ten ranks the matchings are read off bitmaps over all sets of columns, above they are searched for; one matrix per CTA
+    and four, entries up to the largest sums, a matrix that is refused, and a budget that runs out."""
+    few = 40
+    D = random_matrices(few, N, seed=31 * N, **kind)
+    D[0] = 0
+    D[1] = 7
+    D[2] *= (2**31 - 1) // max(1, int(max(D[2].sum(0).max(), D[2].sum(1).max())))
+    D[3, N - 1, 0] = -1
+    for B in (few, 16 * torch.cuda.get_device_properties(0).multi_processor_count + 3):
+        which = np.arange(B) % few
+        for K in (bvn_capacity(N), max(1, N // 2)):
+            g, r = ms.bvn_decompose(dev(D[which]), K, want_aug=True), oracle.bvn_decompose(D, K, threads=8)
+            assert (g.status.cpu().numpy() == r["status"][which]).all() and (g.count.cpu().numpy() == r["count"][which]).all()
+            kk = (np.arange(K)[None, :] < r["count"][:, None])[which]
+            assert (g.perm.cpu().numpy()[kk] == r["perm"][which][kk]).all()
+            assert (g.dur.cpu().numpy()[kk] == r["coef"][which][kk]).all()
+            assert (g.extra.cpu().numpy()[which != 3] == r["aug"][which][which != 3]).all()
