@@ -116,7 +116,9 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
     if (in[s]) sh.claim[s * 32 + lane] = NONE;
   }
   // ---- 1. rows name columns, several at a time; lane l keeps what rows l, l + 32, ... found ----
-  constexpr int ROWS = W <= 2 ? 8 : W <= 4 ? 4 : 2;
+  // (Eight instead of four with three and four words: 300 x 96 ranks 3.27 -> 3.23 ms, 60 x 72 ranks 1.92 -> 1.87; four instead of two with
+  // more: 100 x 160 ranks 4.43 -> 4.57.)
+  constexpr int ROWS = W <= 4 ? 8 : 2;
   int u[W];
   unsigned named[W];
 #pragma unroll
@@ -187,12 +189,15 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
   }
   __syncwarp();
   // ---- 2. free columns raise their duals ----
+  // (Rows in flight: 16 instead of 4 with one-word keys of two words 317 -> 311 us for one plan of 16 matchings, 8 instead of as few as the
+  // compiler took for entries beyond 23 bits 2.18 -> 2.10 ms, 60 x 72 ranks.)
   {
     int best[W];
     unsigned by[W];
     if constexpr (WIDE) {
 #pragma unroll
       for (int s = 0; s < W; ++s) { best[s] = INF32; by[s] = NONE; }
+#pragma unroll 8
       for (int i = 0; i < N; ++i) {
         const auto* row = R.row(i);
         const int ui = sh.urow[i];
@@ -207,7 +212,7 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
       unsigned k[W];
 #pragma unroll
       for (int s = 0; s < W; ++s) k[s] = NONE;
-#pragma unroll 4
+#pragma unroll (W <= 2 ? 16 : 4)
       for (int i = 0; i < N; ++i) {
         const auto* row = R.row(i);
         const unsigned from = sh.claim[i];
