@@ -91,11 +91,11 @@ cudaError_t run_bvn_small(int B, int N, const int32_t* demand, int k_max, uint8_
                           int32_t* aug, int32_t* status, cudaStream_t stream) {
   Geometry ge = {};
   ge.wpb = B >= 16 * sm_count() ? 4 : 1;
+  static_assert(SMALL_MAX_N == 8, "a kernel for every size");
   switch (N) {
 #define MOESCHED_GO(n) \
   case n: return launch_warp_kernel(bvn_small_kernel<n>, ge, B, stream, B, demand, k_max, perm, coef, count, aug, status);
     MOESCHED_GO(1) MOESCHED_GO(2) MOESCHED_GO(3) MOESCHED_GO(4) MOESCHED_GO(5) MOESCHED_GO(6) MOESCHED_GO(7) MOESCHED_GO(8)
-    MOESCHED_GO(9) MOESCHED_GO(10)
 #undef MOESCHED_GO
     default: return cudaErrorInvalidValue;
   }

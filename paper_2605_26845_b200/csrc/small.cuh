@@ -3,8 +3,9 @@
 //
 // Which sets of columns the rows i .. N-1 can fill is a bitmap F_i over all 2^N sets. F_i follows from F_{i+1}: a set can be
 // filled if taking one of row i's columns out of it leaves one that can. Columns 0 .. 4 number a bit within a lane's word, columns
-// 5 .. 9 the lane, so that taking a column out is a shift by a constant or a shuffle, for all sets at once. The matching is then read off from row 0 up: a row takes the lowest of its columns
-// that leaves a set which the rows after it can fill; lane c looks at column c.
+// 5 and up the lane, so that taking a column out is a shift by a constant or a shuffle, for all sets at once. The matching is then
+// read off from row 0 up: a row takes the lowest of its columns that leaves a set which the rows after it can fill; lane c looks at
+// column c.
 // After edges have vanished, F has changed only for their rows and lower ones (the recomputation stops where it comes out as
 // before), rows below the lowest of them keep their columns if that can still be completed, and once the rows above the
 // highest of them see the columns left that they saw before, they keep theirs too. (N = 8: 1.8 bitmaps recomputed and 3.9 rows read
@@ -30,7 +31,7 @@ struct SmallMatcher {
   unsigned rows;              // rows adjacent to the lane's column
   int row;                    // the row matched to it
   unsigned left[N];           // columns that the rows before i leave
-  unsigned F[N + 1];   // F[0] is not used
+  unsigned F[N + 1];          // F[0] is not used
 
   // sets of the bitmap that have column c (c < 5)
   __host__ __device__ static constexpr unsigned having(int c) {
@@ -72,7 +73,7 @@ struct SmallMatcher {
   }
 
   // The matching of the graph without the edges that the rows `gone` have lost (all rows: without anything known before).
-  // False: there is no perfect matching any more (nothing is changed then).
+  // False: there is no perfect matching any more.
   __device__ __forceinline__ bool update(unsigned gone, bool first_time) {
     switch (31 - __clz(gone)) {
 #define MOESCHED_FILL(I)                                                            \
@@ -81,7 +82,7 @@ struct SmallMatcher {
       if (!fill(I, F[I + 1], F[I]) && (gone & ((1u << I) - 1u)) == 0u) break;       \
     }                                                                               \
     [[fallthrough]];
-      MOESCHED_FILL(9) MOESCHED_FILL(8) MOESCHED_FILL(7) MOESCHED_FILL(6)
+      MOESCHED_FILL(7) MOESCHED_FILL(6)
       MOESCHED_FILL(5) MOESCHED_FILL(4) MOESCHED_FILL(3) MOESCHED_FILL(2) MOESCHED_FILL(1)
 #undef MOESCHED_FILL
       default: break;
@@ -102,7 +103,7 @@ struct SmallMatcher {
     }                                                                               \
     [[fallthrough]];
         MOESCHED_TAKE(0) MOESCHED_TAKE(1) MOESCHED_TAKE(2) MOESCHED_TAKE(3) MOESCHED_TAKE(4) MOESCHED_TAKE(5)
-        MOESCHED_TAKE(6) MOESCHED_TAKE(7) MOESCHED_TAKE(8) MOESCHED_TAKE(9)
+        MOESCHED_TAKE(6) MOESCHED_TAKE(7)
 #undef MOESCHED_TAKE
         default: break;
       }
