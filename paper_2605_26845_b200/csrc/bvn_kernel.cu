@@ -7,8 +7,8 @@
 // What bounds it: a dependent chain of searches, about 1200 instructions per matching at N = 64. A full GPU (4096
 // matrices of 64 ranks) issues 2.5 instructions per cycle and SM, 70 % of the integer pipe; with one warp per scheduler
 // or less the time is the chain's latency (3.3 cycles per instruction). Against one row set per column with an
-// OR-reduction per word of every search level, B200: 4096 x N = 64 37.7 -> 25.7 ms, 1024 x N = 128 244 -> 120 ms,
-// 256 x N = 256 1152 -> 490 ms (that was with a CTA of eight warps per matrix), one N = 64 12.9 -> 7.2 ms.
+// OR-reduction per word of every search level, B200: 4096 x N = 64 37.7 -> 25.5 ms, 1024 x N = 128 244 -> 122 ms,
+// 256 x N = 256 1152 -> 493 ms (that was with a CTA of eight warps per matrix), one N = 64 12.9 -> 7.2 ms.
 // (Warps that slept while they were ahead of the others on their scheduler gained 4 % when a matching took 1700
 // instructions; now a full GPU takes the same time with and without it. A team of two, four or eight warps per matrix that
 // exchanges its votes through shared memory is slower at every size, however few the matrices: 148 of 256 ranks, 1200

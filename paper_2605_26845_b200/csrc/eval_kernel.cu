@@ -107,10 +107,10 @@ __host__ __device__ inline EvalLayout eval_layout(int N, int T, int slabs_here, 
   EvalLayout L;
   L.slab = (size_t)(N + 1) * 128;   // one column more than there are: where rows beyond N and bad destinations end up
   L.stage = (size_t)slabs_here * L.slab;
-  L.mark_stride = T;
+  L.mark_stride = T + (mark_buffers == 1 ? 0 : 16);   // (with two buffers the gap costs nothing: one matrix of 129 ranks 110 us without, 106 with)
   L.marks = L.stage + 2 * align16((size_t)CHUNK * N + 16);
-  // A bad destination may mark the first byte of the next matching (or of the 16 behind the last one). Its own matching then lacks a
-  // mark all the same, unless the one before was bad too, and so on up to the first of the chunk, which nothing marks for it.
+  // Without a gap a bad destination may mark the first byte of the next matching (or of the 16 behind the last one). Its own matching
+  // then lacks a mark all the same, unless the one before was bad too, and so on up to the first of the chunk, which nothing marks for it.
   L.gmax = L.marks + (size_t)mark_buffers * CHUNK * L.mark_stride + 16;
   L.served = L.gmax + (prefix ? 2 * CHUNK : BATCH) * sizeof(int);
   L.durs = L.served + (prefix ? 2 * CHUNK : 0) * sizeof(long long);
