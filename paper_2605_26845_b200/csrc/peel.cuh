@@ -291,6 +291,9 @@ struct Peeler {
     }
     __syncwarp();
     unsigned gone = 1u;
+    // (If no row may move, there is nothing to keep from being searched: a vote that pays with one word, where hardly a step of few
+    // ranks has such a row, 64 x 2 ranks 4.07 -> 3.79 us, two matchings; with three 994 -> 1035, 592 x 96.)
+    if constexpr (W == 1) gone = __ballot_sync(FULL, chance[0] > 0);
     while (gone != 0u) {   // every pass takes a row out of `left`
       gone = 0u;
 #pragma unroll
