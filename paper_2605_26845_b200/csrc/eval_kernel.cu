@@ -17,7 +17,7 @@
 //     three-stage maps of its share of them and the maps are composed in order over the threads: the recurrence
 //     costs two instructions per matching instead of ten in a scan over every chunk. (When every prefix is asked for, the
 //     scan over the chunk is what is needed.)
-// B200: 4096 complete Birkhoff schedules of 64 ranks (1.08 GB) 0.89 ms (46 instructions per matching).
+// B200: 4096 complete Birkhoff schedules of 64 ranks (1.08 GB) 0.88 ms (46 instructions per matching).
 #include <type_traits>
 
 #include "common.cuh"
@@ -92,26 +92,29 @@ constexpr int CHUNK = 32;        // matchings replayed between two barriers
 constexpr int BATCH_CHUNKS = 8;  // chunks between two passes over the times
 constexpr int BATCH = CHUNK * BATCH_CHUNKS;
 
-// Buffers for the marks. Two save a barrier per chunk. 16-bit entries are for batches that do not fit the GPU at once, and there one
-// buffer, with no gap between the marks of two matchings, lets an SM hold 14 matrices of 64 ranks instead of 11: 4096 complete Birkhoff
-// schedules 944 -> 886 us, 2000 of 62 ranks 436 -> 406 (two buffers without the gap: 881 and 435).
-__host__ __device__ constexpr int mark_buffers(bool narrow) { return narrow ? 1 : 2; }
-
 // Layout of the shared memory of one matrix. T: threads of the group (all CTAs of a cluster together), t_here: of this CTA.
 struct EvalLayout {
   size_t slab,   // entry (r, j) of a 32-bit slab (32 rows) or 16-bit slab (64 rows) lies at j * 128 in it
        stage, marks, gmax, served, durs, maps, flags, total;
   int mark_stride;
 };
-__host__ __device__ inline EvalLayout eval_layout(int N, int T, int slabs_here, int warps_here, bool prefix, int mark_buffers) {
+// A bad destination's mark may go behind the T bytes of a matching that are looked at. There is a gap for it, or it goes into the first
+// byte of the next matching (or the 16 behind the last one). The bad matching lacks a mark all the same, unless the one before was
+// bad too and marked it for it, and so on up to the first one in the buffers, which nothing else marks.
+// One buffer is there to be small. Two do without the gap for 64 ranks, where an SM then holds 12 matrices instead of 11: 4096 complete
+// Birkhoff schedules 944 -> 881 us, 1658 schedules of 1024 matchings 132 -> 108. (Elsewhere it is as often slower: 16 of 220 ranks 76 ->
+// 80, 300 of 129 106 -> 108.)
+__host__ __device__ constexpr int mark_gap(bool narrow, int mark_buffers, bool exact64) {
+  return narrow && (mark_buffers == 1 || exact64) ? 0 : 16;
+}
+__host__ __device__ inline EvalLayout eval_layout(int N, int T, int slabs_here, int warps_here, bool prefix, int mark_buffers,
+                                                  int mark_gap) {
   EvalLayout L;
   L.slab = (size_t)(N + 1) * 128;   // one column more than there are: where rows beyond N and bad destinations end up
   L.stage = (size_t)slabs_here * L.slab;
-  L.mark_stride = T + (mark_buffers == 1 ? 0 : 16);   // (with two buffers the gap costs nothing: one matrix of 129 ranks 110 us without, 106 with)
+  L.mark_stride = T + mark_gap;
   L.marks = L.stage + 2 * align16((size_t)CHUNK * N + 16);
-  // Without a gap a bad destination may mark the first byte of the next matching (or of the 16 behind the last one). Its own matching
-  // then lacks a mark all the same, unless the one before was bad too, and so on up to the first of the chunk, which nothing marks for it.
-  L.gmax = L.marks + (size_t)mark_buffers * CHUNK * L.mark_stride + 16;
+  L.gmax = L.marks + (size_t)mark_buffers * CHUNK * L.mark_stride + (mark_gap == 0 ? 16 : 0);
   L.served = L.gmax + (prefix ? 2 * CHUNK : BATCH) * sizeof(int);
   L.durs = L.served + (prefix ? 2 * CHUNK : 0) * sizeof(long long);
   L.maps = L.durs + (size_t)warps_here * CHUNK * sizeof(int);
@@ -163,7 +166,8 @@ __device__ __forceinline__ void async_copies_done() { asm volatile("cp.async.wai
 // JOBS (with PREFIX): the two per-matching arrays receive instead the job times of matching k in the
 // three-stage flow shop: reconfiguration + transfer time, and the time of its expert batch.
 // EXACT: N is the number of threads, so that every address of a chunk is a constant away from the thread's own.
-template <int WARPS, bool NARROW, bool CLUSTER, bool PREFIX, bool JOBS, bool EXACT>
+// MARK_BUFFERS: one, at the price of a barrier per chunk, or two (see launch_eval_as).
+template <int WARPS, bool NARROW, bool CLUSTER, bool PREFIX, bool JOBS, bool EXACT, int MARK_BUFFERS>
 __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
     eval_kernel(int B, int n_arg, const int32_t* __restrict__ demand, int k_stride, const uint8_t* __restrict__ perm,
                 const int32_t* __restrict__ dur, const int32_t* __restrict__ count, moesched_model_t model,
@@ -172,7 +176,6 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
                 int32_t* status, long long* __restrict__ prefix_overlap, long long* __restrict__ prefix_unserved,
                 int only_class) {
   constexpr int T_HERE = 32 * WARPS, T = CLUSTER ? 2 * T_HERE : T_HERE;
-  constexpr int MARK_BUFFERS = mark_buffers(NARROW);
   const int N = EXACT ? T : n_arg;
   using Entry = typename std::conditional<NARROW, unsigned short, int>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -186,7 +189,8 @@ __global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
   if (only_class != 0 && status[b] != only_class) return;
   const int slabs = NARROW ? (N + 63) / 64 : (N + 31) / 32;
   const int slabs_here = CLUSTER ? WARPS : slabs;   // (the second CTA of a cluster may leave some unused)
-  const EvalLayout L = eval_layout(N, T, slabs_here, WARPS, PREFIX, MARK_BUFFERS);
+  const EvalLayout L = eval_layout(N, T, slabs_here, WARPS, PREFIX, MARK_BUFFERS,
+                                   mark_gap(NARROW, MARK_BUFFERS, EXACT && T == 64));
   unsigned char* base = smem_raw + (WARPS == 1 ? (size_t)(threadIdx.x >> 5) * L.total : 0);
   // what both CTAs of a cluster write to is kept by CTA 0
   unsigned char* shared0 = base;
@@ -544,31 +548,52 @@ struct EvalArgs {
   long long *prefix_overlap, *prefix_unserved;
   cudaStream_t stream;
 };
-size_t eval_smem(int N, int warps, bool narrow, bool cluster, bool prefix) {
+size_t eval_smem(int N, int warps, bool narrow, bool cluster, bool prefix, int buffers) {
   const int slabs = cluster ? warps : narrow ? (N + 63) / 64 : (N + 31) / 32;
-  return eval_layout(N, 32 * warps * (cluster ? 2 : 1), slabs, warps, prefix, mark_buffers(narrow)).total;
+  const int T = 32 * warps * (cluster ? 2 : 1);
+  return eval_layout(N, T, slabs, warps, prefix, buffers, mark_gap(narrow, buffers, !prefix && N == 64 && T == 64)).total;
 }
 
-template <int WARPS, bool NARROW, bool CLUSTER>
-cudaError_t launch_eval_as(const EvalArgs& a, bool jobs, int only_class) {
+template <int WARPS, bool NARROW, bool CLUSTER, int BUFFERS>
+cudaError_t launch_eval_with(const EvalArgs& a, bool jobs, int only_class) {
   const bool prefix = a.prefix_overlap != nullptr;
   Geometry ge;
   ge.cluster = CLUSTER;
   ge.threads_per_cta = 32 * WARPS;
   ge.wpb = 1;                                    // matrices per CTA
   if (WARPS == 1) { ge.wpb = a.B >= 4 * sm_count() ? 4 : 1; ge.threads_per_cta = 32 * ge.wpb; }
-  ge.smem = eval_smem(a.N, WARPS, NARROW, CLUSTER, prefix) * ge.wpb;
+  ge.smem = eval_smem(a.N, WARPS, NARROW, CLUSTER, prefix, BUFFERS) * ge.wpb;
   const bool full = a.N == 32 * WARPS * (CLUSTER ? 2 : 1);
 #define MOESCHED_GO(P, J, F)                                                                                         \
-  return launch_warp_kernel(eval_kernel<WARPS, NARROW, CLUSTER, P, J, F>, ge, a.B, a.stream, a.B, a.N, a.demand,     \
-                            a.k_stride, a.perm, a.dur, a.count, a.model, a.by_gbps, a.overlap, a.serial, a.idle_ns,  \
-                            a.idle_tok, a.unserved, a.status, a.prefix_overlap, a.prefix_unserved, only_class)
+  return launch_warp_kernel(eval_kernel<WARPS, NARROW, CLUSTER, P, J, F, BUFFERS>, ge, a.B, a.stream, a.B, a.N,      \
+                            a.demand, a.k_stride, a.perm, a.dur, a.count, a.model, a.by_gbps, a.overlap, a.serial,   \
+                            a.idle_ns, a.idle_tok, a.unserved, a.status, a.prefix_overlap, a.prefix_unserved, only_class)
   if (prefix && jobs) MOESCHED_GO(true, true, false);
   if (prefix) MOESCHED_GO(true, false, false);
   if constexpr (!CLUSTER)
     if (full) MOESCHED_GO(false, false, true);
   MOESCHED_GO(false, false, false);
 #undef MOESCHED_GO
+}
+
+// One buffer for the marks leaves room for up to a third more matrices per SM, which is of use where the SMs then hold the whole batch
+// at once (B200, schedules of six matchings per rank: 600 x 112 ranks 86.0 -> 69.4 us, with prefix scores 126.6 -> 89.5; 300 x 140 111.7 ->
+// 95.1 and 161.5 -> 111.7). Otherwise it may as well leave a longer tail (550 x 129, 32 matchings, three at a time instead of two 27.0 ->
+// 33.8; 833 x 112, 28 matchings, 25.4 -> 27.6). Where an SM holds a single matrix either way, the prefix scores are faster with one (256
+// ranks 134.1 -> 130.5 us), the scores as a whole with two (86.4, 87.0). Only 16-bit entries come here: 32-bit ones are for
+// batches that are held at once.
+template <int WARPS, bool NARROW, bool CLUSTER>
+cudaError_t launch_eval_as(const EvalArgs& a, bool jobs, int only_class) {
+  if constexpr (NARROW) {
+    const bool prefix = a.prefix_overlap != nullptr;
+    auto held = [&](int buffers) {   // matrices per SM
+      return (int)((SMEM_LIMIT + 1024) / (eval_smem(a.N, WARPS, true, false, prefix, buffers) + 1024));
+    };
+    const int one = held(1), two = held(2);
+    const long long per_sm = (a.B + sm_count() - 1) / sm_count();
+    if (one == 1 ? prefix : per_sm <= one && per_sm > two) return launch_eval_with<WARPS, NARROW, CLUSTER, 1>(a, jobs, only_class);
+  }
+  return launch_eval_with<WARPS, NARROW, CLUSTER, 2>(a, jobs, only_class);
 }
 }  // namespace
 
@@ -580,7 +605,7 @@ cudaError_t run_eval(int B, int N, const int32_t* demand, int k_stride, const ui
                    idle_ns, idle_tok, unserved, status, prefix_overlap, prefix_unserved, stream};
   if (N <= 32) return launch_eval_as<1, false, false>(a, jobs, 0);
   const int warps = N <= 64 ? 2 : N <= 128 ? 4 : 8;
-  const size_t as_int32 = eval_smem(N, warps, false, false, prefix_overlap != nullptr);
+  const size_t as_int32 = eval_smem(N, warps, false, false, prefix_overlap != nullptr, 2);
   // As in the greedy path: 32-bit entries at once where the whole batch is resident that way, else 16-bit entries first and
   // then the matrices that do not fit them (over a 2-CTA cluster where one CTA cannot hold the matrix).
   int only_class = 0;

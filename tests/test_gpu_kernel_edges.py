@@ -199,3 +199,69 @@ def test_birkhoff_decomposition_of_few_ranks(N, kind):
             assert (g.perm.cpu().numpy()[kk] == r["perm"][which][kk]).all()
             assert (g.dur.cpu().numpy()[kk] == r["coef"][which][kk]).all()
             assert (g.extra.cpu().numpy()[which != 3] == r["aug"][which][which != 3]).all()
+
+
+def faulty_schedules(N, K, seed):
+    """Schedules of K matchings, all but the first and the last with something wrong in them: destinations that do not exist at the
+    edges of chunks of 32 and in a chunk that is not full, alone and in runs, and columns that only the matching before could mark."""
+    perm, dur = random_schedule(1, K, N, seed, 40)
+    none = [N] if N == 255 else [N, 255] if N < 255 else []
+
+    def without_column(p, k, c):                       # row that had column c: the one of another row
+        at = int(np.flatnonzero(p[k] == c)[0])
+        p[k, at] = p[k, (at + 1) % N]
+
+    out = [perm[0]]
+    for k in (0, 15, 31, 32, 63, 64, K - 1):
+        for bad in none:
+            p = perm[0].copy()
+            p[k, (7 * k) % N] = bad
+            out.append(p)
+        p = perm[0].copy()
+        without_column(p, k, 0)
+        out.append(p)
+    for first, last in ((0, 31), (30, 33), (62, K - 1)):
+        for bad in none:
+            p = perm[0].copy()
+            p[first:last + 1, N - 1] = bad             # every one spills into the next
+            out.append(p)
+            for k in range(first + 1, last + 1):       # ... whose only missing column is the first
+                p[k] = perm[0, k]
+                p[k, int(np.flatnonzero(p[k] == 0)[0])] = bad
+            out.append(p.copy())
+    for k in (10, 30, 31, 63):                         # one bad destination, then one column 0 missing
+        for bad in none:
+            p = perm[0].copy()
+            p[k, 3 % N] = bad
+            without_column(p, k + 1, 0)
+            out.append(p)
+    out.append(perm[0])
+    return np.stack(out), np.repeat(dur, len(out), axis=0)
+
+
+@pytest.mark.parametrize("N,B", [(33, 2100), (33, 2500), (62, 1500), (62, 1750), (64, 1500), (64, 1800), (65, 1100), (120, 600), (127, 500),
+                                 (128, 500), (129, 400), (192, 200), (200, 200), (220, 90), (255, 90), (256, 90), (32, 90), (64, 90),
+                                 (128, 90)])
+def test_scoring_of_faulty_schedules(N, B):
+    """Batches of 16-bit entries with one and two buffers for the marks, which may border on the next matching's, and a few of
+    32-bit entries; sound schedules stand beside the faulty ones."""
+    K = 70
+    perm, dur = faulty_schedules(N, K, seed=N)
+    F = len(perm)
+    perm[F - 1, 60:] = 0                               # what lies beyond the count is not looked at
+    count = np.full(F, K, np.int32)
+    count[F - 1] = 60
+    D = random_matrices(F, N, seed=3 * N, high=300)
+    which = np.arange(B) % F
+    which[:3] = 0, F - 1, 0
+    d, p, q, c = dev(D[which]), dev(perm[which]), dev(dur[which]), dev(count[which])
+    r = oracle.schedule_prefix_eval(D, perm, dur, count, PROFILED_MODEL, threads=8)
+    rs = oracle.schedule_eval(D, perm, dur, count, PROFILED_MODEL, threads=8)
+    assert (rs["status"] == np.r_[0, np.full(F - 2, ms.ST_BAD_INPUT), 0]).all()
+    for prefix in (False, True):
+        s = ms.schedule_eval(d, p, q, c, PROFILED_MODEL, prefix=prefix)
+        for name in ms.SCORE_FIELDS + ("status",):
+            assert (s[name].cpu().numpy() == rs[name][which]).all(), name
+        if prefix:
+            for name in ("prefix_overlap_ns", "prefix_unserved_tokens"):
+                assert (s[name].cpu().numpy() == r[name][which]).all(), name
