@@ -257,13 +257,18 @@ void prefer_shared_memory(Kernel kern) {
     (void)cudaGetLastError();
 }
 
+// Dynamic shared memory beyond 48 KB has to be permitted, kernel by kernel and for the whole process. What is permitted is always the
+// most there is, whatever this launch needs: a smaller figure would take it away from a launch of the same kernel on another
+// thread, between that thread's permission and its launch.
+template <typename Kernel>
+cudaError_t permit_shared_memory(Kernel kern, size_t smem) {
+  return smem > 48 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT) : cudaSuccess;
+}
+
 // Launch helper shared by the three kernels.
 template <typename Kernel, typename... Args>
 cudaError_t launch_warp_kernel(Kernel kern, const Geometry& ge, int B, cudaStream_t stream, Args... args) {
-  if (ge.smem > 48 * 1024) {   // up to that much needs no permission
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ge.smem);
-    if (e != cudaSuccess) return e;
-  }
+  if (cudaError_t e = permit_shared_memory(kern, ge.smem); e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(ge.threads_per_cta != 0 ? ge.threads_per_cta : 32 * ge.wpb);
   cfg.dynamicSmemBytes = ge.smem;

@@ -163,8 +163,7 @@ cudaError_t run_order(int B, int k_stride, const long long* leg, const long long
                       const int32_t* eval_status, int32_t* order, long long* best_ns, long long* emission_ns,
                       int32_t* rule, int32_t* status, cudaStream_t stream) {
   const size_t smem = order_smem_bytes(k_stride);
-  cudaError_t e = cudaFuncSetAttribute(order_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
+  if (cudaError_t e = permit_shared_memory(order_kernel, smem); e != cudaSuccess) return e;
   order_kernel<<<B, 32, smem, stream>>>(B, k_stride, leg, comp, count, eval_status, order, best_ns, emission_ns, rule,
                                         status);
   return cudaGetLastError();

@@ -330,10 +330,7 @@ cudaError_t run_sinkhorn(int B, int N, const int32_t* demand, int iters, double 
   const double scale = (double)(1 << scale_bits);
 #define MOESCHED_GO(KERNEL, GRID, THREADS, SMEM, ...)                                                               \
   do {                                                                                                              \
-    if ((SMEM) > 48 * 1024) {                                                                                       \
-      cudaError_t e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SMEM));       \
-      if (e != cudaSuccess) return e;                                                                               \
-    }                                                                                                               \
+    if (cudaError_t e = permit_shared_memory(KERNEL, SMEM); e != cudaSuccess) return e;                             \
     KERNEL<<<GRID, THREADS, SMEM, stream>>>(__VA_ARGS__ N, demand, iters, smooth, scale, scaled, fixed, stretch,    \
                                             row_err, status);                                                       \
     return cudaGetLastError();                                                                                      \
