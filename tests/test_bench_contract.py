@@ -2,8 +2,13 @@
 with the keys the benchmark contract names; needs no GPU."""
 import json
 import os
+import re
 import subprocess
 import sys
+
+import numpy as np
+
+import bench
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -28,3 +33,14 @@ def test_other_ranks_of_the_reference_arm_do_nothing():
     out = subprocess.run([sys.executable, os.path.join(ROOT, "bench.py"), "--impl", "reference", "--gpus", "2"],
                          capture_output=True, text=True, timeout=120, cwd=ROOT, env=env)
     assert out.returncode == 0 and out.stdout.strip() == ""
+
+
+def test_operations_are_those_of_the_kernel_that_is_timed():
+    """Few ranks are decomposed without searches, so what the searching kernel counts is not set against that kernel's time."""
+    work = np.ones((3, 10))
+    few, more = bench.operations(work, work, bench.FEW_RANKS), bench.operations(work, work, bench.FEW_RANKS + 1)
+    assert few["bvn_decompose"] is None and few["mw_decompose"] is not None and more["bvn_decompose"] is not None
+    assert bench.rate_of(None, 1.0) == (None, None) and bench.over(None, 2.0) is None
+    assert bench.rate_of((3e6, 6e6), 1.0) == (3.0, 6.0) and bench.over(3.0, 2.0) == 1.5
+    with open(os.path.join(ROOT, "paper_2605_26845_b200", "csrc", "small.cuh")) as f:
+        assert int(re.search(r"SMALL_MAX_N = (\d+)", f.read()).group(1)) == bench.FEW_RANKS
