@@ -189,6 +189,25 @@ def over(value, peak):
     return None if value is None else value / peak
 
 
+def kernels_in(graph):
+    """Kernel launches among the nodes of a captured graph (a CUgraph handle)."""
+    import ctypes
+    cuda = ctypes.CDLL("libcuda.so.1")
+    n = ctypes.c_size_t(0)
+    if cuda.cuGraphGetNodes(ctypes.c_void_p(graph), None, ctypes.byref(n)) != 0:
+        raise RuntimeError("cuGraphGetNodes failed")
+    nodes = (ctypes.c_void_p * max(1, n.value))()
+    if cuda.cuGraphGetNodes(ctypes.c_void_p(graph), nodes, ctypes.byref(n)) != 0:
+        raise RuntimeError("cuGraphGetNodes failed")
+    kinds = []
+    for node in nodes[:n.value]:
+        kind = ctypes.c_int(-1)
+        if cuda.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) != 0:
+            raise RuntimeError("cuGraphNodeGetType failed")
+        kinds.append(kind.value)
+    return kinds.count(0)            # CU_GRAPH_NODE_TYPE_KERNEL
+
+
 def rank_demand(rank, B):
     """Every rank works on its own B matrices (weak scaling): same recipe, rank-specific seed."""
     return make_demand(CFG, B, seed=SEED + rank)
@@ -461,6 +480,12 @@ def main():
     total_ms, e2e_ms = max_over_ranks([total_ms, e2e_ms], dev, world)
 
     ok = bool((mw.status >= 0).all() and (bv.status == 0).all())
+    # launches of one step, counted in a capture of it (not replayed)
+    counted = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(counted):
+        path.run(d, DEFAULT_MODEL, overlap=not args.no_overlap)
+    launches = kernels_in(counted.raw_cuda_graph())
+    del counted
     # the kernels' work counters (for the algorithmic-operation count) come from one more, untimed pass:
     # the timed steps run the kernels without them
     wk = torch.zeros((2, B, ms.WORK_FIELDS), dtype=torch.int64, device=dev)
@@ -547,9 +572,9 @@ def main():
                     "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h, "steps": e2e_steps,
                     "how": "HostPipeline: upload, kernels and download on three streams, two slots",
                     "results_match_device_run": e2e_ok},
-            # per step: greedy, BvN and two scoring launches; from N = 48 up the greedy and scoring entry
-            # points each add a class pre-pass and a second (wide-class) launch
-            "gpu_launches": (4 if N < 48 else 10) * args.steps,
+            # per step: greedy, BvN and two scoring launches, and one more of the greedy and scoring ones where a batch is held in
+            # 16-bit entries (for the matrices that do not fit them)
+            "gpu_launches": launches * args.steps,
             "clocks": ck,
         }
         if rates_by_k:

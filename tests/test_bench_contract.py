@@ -1,5 +1,5 @@
 """The benchmark's reference arm (the CPU oracle on a bounded sample) prints one JSON line
-with the keys the benchmark contract names; needs no GPU."""
+with the keys the benchmark contract names; what is computed of the counters, and the count of launches."""
 import json
 import os
 import re
@@ -7,6 +7,7 @@ import subprocess
 import sys
 
 import numpy as np
+import pytest
 
 import bench
 
@@ -44,3 +45,20 @@ def test_operations_are_those_of_the_kernel_that_is_timed():
     assert bench.rate_of((3e6, 6e6), 1.0) == (3.0, 6.0) and bench.over(3.0, 2.0) == 1.5
     with open(os.path.join(ROOT, "paper_2605_26845_b200", "csrc", "small.cuh")) as f:
         assert int(re.search(r"SMALL_MAX_N = (\d+)", f.read()).group(1)) == bench.FEW_RANKS
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("N,B,launches", [(8, 3, 4), (64, 100, 4), (64, 1300, 7)])
+def test_launches_are_counted_in_a_capture(N, B, launches):
+    """Greedy, Birkhoff and two scorings; in a batch too large for 32-bit entries the first and the last two launch twice."""
+    import torch
+
+    import paper_2605_26845_b200 as ms
+    d = torch.ones((B, N, N), dtype=torch.int32, device="cuda")
+    path = ms.Path(B, N, 2, 2)
+    path.run(d)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        path.run(d)
+    assert bench.kernels_in(graph.raw_cuda_graph()) == launches
