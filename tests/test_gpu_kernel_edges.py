@@ -182,7 +182,7 @@ def test_decomposers_in_batches_that_are_not_resident(N):
 @pytest.mark.parametrize("N", range(1, 13))
 @pytest.mark.parametrize("kind", [dict(high=9000), dict(kind="ties"), dict(high=5, zero_frac=0.6)])
 def test_birkhoff_decomposition_of_few_ranks(N, kind):
-    """Up to ten ranks the matchings are read off bitmaps over all sets of columns, above they are searched for; one matrix per CTA
+    """Up to eight ranks the matchings are read off bitmaps over all sets of columns, above they are searched for; one matrix per CTA
     and four, entries up to the largest sums, a matrix that is refused, and a budget that runs out."""
     few = 40
     D = random_matrices(few, N, seed=31 * N, **kind)

@@ -36,6 +36,43 @@ def test_lanes_that_run_apart_find_the_same_schedule(program, N, pieces, k_max):
     assert (coef == ref["coef"][0, :count]).all() and (perm == ref["perm"][0, :count]).all()
 
 
+def decompose(program, A, k_max, *how):
+    N = A.shape[0]
+    done = subprocess.run([program, *how], input=np.array([N, k_max], np.int32).tobytes() + A.tobytes(), capture_output=True,
+                          timeout=120, check=True)
+    count = int(np.frombuffer(done.stdout[:4], np.int32)[0])
+    return (count, np.frombuffer(done.stdout[4:4 + 4 * count], np.int32),
+            np.frombuffer(done.stdout[4 + 4 * count:], np.uint8).reshape(count, N))
+
+
+@pytest.mark.parametrize("N,pieces,k_max", [(100, 30, 3), (128, 16, 3), (140, 12, 2), (170, 10, 2), (200, 8, 2)])
+def test_every_number_of_words(program, N, pieces, k_max):
+    """Four to seven words: the first level apart, chances counted or not, rows read back from entries of another layout."""
+    rng = np.random.default_rng(N)
+    A = np.zeros((N, N), np.int32)
+    for _ in range(pieces):
+        A[np.arange(N), rng.permutation(N)] += rng.integers(1, 20)
+    count, coef, perm = decompose(program, A, k_max)
+    ref = oracle.bvn_decompose(A[None], k_max)
+    assert count == ref["count"][0]
+    assert (coef == ref["coef"][0, :count]).all() and (perm == ref["perm"][0, :count]).all()
+
+
+@pytest.mark.parametrize("N", range(1, 9))
+@pytest.mark.parametrize("dense", [False, True])
+def test_bitmaps_of_few_ranks(program, N, dense):
+    rng = np.random.default_rng(10 * N + dense)
+    for _ in range(2):
+        A = np.zeros((N, N), np.int32)
+        for _ in range(30 if dense else N):
+            A[np.arange(N), rng.permutation(N)] += rng.integers(1, 4 if dense else 200)
+        k_max = N * N + 1
+        count, coef, perm = decompose(program, A, k_max, "small")
+        ref = oracle.bvn_decompose(A[None], k_max)
+        assert count == ref["count"][0]
+        assert (coef == ref["coef"][0, :count]).all() and (perm == ref["perm"][0, :count]).all()
+
+
 def smallest_matching(edges, column_of):
     """The lexicographically smallest perfect matching: row by row the lowest column that can be had without touching the rows
     before, by a search for a way to hand the row's own column on."""
