@@ -4,8 +4,8 @@
 // matched entry reached zero are re-matched and the lexicographically smallest perfect matching is restored
 // (Peeler in peel.cuh).
 //
-// What bounds it: a dependent chain of searches, about 1200 instructions per matching at N = 64. A full GPU (4096
-// matrices of 64 ranks) issues 2.5 instructions per cycle and SM, 70 % of the integer pipe; with one warp per scheduler
+// What bounds it: a dependent chain of searches, about 1100 instructions per matching at N = 64. A full GPU (4096
+// matrices of 64 ranks) issues 2.4 instructions per cycle and SM, 70 % of the integer pipe; with one warp per scheduler
 // or less the time is the chain's latency (3.3 cycles per instruction). Against one row set per column with an
 // OR-reduction per word of every search level, B200: 4096 x N = 64 37.7 -> 25.5 ms, 1024 x N = 128 244 -> 122 ms,
 // 256 x N = 256 1152 -> 493 ms (that was with a CTA of eight warps per matrix), one N = 64 12.9 -> 7.2 ms.
@@ -204,7 +204,8 @@ __global__ void __launch_bounds__(128, W <= 2 ? 7 : 0) bvn_kernel(int B, int N, 
 
 cudaError_t run_bvn(int B, int N, const int32_t* demand, int k_max, uint8_t* perm, int32_t* coef, int32_t* count,
                     int32_t* aug, int32_t* scratch, int32_t* status, long long* work, cudaStream_t stream) {
-  // (Work counters count searches, of which the kernel for few ranks has none: with them it is this kernel for any N.)
+  // Up to eight ranks bitmaps are faster than searches whatever the batch (small.cuh has both sides; at eight ranks and beyond 10000
+  // matrices they are even, 2 % behind at 40000). Work counters count searches, of which that kernel has none: with them it is this one.
   if (N <= SMALL_MAX_N && work == nullptr) return run_bvn_small(B, N, demand, k_max, perm, coef, count, aug, status, stream);
   Geometry ge = plan_geometry(N);
 #define MOESCHED_GO(C, M)                                                                                     \

@@ -189,8 +189,9 @@ __device__ __forceinline__ bool solve_assignment(const Residual<STORE>& R, int N
   }
   __syncwarp();
   // ---- 2. free columns raise their duals ----
-  // (Rows in flight: 16 instead of 4 with one-word keys of two words 317 -> 311 us for one plan of 16 matchings, 8 instead of as few as the
-  // compiler took for entries beyond 23 bits 2.18 -> 2.10 ms, 60 x 72 ranks.)
+  // (Rows in flight: 16 instead of 4 with one-word keys of two words 317 -> 311 us for one plan of 16 matchings, of one word 592 x 16 ranks
+  // 66.3 -> 63.7 us and 592 x 32 267 -> 256; below 16 ranks, where the rows go one by one then, 592 x 12 41.1 -> 42.2. 8 instead of as few as
+  // the compiler took for entries beyond 23 bits 2.18 -> 2.10 ms, 60 x 72 ranks.)
   {
     int best[W];
     unsigned by[W];

@@ -12,10 +12,10 @@
 // off per matching.)
 //
 // What bounds it: the chain of shuffle, shift and vote per row read off, 175 cycles, and of 270 cycles per bitmap, with the
-// branches between them. Against the searches of peel.cuh, 64 or 592 matrices, complete decompositions, B200: N = 5 23.6 -> 21.4 us,
-// N = 6 32.1 -> 30.1, N = 7 44.3 -> 38.8, N = 8 56.2 -> 50.4; 4096 of N = 6 62.8 -> 51.5. With eight ranks a single matrix (44.2 and
-// 47.4 us) and 40000 of them (745 and 760) come out the other way round, and from nine ranks on the instructions (4096 of N = 10
-// 169 and 207 us).
+// branches between them. Against the searches of peel.cuh, complete decompositions, back to back in a CUDA graph, B200, for 1, 592 and
+// 4096 matrices: N = 1 1.95 -> 1.24 us, 2.61 -> 1.93, 4.19 -> 2.39; N = 4 7.8 -> 6.3, 9.3 -> 6.6, 19.4 -> 13.5; N = 6 20.6 -> 18.6, 25.6 -> 20.3,
+// 49.4 -> 41.1; N = 8 39.1 -> 38.7, 43.4 -> 41.0, 96.9 -> 93.3. At eight ranks it ends there: 10000 matrices 198 and 199 us, 40000 727 and
+// 741; from nine ranks on the instructions (4096 of N = 10 169 and 207).
 #pragma once
 
 #include "common.cuh"
