@@ -4,17 +4,25 @@
 
 namespace moesched {
 
+// The matrix lies in shared memory, no more of it than the warps of the CTA need: with a fixed 4 KB a CTA, for one warp or for four, the
+// CTAs of a thousand matrices took a division of the SMs' memory beside which no greedy CTA could start, and a step of greedy
+// and Birkhoff became as long as one after the other (paths run one after another, 800 matrices of 8 ranks 91 us, now 45; by searches 51).
+// Up to three ranks it is in registers (1000 of 3 ranks 22.5 -> 18.6 us; with more, choosing a register costs more than the load:
+// decompositions of 592 matrices of 8 ranks 41 -> 50).
+template <int N>
+constexpr bool IN_REGISTERS = N <= 3;
+
 template <int N>
 __global__ void __launch_bounds__(128) bvn_small_kernel(int B, const int32_t* __restrict__ demand, int k_max,
                                                         uint8_t* __restrict__ perm, int32_t* __restrict__ coef,
                                                         int32_t* __restrict__ count, int32_t* __restrict__ aug,
                                                         int32_t* __restrict__ status) {
-  __shared__ int cells[4][N * 32];
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b = blockIdx.x * (blockDim.x >> 5) + warp;
   if (b >= B) return;
   const bool in = lane < N;
-  int* A = cells[warp] + lane;   // column `lane`, 32 apart
+  int* A = reinterpret_cast<int*>(smem_raw) + warp * (N * 32) + lane;   // column `lane`, 32 apart
 
   // ---- the matrix, row and column sums, validation: lane i owns row and column i ----
   const int32_t* D = demand + (size_t)b * N * N;
@@ -52,7 +60,7 @@ __global__ void __launch_bounds__(128) bvn_small_kernel(int B, const int32_t* __
       r_from = r_to;
       if (in && more > 0) v[r] += (int)more;
       if (v[r] > 0) rows |= 1u << r;
-      A[r * 32] = v[r];
+      if constexpr (!IN_REGISTERS<N>) A[r * 32] = v[r];
       if (aug != nullptr && in) aug[(size_t)b * N * N + r * N + lane] = v[r];
     }
 
@@ -66,10 +74,21 @@ __global__ void __launch_bounds__(128) bvn_small_kernel(int B, const int32_t* __
       if (!m.update(gone, k == 0)) { st_code = MOESCHED_ST_INTERNAL; break; }
       // coefficient = smallest matched entry; subtract it along the matching; what reaches zero leaves the graph
       int* cell = A + MS_AT(m.row, N) * 32;
-      int val = *cell;
+      int val = v[0];
+      if constexpr (IN_REGISTERS<N>) {
+#pragma unroll
+        for (int r = 1; r < N; ++r) val = m.row == r ? v[r] : val;
+      } else {
+        val = *cell;
+      }
       const int c = (int)__reduce_min_sync(FULL, in ? (unsigned)val : 0x7fffffffu);
       val -= c;
-      if (in) *cell = val;
+      if constexpr (IN_REGISTERS<N>) {
+#pragma unroll
+        for (int r = 0; r < N; ++r) v[r] = m.row == r ? val : v[r];
+      } else {
+        if (in) *cell = val;
+      }
       const unsigned lost = in && val == 0 ? 1u << m.row : 0u;
       m.rows &= ~lost;
       gone = __reduce_or_sync(FULL, lost);
@@ -94,7 +113,9 @@ cudaError_t run_bvn_small(int B, int N, const int32_t* demand, int k_max, uint8_
   static_assert(SMALL_MAX_N == 8, "a kernel for every size");
   switch (N) {
 #define MOESCHED_GO(n) \
-  case n: return launch_warp_kernel(bvn_small_kernel<n>, ge, B, stream, B, demand, k_max, perm, coef, count, aug, status);
+  case n:                                                                    \
+    if (!IN_REGISTERS<n>) ge.smem = (size_t)ge.wpb * n * 32 * sizeof(int);   \
+    return launch_warp_kernel(bvn_small_kernel<n>, ge, B, stream, B, demand, k_max, perm, coef, count, aug, status);
     MOESCHED_GO(1) MOESCHED_GO(2) MOESCHED_GO(3) MOESCHED_GO(4) MOESCHED_GO(5) MOESCHED_GO(6) MOESCHED_GO(7) MOESCHED_GO(8)
 #undef MOESCHED_GO
     default: return cudaErrorInvalidValue;

@@ -570,7 +570,7 @@ cudaError_t launch_eval_with(const EvalArgs& a, bool jobs, int only_class) {
                             a.idle_ns, a.idle_tok, a.unserved, a.status, a.prefix_overlap, a.prefix_unserved, only_class)
   if (prefix && jobs) MOESCHED_GO(true, true, false);
   if (prefix) MOESCHED_GO(true, false, false);
-  if constexpr (!CLUSTER)
+  if constexpr (!CLUSTER && (BUFFERS == 2 || WARPS == 2))   // (128 and 256 ranks never have one buffer here)
     if (full) MOESCHED_GO(false, false, true);
   MOESCHED_GO(false, false, false);
 #undef MOESCHED_GO

@@ -202,9 +202,9 @@ struct Peeler {
   static constexpr bool COUNTED = W <= 4;
   // A branch that all lanes take together costs about 20 cycles of the chain, so the ways out of a search lead straight to what comes
   // next instead of through a common test (one of N = 64 7.84 -> 7.47 ms, 4096 27.1 -> 25.9, 256 of N = 256 530 -> 514). Likewise:
-  // the first level, where 67 % of the searches of 16 ranks, 44 % of 64 and 31 % of 128 end, is taken apart and followed by the exchange (1024 of N = 16 271 -> 267 us, one of
-  // N = 64 7.47 -> 7.24 ms, 148 of N = 96 27.1 -> 26.4, 100 of N = 192 168.9 -> 165.3; 1024 of N = 128 123.7 -> 124.9; with eight words the
-  // code that this adds costs more: 514 -> 581);
+  // the first level, where 67 % of the searches of 16 ranks, 44 % of 64 and 31 % of 128 end, is taken apart and followed by the exchange
+  // (1024 of N = 16 271 -> 267 us, one of N = 64 7.47 -> 7.24 ms, 148 of N = 96 27.1 -> 26.4, 100 of N = 192 168.9 -> 165.3; 1024 of N = 128
+  // 123.7 -> 124.9; with eight words the code that this adds costs more: 514 -> 581);
   static constexpr bool FIRST_APART = W <= 6;
   // a first level without members has a way of its own (267 -> 261 us, 4096 of N = 64 26.0 -> 25.7 ms; 100 of N = 160 153.9 -> 158.3);
   static constexpr bool NONE_APART = W <= 2;
